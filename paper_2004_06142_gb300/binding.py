@@ -532,10 +532,13 @@ class DonofEnergy(torch.autograd.Function):
         E, lam, _ = builder.forward(h, C.contiguous(), gamma.contiguous(), pair_map)
         ctx.builder = builder
         ctx.mark_non_differentiable(lam)
+        ctx.set_materialize_grads(False)  # no nbf x nbf zeros for lambda's gradient
         return E.reshape(()), lam
 
     @staticmethod
     def backward(ctx, gE, glam):
+        if gE is None:  # E took no part in what was differentiated
+            return None, None, None, None, None
         Ebar = gE.reshape(1).to(torch.float64).contiguous()
         dC, dg = ctx.builder.backward(Ebar)
         return dC, dg, None, None, None
