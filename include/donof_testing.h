@@ -9,6 +9,7 @@
 #ifndef DONOF_TESTING_H
 #define DONOF_TESTING_H
 
+#include <stddef.h>
 #include <stdint.h>
 
 #ifdef __cplusplus
@@ -48,6 +49,15 @@ int donof_testing_tc_gemm_il8(const uint16_t* A_hi, const uint16_t* A_lo, const 
 int donof_testing_tc_gemm_ex(const uint16_t* A_hi, const uint16_t* A_lo, const uint16_t* B_hi,
                              const uint16_t* B_lo, float* D, int32_t M, int32_t N, int32_t K,
                              int32_t layout, int32_t pair, void* stream);
+
+/* C = A B in double by exact digit products on the tensor cores (the FP64 path's contraction):
+ * A(m, k) at A[m sAm + k sAk] with sAm = 1 or sAk = 1, B(k, n) at B[k ldb + n], C(m, n) at
+ * C[m ldc + n]; device pointers, 1 <= K <= 16384.  workspace: device, 256-byte aligned, at least
+ * 1024 + 4 (M + N) + 16 (N + 64) (K + 32) bytes; its first word receives the status of the
+ * bounded waits. */
+int donof_testing_digit_product(const double* A, int64_t sAm, int64_t sAk, const double* B,
+                                int64_t ldb, double* C, int64_t ldc, int32_t M, int32_t N,
+                                int32_t K, void* workspace, size_t workspace_bytes, void* stream);
 
 /* The bounded device wait of the tensor-core kernel, run out on purpose: one CTA whose two
  * roles wait on mbarriers that nothing completes, the first with a limit of limit_a_ns

@@ -15,7 +15,7 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libdonof.so")
 SOURCES = ["api.cu", "fp64.cu", "tc.cu", "noalloc.cu", "batch.cu", "orbital.cu", "occopt.cu", "mid.cu",
-           "nofmp2.cu", "eigh.cu"]
+           "nofmp2.cu", "eigh.cu", "digits.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -41,7 +41,8 @@ def _compile(src: str, extra: list[str]) -> str:
 def build(verbose_ptxas: bool = False, force: bool = False) -> str:
     os.makedirs(OBJ, exist_ok=True)
     srcs = [os.path.join(CSRC, s) for s in SOURCES]
-    deps = srcs + [os.path.join(CSRC, "common.cuh"),
+    deps = srcs + [os.path.join(CSRC, "common.cuh"), os.path.join(CSRC, "occ.cuh"),
+                   os.path.join(CSRC, "tcptx.cuh"),
                    os.path.join(os.path.dirname(HERE), "include", "donof.h")]
     if not force and os.path.exists(LIB):
         t = os.path.getmtime(LIB)

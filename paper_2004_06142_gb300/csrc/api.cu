@@ -18,6 +18,57 @@
 
 namespace donof {
 
+namespace {
+// Bytes per auxiliary slice of the FP64 path's buffers (make_layout): X, b, Y and an unpacked
+// slice on the FP64 pipe (digit 0), X, b, Y's stage images, w and X's exponents on digit products.
+size_t per_slice_fp64(const Dims& d, int digit) {
+  const size_t N = d.N, A = d.A;
+  const size_t common = N * A * 8 + A * A * 8 + (d.layout == DONOF_B_PACKED ? N * N * 8 : 0);
+  if (!digit) return common + A * A * 8;
+  const DigitShape t = digit_shape(d.A, 32);
+  return common + (size_t)round_up_int(d.A, 8) * t.ntiles * t.NT * 16 + A * 12;
+}
+
+void set_blocks(Dims& d, long long pb) {
+  d.pb = (int)pb;
+  d.nblk = (d.Q + d.pb - 1) / d.pb;
+}
+
+// The FP64 path takes its contractions as digit products wherever their buffers fit what the
+// path on the FP64 pipe asks for (small problems, up to 64 MiB: half as much again and 4 MiB),
+// in up to four times as many blocks of slices; callers that size or bound their memory by
+// donof_workspace_size or x_budget_bytes are served as before.
+void choose_digit(Dims& d, uint64_t x_budget) {
+  const size_t plain = make_layout(d).total;
+  d.ws_total = plain;
+  if (d.N > 16384) return;  // (the sums over k of group 0 in 32 bits)
+  constexpr size_t kSmall = (size_t)64 << 20;
+  size_t limit = plain;
+  if (plain <= kSmall) {
+    limit = plain + plain / 2 + ((size_t)4 << 20);
+    if (limit > kSmall) limit = kSmall;
+  }
+  const int nblk0 = d.nblk, pb0 = d.pb;
+  const size_t per = per_slice_fp64(d, 1);
+  d.digit = 1;
+  for (int nblk = nblk0; nblk <= 4 * nblk0; ++nblk) {
+    const long long pb = (d.Q + nblk - 1) / nblk;
+    if (x_budget > 0 && pb > 1 && (size_t)pb * per > x_budget) continue;
+    set_blocks(d, pb);
+    if ((long long)d.pb * d.N > (1ll << 30)) continue;  // row and unit indices in 32 bits
+    const size_t total = make_layout(d).total;
+    if (total <= limit) {
+      d.ws_total = total > plain ? total : plain;
+      return;
+    }
+    if (pb == 1) break;
+  }
+  d.digit = 0;
+  set_blocks(d, pb0);
+  d.ws_total = plain;
+}
+}  // namespace
+
 Dims make_dims(const donof_problem* p) {
   Dims d{};
   d.N = p->nbf;
@@ -34,8 +85,7 @@ Dims make_dims(const donof_problem* p) {
   d.precision = p->precision;
   size_t perP;
   if (d.precision == DONOF_FP64) {
-    perP = (size_t)d.N * d.A * 8 + 2 * (size_t)d.A * d.A * 8 +
-           (d.layout == DONOF_B_PACKED ? (size_t)d.N * d.N * 8 : 0);
+    perP = per_slice_fp64(d, 0);
   } else {
     perP = (size_t)d.Np * d.Ap * 4 + (size_t)d.Ap * d.Np * 4 + (size_t)d.Ap * d.Ap * (4 + 4 + 4) +
            (size_t)d.Ap * 4 + (size_t)d.A * 8;
@@ -47,8 +97,11 @@ Dims make_dims(const donof_problem* p) {
     if (pb > d.Q) pb = d.Q;
   }
   if (pb > 65535) pb = 65535;  // batch index of the double GEMMs lives in gridDim.z
-  d.pb = (int)pb;
-  d.nblk = (d.Q + d.pb - 1) / d.pb;
+  set_blocks(d, pb);
+  if (d.precision == DONOF_FP64) {
+    choose_digit(d, p->x_budget_bytes);
+    return d;
+  }
   // split-K of the G contraction: at most 64 slices per split, enough units (row tiles x
   // splits) for 2 waves over the 152 SMs but at least 32 slices per split (short splits
   // only add partials to reduce), and where a few more splits make the units a whole
@@ -106,18 +159,39 @@ Layout make_layout(const Dims& d) {
   L.Epart = take(4 * A * 8);
   {  // split-K partials of the FP64 products with N x A outputs (h C_act, lambda, G)
     size_t ks = 0;
-    if (d.precision == DONOF_FP64) {
+    if (d.precision == DONOF_FP64 && d.digit) {
+      // of G on digit products, and of J and K
+      const size_t g = (size_t)g_splits_digit((int)N, (int)A, (int)pb) * N * A;
+      const size_t jk = (size_t)jk_splits64((int)A, (int)pb) * A * (A + 1);
+      L.skp = take((g > jk ? g : jk) * 8);
+    } else if (d.precision == DONOF_FP64) {
       ks = (size_t)splitk_count((int)N, (int)A, (int)N);
       const size_t kg = (size_t)g_splits_fp64((int)N, (int)A, (int)pb);
       if (kg > ks) ks = kg;
     }
-    L.skp = take(ks > 1 ? ks * N * A * 8 : 0);
+    if (!d.digit) L.skp = take(ks > 1 ? ks * N * A * 8 : 0);
   }
   if (d.precision == DONOF_FP64) {
     L.X64 = take(pb * N * A * 8);
     L.b64 = take(pb * A * A * 8);
-    L.Y64 = take(pb * A * A * 8);
     L.Bun = d.layout == DONOF_B_PACKED ? take(pb * N * N * 8) : 0;
+    if (d.digit) {
+      L.eRow = take((size_t)d.Q * N * 4);
+      L.eH64 = take(N * 4);
+      L.eC64 = take(N * 4);      // eC64 .. exend: zeroed per build
+      L.eG64 = take(A * 4);
+      L.exq = take(pb * A * 4);  // exq .. exend: zeroed per block
+      L.exm = take(N * 4);
+      L.bmax = take(A * (A + 1) / 2 * 4);
+      L.wmax = take(A * 4);
+      L.exend = off;
+      L.eY64 = take(A * 4);
+      L.Cimg = take(digit_shape(d.A, d.N).bytes);
+      L.Yimg = take(digit_shape(d.A, (long long)pb * round_up_int(d.A, 8)).bytes);
+      L.W64 = take(pb * A * 8);
+    } else {
+      L.Y64 = take(pb * A * A * 8);
+    }
   } else {
     const size_t Q = d.Q;
     // split B in symmetric lower-triangle tiles, per plane Q x SymTiles::perP halves
@@ -165,7 +239,7 @@ Layout make_layout(const Dims& d) {
     L.eh = take(N * 4);
     L.hpart = take(4 * N * Ap * 4);
   }
-  L.total = off;
+  L.total = off > d.ws_total ? off : d.ws_total;
   return L;
 }
 
@@ -262,9 +336,11 @@ int check_problem(const donof_problem* p) {
   return DONOF_OK;
 }
 
-int check_ws(const donof_problem* p, const void* ws, size_t bytes) {
+// Checks the workspace and gives the problem's sizes and the workspace's carving.
+int check_ws(const donof_problem* p, const void* ws, size_t bytes, Dims& d, Layout& L) {
   if (!ws || ((uintptr_t)ws % kAlign) != 0) return DONOF_ERR_WORKSPACE;
-  const Layout L = make_layout(make_dims(p));
+  d = make_dims(p);
+  L = make_layout(d);
   return bytes >= L.total ? DONOF_OK : DONOF_ERR_WORKSPACE;
 }
 
@@ -332,11 +408,11 @@ extern "C" int donof_prepare_B(const donof_problem* prob, const double* B, void*
   int rc = check_problem(prob);
   if (rc != DONOF_OK) return rc;
   if (!B) return DONOF_ERR_INVALID_ARG;
-  rc = check_ws(prob, workspace, workspace_bytes);
+  Dims d;
+  Layout L;
+  rc = check_ws(prob, workspace, workspace_bytes, d, L);
   if (rc != DONOF_OK) return rc;
   cudaStream_t s = (cudaStream_t)stream;
-  const Dims d = make_dims(prob);
-  const Layout L = make_layout(d);
   char* ws = (char*)workspace;
   prof_begin(DONOF_PHASE_PREPARE_B, s);
   CK(cudaMemsetAsync(ws + L.header, 0, sizeof(DevHeader), s));
@@ -348,6 +424,8 @@ extern "C" int donof_prepare_B(const donof_problem* prob, const double* B, void*
     CK(cudaMemsetAsync(ws + L.hAF, 0, u, s));
     CK(cudaMemsetAsync(ws + L.cPH, 0, v, s));
     CK(cudaMemsetAsync(ws + L.cPF, 0, v, s));
+  } else if (d.digit) {
+    CK(digit_prepare_B(d, B, ws, L, s));
   }
   prof_end(DONOF_PHASE_PREPARE_B, s);
   std::lock_guard<std::mutex> lk(g_mu);
@@ -372,7 +450,9 @@ int run_build(const donof_problem* prob, const double* h, const double* B, const
   if (mode != kPartial && !E) return DONOF_ERR_INVALID_ARG;
   if (mode != kFull && !partial) return DONOF_ERR_INVALID_ARG;
   if (mode != kFinish && !B) return DONOF_ERR_INVALID_ARG;
-  rc = check_ws(prob, workspace, workspace_bytes);
+  Dims d;
+  Layout L;
+  rc = check_ws(prob, workspace, workspace_bytes, d, L);
   if (rc != DONOF_OK) return rc;
   if (mode != kFinish) {
     std::lock_guard<std::mutex> lk(g_mu);
@@ -380,8 +460,6 @@ int run_build(const donof_problem* prob, const double* h, const double* B, const
     if (it == g_reg.end() || it->second.B != B || !same_problem(it->second.prob, *prob))
       return DONOF_ERR_NOT_PREPARED;
   }
-  const Dims d = make_dims(prob);
-  const Layout L = make_layout(d);
   char* ws = (char*)workspace;
   const int N = d.N, A = d.A;
   const size_t AA = (size_t)A * A * 8;
@@ -398,6 +476,8 @@ int run_build(const donof_problem* prob, const double* h, const double* B, const
     if (rc != DONOF_OK) return rc;
     // bound on ||C_act||_2 for the exponents of X in the G contraction
     if (mode != kFinish) CK(launch_gram_bound(d, C, ws, L, s));
+  } else if (d.digit) {
+    CK(digit_hc(d, h, C, ws, L, s));
   } else {
     CK(cudaMemsetAsync(ws + L.hC, 0, (size_t)N * A * 8, s));
     CK(launch_dgemm(split_k_args(N, A, N, h, N, 1, C, N, 1, (double*)(ws + L.hC), A, 1,
@@ -408,9 +488,8 @@ int run_build(const donof_problem* prob, const double* h, const double* B, const
     CK(cudaMemcpyAsync(ws + L.J, partial, AA, cudaMemcpyDeviceToDevice, s));
     CK(cudaMemcpyAsync(ws + L.K, partial + (size_t)A * A, AA, cudaMemcpyDeviceToDevice, s));
     CK(launch_add((double*)(ws + L.G), partial + 2 * (size_t)A * A, (long long)N * A, s));
-  } else {
-    CK(cudaMemsetAsync(ws + L.J, 0, AA, s));
-    CK(cudaMemsetAsync(ws + L.K, 0, AA, s));
+  } else if (!d.digit) {  // (the digit products' first block sets J and K)
+    CK(cudaMemsetAsync(ws + L.J, 0, L.K + AA - L.J, s));  // K follows J
   }
   prof_end(DONOF_PHASE_PREP, s);
 
@@ -429,6 +508,12 @@ int run_build(const donof_problem* prob, const double* h, const double* B, const
       Bblk = (const double*)(ws + L.Bun);
     } else {
       Bblk = B + (size_t)p0 * N * N;
+    }
+    if (d.digit) {
+      rc = digit_block(d, Bblk, p0, np, ws, L, s);
+      if (rc != DONOF_OK) return rc;
+      prof_end(DONOF_PHASE_G_BUILD, s);
+      continue;
     }
     double* X = (double*)(ws + L.X64);
     double* b = (double*)(ws + L.b64);
@@ -488,6 +573,8 @@ int run_build(const donof_problem* prob, const double* h, const double* B, const
     if (d.precision == DONOF_MIXED) {
       rc = run_lambda_tc(d, C, ws, L, lam, s);
       if (rc != DONOF_OK) return rc;
+    } else if (d.digit) {
+      CK(digit_lambda(d, C, ws, L, lam, s));
     } else {
       CK(launch_dgemm(split_k_args(N, A, N, C, 1, N, (const double*)(ws + L.G), A, 1, lam, N, 1,
                                    (double*)(ws + L.skp)),
@@ -542,10 +629,10 @@ extern "C" int donof_energy_backward(const donof_problem* prob, const double* Eb
   int rc = check_problem(prob);
   if (rc != DONOF_OK) return rc;
   if (!Ebar) return DONOF_ERR_INVALID_ARG;
-  rc = check_ws(prob, workspace, workspace_bytes);
+  Dims d;
+  Layout L;
+  rc = check_ws(prob, workspace, workspace_bytes, d, L);
   if (rc != DONOF_OK) return rc;
-  const Dims d = make_dims(prob);
-  const Layout L = make_layout(d);
   prof_begin(DONOF_PHASE_BACKWARD, (cudaStream_t)stream);
   CK(launch_backward(d, Ebar, (const char*)workspace, L, dE_dC, dE_dgamma, (cudaStream_t)stream));
   prof_end(DONOF_PHASE_BACKWARD, (cudaStream_t)stream);
@@ -556,10 +643,10 @@ extern "C" int donof_get_jk(const donof_problem* prob, const void* workspace,
                             size_t workspace_bytes, double* J, double* K, void* stream) {
   int rc = check_problem(prob);
   if (rc != DONOF_OK) return rc;
-  rc = check_ws(prob, workspace, workspace_bytes);
+  Dims d;
+  Layout L;
+  rc = check_ws(prob, workspace, workspace_bytes, d, L);
   if (rc != DONOF_OK) return rc;
-  const Dims d = make_dims(prob);
-  const Layout L = make_layout(d);
   const size_t bytes = (size_t)d.A * d.A * 8;
   cudaStream_t s = (cudaStream_t)stream;
   if (J) CK(cudaMemcpyAsync(J, (const char*)workspace + L.J, bytes, cudaMemcpyDeviceToDevice, s));

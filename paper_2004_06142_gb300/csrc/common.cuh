@@ -32,6 +32,8 @@ struct Dims {
   int N, Q, A, Ap, Np, npair, ncwo, ng, pb, nblk, functional, layout, precision;
   int nsingle;  // singly occupied orbitals (Omega_I) at npair .. npair + nsingle - 1
   int splits;  // split-K factor of the G contraction (mixed path)
+  int digit;   // FP64: the contractions as exact digit products on the tensor cores (digits.cu)
+  size_t ws_total;  // bytes of the workspace (at least; FP64)
 };
 
 // Byte offsets of every buffer inside the workspace.
@@ -42,6 +44,10 @@ struct Layout {
   size_t skp;  // deterministic split-K partials of the FP64 N x A products
   // FP64 path
   size_t X64, b64, Y64, Bun;
+  // FP64 path on digit products: largest biased exponents of B's rows (eRow, from
+  // prepare), of C's columns, h's rows and G's columns, of X per (P, q) and per mu, of b and
+  // w, and Y's columns; the stage images of C_act (then of G) and of Y; w^P
+  size_t eRow, eC64, eH64, eG64, exq, exm, bmax, wmax, exend, eY64, Cimg, Yimg, W64;
   // mixed path
   // integer + fraction planes (h, f) of the tensor-core operands and their per-row
   // exponents: B (Bhi/Blo, eB), C_act^T (Chi/Clo, eC), X^T for b (Xthi/Xtlo, eXt), X for G
@@ -302,6 +308,80 @@ struct DgemmArgs {
   double* part;  // ksplit x M x N scratch when ksplit > 1
 };
 cudaError_t launch_dgemm(const DgemmArgs& a, cudaStream_t s);
+
+// Products of doubles as exact digit products on the tensor cores (digits.cu).
+struct DigitArgs {
+  // A(m, k): row m = b Mb + r at A + b sAb + r sAm; k = kb Kpad + q at kb sAkb + q sAk
+  // (q < Kin; Kpad a multiple of 8 pads each kb with zeros)
+  const double* A;
+  long long sAb, sAm, sAk, sAkb;
+  int M, Mb, Kin, Kpad, KB;
+  const int* eA;        // per row: the largest biased exponent in it (k_row_exp, k_col_exp)
+  const __half* Bimg;   // stage images of B (k_digit_planes)
+  const int* eB;        // per column, as eA
+  int N, NT, ntiles, mtiles, nstages, splits;
+  // C(m, n) at C + split sCs + (m / Mb) sCb + (m % Mb) sCm + n
+  double* C;
+  long long sCs, sCb, sCm;
+  // when set: the largest biased exponents of the result, per (m / Mb, n) in exq[.. exq_ld + n]
+  // and per m % Mb in exm (atomic maxima; zeroed by the caller)
+  int *exq, *exm;
+  int exq_ld;
+  int vecA, vecC;       // 16-byte loads of A / stores of C are aligned
+  int *status, *abort_flag;
+  uint32_t k64;         // the half2 word 1024, an argument so that it stays in a register
+};
+// Tiling of an operand B of N columns over a contraction of K (padded) elements: column tiles of
+// NT (a multiple of 16, at most 64, as even as the width allows), stages of 32 elements, and
+// the bytes of its stage images.
+struct DigitShape {
+  int NT, ntiles, nstages;
+  size_t bytes;
+};
+inline DigitShape digit_shape(int N, long long K) {
+  DigitShape t;
+  const int c = (N + 15) / 16;
+  t.ntiles = (c + 3) / 4;
+  t.NT = 16 * ((c + t.ntiles - 1) / t.ntiles);
+  t.nstages = (int)((K + 31) / 32);
+  t.bytes = (size_t)t.ntiles * t.nstages * 8 * t.NT * 64;
+  return t;
+}
+// Splits of the G contraction (about one unit per SM, at least four stages and at most 64
+// chunks of 256 elements each, so that group 0 stays below 2^30) and of the
+// sums over slices of J and K (about 300 CTAs, at least 8 slices each).
+inline int g_splits_digit(int N, int A, int np) {
+  const DigitShape t = digit_shape(A, (long long)np * round_up_int(A, 8));
+  const int tiles = t.ntiles * ((N + 127) / 128);
+  int sp = 152 / tiles;
+  if (sp > t.nstages / 4) sp = t.nstages / 4;
+  const int least = (t.nstages + 511) / 512;
+  return sp < least ? least : sp;
+}
+inline int jk_splits64(int A, int np) {
+  const int nb = (A * (A + 1) / 2 + 255) / 256;
+  int sp = (300 + nb - 1) / nb;
+  if (sp > (np + 7) / 8) sp = (np + 7) / 8;
+  return sp < 1 ? 1 : sp;
+}
+// C = A B (M x N, C's rows ldc apart; A(m, k) at m sAm + k sAk, one of the strides 1; B(k, n) at
+// k ldb + n; K <= 16384) with the operands' exponents and B's digits in `scratch`
+// (digit_product_bytes, 256-byte aligned); status and abort_flag: device words of the bounded
+// waits.
+size_t digit_product_bytes(int M, int N, int K);
+cudaError_t digit_product(int M, int N, int K, const double* A, long long sAm, long long sAk,
+                          const double* B, long long ldb, double* C, long long ldc, char* scratch,
+                          int* status, int* abort_flag, cudaStream_t s);
+// The FP64 path's parts on digit products: the exponents of B's rows, h C_act, one block of
+// slices (X, b, J, K, G; Bblk: its slices, dense), lambda.
+cudaError_t digit_prepare_B(const Dims& d, const double* B, char* ws, const Layout& L,
+                            cudaStream_t s);
+cudaError_t digit_hc(const Dims& d, const double* h, const double* C, char* ws, const Layout& L,
+                     cudaStream_t s);
+int digit_block(const Dims& d, const double* Bblk, int p0, int np, char* ws, const Layout& L,
+                cudaStream_t s);
+cudaError_t digit_lambda(const Dims& d, const double* C, char* ws, const Layout& L, double* lam,
+                         cudaStream_t s);
 // The split count split_k_args uses for an M x N output with contraction length K.
 int splitk_count(int M, int N, int K);
 // Symmetric FP64 eigensolver (eigh.cu): A (N x N, row-major, symmetric; not modified) =

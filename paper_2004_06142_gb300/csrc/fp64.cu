@@ -202,11 +202,10 @@ __global__ void k_occupations(Dims d, const double* __restrict__ gamma,
 
 cudaError_t launch_occupations(const Dims& d, const double* gamma, const int32_t* pm, char* ws,
                                const Layout& L, cudaStream_t s) {
+  // the three Jacobians follow one another
   const size_t jac = (size_t)d.A * d.ng * sizeof(double);
-  for (size_t off : {L.dn, L.dsq, L.dphi}) {
-    const cudaError_t e = cudaMemsetAsync(ws + off, 0, jac, s);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = cudaMemsetAsync(ws + L.dn, 0, L.dphi + jac - L.dn, s);
+  if (e != cudaSuccess) return e;
   DevHeader* hdr = (DevHeader*)(ws + L.header);
   double *n = (double*)(ws + L.n), *sqn = (double*)(ws + L.sqn), *phi = (double*)(ws + L.phi);
   double *dn = (double*)(ws + L.dn), *dsq = (double*)(ws + L.dsq), *dphi = (double*)(ws + L.dphi);
