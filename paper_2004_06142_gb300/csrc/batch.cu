@@ -316,8 +316,8 @@ int enqueue_grouped(int32_t ninst, char* ws, int32_t flags, const Plan& pl, cuda
   return DONOF_OK;
 }
 
-// The plan last copied into each batched workspace (so that an unchanged plan is not copied
-// again).
+// The plan last copied into each batched workspace since it was prepared (so that an unchanged
+// plan is not copied again).
 std::map<const void*, std::vector<char>> g_uploaded;
 
 int upload_plan(char* ws, const Plan& pl, cudaStream_t s) {
@@ -381,6 +381,10 @@ extern "C" int donof_prepare_B_batched(int32_t ninst, const donof_problem* probs
   if (!inst || !workspace || workspace_bytes < need || ((uintptr_t)workspace % kAlign) != 0)
     return DONOF_ERR_WORKSPACE;
   cudaStream_t s = (cudaStream_t)stream;
+  {  // a workspace prepared anew may be other memory at an old address: its tables are copied again
+    std::lock_guard<std::mutex> lk(g_batch_mu);
+    g_uploaded.erase(workspace);
+  }
   // the batch's status header cleared, the constant 1.0 set
   if (cudaMemsetAsync(workspace, 0, sizeof(DevHeader), s) != cudaSuccess) return DONOF_ERR_CUDA;
   const double one = 1.0;
