@@ -1046,44 +1046,263 @@ __device__ inline double load_B_elem(const double* __restrict__ B, int layout, l
   return B[P * npk + (long long)a * (a + 1) / 2 + b];
 }
 
-// Per row (P, mu) of B: its squared L2 norm (rn2, fp32 rounded up, for the exponents of X
-// in the G contraction), the slice's largest row L1 norm (L1max, the bound on X^T rows) and the AO
-// index's largest row norm over the slices (rnmax, for the symmetric scaling); any
-// non-finite element raises DONOF_ERR_NONFINITE.
-__global__ void k_b_stats(const double* __restrict__ B, int layout, long long Q, int N,
-                          DevHeader* hdr, unsigned long long* L1max_bits, float* rn2,
-                          unsigned long long* rnmax_bits) {
-  const long long rows = Q * N;
-  const int lane = threadIdx.x % 32;
-  const long long npk = (long long)N * (N + 1) / 2;
-  double mx = 0.0, mr = 0.0;
-  for (long long row = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / 32; row < rows;
-       row += (long long)gridDim.x * blockDim.x / 32) {
-    const long long P = row / N;
-    const int mu = (int)(row % N);
-    double ss = 0.0, m = 0.0, l1 = 0.0;
-    for (int nu = lane; nu < N; nu += 32) {
-      const double v = load_B_elem(B, layout, P, row, mu, nu, N, npk);
-      ss = fma(v, v, ss);
-      m = fmax(m, fabs(v));
-      l1 += fabs(v);
+// The passes over B below work in fp32 on elements scaled by a power of two per slice (this
+// GPU's FP64 pipe gives 1.6 operations per clock and SM, its double-to-float conversion 100): a
+// CTA per slice finds the largest (scaled) exponent, then sums elements brought to at most 2.
+// two_floats: v 2^k (biased exponent e of v, e + k within a float's range) as xh + xl, xh the
+// upper 24 bits rounded half up, xl the lower 29 bits (rounded to 24), from the bits alone.
+__device__ __forceinline__ void two_floats(double v, int k, float& xh, float& xl) {
+  const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+  const int e = (int)((hi >> 20) & 0x7ffu) + k;
+  const bool tiny = (hi & 0x7ff00000u) == 0 || e < 1023 - 120;  // taken as zero
+  uint32_t h2 = hi + ((uint32_t)k << 20), l2 = lo;
+  asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, 0;" : "+r"(l2), "+r"(h2) : "r"(0x10000000u));
+  xh = tiny ? 0.f : (float)__hiloint2double((int)h2, (int)(l2 & 0xe0000000u));
+  // the lower bits as a signed number of 2^-3: weight 2^(e - 1023 - 52 - 3)
+  const float w = __int_as_float(max(e - 1078 + 127, 0) << 23);
+  const float r = (float)(int)(lo << 3) * w;
+  xl = tiny ? 0.f : ((int)hi < 0 ? -r : r);
+}
+// |v| 2^k rounded to a float, for sums that a few roundings do not matter to.
+__device__ __forceinline__ float one_float(double v, int k) {
+  const int hi = __double2hiint(v), e = ((hi >> 20) & 0x7ff) + k;
+  const bool tiny = (hi & 0x7ff00000) == 0 || e < 1023 - 120;
+  return tiny ? 0.f : (float)__hiloint2double((hi & 0xfffff) | (e << 20), __double2loint(v));
+}
+// s + c += p, the rounding of s kept in c (Knuth's two-sum)
+__device__ __forceinline__ void add_comp(float& s, float& c, float p) {
+  const float t = __fadd_rn(s, p), z = __fsub_rn(t, s);
+  c += __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z));
+  s = t;
+}
+// What elements too small for their square to be a float can add to a row's sum, per element.
+constexpr double kStatsLost = 0x1p-118;
+
+// Row sums of slice P (N x N, symmetric) over its elements times 2^(-s_mu - s_nu) (s null: 0) in
+// units of 2^top: row(mu, squares, magnitudes), called by one thread per row.  EXACT: compensated
+// sums, to about 2^-40; otherwise squares only, to sum_margin.  Dense: a warp per row.  Packed: a
+// warp per stored row, whose elements also count for their columns (partial sums per warp in
+// shared memory, added in the order of the warps).  Returns top (above 4096: a NaN or an infinity).
+// All threads of the CTA call it; sh holds kSums N floats per warp and once more (packed), red 33
+// ints.
+template <bool PACKED, bool EXACT, class Row>
+__device__ __forceinline__ int slice_row_sums(const double* __restrict__ B, int N,
+                                              const int* __restrict__ s, float* sh, int* red,
+                                              const Row& row) {
+  constexpr int kSums = EXACT ? 4 : 1;  // squares, their compensation, magnitudes, theirs
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  int m = 0;  // biased; 0: the slice is zero
+  for (int mu = w; mu < N; mu += nw) {
+    const double* r = B + (PACKED ? (long long)mu * (mu + 1) / 2 : (long long)mu * N);
+    const int n = PACKED ? mu + 1 : N, smu = s ? s[mu] : 0;
+#pragma unroll 4
+    for (int nu = lane; nu < n; nu += 32) {
+      const int e = (__double2hiint(r[nu]) >> 20) & 0x7ff;
+      if (e > 0) m = max(m, e == 2047 ? 1 << 20 : e + 4096 - smu - (s ? s[nu] : 0));
     }
-    for (int o = 16; o > 0; o >>= 1) {
-      ss += __shfl_xor_sync(0xffffffffu, ss, o);
-      m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-      l1 += __shfl_xor_sync(0xffffffffu, l1, o);
-    }
-    const double nr = sqrt(ss);
-    if (lane == 0) {
-      rn2[row] = __double2float_ru(ss);
-      atomic_max_nonneg(L1max_bits + P, l1);
-      atomic_max_nonneg(rnmax_bits + mu, nr);
-    }
-    mx = fmax(mx, m);
-    mr = fmax(mr, nr);
   }
-  if (lane == 0) {
-    if (!isfinite(mx) || !isfinite(mr)) set_status(hdr, DONOF_ERR_NONFINITE);
+  m = __reduce_max_sync(0xffffffffu, m);
+  __syncthreads();  // red and sh are free
+  if (lane == 0) red[w] = m;
+  if (PACKED)
+    for (int i = threadIdx.x; i < kSums * N * nw; i += blockDim.x) sh[i] = 0.f;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    m = threadIdx.x < nw ? red[threadIdx.x] : 0;
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (threadIdx.x == 0) red[32] = m;
+  }
+  __syncthreads();
+  const int top = red[32] - 4096;  // the largest scaled biased exponent
+  float* cs = sh + kSums * N * w;  // this warp's partial sums of the columns
+  for (int mu = w; mu < N; mu += nw) {
+    const double* r = B + (PACKED ? (long long)mu * (mu + 1) / 2 : (long long)mu * N);
+    const int n = PACKED ? mu + 1 : N, k = 1023 - top - (s ? s[mu] : 0);
+    float ss = 0.f, sc = 0.f, l1 = 0.f, lc = 0.f;
+#pragma unroll 4
+    for (int nu = lane; nu < n; nu += 32) {
+      if (EXACT) {
+        float xh, xl;
+        two_floats(r[nu], k - (s ? s[nu] : 0), xh, xl);
+        const float q = __fmul_rn(xh, xh);
+        const float qe = fmaf(2.f * xh, xl, fmaf(xh, xh, -q)), a = fabsf(xh);
+        const float al = xh < 0.f ? -xl : xl;
+        add_comp(ss, sc, q);
+        sc += qe;
+        add_comp(l1, lc, a);
+        lc += al;
+        if (PACKED && nu < mu) {
+          float ts = cs[nu], tc = cs[N + nu], tl = cs[2 * N + nu], td = cs[3 * N + nu];
+          add_comp(ts, tc, q);
+          add_comp(tl, td, a);
+          cs[nu] = ts;
+          cs[N + nu] = tc + qe;
+          cs[2 * N + nu] = tl;
+          cs[3 * N + nu] = td + al;
+        }
+      } else {
+        const float x = one_float(r[nu], k - (s ? s[nu] : 0));
+        ss = fmaf(x, x, ss);
+        if (PACKED && nu < mu) cs[nu] = fmaf(x, x, cs[nu]);
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      if (EXACT) {
+        const float c2 = __shfl_xor_sync(0xffffffffu, sc, o), d2 = __shfl_xor_sync(0xffffffffu, lc, o);
+        add_comp(ss, sc, __shfl_xor_sync(0xffffffffu, ss, o));
+        add_comp(l1, lc, __shfl_xor_sync(0xffffffffu, l1, o));
+        sc += c2;
+        lc += d2;
+      } else {
+        ss += __shfl_xor_sync(0xffffffffu, ss, o);
+      }
+    }
+    if (lane == 0) {
+      if (PACKED) {  // the row's own part, behind the warps' column sums
+        float* o = sh + kSums * N * nw + mu;
+        o[0] = ss;
+        if (EXACT) {
+          o[N] = sc;
+          o[2 * N] = l1;
+          o[3 * N] = lc;
+        }
+      } else {
+        row(mu, (double)ss + (double)sc, (double)l1 + (double)lc);
+      }
+    }
+  }
+  if (PACKED) {
+    __syncthreads();
+    for (int mu = threadIdx.x; mu < N; mu += blockDim.x) {
+      float t[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int i = 0; i <= nw; ++i) {
+        const float* c = sh + kSums * N * i + mu;
+        if (EXACT) {
+          add_comp(t[0], t[1], c[0]);
+          add_comp(t[2], t[3], c[2 * N]);
+          t[1] += c[N];
+          t[3] += c[3 * N];
+        } else {
+          t[0] += c[0];
+        }
+      }
+      row(mu, (double)t[0] + (double)t[1], (double)t[2] + (double)t[3]);
+    }
+  }
+  return top;
+}
+// The largest of the threads' non-negative doubles, in every thread (red: 33 64-bit words).
+__device__ __forceinline__ double block_max(double v, unsigned long long* red) {
+  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = (unsigned long long)__double_as_longlong(v);
+  __syncthreads();
+  unsigned long long t = 0;
+  for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t = max(t, red[i]);
+  return __longlong_as_double((long long)t);
+}
+// Warps of a slice's CTA and its shared memory (the largest N of packed slices whose sums fit one
+// warp's share is 6400; no B of that size fits the device).
+constexpr int kPackedStatsMaxN = 6400;
+inline int slice_warps(bool packed, int N) {
+  int nw = 8;
+  while (packed && nw > 1 && (size_t)(nw + 1) * 16 * N > 200 * 1024) --nw;
+  return nw;
+}
+inline size_t slice_smem(bool packed, int N) {
+  return packed ? (size_t)(slice_warps(true, N) + 1) * 16 * N : 0;  // (k_b_stats)
+}
+
+// Per row (P, mu) of B: its squared L2 norm (rn2, fp32 rounded up, for the exponents of X in the
+// G contraction), the slice's largest row L1 norm (L1max, the bound on X^T rows) and the AO
+// index's largest row norm over the slices (rnmax, for the symmetric scaling); any
+// non-finite element raises DONOF_ERR_NONFINITE.  1103 packed slices of 301: 0.26 ms (in double,
+// every element gathered twice: 1.18 ms).
+template <bool PACKED>
+__global__ void __launch_bounds__(256) k_b_stats(const double* __restrict__ B, int Q, int N,
+                                                 DevHeader* hdr, double* L1max, float* rn2,
+                                                 unsigned long long* rnmax_bits) {
+  extern __shared__ float sh_f[];
+  __shared__ int red[33];
+  __shared__ unsigned long long redl[33];
+  const long long per = PACKED ? (long long)N * (N + 1) / 2 : (long long)N * N;
+  constexpr double kUp = 1.0 + 0x1p-36;  // above the compensated sums' error
+  const double lost = N * kStatsLost;
+  for (int P = blockIdx.x; P < Q; P += gridDim.x) {
+    double mx = 0.0;
+    float* out = rn2 + (size_t)P * N;
+    // the slice's scale is known to every thread only after the call: the rows are scaled by
+    // the exponent that the call found, which it leaves in red
+    const int top = slice_row_sums<PACKED, true>(
+        B + P * per, N, nullptr, sh_f, red, [&](int mu, double ss, double l1) {
+          const int t = red[32] - 4096;
+          if (t > 4096) {
+            out[mu] = __int_as_float(0x7fc00000);
+            return;
+          }
+          const double sc = pow2d(t - 1023);
+          out[mu] = __double2float_ru((ss * kUp + lost) * sc * sc);
+          atomic_max_nonneg(rnmax_bits + mu, sqrt(ss) * sc);
+          mx = fmax(mx, l1);
+        });
+    const double l1 = block_max(mx, redl);
+    if (threadIdx.x == 0) {
+      if (top > 4096) {
+        set_status(hdr, DONOF_ERR_NONFINITE);
+        L1max[P] = __longlong_as_double(0x7ff8000000000000ll);
+      } else {
+        L1max[P] = (l1 * kUp + lost) * pow2d(top - 1023);
+      }
+    }
+  }
+}
+
+// Per slice: t_P, the exponent of the largest row norm of Bt^P without t_P.  Where the fp32 sums
+// cannot tell on which side of a power of two the norm lies, the slice's sums are taken in
+// double.  1103 packed slices of 301: 0.2 ms (in double, with an ldexp per element: 1.35 ms).
+template <bool PACKED>
+__global__ void __launch_bounds__(256) k_p_scale(const double* __restrict__ B, int Q, int N,
+                                                 const int* __restrict__ eS, double invT,
+                                                 int* tP) {
+  extern __shared__ float sh_f[];
+  __shared__ int red[33];
+  __shared__ unsigned long long redl[33];
+  const long long npk = (long long)N * (N + 1) / 2, per = PACKED ? npk : (long long)N * N;
+  // rounding of the sums: N / 32 terms a lane, N / nw in a warp's sum of a column, the tree over
+  // lanes, the warps' sums, every term rounded before
+  const int nw = blockDim.x >> 5;
+  int* sS = (int*)(sh_f + (PACKED ? (nw + 1) * N : 0));  // the scale exponents, behind the sums
+  for (int i = threadIdx.x; i < N; i += blockDim.x) sS[i] = eS[i];
+  __syncthreads();
+  const double mg = (N / 32 + (PACKED ? N / nw : 0) + 32) * 0x1p-24;
+  for (int P = blockIdx.x; P < Q; P += gridDim.x) {
+    const double* Bp = B + P * per;
+    double mx = 0.0;
+    const int top = slice_row_sums<PACKED, false>(
+        Bp, N, sS, sh_f, red, [&](int, double ss, double) { mx = fmax(mx, ss); });
+    const double ss = block_max(mx, redl);
+    const double sc = pow2d(top - 1023);
+    const int e0 = intfrac_exponent_inv(sqrt(ss * (1.0 - mg)) * sc, invT);
+    const int e1 = intfrac_exponent_inv(sqrt(ss * (1.0 + mg)) * sc, invT);
+    if (e0 == e1) {  // (the same in every thread)
+      if (threadIdx.x == 0) tP[P] = top > 4096 ? 0 : e0;
+      continue;
+    }
+    double t2 = 0.0;
+    for (int mu = threadIdx.x >> 5; mu < N; mu += nw) {
+      double t = 0.0;
+      for (int nu = threadIdx.x & 31; nu < N; nu += 32) {
+        const double v = ldexp(load_B_elem(Bp, PACKED ? DONOF_B_PACKED : DONOF_B_DENSE, 0, mu, mu,
+                                           nu, N, npk),
+                               -eS[mu] - eS[nu]);
+        t = fma(v, v, t);
+      }
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      t2 = fmax(t2, t);
+    }
+    const double exact = block_max(sqrt(t2), redl);
+    if (threadIdx.x == 0) tP[P] = intfrac_exponent_inv(exact, invT);
   }
 }
 
@@ -1113,100 +1332,109 @@ __global__ void __launch_bounds__(1024) k_sym_scale(const double* __restrict__ r
   }
 }
 
-// Per slice: the largest row norm of Bt^P without t_P (one warp per row).
-__global__ void k_p_scale(const double* __restrict__ B, int layout, long long Q, int N,
-                          const int* __restrict__ eS, unsigned long long* tmax_bits) {
-  const long long rows = Q * N;
-  const int lane = threadIdx.x % 32;
-  const long long npk = (long long)N * (N + 1) / 2;
-  for (long long row = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / 32; row < rows;
-       row += (long long)gridDim.x * blockDim.x / 32) {
-    const long long P = row / N;
-    const int mu = (int)(row % N);
-    double ss = 0.0;
-    for (int nu = lane; nu < N; nu += 32) {
-      const double v = ldexp(load_B_elem(B, layout, P, row, mu, nu, N, npk), -eS[mu] - eS[nu]);
-      ss = fma(v, v, ss);
-    }
-    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    if (lane == 0) atomic_max_nonneg(tmax_bits + P, sqrt(ss));
-  }
-}
-
 // eA[P][mu] = t_P + s_mu: the exponent of output row (P, mu) of the half transform.
-__global__ void k_sym_exps(const double* __restrict__ tmax, const int* __restrict__ eS,
-                           long long Q, int N, double invT, int* eA) {
+__global__ void k_sym_exps(const int* __restrict__ tP, const int* __restrict__ eS,
+                           long long Q, int N, int* eA) {
   const long long tot = Q * N;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < tot;
        i += (long long)gridDim.x * blockDim.x)
-    eA[i] = intfrac_exponent_inv(tmax[i / N], invT) + eS[i % N];
+    eA[i] = tP[i / N] + eS[i % N];
 }
 
-// Bt^P 2^-t_P -> integer + fraction planes in the lower-triangle tile storage (SymTiles).
-// One thread per 8 consecutive stored elements: slice P, stored row mu (rows of the last
-// tile padded to Rlast), 64-wide k block kb of a tile column not right of mu's tile.
-__global__ void k_split_B_sym(const double* __restrict__ B, int layout, long long Q, int N,
-                              SymTiles st, DevHeader* hdr, const int* __restrict__ eS,
-                              const double* __restrict__ tmax, double invT, __half* H,
-                              __half* F) {
+// The integer + fraction split of y = v 2^k, |y| < 4096, as the double split forms it (h =
+// fp16(rint(y)), f = fp16(fl32(y - h))), without an FP64 operation: y = yh + yl (two_floats); rint(y)
+// is rint(yh) except where yh lies half-way between two integers and yl decides; y - h =
+// (yh - h) + yl with an exact difference.
+__device__ __forceinline__ void intfrac_split_scaled(double v, int k, __half& h, __half& f) {
+  float yh, yl;
+  two_floats(v, k, yh, yl);
+  float t = rintf(yh);
+  const float d = yh - t;
+  t += (d == 0.5f && yl > 0.f) ? 1.f : ((d == -0.5f && yl < 0.f) ? -1.f : 0.f);
+  h = __float2half_rn(t);
+  f = __float2half_rn((yh - __half2float(h)) + yl);
+}
+
+// Bt^P 2^-t_P -> integer + fraction planes in the lower-triangle tile storage (SymTiles).  A warp
+// per stored row mu of a slice (rows of the last tile padded to Rlast), a lane per 8
+// consecutive stored elements; the columns reach to the end of mu's tile.
+__global__ void __launch_bounds__(256) k_split_B_sym(const double* __restrict__ B, int layout,
+                                                     int Q, int N, SymTiles st,
+                                                     const int* __restrict__ eS,
+                                                     const int* __restrict__ tP, __half* H,
+                                                     __half* F) {
   const long long npk = (long long)N * (N + 1) / 2;
   const int rows = 128 * (st.T - 1) + st.Rlast;  // stored rows (= columns) per slice
-  const int KB = rows / 64;
-  const long long tot = Q * rows * KB * 8;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < tot;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int j8 = (int)(i % 8);
-    long long t = i / 8;
-    const int kb = (int)(t % KB);
-    t /= KB;
-    const int mu = (int)(t % rows);
-    const long long P = t / rows;
-    const int ti = mu / 128, tj = kb / 2;
-    if (tj > ti) continue;  // upper triangle: not stored
-    const int r = mu - 128 * ti, c = kb - 2 * tj;
-    const int Ri = sym_R(st, ti);
-    const int tP = intfrac_exponent_inv(tmax[P], invT);
-    __align__(16) __half hv[8], fv[8];
+  const int lane = threadIdx.x & 31, rb = (rows + 7) / 8;
+  const long long tot = (long long)Q * rb;
+  for (long long u = blockIdx.x; u < tot; u += gridDim.x) {  // 8 rows of a slice per CTA
+    const int P = (int)(u / rb), mu = (int)(u - (long long)P * rb) * 8 + (threadIdx.x >> 5);
+    if (mu >= rows) continue;
+    const int ti = mu >> 7, r = mu & 127, Ri = sym_R(st, ti);
+    const int k0 = -tP[P] - (mu < N ? eS[mu] : 0);
+    const double* Bp = B + (layout == DONOF_B_DENSE ? (size_t)P * N * N : (size_t)P * npk);
+    const size_t base = (size_t)P * st.perP;
+    const int ncols = 128 * ti + (ti == st.T - 1 ? st.Rlast : 128);
+    const double* row = Bp + (layout == DONOF_B_DENSE ? (size_t)mu * N
+                                                      : (size_t)((long long)mu * (mu + 1) / 2));
+    for (int c8 = lane; c8 < ncols / 8; c8 += 32) {
+      __align__(16) __half hv[8], fv[8];
+      const int nu0 = 8 * c8;
+      double v[8];
+      int k[8];
+      if (mu < N && (layout == DONOF_B_DENSE ? nu0 + 7 < N : nu0 + 7 <= mu)) {  // stored in a row
+        *(int4*)k = *(const int4*)(eS + nu0);
+        *(int4*)(k + 4) = *(const int4*)(eS + nu0 + 4);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int nu = kb * 64 + j8 * 8 + k;
-      double y = 0.0;
-      if (mu < N && nu < N)
-        y = ldexp(load_B_elem(B, layout, P, P * N + mu, mu, nu, N, npk), -tP - eS[mu] - eS[nu]);
-      intfrac_split(y, hv[k], fv[k]);
+        for (int j = 0; j < 8; ++j) {
+          v[j] = __ldg(row + nu0 + j);
+          k[j] = k0 - k[j];
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int nu = nu0 + j;
+          const bool in = mu < N && nu < N;
+          v[j] = in ? load_B_elem(Bp, layout, 0, mu, mu, nu, N, npk) : 0.0;
+          k[j] = in ? k0 - eS[nu] : 0;
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) intfrac_split_scaled(v[j], k[j], hv[j], fv[j]);
+      const int tj = c8 >> 4, c = (c8 >> 3) & 1, j8 = c8 & 7;
+      const size_t o = base + sym_tile_off(st, ti, tj) + ((size_t)c * Ri + r) * 64 +
+                       (size_t)((j8 ^ (r & 7)) * 8);
+      *(uint4*)(H + o) = *(const uint4*)hv;
+      *(uint4*)(F + o) = *(const uint4*)fv;
     }
-    const size_t o = (size_t)P * st.perP + sym_tile_off(st, ti, tj) +
-                     ((size_t)c * Ri + r) * 64 + (size_t)((j8 ^ (r & 7)) * 8);
-    *(uint4*)(H + o) = *(const uint4*)hv;
-    *(uint4*)(F + o) = *(const uint4*)fv;
   }
 }
 
 // Bt^P 2^-t_P -> integer + fraction planes in the dense storage, [P][mu][ld] (columns
-// nu >= N zero).  One thread per 8 consecutive stored elements of a row.
-__global__ void k_split_B_dense(const double* __restrict__ B, int layout, long long Q, int N,
-                                int ld, const int* __restrict__ eS,
-                                const double* __restrict__ tmax, double invT, __half* H,
-                                __half* F) {
+// nu >= N zero).  A lane per 8 consecutive stored elements of a row; the rows of a slice share
+// a warp when they are short.
+__global__ void __launch_bounds__(256) k_split_B_dense(const double* __restrict__ B, int layout,
+                                                       long long Q, int N, int ld,
+                                                       const int* __restrict__ eS,
+                                                       const int* __restrict__ tP, __half* H,
+                                                       __half* F) {
   const long long npk = (long long)N * (N + 1) / 2;
-  const int n8 = ld / 8;
-  const long long tot = Q * N * n8;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < tot;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int j8 = (int)(i % n8);
-    const long long row = i / n8;  // P * N + mu
-    const long long P = row / N;
-    const int mu = (int)(row % N);
-    const int tP = intfrac_exponent_inv(tmax[P], invT);
+  const int n8 = ld / 8, per = N * n8;  // 8-element pieces of a slice (N <= 256)
+  const int ctas = (per + 255) / 256;
+  for (long long u = blockIdx.x; u < Q * ctas; u += gridDim.x) {
+    const int P = (int)(u / ctas), i = (int)(u - (long long)P * ctas) * 256 + threadIdx.x;
+    if (i >= per) continue;
+    const int mu = i / n8, j8 = i - mu * n8;
+    const int k0 = -tP[P] - eS[mu];
+    const double* Bp = B + (layout == DONOF_B_DENSE ? (size_t)P * N * N : (size_t)P * npk);
     __align__(16) __half hv[8], fv[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int nu = j8 * 8 + k;
-      double y = 0.0;
-      if (nu < N) y = ldexp(load_B_elem(B, layout, P, row, mu, nu, N, npk), -tP - eS[mu] - eS[nu]);
-      intfrac_split(y, hv[k], fv[k]);
+    for (int j = 0; j < 8; ++j) {
+      const int nu = j8 * 8 + j;
+      const double v = nu < N ? load_B_elem(Bp, layout, 0, mu, mu, nu, N, npk) : 0.0;
+      intfrac_split_scaled(v, nu < N ? k0 - eS[nu] : 0, hv[j], fv[j]);
     }
-    const size_t o = (size_t)row * ld + (size_t)j8 * 8;
+    const size_t o = ((size_t)P * N + mu) * ld + (size_t)j8 * 8;
     *(uint4*)(H + o) = *(const uint4*)hv;
     *(uint4*)(F + o) = *(const uint4*)fv;
   }
@@ -1646,35 +1874,38 @@ __global__ void k_reduce_G(const float* __restrict__ Gp, int S, int N, int A, in
 cudaError_t launch_prepare_split_B(const Dims& d, const double* B, char* ws, const Layout& L,
                                    cudaStream_t s) {
   DevHeader* hdr = (DevHeader*)(ws + L.header);
-  cudaError_t e = cudaMemsetAsync(ws + L.L1max, 0, (size_t)d.Q * sizeof(double), s);
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(ws + L.rnmax, 0, (size_t)d.N * sizeof(double), s);
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(ws + L.tmax, 0, (size_t)d.Q * sizeof(double), s);
-  if (e != cudaSuccess) return e;
-  k_b_stats<<<num_sms() * 8, 256, 0, s>>>(B, d.layout, d.Q, d.N, hdr,
-                                          (unsigned long long*)(ws + L.L1max),
-                                          (float*)(ws + L.rn2),
-                                          (unsigned long long*)(ws + L.rnmax));
+  const cudaError_t e0 = cudaMemsetAsync(ws + L.rnmax, 0, (size_t)d.N * sizeof(double), s);
+  if (e0 != cudaSuccess) return e0;
+  int* tP = (int*)(ws + L.tmax);
+  const int* eS = (const int*)(ws + L.eS);
+  const double invT = intfrac_inv_target(d.N);
+  const bool packed = d.layout == DONOF_B_PACKED;
+  if (packed && d.N > kPackedStatsMaxN) return cudaErrorInvalidValue;  // (no B of that size fits)
+  const size_t smem = slice_smem(packed, d.N);
+  const int threads = 32 * slice_warps(packed, d.N), ctas = d.Q < num_sms() * 8 ? d.Q : num_sms() * 8;
+  auto stats = packed ? k_b_stats<true> : k_b_stats<false>;
+  auto scale = packed ? k_p_scale<true> : k_p_scale<false>;
+  if (smem > 48 * 1024 || (size_t)d.N * 4 > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(stats, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(scale, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)((packed ? smem / 4 : 0) + (size_t)d.N * 4));
+    if (e != cudaSuccess) return e;
+  }
+  stats<<<ctas, threads, smem, s>>>(B, d.Q, d.N, hdr, (double*)(ws + L.L1max),
+                                    (float*)(ws + L.rn2), (unsigned long long*)(ws + L.rnmax));
   k_sym_scale<<<1, 1024, 0, s>>>((const double*)(ws + L.rnmax), d.N, (int*)(ws + L.eS));
-  k_p_scale<<<num_sms() * 8, 256, 0, s>>>(B, d.layout, d.Q, d.N, (const int*)(ws + L.eS),
-                                          (unsigned long long*)(ws + L.tmax));
-  k_sym_exps<<<num_sms() * 4, 256, 0, s>>>((const double*)(ws + L.tmax),
-                                           (const int*)(ws + L.eS), d.Q, d.N,
-                                           intfrac_inv_target(d.N), (int*)(ws + L.eB));
+  const size_t smem2 = (packed ? smem / 4 : 0) + (size_t)d.N * 4;
+  scale<<<ctas, threads, smem2, s>>>(B, d.Q, d.N, eS, invT, tP);
+  k_sym_exps<<<num_sms() * 4, 256, 0, s>>>(tP, eS, d.Q, d.N, (int*)(ws + L.eB));
   const SymTiles st = sym_tiles(d.N);
   if (st.dense)
-    k_split_B_dense<<<num_sms() * 8, 256, 0, s>>>(B, d.layout, d.Q, d.N, st.ld,
-                                                  (const int*)(ws + L.eS),
-                                                  (const double*)(ws + L.tmax),
-                                                  intfrac_inv_target(d.N), (__half*)(ws + L.Bhi),
-                                                  (__half*)(ws + L.Blo));
+    k_split_B_dense<<<num_sms() * 8, 256, 0, s>>>(B, d.layout, d.Q, d.N, st.ld, eS, tP,
+                                                  (__half*)(ws + L.Bhi), (__half*)(ws + L.Blo));
   else
-    k_split_B_sym<<<num_sms() * 8, 256, 0, s>>>(B, d.layout, d.Q, d.N, st, hdr,
-                                                (const int*)(ws + L.eS),
-                                                (const double*)(ws + L.tmax),
-                                                intfrac_inv_target(d.N), (__half*)(ws + L.Bhi),
-                                                (__half*)(ws + L.Blo));
+    k_split_B_sym<<<num_sms() * 8, 256, 0, s>>>(B, d.layout, d.Q, d.N, st, eS, tP,
+                                                (__half*)(ws + L.Bhi), (__half*)(ws + L.Blo));
   count_launch(5);
   return cudaGetLastError();
 }
