@@ -300,7 +300,6 @@ inline int dgemm_tile_n(int N) { return (N + 31) / 32 * 32 < (N + 63) / 64 * 64 
 // order of ks (C += sum, so beta must be 1): the result does not depend on scheduling.
 struct DgemmArgs {
   int M, N, K, KB, batch, ksplit, Ktot;
-  int lower;  // 1: only output tiles that reach the lower triangle (m >= n); ksplit == 1
   const double* A; long long sAb, sAm, sAk, sAkb;
   const double* B; long long sBb, sBk, sBn, sBkb;
   double* C; long long sCb, sCm, sCn;
@@ -316,7 +315,7 @@ struct DigitArgs {
   const double* A;
   long long sAb, sAm, sAk, sAkb;
   int M, Mb, Kin, Kpad, KB;
-  const int* eA;        // per row: the largest biased exponent in it (k_row_exp, k_col_exp)
+  const int* eA;        // per row: the largest biased exponent in it, or a larger one; null: 1023
   const __half* Bimg;   // stage images of B (k_digit_planes)
   const int* eB;        // per column, as eA
   int N, NT, ntiles, mtiles, nstages, splits;
@@ -327,6 +326,7 @@ struct DigitArgs {
   // and per m % Mb in exm (atomic maxima; zeroed by the caller)
   int *exq, *exm;
   int exq_ld;
+  int sub;              // C -= A B
   int vecA, vecC;       // 16-byte loads of A / stores of C are aligned
   int *status, *abort_flag;
   uint32_t k64;         // the half2 word 1024, an argument so that it stays in a register
@@ -364,13 +364,20 @@ inline int jk_splits64(int A, int np) {
   if (sp > (np + 7) / 8) sp = (np + 7) / 8;
   return sp < 1 ? 1 : sp;
 }
-// C = A B (M x N, C's rows ldc apart; A(m, k) at m sAm + k sAk, one of the strides 1; B(k, n) at
-// k ldb + n; K <= 16384) with the operands' exponents and B's digits in `scratch`
+// C = A B (M x N, C's rows ldc apart; A(m, k) at m sAm + k sAk, B(k, n) at k sBk + n sBn, one
+// stride of each 1; K <= 16384) with the operands' exponents and B's digits in `scratch`
 // (digit_product_bytes, 256-byte aligned); status and abort_flag: device words of the bounded
 // waits.
 size_t digit_product_bytes(int M, int N, int K);
 cudaError_t digit_product(int M, int N, int K, const double* A, long long sAm, long long sAk,
-                          const double* B, long long ldb, double* C, long long ldc, char* scratch,
+                          const double* B, long long sBk, long long sBn, double* C, long long ldc,
+                          char* scratch, int* status, int* abort_flag, cudaStream_t s);
+// V = Q Z for Q = H_0 .. H_{nref-1} in blocks of 64 reflectors (rows of Yr, unit first element,
+// zeros before it; T: the blocks' triangular factors, 64 x 64 each), Z = V in place, its elements
+// at most 1: per block W = T Y^T Z and Z -= Y W as digit products.  img holds
+// digit_reflect_bytes(N) bytes.
+size_t digit_reflect_bytes(int N);
+cudaError_t digit_reflect(int N, int nref, const double* Yr, const double* T, double* V, char* img,
                           int* status, int* abort_flag, cudaStream_t s);
 // The FP64 path's parts on digit products: the exponents of B's rows, h C_act, one block of
 // slices (X, b, J, K, G; Bblk: its slices, dense), lambda.
@@ -391,6 +398,13 @@ int splitk_count(int M, int N, int K);
 constexpr int kEighMaxN = 4096;
 size_t eigh_workspace_bytes(int N);
 int eigh_run(int N, const double* A, double* V, double* w, char* ws, cudaStream_t s);
+// The part of the solver's workspace that is free between its calls, at least
+// digit_product_bytes(N, N, N), with the status and abort words of bounded waits.
+struct EighScratch {
+  char* mem;
+  int *status, *abort_flag;
+};
+EighScratch eigh_scratch(int N, char* ws);
 int g_splits_fp64(int N, int A, int np);
 // C(m, n) += sum_k A(m, k) B(k, n) with the contraction cut into 64-wide (or 16-wide) chunks
 // shared by enough CTAs to fill the GPU; `part` holds splitk_count(M, N, K) x M x N doubles

@@ -211,7 +211,7 @@ struct Cursor {
     left = -(1 << 30);
     p = a.A;
     if (row < a.M) {
-      e20 = split_exp(__ldg(a.eA + row));
+      e20 = split_exp(a.eA ? __ldg(a.eA + row) : 1023);
       const int b = row / a.Mb, r = row - b * a.Mb;
       p = a.A + (long long)b * a.sAb + (long long)r * a.sAm + (long long)kb * a.sAkb +
           (long long)q * a.sAk;
@@ -395,7 +395,7 @@ __global__ void __launch_bounds__(kDigThreads, 1)
       const int row = m * kTileM + q4 * 32 + lane;
       const bool rv = row < a.M;
       const int b = rv ? row / a.Mb : 0, r = rv ? row - b * a.Mb : 0;
-      const int ea = (rv ? scale_exp(__ldg(a.eA + row)) : 0) - 1086;
+      const int ea = (rv ? (a.eA ? scale_exp(__ldg(a.eA + row)) : 1023) : 0) - 1086;
       double* Crow = a.C + (long long)sp * a.sCs + (long long)b * a.sCb + (long long)r * a.sCm + n0;
       int rmax = 0;
       // exponents of the result per (b, column): the lanes of a warp span one or two b when a
@@ -432,7 +432,7 @@ __global__ void __launch_bounds__(kDigThreads, 1)
           top[h + j] = 0;
           // (columns past N, whose digits are zero, take the last column's exponent)
           v[j] = fixed_to_double(hi, (uint32_t)lo & 0x0fffffffu,
-                                 ea + scale_exp(__ldg(a.eB + (n < a.N ? n : a.N - 1))));
+                                 ea + (a.eB ? scale_exp(__ldg(a.eB + (n < a.N ? n : a.N - 1))) : 1023));
           if (a.exq) {
             const int e = rv ? (__double2hiint(v[j]) >> 20) & 0x7ff : 0;
             rmax = max(rmax, e);
@@ -447,6 +447,11 @@ __global__ void __launch_bounds__(kDigThreads, 1)
               atomicMax(a.exq + (size_t)b * a.exq_ld + n, e);
             }
           }
+        }
+        if (a.sub && rv) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (n0 + h + j < a.N) v[j] = Crow[h + j] - v[j];
         }
         if (rv) {
           if (a.vecC && n0 + h + 3 < a.N) {
@@ -628,10 +633,10 @@ __device__ __forceinline__ void put_planes(const double (&x)[8], int em, uint32_
   });
 }
 
-// Stage images of a matrix S[k ld + n]: a thread per column and 8 elements of k (columns past
-// N and elements past K are zero).
-__global__ void __launch_bounds__(256) k_digit_planes(const double* __restrict__ S, long long ld,
-                                                      int K, int N, uint32_t k64,
+// Stage images of a matrix S[k sk + n sn]: a thread per column and 8 elements of k (columns past
+// N and elements past K are zero; ex null: exponent 1023).
+__global__ void __launch_bounds__(256) k_digit_planes(const double* __restrict__ S, long long sk,
+                                                      long long sn, int K, int N, uint32_t k64,
                                                       const int* __restrict__ ex,
                                                       __half* img, int NT, int ntiles,
                                                       int nstages) {
@@ -643,9 +648,9 @@ __global__ void __launch_bounds__(256) k_digit_planes(const double* __restrict__
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int k = 8 * kc + j;
-      x[j] = (n < N && k < K) ? S[(long long)k * ld + n] : 0.0;
+      x[j] = (n < N && k < K) ? S[(long long)k * sk + (long long)n * sn] : 0.0;
     }
-    put_planes(x, n < N ? ex[n] : 2047, k64, img, img_addr(n, kc, NT, nstages), NT);
+    put_planes(x, n < N ? (ex ? ex[n] : 1023) : 2047, k64, img, img_addr(n, kc, NT, nstages), NT);
   }
 }
 
@@ -895,11 +900,11 @@ cudaError_t launch_exps(const ExpJob* jobs, int count, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_planes(const double* S, long long ld, int K, int N, const int* ex, void* img,
-                          cudaStream_t s) {
+cudaError_t launch_planes(const double* S, long long sk, long long sn, int K, int N, const int* ex,
+                          void* img, cudaStream_t s) {
   const DigitShape sh = digit_shape(N, K);
   k_digit_planes<<<grid_for((long long)sh.NT * sh.ntiles * sh.nstages * 4), 256, 0, s>>>(
-      S, ld, K, N, kK64, ex, (__half*)img, sh.NT, sh.ntiles, sh.nstages);
+      S, sk, sn, K, N, kK64, ex, (__half*)img, sh.NT, sh.ntiles, sh.nstages);
   count_launch(1);
   return cudaGetLastError();
 }
@@ -979,16 +984,18 @@ size_t digit_product_bytes(int M, int N, int K) {
 }
 
 cudaError_t digit_product(int M, int N, int K, const double* A, long long sAm, long long sAk,
-                          const double* B, long long ldb, double* C, long long ldc, char* scratch,
-                          int* status, int* abort_flag, cudaStream_t s) {
+                          const double* B, long long sBk, long long sBn, double* C, long long ldc,
+                          char* scratch, int* status, int* abort_flag, cudaStream_t s) {
   int* eA = (int*)scratch;
   int* eB = (int*)(scratch + align_up((size_t)M * 4));
   char* img = (char*)eB + align_up((size_t)N * 4);
-  CKE(cudaMemsetAsync(scratch, 0, (size_t)(img - scratch), s));
-  ExpJob jobs[2] = {{B, ldb, K, N, 1, eB}, {A, sAm, M, K, 0, eA}};
+  if (sAk != 1 || sBn == 1)  // a matrix read down its columns accumulates maxima
+    CKE(cudaMemsetAsync(scratch, 0, (size_t)(img - scratch), s));
+  ExpJob jobs[2] = {{B, sBk, K, N, 1, eB}, {A, sAm, M, K, 0, eA}};
+  if (sBn != 1) jobs[0] = ExpJob{B, sBn, N, K, 0, eB};
   if (sAk != 1) jobs[1] = ExpJob{A, sAk, K, M, 1, eA};
   CKE(launch_exps(jobs, 2, s));
-  CKE(launch_planes(B, ldb, K, N, eB, img, s));
+  CKE(launch_planes(B, sBk, sBn, K, N, eB, img, s));
   DigitArgs a{};
   a.KB = 1; a.splits = 1;
   a.A = A; a.sAm = sAm; a.sAk = sAk; a.M = M; a.Mb = M; a.Kin = K; a.eA = eA;
@@ -996,6 +1003,139 @@ cudaError_t digit_product(int M, int N, int K, const double* A, long long sAm, l
   a.C = C; a.sCm = ldc;
   a.status = status; a.abort_flag = abort_flag;
   return launch_digit_gemm(a, K, s);
+}
+
+// ------------------------------------------------------------------ reflectors
+namespace {
+constexpr int kRefBlk = 64;   // reflectors per block
+constexpr int kRefCols = 8;   // columns of Z per CTA of k_reflect_w
+// W = T (sum over the splits of part[s][n][c]) for the columns n of Z, c < 64 reflectors, and its
+// stage images (k = c, two stages): the sums and W in shared memory, a thread per reflector and
+// two columns; then a thread per column and 8 reflectors.
+__global__ void __launch_bounds__(256) k_reflect_w(const double* __restrict__ part, int splits,
+                                                   int N, const double* __restrict__ T,
+                                                   uint32_t k64, int* eW, __half* img, int NT,
+                                                   int ntiles) {
+  __shared__ double Ts[kRefBlk][kRefBlk + 1];
+  __shared__ double Ws[kRefCols][kRefBlk], Wt[kRefCols][kRefBlk];
+  const int tid = threadIdx.x, n0 = blockIdx.x * kRefCols;
+  for (int i = tid; i < kRefBlk * kRefBlk; i += 256) Ts[i / kRefBlk][i % kRefBlk] = T[i];
+  for (int i = tid; i < kRefCols * kRefBlk; i += 256) {
+    const int n = n0 + i / kRefBlk, c = i % kRefBlk;
+    double t = 0.0;
+    if (n < N)
+      for (int s = 0; s < splits; ++s) t += part[((size_t)s * N + n) * kRefBlk + c];
+    Ws[i / kRefBlk][c] = t;
+  }
+  __syncthreads();
+  {
+    const int r = tid % kRefBlk, g = tid / kRefBlk * 2;  // T is upper triangular
+    double a0 = 0.0, a1 = 0.0, b0 = 0.0, b1 = 0.0;       // two chains each
+    int c = r;
+    for (; c + 1 < kRefBlk; c += 2) {
+      a0 = fma(Ts[r][c], Ws[g][c], a0);
+      b0 = fma(Ts[r][c], Ws[g + 1][c], b0);
+      a1 = fma(Ts[r][c + 1], Ws[g][c + 1], a1);
+      b1 = fma(Ts[r][c + 1], Ws[g + 1][c + 1], b1);
+    }
+    if (c < kRefBlk) {
+      a0 = fma(Ts[r][c], Ws[g][c], a0);
+      b0 = fma(Ts[r][c], Ws[g + 1][c], b0);
+    }
+    Wt[g][r] = a0 + a1;
+    Wt[g + 1][r] = b0 + b1;
+  }
+  __syncthreads();
+  if (tid < kRefCols * 8) {  // (two whole warps; 8 neighbouring lanes per column)
+    const int j = tid / 8, kc = tid % 8, n = n0 + j;
+    double x[8];
+    int m = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      x[i] = Wt[j][8 * kc + i];
+      m = max(m, exp_field(x[i]));
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (n < N && kc == 0) eW[n] = m;
+    if (n < NT * ntiles) put_planes(x, n < N ? m : 2047, k64, img, img_addr(n, kc, NT, 2), NT);
+  }
+}
+int reflect_splits(int N, int stages) {
+  const int mt = (N + kTileM - 1) / kTileM;
+  int sp = 152 / mt;
+  if (sp > (stages + 1) / 2) sp = (stages + 1) / 2;
+  return sp < 1 ? 1 : sp;
+}
+struct ReflectLayout {
+  size_t y, w, eW, part, total;
+};
+ReflectLayout reflect_layout(int N) {
+  ReflectLayout L{};
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    const size_t o = off;
+    off = align_up(off + bytes);
+    return o;
+  };
+  const DigitShape one = digit_shape(kRefBlk, N);
+  L.y = take((size_t)((N + kRefBlk - 1) / kRefBlk) * one.bytes);
+  L.w = take(digit_shape(N, kRefBlk).bytes);
+  L.eW = take((size_t)N * 4);
+  L.part = take((size_t)reflect_splits(N, one.nstages) * N * kRefBlk * 8);
+  L.total = off;
+  return L;
+}
+}  // namespace
+
+size_t digit_reflect_bytes(int N) { return reflect_layout(N).total; }
+
+cudaError_t digit_reflect(int N, int nref, const double* Yr, const double* T, double* V, char* img,
+                          int* status, int* abort_flag, cudaStream_t s) {
+  const ReflectLayout L = reflect_layout(N);
+  const int nblk = (nref + kRefBlk - 1) / kRefBlk;
+  // every block's reflectors as column tiles of one image over k = 0 .. N - 1 (|y| <= 1)
+  const DigitShape ysh = digit_shape(kRefBlk, N);  // NT 64, one tile per block
+  const int W = nblk * kRefBlk;
+  k_digit_planes<<<grid_for((long long)W * ysh.nstages * 4), 256, 0, s>>>(
+      Yr, 1, N, N, nref, kK64, nullptr, (__half*)(img + L.y), kRefBlk, nblk, ysh.nstages);
+  count_launch(1);
+  CKE(cudaGetLastError());
+  const DigitShape wsh = digit_shape(N, kRefBlk);
+  double* part = (double*)(img + L.part);
+  int* eW = (int*)(img + L.eW);
+  for (int b = nblk - 1; b >= 0; --b) {
+    const int k0 = b * kRefBlk, R0 = k0 + 1;
+    const int st0 = R0 / kStageK, Ra = st0 * kStageK;  // (the rows Ra .. R0 - 1 of Y are zero)
+    const int stages = ysh.nstages - st0;
+    // part[s][n][c] = sum over the split's rows of Z[j][n] Y[j][c]
+    DigitArgs a{};
+    a.KB = 1;
+    a.splits = reflect_splits(N, stages);
+    a.A = V + (size_t)Ra * N; a.sAm = 1; a.sAk = N; a.M = N; a.Mb = N; a.Kin = N - Ra;
+    a.Bimg = (const __half*)(img + L.y) +
+             ((size_t)b * ysh.nstages + st0) * (kD * kRefBlk * kStageK);
+    a.N = kRefBlk;
+    a.C = part; a.sCs = (long long)N * kRefBlk; a.sCm = kRefBlk;
+    a.status = status; a.abort_flag = abort_flag;
+    CKE(launch_digit_gemm(a, N - Ra, s));
+    k_reflect_w<<<(wsh.NT * wsh.ntiles + kRefCols - 1) / kRefCols, 256, 0, s>>>(
+        part, a.splits, N, T + (size_t)b * kRefBlk * kRefBlk, kK64, eW, (__half*)(img + L.w), wsh.NT,
+        wsh.ntiles);
+    count_launch(1);
+    CKE(cudaGetLastError());
+    // Z[R0 ..] -= Y W
+    DigitArgs u{};
+    u.KB = 1;
+    u.splits = 1;
+    u.A = Yr + (size_t)k0 * N + R0; u.sAm = 1; u.sAk = N; u.M = N - R0; u.Mb = N - R0;
+    u.Kin = nref - k0 < kRefBlk ? nref - k0 : kRefBlk;
+    u.Bimg = (const __half*)(img + L.w); u.eB = eW; u.N = N;
+    u.C = V + (size_t)R0 * N; u.sCm = N; u.sub = 1;
+    u.status = status; u.abort_flag = abort_flag;
+    CKE(launch_digit_gemm(u, kRefBlk, s));
+  }
+  return cudaSuccess;
 }
 
 namespace {
@@ -1035,7 +1175,7 @@ cudaError_t digit_hc(const Dims& d, const double* h, const double* C, char* ws, 
     const ExpJob jobs[2] = {{C, N, N, N, 1, (int*)(ws + L.eC64)},
                             {h, N, N, N, 0, (int*)(ws + L.eH64)}};
     CKE(launch_exps(jobs, 2, s));
-    CKE(launch_planes(C, N, N, d.A, (const int*)(ws + L.eC64), ws + L.Cimg, s));
+    CKE(launch_planes(C, N, 1, N, d.A, (const int*)(ws + L.eC64), ws + L.Cimg, s));
   }
   DigitArgs a = digit_args(ws, L);
   a.A = h; a.sAm = N; a.sAk = 1; a.M = N; a.Mb = N; a.Kin = N;
@@ -1132,7 +1272,7 @@ cudaError_t digit_lambda(const Dims& d, const double* C, char* ws, const Layout&
   } else {
     const ExpJob jobs[1] = {{G, A, N, A, 1, eG}};
     CKE(launch_exps(jobs, 1, s));
-    CKE(launch_planes(G, A, N, A, eG, ws + L.Cimg, s));
+    CKE(launch_planes(G, A, 1, N, A, eG, ws + L.Cimg, s));
   }
   DigitArgs a = digit_args(ws, L);
   a.A = C; a.sAm = 1; a.sAk = N; a.M = N; a.Mb = N; a.Kin = N;
@@ -1160,7 +1300,7 @@ extern "C" int donof_testing_digit_product(const double* A, int64_t sAm, int64_t
   cudaStream_t s = (cudaStream_t)stream;
   int* words = (int*)workspace;  // status, abort flag
   if (cudaMemsetAsync(words, 0, kAlign, s) != cudaSuccess ||
-      digit_product(M, N, K, A, sAm, sAk, B, ldb, C, ldc, (char*)workspace + kAlign, words,
+      digit_product(M, N, K, A, sAm, sAk, B, ldb, 1, C, ldc, (char*)workspace + kAlign, words,
                     words + 1, s) != cudaSuccess)
     return DONOF_ERR_CUDA;
   return DONOF_OK;

@@ -34,35 +34,16 @@ __global__ void k_newton_schulz(const double* __restrict__ S, int N, double* M) 
   }
 }
 
-DgemmArgs plain(int M, int N, int K, const double* A, long long sAm, long long sAk,
-                const double* B, long long sBk, long long sBn, double* C, double beta = 0.0) {
-  DgemmArgs a{};
-  a.M = M; a.N = N; a.K = K; a.KB = 1; a.batch = 1; a.ksplit = 1;
-  a.A = A; a.sAm = sAm; a.sAk = sAk;
-  a.B = B; a.sBk = sBk; a.sBn = sBn;
-  a.C = C; a.sCm = N; a.sCn = 1;
-  a.alpha = 1.0; a.beta = beta;
-  return a;
-}
-
-// M[i][j] = M[j][i] for i < j: the upper triangle from the lower one (a symmetric product
-// formed on its lower-triangle tiles only)
-__global__ void k_mirror_lower(double* M, int N) {
-  const long long tot = (long long)N * N;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < tot;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int r = (int)(i / N), c = (int)(i % N);
-    if (r < c) M[i] = M[(size_t)c * N + r];
-  }
-}
-
-// A symmetric product C_out (+)= A B formed on the lower-triangle tiles, then mirrored.
-int sym_product(DgemmArgs a, cudaStream_t s) {
-  a.lower = 1;
-  if (launch_dgemm(a, s) != cudaSuccess) return DONOF_ERR_CUDA;
-  k_mirror_lower<<<152 * 4, 256, 0, s>>>(a.C, a.N);
-  count_launch(1);
-  return cudaGetLastError() == cudaSuccess ? DONOF_OK : DONOF_ERR_CUDA;
+// C = A B to double precision (M x N, row-major; A(m, k) at m sAm + k sAk, B(k, n) at k sBk +
+// n sBn, one stride of each 1), by exact digit products on the tensor cores: 0.17 ms at 1200^3
+// (1.7 ms and more on the FP64 pipe).  The operands' digits go to the eigensolver's workspace,
+// which is free between its calls.
+int product(int M, int N, int K, const double* A, long long sAm, long long sAk, const double* B,
+            long long sBk, long long sBn, double* C, const EighScratch& w, cudaStream_t s) {
+  return digit_product(M, N, K, A, sAm, sAk, B, sBk, sBn, C, N, w.mem, w.status, w.abort_flag, s) ==
+                 cudaSuccess
+             ? DONOF_OK
+             : DONOF_ERR_CUDA;
 }
 
 }  // namespace
@@ -103,14 +84,15 @@ extern "C" int donof_orbital_update(int32_t nbf, const double* lam, const double
   rc = eigh_run(N, F, F, eps, ews, s);
   if (rc != DONOF_OK) return rc;
   // T[mu][j] = sum_i C[mu][i] V[i][j]
-  if (launch_dgemm(plain(N, N, N, C, N, 1, F, N, 1, T), s) != cudaSuccess) return DONOF_ERR_CUDA;
-  // S = T^T T;  M = (3I - S) / 2;  C_new = T M
-  if (sym_product(plain(N, N, N, T, 1, N, T, N, 1, S), s) != DONOF_OK) return DONOF_ERR_CUDA;
+  const EighScratch sc = eigh_scratch(N, ews);
+  if (product(N, N, N, C, N, 1, F, N, 1, T, sc, s) != DONOF_OK) return DONOF_ERR_CUDA;
+  // S = T^T T (both triangles from the same digits: exactly symmetric);  M = (3I - S) / 2;
+  // C_new = T M
+  if (product(N, N, N, T, 1, N, T, N, 1, S, sc, s) != DONOF_OK) return DONOF_ERR_CUDA;
   k_newton_schulz<<<152 * 4, 256, 0, s>>>(S, N, S);
   count_launch(1);
   if (cudaGetLastError() != cudaSuccess) return DONOF_ERR_CUDA;
-  if (launch_dgemm(plain(N, N, N, T, N, 1, S, N, 1, C_new), s) != cudaSuccess)
-    return DONOF_ERR_CUDA;
+  if (product(N, N, N, T, N, 1, S, N, 1, C_new, sc, s) != DONOF_OK) return DONOF_ERR_CUDA;
   prof_end(DONOF_PHASE_ORBITAL_UPDATE, s);
   return DONOF_OK;
 }
@@ -145,7 +127,6 @@ struct Slots {
 
 struct OptLayout {
   size_t lam, Emo, T1, T2, Fbar, hist, eps, scal, B, c, work;
-  size_t skp;  // split-K partials of R_a C^T (nact x N)
   size_t total;
 };
 
@@ -169,8 +150,7 @@ int opt_layout(int N, int A, int depth, OptLayout* o) {
   o->B = take((size_t)kMaxDepth * kMaxDepth * 8);
   o->c = take((size_t)(kMaxDepth + 2) * 8);  // c[0..n]; the restart flag kept at [kMaxDepth + 1]
   o->work = take(eigh_workspace_bytes(N));  // the eigensolver's workspace
-  const int ks = splitk_count(A, N, N);
-  o->skp = take(ks > 1 ? (size_t)ks * A * N * 8 : 0);
+  (void)A;
   o->total = off;
   return DONOF_OK;
 }
@@ -218,6 +198,17 @@ __global__ void k_sym_sum(const double* __restrict__ Z, int N, double* S) {
        i += (long long)gridDim.x * blockDim.x) {
     const int r = (int)(i / N), c = (int)(i % N);
     S[i] = Z[i] + Z[(size_t)c * N + r];
+  }
+}
+
+// S = E + P with the lower triangle of P for both (E symmetric)
+__global__ void k_add_lower(const double* __restrict__ E, const double* __restrict__ P, int N,
+                            double* S) {
+  const long long tot = (long long)N * N;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < tot;
+       i += (long long)gridDim.x * blockDim.x) {
+    const int r = (int)(i / N), c = (int)(i % N);
+    S[i] = E[i] + (r >= c ? P[i] : P[(size_t)c * N + r]);
   }
 }
 
@@ -394,11 +385,11 @@ int loop_reorthonormalise(Loop& lp) {
   const int N = lp.N;
   double* T1 = (double*)(lp.ows + lp.L.T1);
   double* T2 = (double*)(lp.ows + lp.L.T2);
-  if (sym_product(plain(N, N, N, lp.C, 1, N, lp.C, N, 1, T1), lp.s) != DONOF_OK)
-    return DONOF_ERR_CUDA;
+  const EighScratch sc = eigh_scratch(N, lp.ows + lp.L.work);
+  if (product(N, N, N, lp.C, 1, N, lp.C, N, 1, T1, sc, lp.s) != DONOF_OK) return DONOF_ERR_CUDA;
   k_newton_schulz<<<152 * 4, 256, 0, lp.s>>>(T1, N, T1);
   count_launch(1);
-  if (!ok(launch_dgemm(plain(N, N, N, lp.C, N, 1, T1, N, 1, T2), lp.s))) return DONOF_ERR_CUDA;
+  if (product(N, N, N, lp.C, N, 1, T1, N, 1, T2, sc, lp.s) != DONOF_OK) return DONOF_ERR_CUDA;
   if (!ok(cudaMemcpyAsync(lp.C, T2, (size_t)N * N * 8, cudaMemcpyDeviceToDevice, lp.s)))
     return DONOF_ERR_CUDA;
   return DONOF_OK;
@@ -432,21 +423,19 @@ int loop_orbital_step(Loop& lp, double zeta, int depth, std::vector<int>& active
   double* W = (double*)(o + lp.L.T2);  // R_a C^T, nact x N
   k_halve_block<<<152, 256, 0, lp.s>>>(Emo, N, A);
   count_launch(1);
-  if (!ok(cudaMemsetAsync(W, 0, (size_t)A * N * 8, lp.s)) ||
-      !ok(launch_dgemm(split_k_args(A, N, N, Emo, N, 1, lp.C, 1, N, W, N, 1,
-                                    (double*)(o + lp.L.skp)),
-                       lp.s)) ||
-      !ok(launch_dgemm(plain(N, N, A, lp.C, N, 1, W, N, 1, T1), lp.s)))
+  const EighScratch sc = eigh_scratch(N, o + lp.L.work);
+  if (product(A, N, N, Emo, N, 1, lp.C, 1, N, W, sc, lp.s) != DONOF_OK ||
+      product(N, N, A, lp.C, N, 1, W, N, 1, T1, sc, lp.s) != DONOF_OK)
     return DONOF_ERR_CUDA;
   k_sym_sum<<<152 * 4, 256, 0, lp.s>>>(T1, N, e_ao);
   count_launch(1);
-  // F_AO = e_AO + (C diag(Fdiag)) C^T, symmetric
+  // F_AO = e_AO + (C diag(Fdiag)) C^T, symmetric: the lower triangle of the product for both
   k_scale_cols<<<152 * 4, 256, 0, lp.s>>>(lp.C, lp.Fdiag, N, T1);
   count_launch(1);
-  if (!ok(cudaMemcpyAsync(F_ao, e_ao, nn * 8, cudaMemcpyDeviceToDevice, lp.s)) ||
-      sym_product(plain(N, N, N, T1, N, 1, lp.C, 1, N, F_ao, 1.0), lp.s) != DONOF_OK ||
-      !ok(cudaMemsetAsync(c + kMaxDepth + 1, 0, 8, lp.s)))
-    return DONOF_ERR_CUDA;
+  if (product(N, N, N, T1, N, 1, lp.C, 1, N, W, sc, lp.s) != DONOF_OK) return DONOF_ERR_CUDA;
+  k_add_lower<<<152 * 4, 256, 0, lp.s>>>(e_ao, W, N, F_ao);
+  count_launch(1);
+  if (!ok(cudaMemsetAsync(c + kMaxDepth + 1, 0, 8, lp.s))) return DONOF_ERR_CUDA;
   Slots sl{};
   sl.n = (int)active.size();
   for (int i = 0; i < sl.n; ++i) sl.idx[i] = active[i];
@@ -499,7 +488,7 @@ int loop_initial_diagonal(Loop& lp) {
   const int rc = eigh_run(N, S, S, (double*)(o + lp.L.eps), o + lp.L.work, lp.s);
   if (rc != DONOF_OK) return rc;
   // T1 = C V, V[i][j] = S[i * N + j] (ascending eigenvalues)
-  if (!ok(launch_dgemm(plain(N, N, N, lp.C, N, 1, S, N, 1, T1), lp.s)) ||
+  if (product(N, N, N, lp.C, N, 1, S, N, 1, T1, eigh_scratch(N, o + lp.L.work), lp.s) != DONOF_OK ||
       !ok(cudaMemcpyAsync(lp.C, T1, (size_t)N * N * 8, cudaMemcpyDeviceToDevice, lp.s)))
     return DONOF_ERR_CUDA;
   k_negate<<<8, 256, 0, lp.s>>>((const double*)(o + lp.L.eps), N, lp.Fdiag);
