@@ -465,31 +465,37 @@ int run_build(const donof_problem* prob, const double* h, const double* B, const
   const size_t AA = (size_t)A * A * 8;
 
   prof_begin(DONOF_PHASE_PREP, s);
-  CK(cudaMemsetAsync(&((DevHeader*)(ws + L.header))->abort_flag, 0, sizeof(int32_t), s));
-  CK(launch_occupations(d, gamma, pair_map, ws, L, s));
-  CK(launch_coefficients(d, pair_map, ws, L, s));
-  // hC = h C_act (FP64 DGEMM, or on the tensor cores with residual-extended operands), then
-  // H_pp and G = n o hC
+  // what the build accumulates into or writes only in part
+  ZeroJob zero{};
+  zero.flag = &((DevHeader*)(ws + L.header))->abort_flag;
+  zero.add(ws + L.dn, L.dphi + (size_t)A * d.ng * 8 - L.dn);  // the three Jacobians, in a row
+  if (mode != kFinish && !d.digit) zero.add(ws + L.J, L.K + AA - L.J);  // K follows J
+  if (d.precision == DONOF_MIXED) zero.add(&((DevHeader*)(ws + L.header))->sC2, 8);
+  // hC = h C_act (FP64 DGEMM, or on the tensor cores with residual-extended operands, or as digit
+  // products), then H_pp and G = n o hC
   if (d.precision == DONOF_MIXED) {
-    CK(launch_split_C(d, C, h, ws, L, mode != kFinish, s));
+    CK(launch_split_C(d, C, h, ws, L, mode != kFinish, zero, s));
     rc = run_hc_tc(d, ws, L, s);
     if (rc != DONOF_OK) return rc;
-    // bound on ||C_act||_2 for the exponents of X in the G contraction
-    if (mode != kFinish) CK(launch_gram_bound(d, C, ws, L, s));
   } else if (d.digit) {
-    CK(digit_hc(d, h, C, ws, L, s));
+    CK(digit_hc(d, h, C, ws, L, zero, s));
   } else {
+    CK(cudaMemsetAsync(zero.flag, 0, sizeof(int32_t), s));
+    for (int i = 0; i < 4; ++i)
+      if (zero.n[i] > 0) CK(cudaMemsetAsync(zero.p[i], 0, (size_t)zero.n[i] * 8, s));
     CK(cudaMemsetAsync(ws + L.hC, 0, (size_t)N * A * 8, s));
     CK(launch_dgemm(split_k_args(N, A, N, h, N, 1, C, N, 1, (double*)(ws + L.hC), A, 1,
                                  (double*)(ws + L.skp)), s));
   }
+  CK(launch_occupations(d, gamma, pair_map, ws, L, s));
+  CK(launch_coefficients(d, pair_map, ws, L, s));
+  // bound on ||C_act||_2 for the exponents of X in the G contraction
+  if (d.precision == DONOF_MIXED && mode != kFinish) CK(launch_gram_bound(d, C, ws, L, s));
   CK(launch_hdiag_ginit(d, C, ws, L, mode != kPartial, s));
   if (mode == kFinish) {  // the summed two-electron parts of every shard
     CK(cudaMemcpyAsync(ws + L.J, partial, AA, cudaMemcpyDeviceToDevice, s));
     CK(cudaMemcpyAsync(ws + L.K, partial + (size_t)A * A, AA, cudaMemcpyDeviceToDevice, s));
     CK(launch_add((double*)(ws + L.G), partial + 2 * (size_t)A * A, (long long)N * A, s));
-  } else if (!d.digit) {  // (the digit products' first block sets J and K)
-    CK(cudaMemsetAsync(ws + L.J, 0, L.K + AA - L.J, s));  // K follows J
   }
   prof_end(DONOF_PHASE_PREP, s);
 
@@ -569,13 +575,13 @@ int run_build(const donof_problem* prob, const double* h, const double* B, const
   prof_begin(DONOF_PHASE_ENERGY_LAMBDA, s);
   CK(launch_energy(d, pair_map, ws, L, E, dE_dgamma, s));
   if (lam) {  // lambda_qp = C_q^T G_p (q < N, p < nact), zero for p >= nact
-    CK(cudaMemsetAsync(lam, 0, (size_t)N * N * 8, s));
     if (d.precision == DONOF_MIXED) {
       rc = run_lambda_tc(d, C, ws, L, lam, s);
       if (rc != DONOF_OK) return rc;
     } else if (d.digit) {
       CK(digit_lambda(d, C, ws, L, lam, s));
     } else {
+      CK(cudaMemsetAsync(lam, 0, (size_t)N * N * 8, s));
       CK(launch_dgemm(split_k_args(N, A, N, C, 1, N, (const double*)(ws + L.G), A, 1, lam, N, 1,
                                    (double*)(ws + L.skp)),
                       s));

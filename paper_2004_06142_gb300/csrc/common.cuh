@@ -2,6 +2,7 @@
 // Nothing here is part of the C ABI (include/donof.h is).
 #pragma once
 
+#include <utility>
 #include <cuda_runtime.h>
 #include <cuda_fp16.h>
 #include <stdint.h>
@@ -103,6 +104,64 @@ __host__ __device__ inline SymTiles sym_tiles(int N) {
 }
 
 // ---------------------------------------------------------------------------
+// Chained launches (programmatic dependent launch).  A build is a chain of some 25 kernels, most
+// of them a few microseconds long on the small molecules, and between two of them a plain launch
+// leaves the chip idle while the first one drains and the next one is set up.  A chained kernel is
+// set up while the one before it runs: every kernel of the chain lets its successor be launched as
+// soon as its own CTAs are resident (the contractions: as they leave, because CTAs parked beside
+// one slow it down), and waits before its first access to memory until the kernel before it is
+// complete and its writes are visible.  The wait is transitive, as each kernel completes only after
+// its own wait.  A call's first kernel is launched plainly, so that nothing is assumed of the
+// caller's kernels; behind a copy or a memset a chained launch is a plain one.  The tridiagonal
+// reduction, whose CTAs wait on one another, takes no part.  24 / 96 / 10 orbitals, mixed: 157 ->
+// 115 us a build and adjoint; 97 / 331 / 19, double, with integrals: 216 -> 183.
+//
+// Only grids of up to kChainCtas CTAs (two per SM) are chained: the CTAs of a chained kernel are
+// placed where the kernel before leaves room, unevenly, which costs wide kernels more than the gap
+// (500 / 2000 / 80: J, K and Y with 785 and 1216 CTAs 86 us plainly, 154 chained).  The same holds
+// for the fp16 contractions that fill the chip, which find the units of their neighbours in L2
+// (launch_tc).  Grouped launches are wide and stay plain (64 instances: 1778 us, 1820 chained).
+// ---------------------------------------------------------------------------
+// First statement of a chained kernel (a plainly launched one passes through).  Returns 0, through
+// the wait: loads through read-only pointers may be moved over a memory clobber, so that every such
+// load has to take its address from this value (the block's coordinates, Blk::zero).
+__device__ __forceinline__ int chain_begin() {
+  int z;
+  asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;\n\tmov.u32 %0, 0;"
+               : "=r"(z)
+               :
+               : "memory");
+  return z;
+}
+// The same for a kernel whose successor is launched only as its CTAs leave.
+__device__ __forceinline__ int chain_wait() {
+  int z;
+  asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(z) : : "memory");
+  return z;
+}
+constexpr int kChainCtas = 304;
+template <class... P, class... Args>
+cudaError_t launch_chained_to(int max_ctas, void (*kernel)(P...), dim3 grid, dim3 block,
+                              size_t smem, cudaStream_t s, Args&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = (long long)grid.x * grid.y * grid.z <= max_ctas ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+template <class... P, class... Args>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                           cudaStream_t s, Args&&... args) {
+  return launch_chained_to(kChainCtas, kernel, grid, block, smem, s, std::forward<Args>(args)...);
+}
+
+// ---------------------------------------------------------------------------
 // Grouped launches (batch.cu): one launch runs a kernel for every instance of a batch.  A
 // kernel body takes its block coordinates as a Blk (the native ones for a single instance);
 // in a grouped launch instance i owns the blocks [start[i], start[i+1]) of the flat grid,
@@ -110,10 +169,12 @@ __host__ __device__ inline SymTiles sym_tiles(int N) {
 // ---------------------------------------------------------------------------
 struct Blk {
   int x, y, z, gx, gy, gz;
+  int zero;  // 0, known only once the kernels before are complete (chain_begin)
 };
 __device__ __forceinline__ Blk native_blk() {
-  return Blk{(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z,
-             (int)gridDim.x,  (int)gridDim.y,  (int)gridDim.z};
+  const int z = chain_begin();
+  return Blk{(int)blockIdx.x + z, (int)blockIdx.y + z, (int)blockIdx.z + z,
+             (int)gridDim.x,      (int)gridDim.y,      (int)gridDim.z,      z};
 }
 // One instance of a batch: its sizes, workspace carving and pointers.
 struct InstRec {
@@ -148,7 +209,33 @@ __device__ __forceinline__ int group_locate(const GroupLaunch& g, Blk& b) {
   b.gx = gx;
   b.gy = gy;
   b.gz = gz;
+  b.zero = 0;
   return lo;
+}
+
+// What a build accumulates into or writes only in part, cleared by spare CTAs of its first kernel
+// (a memset each was a launch and broke the chain; 24 / 96 / 10 orbitals, mixed: 115 -> 109 us a
+// build and adjoint).
+struct ZeroJob {
+  int* flag;          // one word, may be null
+  double* p[4];       // n[i] doubles each (0: none)
+  long long n[4];
+  __host__ void add(void* at, size_t bytes) {
+    for (int i = 0; i < 4; ++i)
+      if (n[i] == 0) {
+        p[i] = (double*)at;
+        n[i] = (long long)(bytes / 8);
+        return;
+      }
+  }
+};
+__device__ __forceinline__ void zero_ranges(const ZeroJob& z, int cta, int ctas) {
+  if (z.flag && cta == 0 && threadIdx.x == 0) *z.flag = 0;
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+    for (long long i = cta * (long long)blockDim.x + threadIdx.x; i < z.n[r];
+         i += (long long)ctas * blockDim.x)
+      z.p[r][i] = 0.0;
 }
 
 // The K and J partials' entries (q, p0..p0+3) on and below the diagonal (p0 <= q, p0 a
@@ -384,7 +471,7 @@ cudaError_t digit_reflect(int N, int nref, const double* Yr, const double* T, do
 cudaError_t digit_prepare_B(const Dims& d, const double* B, char* ws, const Layout& L,
                             cudaStream_t s);
 cudaError_t digit_hc(const Dims& d, const double* h, const double* C, char* ws, const Layout& L,
-                     cudaStream_t s);
+                     ZeroJob zero, cudaStream_t s);
 int digit_block(const Dims& d, const double* Bblk, int p0, int np, char* ws, const Layout& L,
                 cudaStream_t s);
 cudaError_t digit_lambda(const Dims& d, const double* C, char* ws, const Layout& L, double* lam,
@@ -413,6 +500,7 @@ DgemmArgs split_k_args(int M, int N, int K, const double* A, long long sAm, long
                        const double* B, long long sBk, long long sBn, double* C, long long sCm,
                        long long sCn, double* part);
 
+// (the Jacobians are zero already)
 cudaError_t launch_occupations(const Dims& d, const double* gamma, const int32_t* pair_map,
                                char* ws, const Layout& L, cudaStream_t s);
 cudaError_t launch_coefficients(const Dims& d, const int32_t* pair_map, char* ws, const Layout& L,
@@ -448,7 +536,8 @@ cudaError_t launch_prepare_split_B(const Dims& d, const double* B, char* ws, con
 // with_half_transform = false leaves out the operand of the half transform (its exponents
 // come from the prepared B), for a build that runs no contraction over B.
 cudaError_t launch_split_C(const Dims& d, const double* C, const double* h, char* ws,
-                           const Layout& L, bool with_half_transform, cudaStream_t s);
+                           const Layout& L, bool with_half_transform, const ZeroJob& zero,
+                           cudaStream_t s);
 // hC = h C_act on the tensor cores from the planes written by launch_split_C (mixed path).
 int run_hc_tc(const Dims& d, char* ws, const Layout& L, cudaStream_t s);
 cudaError_t launch_reduce_G(const Dims& d, char* ws, const Layout& L, cudaStream_t s);

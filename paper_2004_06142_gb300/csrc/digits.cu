@@ -193,16 +193,16 @@ struct Cursor {
   uint32_t e20;    // split_exp of the row
   const double* p;
   int kb;
-  __device__ __forceinline__ Cursor(const DigitArgs& a, int units) {
-    u = (int)blockIdx.x;
+  __device__ __forceinline__ Cursor(const DigitArgs& a, int units, int zero) {
+    u = (int)blockIdx.x;  // (warp-uniform; the addresses of the first loads carry `zero`)
     st = st_end = 0;
-    if (u < units) enter(a);
+    if (u < units) enter(a, zero);
   }
-  __device__ __forceinline__ void enter(const DigitArgs& a) {
+  __device__ __forceinline__ void enter(const DigitArgs& a, int zero = 0) {
     const int m = (u / a.ntiles) % a.mtiles, sp = u / (a.ntiles * a.mtiles);
     st = (int)((long long)a.nstages * sp / a.splits);
     st_end = (int)((long long)a.nstages * (sp + 1) / a.splits);
-    const int tid = (int)threadIdx.x;
+    const int tid = (int)threadIdx.x + zero;
     const int row = m * kTileM + (KC ? tid >> 2 : tid & 127);
     const long long kk = (long long)st * kStageK + 8 * (KC ? tid & 3 : tid >> 7);
     kb = (int)(kk / a.Kpad);
@@ -280,6 +280,8 @@ __global__ void __launch_bounds__(kDigThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *(volatile uint32_t*)tmem_slot;
+  // all of the above while the kernel before runs
+  const int zero = chain_wait();
 
   if (warp == kWorkers) {
     if (lane == 0) {  // ------------------------------------------------ MMA issuer
@@ -343,7 +345,7 @@ __global__ void __launch_bounds__(kDigThreads, 1)
     int top[kCols];
 #pragma unroll
     for (int j = 0; j < kCols; ++j) top[j] = 0;
-    Cursor<KC> cur(a, units);
+    Cursor<KC> cur(a, units, zero);
     double x[8];
     if (cur.u < units) cur.load(a, x);
     uint32_t it = 0, nflush = 0;
@@ -551,13 +553,14 @@ constexpr int kExpRows = 64;  // rows of a column job per CTA
 __device__ __forceinline__ int exp_field(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
 
 __global__ void __launch_bounds__(256) k_exps(ExpJobs jobs) {
-  const ExpJob jb = jobs.j[blockIdx.y];
+  const int z = chain_begin(), bx = (int)blockIdx.x + z;
+  const ExpJob jb = jobs.j[blockIdx.y + z];
   const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
   if (jb.by_col) {
     __shared__ int red[8][32];
     const int ncb = (jb.cols + 31) / 32;
     const long long tiles = (long long)ncb * ((jb.rows + kExpRows - 1) / kExpRows);
-    for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
+    for (long long t = bx; t < tiles; t += gridDim.x) {
       const int c = (int)(t % ncb) * 32 + tx;
       const long long r0 = t / ncb * kExpRows;
       int m = 0;
@@ -578,7 +581,7 @@ __global__ void __launch_bounds__(256) k_exps(ExpJobs jobs) {
       __syncthreads();
     }
   } else {
-    for (long long r = (long long)blockIdx.x * 8 + ty; r < jb.rows; r += (long long)gridDim.x * 8) {
+    for (long long r = (long long)bx * 8 + ty; r < jb.rows; r += (long long)gridDim.x * 8) {
       const double* row = jb.S + r * jb.ld;
       int m = 0;
 #pragma unroll 4
@@ -593,9 +596,10 @@ __global__ void __launch_bounds__(256) k_exps(ExpJobs jobs) {
 // slice's maxima in shared memory (in the output itself when N is too large for it).
 __global__ void __launch_bounds__(256) k_packed_exps(const double* __restrict__ Bp, int Q, int N,
                                                      int in_smem, int* out) {
+  const int z = chain_begin(), bx = (int)blockIdx.x + z;
   extern __shared__ int sh_max[];
   const long long npk = (long long)N * (N + 1) / 2;
-  for (int P = blockIdx.x; P < Q; P += gridDim.x) {
+  for (int P = bx; P < Q; P += gridDim.x) {
     int* ex = in_smem ? sh_max : out + (size_t)P * N;
     for (int i = threadIdx.x; i < N; i += 256) ex[i] = 0;
     __syncthreads();
@@ -640,9 +644,10 @@ __global__ void __launch_bounds__(256) k_digit_planes(const double* __restrict__
                                                       const int* __restrict__ ex,
                                                       __half* img, int NT, int ntiles,
                                                       int nstages) {
+  const int z = chain_begin(), bx = (int)blockIdx.x + z;
   const int W = NT * ntiles;
   const long long tot = (long long)W * nstages * 4;
-  for (long long i = blockIdx.x * 256ll + threadIdx.x; i < tot; i += 256ll * gridDim.x) {
+  for (long long i = bx * 256ll + threadIdx.x; i < tot; i += 256ll * gridDim.x) {
     const int kc = (int)(i / W), n = (int)(i - (long long)kc * W);
     double x[8];
 #pragma unroll
@@ -657,17 +662,22 @@ __global__ void __launch_bounds__(256) k_digit_planes(const double* __restrict__
 // The same with the exponents found on the way, for K <= kFuseK: a CTA per 32 columns passes over
 // them twice (the second time from L1 or L2), so that a short product needs one launch less;
 // the CTAs from col_ctas on find the rows' exponents of a second matrix (R, rows of `rows_k`
-// elements), a warp per row.
+// elements), a warp per row, and those behind them clear `zero`.
 constexpr int kFuseK = 640;
 __global__ void __launch_bounds__(256) k_exps_planes(const double* __restrict__ S, long long ld,
                                                      int K, int ncols, int N, uint32_t k64,
                                                      int* ex, __half* img, int NT, int nstages,
                                                      int col_ctas, const double* __restrict__ R,
-                                                     int rows, int rows_k, int* ex_rows) {
+                                                     int rows, int rows_k, int* ex_rows,
+                                                     int row_ctas, const ZeroJob zero) {
+  const int z = chain_begin(), bx = (int)blockIdx.x + z;
   const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
-  if ((int)blockIdx.x >= col_ctas) {
-    for (int r = ((int)blockIdx.x - col_ctas) * 8 + ty; r < rows;
-         r += ((int)gridDim.x - col_ctas) * 8) {
+  if (bx >= col_ctas + row_ctas) {
+    zero_ranges(zero, bx - col_ctas - row_ctas, (int)gridDim.x - col_ctas - row_ctas);
+    return;
+  }
+  if (bx >= col_ctas) {
+    for (int r = (bx - col_ctas) * 8 + ty; r < rows; r += row_ctas * 8) {
       int m = 0;
 #pragma unroll 4
       for (int c = tx; c < rows_k; c += 32) m = max(m, exp_field(__ldg(R + (long long)r * rows_k + c)));
@@ -677,7 +687,7 @@ __global__ void __launch_bounds__(256) k_exps_planes(const double* __restrict__ 
     return;
   }
   __shared__ int red[8][32];
-  const int n = (int)blockIdx.x * 32 + tx;  // columns past N: to the width of the images
+  const int n = bx * 32 + tx;  // columns past N: to the width of the images
   int m = 0;
   if (n < ncols) {
 #pragma unroll 4
@@ -709,13 +719,14 @@ __global__ void __launch_bounds__(256) k_w_jk64(const double* __restrict__ b, in
                                                 const double* __restrict__ Ac, double* W,
                                                 int* wmax, int w_ctas, int splits, double* part,
                                                 int* bmax) {
+  const int z = chain_begin(), bx = (int)blockIdx.x + z;
   extern __shared__ double dv[];
-  if ((int)blockIdx.x < w_ctas) {
-    for (int P = blockIdx.x; P < np; P += w_ctas) {
+  if (bx < w_ctas) {
+    for (int P = bx; P < np; P += w_ctas) {
       const double* bp = b + (size_t)P * A * A;
       for (int r = threadIdx.x; r < A; r += 256) dv[r] = bp[(size_t)r * A + r];
       __syncthreads();
-      for (int p = threadIdx.x; p < A; p += 256) {
+      for (int p = threadIdx.x + z; p < A; p += 256) {
         double w[4] = {0.0, 0.0, 0.0, 0.0};  // four chains: the FP64 latency bounds this part
         const double* row = Ac + p;          // Acoef is symmetric: read down its columns
         int r = 0;
@@ -732,7 +743,7 @@ __global__ void __launch_bounds__(256) k_w_jk64(const double* __restrict__ b, in
     }
     return;
   }
-  const int cta = (int)blockIdx.x - w_ctas, split = cta % splits;
+  const int cta = bx - w_ctas, split = cta % splits;
   const int tri = A * (A + 1) / 2, i = cta / splits * 256 + threadIdx.x;
   if (i >= tri) return;
   int p = (int)((sqrtf(8.0f * (float)i + 1.0f) - 1.0f) * 0.5f);
@@ -783,9 +794,10 @@ __global__ void __launch_bounds__(256) k_jk_final64(const double* __restrict__ p
                                                     const int* __restrict__ wmax, double* J,
                                                     double* K, int* eY, int jk_blocks,
                                                     int first) {
+  const int z = chain_begin(), bx = (int)blockIdx.x + z;
   const int tri = A * (A + 1) / 2;
-  if ((int)blockIdx.x < jk_blocks) {
-    const int i = blockIdx.x * 256 + threadIdx.x;
+  if (bx < jk_blocks) {
+    const int i = bx * 256 + threadIdx.x;
     if (i >= tri) return;
     int p = (int)((sqrtf(8.0f * (float)i + 1.0f) - 1.0f) * 0.5f);
     while (p * (p + 1) / 2 > i) --p;
@@ -807,7 +819,7 @@ __global__ void __launch_bounds__(256) k_jk_final64(const double* __restrict__ p
     }
     return;
   }
-  const int p = ((int)blockIdx.x - jk_blocks) * 8 + threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int p = (bx - jk_blocks) * 8 + threadIdx.x / 32, lane = threadIdx.x % 32;
   if (p >= A) return;
   // 2^(f - 1022) bounds every |Y_qp|, f = e(Bcoef) + e(b) - 1022 for a product, one more for
   // the rounding of b_qp against b_pq and one for the sum with w
@@ -829,9 +841,10 @@ __global__ void __launch_bounds__(256) k_y_planes(const double* __restrict__ b, 
                                                   const double* __restrict__ W,
                                                   const int* __restrict__ eY, __half* img, int NT,
                                                   int ntiles, int nstages) {
+  const int z = chain_begin(), bx = (int)blockIdx.x + z;
   const int Wd = NT * ntiles;
   const long long tot = (long long)Wd * nstages * 4;
-  for (long long i = blockIdx.x * 256ll + threadIdx.x; i < tot; i += 256ll * gridDim.x) {
+  for (long long i = bx * 256ll + threadIdx.x; i < tot; i += 256ll * gridDim.x) {
     const int kc = (int)(i / Wd), n = (int)(i - (long long)kc * Wd);
     const int P = (int)(8ll * kc / Kpad), q0 = (int)(8ll * kc - (long long)P * Kpad);
     double x[8];
@@ -852,9 +865,10 @@ __global__ void __launch_bounds__(256) k_y_planes(const double* __restrict__ b, 
 // split, their sums added in order.
 __global__ void __launch_bounds__(256) k_split_sum(const double* __restrict__ part, int splits,
                                                    long long tot, double* C) {
+  const int z = chain_begin(), bx = (int)blockIdx.x + z;
   __shared__ double red[8][32];
   const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
-  const long long i = blockIdx.x * 32ll + tx;
+  const long long i = bx * 32ll + tx;
   double t = 0.0;
   if (i < tot) {
 #pragma unroll 4
@@ -895,7 +909,7 @@ cudaError_t launch_exps(const ExpJob* jobs, int count, cudaStream_t s) {
                                        : (jobs[i].rows + 7) / 8;
     if (t > nb) nb = t;
   }
-  k_exps<<<dim3((unsigned)(nb < 152 * 8 ? nb : 152 * 8), count), 256, 0, s>>>(js);
+  launch_chained(k_exps, dim3((unsigned)(nb < 152 * 8 ? nb : 152 * 8), count), 256, 0, s, js);
   count_launch(1);
   return cudaGetLastError();
 }
@@ -903,22 +917,26 @@ cudaError_t launch_exps(const ExpJob* jobs, int count, cudaStream_t s) {
 cudaError_t launch_planes(const double* S, long long sk, long long sn, int K, int N, const int* ex,
                           void* img, cudaStream_t s) {
   const DigitShape sh = digit_shape(N, K);
-  k_digit_planes<<<grid_for((long long)sh.NT * sh.ntiles * sh.nstages * 4), 256, 0, s>>>(
+  launch_chained(k_digit_planes, grid_for((long long)sh.NT * sh.ntiles * sh.nstages * 4), 256, 0, s,
       S, sk, sn, K, N, kK64, ex, (__half*)img, sh.NT, sh.ntiles, sh.nstages);
   count_launch(1);
   return cudaGetLastError();
 }
 
-// ncols columns' exponents and the planes of the first N, K <= kFuseK; rows' exponents of R.
+// ncols columns' exponents and the planes of the first N, K <= kFuseK; rows' exponents of R; zero
+// cleared.  `first`: the first launch of a call.
 cudaError_t launch_exps_planes(const double* S, long long ld, int K, int ncols, int N, int* ex,
                                void* img, const double* R, int rows, int rows_k, int* ex_rows,
-                               cudaStream_t s) {
+                               const ZeroJob& zero, bool first, cudaStream_t s) {
   const DigitShape sh = digit_shape(N, K);
   const int width = ncols > sh.NT * sh.ntiles ? ncols : sh.NT * sh.ntiles;
-  const int cc = (width + 31) / 32;
-  k_exps_planes<<<cc + (rows + 7) / 8, 256, 0, s>>>(S, ld, K, ncols, N, kK64, ex, (__half*)img,
-                                                    sh.NT, sh.nstages, cc, R, rows, rows_k,
-                                                    ex_rows);
+  const int cc = (width + 31) / 32, rc = (rows + 7) / 8;
+  long long nz = 0;
+  for (int i = 0; i < 4; ++i) nz += zero.n[i];
+  const int zc = (int)(nz < 2048 * 32 ? (nz + 2047) / 2048 : 32);
+  launch_chained_to(first ? 0 : kChainCtas, k_exps_planes, cc + rc + (zero.flag && !zc ? 1 : zc),
+                    256, 0, s, S, ld, K, ncols, N, kK64, ex, (__half*)img, sh.NT, sh.nstages, cc, R,
+                    rows, rows_k, ex_rows, rc, zero);
   count_launch(1);
   return cudaGetLastError();
 }
@@ -963,7 +981,7 @@ cudaError_t launch_digit_gemm(DigitArgs a, long long K, cudaStream_t s) {
       if (e != cudaSuccess) return e;
       mask |= bit;
     }
-    fn<<<grid, kDigThreads, smem, s>>>(a);
+    launch_chained(fn, grid, kDigThreads, smem, s, a);
     e = cudaGetLastError();
     if (e == cudaSuccess || raise) break;
   }
@@ -1016,10 +1034,11 @@ __global__ void __launch_bounds__(256) k_reflect_w(const double* __restrict__ pa
                                                    int N, const double* __restrict__ T,
                                                    uint32_t k64, int* eW, __half* img, int NT,
                                                    int ntiles) {
+  const int z = chain_begin(), bx = (int)blockIdx.x + z;
   __shared__ double Ts[kRefBlk][kRefBlk + 1];
   __shared__ double Ws[kRefCols][kRefBlk], Wt[kRefCols][kRefBlk];
-  const int tid = threadIdx.x, n0 = blockIdx.x * kRefCols;
-  for (int i = tid; i < kRefBlk * kRefBlk; i += 256) Ts[i / kRefBlk][i % kRefBlk] = T[i];
+  const int tid = threadIdx.x, n0 = bx * kRefCols;
+  for (int i = tid; i < kRefBlk * kRefBlk; i += 256) Ts[i / kRefBlk][i % kRefBlk] = T[i + z];
   for (int i = tid; i < kRefCols * kRefBlk; i += 256) {
     const int n = n0 + i / kRefBlk, c = i % kRefBlk;
     double t = 0.0;
@@ -1097,7 +1116,7 @@ cudaError_t digit_reflect(int N, int nref, const double* Yr, const double* T, do
   // every block's reflectors as column tiles of one image over k = 0 .. N - 1 (|y| <= 1)
   const DigitShape ysh = digit_shape(kRefBlk, N);  // NT 64, one tile per block
   const int W = nblk * kRefBlk;
-  k_digit_planes<<<grid_for((long long)W * ysh.nstages * 4), 256, 0, s>>>(
+  launch_chained(k_digit_planes, grid_for((long long)W * ysh.nstages * 4), 256, 0, s,
       Yr, 1, N, N, nref, kK64, nullptr, (__half*)(img + L.y), kRefBlk, nblk, ysh.nstages);
   count_launch(1);
   CKE(cudaGetLastError());
@@ -1119,7 +1138,7 @@ cudaError_t digit_reflect(int N, int nref, const double* Yr, const double* T, do
     a.C = part; a.sCs = (long long)N * kRefBlk; a.sCm = kRefBlk;
     a.status = status; a.abort_flag = abort_flag;
     CKE(launch_digit_gemm(a, N - Ra, s));
-    k_reflect_w<<<(wsh.NT * wsh.ntiles + kRefCols - 1) / kRefCols, 256, 0, s>>>(
+    launch_chained(k_reflect_w, (wsh.NT * wsh.ntiles + kRefCols - 1) / kRefCols, 256, 0, s,
         part, a.splits, N, T + (size_t)b * kRefBlk * kRefBlk, kK64, eW, (__half*)(img + L.w), wsh.NT,
         wsh.ntiles);
     count_launch(1);
@@ -1164,14 +1183,18 @@ cudaError_t digit_prepare_B(const Dims& d, const double* B, char* ws, const Layo
 }
 
 cudaError_t digit_hc(const Dims& d, const double* h, const double* C, char* ws, const Layout& L,
-                     cudaStream_t s) {
+                     ZeroJob zero, cudaStream_t s) {
   const int N = d.N;
   // exponents of C's columns (the operand planes, and lambda's rows) and of h's rows
-  CKE(cudaMemsetAsync(ws + L.eC64, 0, L.exend - L.eC64, s));
   if (N <= kFuseK) {
+    zero.add(ws + L.exq, L.exend - L.exq);
     CKE(launch_exps_planes(C, N, N, N, d.A, (int*)(ws + L.eC64), ws + L.Cimg, h, N, N,
-                           (int*)(ws + L.eH64), s));
+                           (int*)(ws + L.eH64), zero, true, s));
   } else {
+    CKE(cudaMemsetAsync(ws + L.eC64, 0, L.exend - L.eC64, s));
+    if (zero.flag) CKE(cudaMemsetAsync(zero.flag, 0, sizeof(int), s));
+    for (int i = 0; i < 4; ++i)
+      if (zero.n[i] > 0) CKE(cudaMemsetAsync(zero.p[i], 0, (size_t)zero.n[i] * 8, s));
     const ExpJob jobs[2] = {{C, N, N, N, 1, (int*)(ws + L.eC64)},
                             {h, N, N, N, 0, (int*)(ws + L.eH64)}};
     CKE(launch_exps(jobs, 2, s));
@@ -1232,11 +1255,11 @@ int digit_block(const Dims& d, const double* Bblk, int p0, int np, char* ws, con
     int *bmax = (int*)(ws + L.bmax), *wmax = (int*)(ws + L.wmax), *eY = (int*)(ws + L.eY64);
     const double *Ac = (const double*)(ws + L.Acoef), *Bc = (const double*)(ws + L.Bcoef);
     const int js = jk_splits64(A, np), wc = np < 152 * 4 ? np : 152 * 4;
-    k_w_jk64<<<wc + jb * js, 256, (size_t)A * 8, s>>>(b, np, A, Ac, W, wmax, wc, js, part, bmax);
-    k_jk_final64<<<jb + (A + 7) / 8, 256, 0, s>>>(part, js, A, Bc, bmax, wmax,
-                                                  (double*)(ws + L.J), (double*)(ws + L.K), eY, jb,
-                                                  p0 == 0 ? 1 : 0);
-    k_y_planes<<<grid_for((long long)ys.NT * ys.ntiles * ys.nstages * 4), 256, 0, s>>>(
+    launch_chained(k_w_jk64, wc + jb * js, 256, (size_t)A * 8, s, b, np, A, Ac, W, wmax, wc, js,
+                   part, bmax);
+    launch_chained(k_jk_final64, jb + (A + 7) / 8, 256, 0, s, part, js, A, Bc, bmax, wmax,
+                   (double*)(ws + L.J), (double*)(ws + L.K), eY, jb, p0 == 0 ? 1 : 0);
+    launch_chained(k_y_planes, grid_for((long long)ys.NT * ys.ntiles * ys.nstages * 4), 256, 0, s,
         b, np, A, Kpad, kK64, Bc, W, eY, (__half*)(ws + L.Yimg), ys.NT, ys.ntiles, ys.nstages);
     count_launch(3);
     CKI(cudaGetLastError());
@@ -1253,7 +1276,7 @@ int digit_block(const Dims& d, const double* Bblk, int p0, int np, char* ws, con
     a.splits = g_splits_digit(N, A, np);
     a.C = (double*)(ws + L.skp); a.sCs = (long long)N * A; a.sCm = A;
     CKI(launch_digit_gemm(a, (long long)np * Kpad, s));
-    k_split_sum<<<(unsigned)(((long long)N * A + 31) / 32), 256, 0, s>>>(
+    launch_chained(k_split_sum, (unsigned)(((long long)N * A + 31) / 32), 256, 0, s,
         (const double*)(ws + L.skp), a.splits, (long long)N * A, (double*)(ws + L.G));
     count_launch(1);
     CKI(cudaGetLastError());
@@ -1268,8 +1291,11 @@ cudaError_t digit_lambda(const Dims& d, const double* C, char* ws, const Layout&
   int* eG = (int*)(ws + L.eG64);
   // C's planes are done with
   if (N <= kFuseK) {
-    CKE(launch_exps_planes(G, A, N, A, A, eG, ws + L.Cimg, nullptr, 0, 0, nullptr, s));
+    ZeroJob zero{};
+    zero.add(lam, (size_t)N * N * 8);
+    CKE(launch_exps_planes(G, A, N, A, A, eG, ws + L.Cimg, nullptr, 0, 0, nullptr, zero, false, s));
   } else {
+    CKE(cudaMemsetAsync(lam, 0, (size_t)N * N * 8, s));
     const ExpJob jobs[1] = {{G, A, N, A, 1, eG}};
     CKE(launch_exps(jobs, 1, s));
     CKE(launch_planes(G, A, 1, N, A, eG, ws + L.Cimg, s));

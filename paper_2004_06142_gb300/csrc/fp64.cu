@@ -154,7 +154,7 @@ __device__ __forceinline__ void k_occupations_body(const Blk& B_, Dims d, const 
     }
   }
   if (kTable) __syncthreads();
-  const int p = threadIdx.x + B_.x * blockDim.x;
+  const int p = threadIdx.x + B_.zero + B_.x * blockDim.x;
   if (p >= A) return;
   const int nsub = npair + d.nsingle;  // subspaces: pairs, then the singly occupied orbitals
   const int g = pm[p];
@@ -201,21 +201,19 @@ __global__ void k_occupations(Dims d, const double* __restrict__ gamma,
 
 cudaError_t launch_occupations(const Dims& d, const double* gamma, const int32_t* pm, char* ws,
                                const Layout& L, cudaStream_t s) {
-  // the three Jacobians follow one another
-  const size_t jac = (size_t)d.A * d.ng * sizeof(double);
-  const cudaError_t e = cudaMemsetAsync(ws + L.dn, 0, L.dphi + jac - L.dn, s);
-  if (e != cudaSuccess) return e;
   DevHeader* hdr = (DevHeader*)(ws + L.header);
   double *n = (double*)(ws + L.n), *sqn = (double*)(ws + L.sqn), *phi = (double*)(ws + L.phi);
   double *dn = (double*)(ws + L.dn), *dsq = (double*)(ws + L.dsq), *dphi = (double*)(ws + L.dphi);
   if (d.A <= 1024) {  // one CTA with the sin/cos table (at most 16 KB: ng < nact)
     const int threads = (d.A + 31) / 32 * 32;
     const size_t smem = (size_t)(d.ng > 0 ? d.ng : 1) * 2 * sizeof(double);
-    k_occupations<true><<<1, threads, smem, s>>>(d, gamma, pm, hdr, n, sqn, phi, dn, dsq, dphi);
+    launch_chained(k_occupations<true>, 1, threads, smem, s, d, gamma, pm, hdr, n, sqn, phi, dn,
+                   dsq, dphi);
   } else {
     const int threads = 128;
-    k_occupations<false><<<(d.A + threads - 1) / threads, threads, 0, s>>>(
-        d, gamma, pm, hdr, n, sqn, phi, dn, dsq, dphi);
+    launch_chained(
+        k_occupations<false>, (d.A + threads - 1) / threads, threads, 0, s, d, gamma, pm, hdr, n,
+        sqn, phi, dn, dsq, dphi);
   }
   count_launch(1);
   return cudaGetLastError();
@@ -260,7 +258,7 @@ cudaError_t launch_coefficients(const Dims& d, const int32_t* pm, char* ws, cons
                                 cudaStream_t s) {
   const bool mixed = d.precision == DONOF_MIXED;
   const long long W = mixed ? d.Ap : d.A;
-  k_coefficients<<<(unsigned)((W * W + 255) / 256), 256, 0, s>>>(
+  launch_chained(k_coefficients, (unsigned)((W * W + 255) / 256), 256, 0, s,
       d, pm, (const double*)(ws + L.n), (const double*)(ws + L.sqn), (const double*)(ws + L.phi),
       (double*)(ws + L.Acoef), (double*)(ws + L.Bcoef), mixed ? (float*)(ws + L.AcF) : nullptr,
       mixed ? (float*)(ws + L.BcF) : nullptr);
@@ -321,9 +319,9 @@ __global__ void k_hdiag_ginit(Dims d, const double* __restrict__ C, const double
 
 cudaError_t launch_hdiag_ginit(const Dims& d, const double* C, char* ws, const Layout& L,
                                bool one_electron_G, cudaStream_t s) {
-  k_hdiag_ginit<<<(d.A + 7) / 8, 256, 0, s>>>(d, C, (const double*)(ws + L.hC),
-                                              (const double*)(ws + L.n), (double*)(ws + L.Hd),
-                                              (double*)(ws + L.G), one_electron_G ? 1.0 : 0.0);
+  launch_chained(k_hdiag_ginit, (d.A + 7) / 8, 256, 0, s, d, C, (const double*)(ws + L.hC),
+                 (const double*)(ws + L.n), (double*)(ws + L.Hd), (double*)(ws + L.G),
+                 one_electron_G ? 1.0 : 0.0);
   count_launch(1);
   return cudaGetLastError();
 }
@@ -443,7 +441,7 @@ __device__ __forceinline__ void k_energy_rows_body(const Blk& B_, Dims d, const 
                               const double* __restrict__ K, double* part) {
   const int A = d.A;
   const int p = B_.x * (blockDim.x / 32) + threadIdx.x / 32;
-  const int lane = threadIdx.x % 32;
+  const int lane = threadIdx.x % 32 + B_.zero;
   if (p >= A) return;
   const int g = pm[p];
   double e = 0.0, a_n = 0.0, a_s = 0.0, a_p = 0.0, a_7s = 0.0;
@@ -495,7 +493,7 @@ __device__ __forceinline__ void k_energy_final_body(const Blk& B_, Dims d, const
   // one warp per output (E first, then each dE/dgamma_k), lanes over orbitals, a fixed
   // shuffle tree: the sums do not depend on scheduling
   const int A = d.A;
-  const int lane = threadIdx.x % 32, nw = B_.gx * (blockDim.x / 32);
+  const int lane = threadIdx.x % 32 + B_.zero, nw = B_.gx * (blockDim.x / 32);
   const int warp = B_.x * (blockDim.x / 32) + threadIdx.x / 32;
   const double* gn = part + A;
   const double* gs = part + 2 * A;
@@ -536,14 +534,14 @@ __global__ void __launch_bounds__(256) k_energy_final(Dims d, const double* __re
 cudaError_t launch_energy(const Dims& d, const int32_t* pm, char* ws, const Layout& L,
                           double* E_out, double* dEdg_out, cudaStream_t s) {
   double* part = (double*)(ws + L.Epart);
-  k_energy_rows<<<(d.A + 7) / 8, 256, 0, s>>>(
+  launch_chained(k_energy_rows, (d.A + 7) / 8, 256, 0, s,
       d, pm, (const double*)(ws + L.n), (const double*)(ws + L.sqn), (const double*)(ws + L.phi),
       (const double*)(ws + L.Acoef), (const double*)(ws + L.Bcoef), (const double*)(ws + L.Hd),
       (const double*)(ws + L.J), (const double*)(ws + L.K), part);
-  k_energy_final<<<(d.ng + 1 + 7) / 8, 256, 0, s>>>(d, part, (const double*)(ws + L.dn),
-                                   (const double*)(ws + L.dsq), (const double*)(ws + L.dphi),
-                                   (DevHeader*)(ws + L.header), (double*)(ws + L.dEdg), E_out,
-                                   dEdg_out);
+  launch_chained(k_energy_final, (d.ng + 1 + 7) / 8, 256, 0, s, d, part,
+                 (const double*)(ws + L.dn), (const double*)(ws + L.dsq),
+                 (const double*)(ws + L.dphi), (DevHeader*)(ws + L.header),
+                 (double*)(ws + L.dEdg), E_out, dEdg_out);
   count_launch(2);
   return cudaGetLastError();
 }

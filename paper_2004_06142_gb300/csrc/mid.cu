@@ -242,7 +242,7 @@ __device__ __forceinline__ void k_y_quant_body(const Blk& B_, const float* __res
                           __half* __restrict__ H, __half* __restrict__ F, DevHeader* hdr) {
   if (B_.x == 0 && threadIdx.x == 0 && threadIdx.y == 0)
     hdr->e3 = 0;  // G partials are in true units
-  const int r4 = Ap / 4, c4 = threadIdx.x, c0 = 4 * c4;
+  const int r4 = Ap / 4, c4 = threadIdx.x + B_.zero, c0 = 4 * c4;
   const float4* Bc4 = (const float4*)BcF;
   for (int P = B_.x; P < np; P += B_.gx) {
     const float4* b4 = (const float4*)b + (size_t)P * Ap * r4;
@@ -360,17 +360,15 @@ cudaError_t launch_mid_mixed(const Dims& d, int np, int splits, char* ws, const 
   float* W = (float*)(ws + L.W);
   const float* AcF = (const float*)(ws + L.AcF);
   const float* BcF = (const float*)(ws + L.BcF);
-  k_diag_w<<<dim3((np + kDwS - 1) / kDwS, (A + kDwP - 1) / kDwP), 256, 0, s>>>(D, np, A, Ap, AcF,
-                                                                           W);
-  k_kpart<<<dim3((kpart_quads(A) + 255) / 256, splits), 256, 0, s>>>(b, D, np, A, Ap, splits,
-                                                         (double*)(ws + L.Ksp),
-                                                         (double*)(ws + L.Jsp));
+  launch_chained(k_diag_w, dim3((np + kDwS - 1) / kDwS, (A + kDwP - 1) / kDwP), 256, 0, s, D, np,
+                 A, Ap, AcF, W);
+  launch_chained(k_kpart, dim3((kpart_quads(A) + 255) / 256, splits), 256, 0, s, b, D, np, A, Ap,
+                 splits, (double*)(ws + L.Ksp), (double*)(ws + L.Jsp));
   const int ncta_e = (splits * Ap + 7) / 8;  // a warp per (split, row) of the exponents
-  k_jk_eY<<<(A * A + 255) / 256 + ncta_e, 256, 0, s>>>((const double*)(ws + L.Ksp),
-                                             (const double*)(ws + L.Jsp), D, W, BcF, np, A, Ap,
-                                             splits, (double*)(ws + L.K), (double*)(ws + L.J),
-                                             (int*)(ws + L.eY));
-  k_y_quant<<<np < sm_count() * 8 ? np : sm_count() * 8, dim3(Ap / 4, 8), 0, s>>>(
+  launch_chained(k_jk_eY, (A * A + 255) / 256 + ncta_e, 256, 0, s, (const double*)(ws + L.Ksp),
+                 (const double*)(ws + L.Jsp), D, W, BcF, np, A, Ap, splits, (double*)(ws + L.K),
+                 (double*)(ws + L.J), (int*)(ws + L.eY));
+  launch_chained(k_y_quant, np < sm_count() * 8 ? np : sm_count() * 8, dim3(Ap / 4, 8), 0, s,
       b, W, BcF, np, A, Ap, (const int*)(ws + L.spOf), (const int*)(ws + L.eY),
       (__half*)(ws + L.Yhi), (__half*)(ws + L.Ylo), (DevHeader*)(ws + L.header));
   count_launch(4);

@@ -240,6 +240,9 @@ __device__ __forceinline__ void tc_body(const TcArgs* __restrict__ targs,
   if (PAIR) cluster_sync_all();  // the peer's barriers are initialised before any remote use
   tc_fence_after();
   const uint32_t tmem_base = *(volatile uint32_t*)tmem_slot;
+  // all of the above while the kernel before runs (it holds no TMEM: one CTA of this kind per SM);
+  // no load below goes through a read-only pointer
+  chain_wait();
 
   // work units: (z, row tile, split) of each problem; PAIR: a unit is the M = 256 tile of the
   // cluster, rows of slice pair (2 zp, 2 zp + 1) in the symmetric mode, row tiles
@@ -1016,7 +1019,9 @@ cudaError_t launch_tc(const TcMaps& m, TcArgs a, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
   }
-  k_tc_gemm<BK, NUM, PAIR><<<work, kThreads, smem, s>>>(m, a);
+  // chained while it leaves SMs free (500 / 2000 / 80: 989 us a build with no contraction chained,
+  // 960 with the small ones, 991 with all)
+  launch_chained_to(num_sms() - 1, k_tc_gemm<BK, NUM, PAIR>, work, kThreads, smem, s, m, a);
   count_launch(1);
   return cudaGetLastError();
 }
@@ -1527,8 +1532,15 @@ __device__ __forceinline__ void k_colnorms_body(const Blk& B_, SplitJobs jobs, d
   __syncthreads();
   if (ty == 0 && c < jb.nrows_out) colnorm_finish(jb, c, red, tx, G, invT, hdr);
 }
-__global__ void __launch_bounds__(1024) k_colnorms(SplitJobs jobs, double invT, DevHeader* hdr) {
-  k_colnorms_body(native_blk(), jobs, invT, hdr);
+// The row of CTAs behind the jobs', if any, clears `zero`.
+__global__ void __launch_bounds__(1024) k_colnorms(SplitJobs jobs, double invT, DevHeader* hdr,
+                                                   const ZeroJob zero) {
+  const Blk b = native_blk();
+  if (b.y == jobs.count) {
+    zero_ranges(zero, b.x, b.gx);
+    return;
+  }
+  k_colnorms_body(b, jobs, invT, hdr);
 }
 
 // The split itself, as rows c < nrows_out of Np halves (zero for c >= ncols or mu >= N):
@@ -1690,14 +1702,17 @@ __host__ __device__ inline SplitJobs lambda_jobs(const Dims& d, const Layout& L,
   return jobs;
 }
 
-// All jobs' norms, then all splits: two launches.
+// All jobs' norms, then all splits: two launches.  `first`: the first of a call (launched plainly).
 cudaError_t launch_split_jobs(const SplitJobs& jobs, int Np, double invT, DevHeader* hdr,
-                              cudaStream_t s) {
+                              const ZeroJob& zero, bool first, cudaStream_t s) {
   int rmax = 0;
   for (int k = 0; k < jobs.count; ++k)
     if (jobs.j[k].nrows_out > rmax) rmax = jobs.j[k].nrows_out;
-  k_colnorms<<<dim3((rmax + 31) / 32, jobs.count), 32 * norm_groups(jobs.j[0].N), 0, s>>>(jobs, invT, hdr);
-  k_split_T<<<dim3((Np + 31) / 32, (rmax + 31) / 32, jobs.count), 256, 0, s>>>(jobs, Np);
+  const bool clear = zero.flag || zero.n[0] > 0;
+  launch_chained_to(first ? 0 : kChainCtas, k_colnorms,
+                    dim3((rmax + 31) / 32, jobs.count + (clear ? 1 : 0)),
+                    32 * norm_groups(jobs.j[0].N), 0, s, jobs, invT, hdr, zero);
+  launch_chained(k_split_T, dim3((Np + 31) / 32, (rmax + 31) / 32, jobs.count), 256, 0, s, jobs, Np);
   count_launch(2);
   return cudaGetLastError();
 }
@@ -1911,27 +1926,26 @@ cudaError_t launch_prepare_split_B(const Dims& d, const double* B, char* ws, con
 }
 
 cudaError_t launch_split_C(const Dims& d, const double* C, const double* h, char* ws,
-                           const Layout& L, bool with_half_transform, cudaStream_t s) {
+                           const Layout& L, bool with_half_transform, const ZeroJob& zero,
+                           cudaStream_t s) {
   return launch_split_jobs(split_c_jobs(d, L, ws, C, h, with_half_transform), d.Np,
-                           intfrac_inv_target(d.N), (DevHeader*)(ws + L.header), s);
+                           intfrac_inv_target(d.N), (DevHeader*)(ws + L.header), zero, true, s);
 }
 
 cudaError_t launch_gram_bound(const Dims& d, const double* C, char* ws, const Layout& L,
                               cudaStream_t s) {
   DevHeader* hdr = (DevHeader*)(ws + L.header);
-  cudaError_t e = cudaMemsetAsync(&hdr->sC2, 0, sizeof(double), s);
-  if (e != cudaSuccess) return e;
   const int nch = (d.N + kGramChunk - 1) / kGramChunk;
   float* part = (float*)(ws + L.gram);
-  k_gram_part<<<dim3(nch, (d.A + 15) / 16), 256, 0, s>>>(C, d.N, d.A, part);
-  k_gram_final<<<d.A, 256, 0, s>>>(part, nch, d.A, hdr);
+  launch_chained(k_gram_part, dim3(nch, (d.A + 15) / 16), 256, 0, s, C, d.N, d.A, part);
+  launch_chained(k_gram_final, d.A, 256, 0, s, part, nch, d.A, hdr);
   count_launch(2);
   return cudaGetLastError();
 }
 
 cudaError_t launch_reduce_G(const Dims& d, char* ws, const Layout& L, cudaStream_t s) {
   const int nb = (int)(((long long)d.N * (d.Ap / 4) + 255) / 256);
-  k_reduce_G<<<nb, 256, 0, s>>>((const float*)(ws + L.Gpart), d.splits, d.N, d.A, d.Ap,
+  launch_chained(k_reduce_G, nb, 256, 0, s, (const float*)(ws + L.Gpart), d.splits, d.N, d.A, d.Ap,
                                            (const DevHeader*)(ws + L.header), (double*)(ws + L.G));
   count_launch(1);
   return cudaGetLastError();
@@ -1993,7 +2007,7 @@ int run_extended_product(const Dims& d, int M, const int* eU, const int* eV, int
   if (launch_tc<64, kIntFrac, 0>(m, a, s) != cudaSuccess)
     return DONOF_ERR_CUDA;
   const long long nb = ((long long)M * ncols + 255) / 256;
-  k_sum_blocks<<<(int)(nb < num_sms() * 8 ? nb : num_sms() * 8), 256, 0, s>>>(
+  launch_chained(k_sum_blocks, (int)(nb < num_sms() * 8 ? nb : num_sms() * 8), 256, 0, s,
       (const float*)(ws + L.hpart), M, ncols, d.Ap, out, ld);
   count_launch(1);
   return cudaGetLastError() == cudaSuccess ? DONOF_OK : DONOF_ERR_CUDA;
@@ -2013,8 +2027,10 @@ int run_lambda_tc(const Dims& d, const double* C, char* ws, const Layout& L, dou
                   cudaStream_t s) {
   DevHeader* hdr = (DevHeader*)(ws + L.header);
   const int N = d.N, A = d.A;
-  if (launch_split_jobs(lambda_jobs(d, L, ws, C), d.Np, intfrac_inv_target(N), hdr, s) !=
-      cudaSuccess)
+  ZeroJob zero{};
+  zero.add(lam, (size_t)N * N * 8);
+  if (launch_split_jobs(lambda_jobs(d, L, ws, C), d.Np, intfrac_inv_target(N), hdr, zero, false,
+                        s) != cudaSuccess)
     return DONOF_ERR_CUDA;
   return run_extended_product(d, N, (const int*)(ws + L.eCf), (const int*)(ws + L.eG), A, lam,
                               N, ws, L, s);
@@ -2150,7 +2166,9 @@ int run_tc_block(const Dims& d, int p0, int np, char* ws, const Layout& L, cudaS
   // the G contraction's rows run over (slices of a split) x Ap: the largest split's length
   const double invT2 = intfrac_inv_target_sq((double)((np + splits3 - 1) / splits3) * Ap);
   const int gx3 = (splits3 * N + 255) / 256;
-  k_x_exponents<<<dim3(gx3 > num_sms() * 4 ? gx3 : num_sms() * 4, 2), 256, 0, s>>>(
+  const long long gx1 = std::min(((long long)np * Ap + 255) / 256, num_sms() * 4ll);
+  launch_chained(
+      k_x_exponents, dim3((unsigned)std::max<long long>(gx3, gx1), 2), 256, 0, s,
       (const double*)(ws + L.L1max) + p0, (const double*)(ws + L.cnorm), Ap,
       intfrac_inv_target(N), (int*)(ws + L.eXt), (const float*)(ws + L.rn2) + (size_t)p0 * N,
       (const DevHeader*)hdr, np, splits3, N, invT2, (int*)(ws + L.spOf), (int*)(ws + L.eX3));
