@@ -35,8 +35,7 @@ namespace {
 constexpr int kRowWarps = 8;                  // warps of a tridiagonal-reduction CTA that own rows
 constexpr int kTriWarps = kRowWarps + 1;      // ... and the scalar warp
 constexpr int kTriThreads = 32 * kTriWarps;
-constexpr int kScalarTid = 32 * kRowWarps;    // lane 0 of the scalar warp
-static_assert(kTriWarps <= 16, "block_sum_d sums at most 16 warps");
+static_assert(kTriWarps <= 16, "warps_sum_d adds at most 16 sums");
 constexpr int kNb = 64;           // reflectors per WY block
 constexpr int kFixCTAs = 32;      // CTAs (one warp each) of the small-cluster kernel
 constexpr int kSmallCl = 32;      // clusters up to this size are orthonormalised by one warp
@@ -141,33 +140,34 @@ __device__ __forceinline__ double warp_sum_d(double v) {
   return v;
 }
 
-// Sum over the CTA in a fixed order (a fixed shuffle tree in each warp, then warp 0 adds the
-// warps' sums by a fixed tree): every thread gets the same value.  red holds kTriWarps + 1.
-__device__ __forceinline__ double block_sum_d(double v, double* red) {
-  v = warp_sum_d(v);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double t = threadIdx.x < kTriWarps ? red[threadIdx.x] : 0.0;
+// The sum of the warps' sums in red[kTriWarps], in a fixed order; in lanes 0 .. 15 of the warp that
+// calls it.
+__device__ __forceinline__ double warps_sum_d(const double* red) {
+  const int lane = threadIdx.x & 31;
+  double t = lane < kTriWarps ? red[lane] : 0.0;
 #pragma unroll
-    for (int o = 8; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (threadIdx.x == 0) red[kTriWarps] = t;
-  }
-  __syncthreads();
-  return red[kTriWarps];
+  for (int o = 8; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return t;
 }
 
 // Grid barrier of the cooperative launch: arrivals counted in hdr->ctr (zeroed before the
 // launch); the wait gives up after kBarrierLimitNs and raises hdr->abort, which ends every
-// other CTA's wait at once.  Returns false when the CTA must leave.
-__device__ __forceinline__ bool grid_barrier(EighHdr* h, unsigned target, int* s_flag) {
+// other CTA's wait at once.  grid_wait returns false when the CTA must leave.  Release and acquire
+// at device scope, cumulative over what the CTA's own barrier ordered before.
+__device__ __forceinline__ void grid_arrive(EighHdr* h) {
   __syncthreads();
+  if (threadIdx.x == 0)
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&h->ctr) : "memory");
+}
+__device__ __forceinline__ bool grid_wait(EighHdr* h, unsigned target, int* s_flag) {
   if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(&h->ctr, 1u);
     const unsigned long long t0 = gtimer();
     int ok = 1;
-    while (*(volatile unsigned*)&h->ctr < target) {
+    for (unsigned it = 1;; ++it) {
+      unsigned c;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(&h->ctr) : "memory");
+      if (c >= target) break;
+      if (it & 15) continue;
       if (*(volatile int*)&h->abort) { ok = 0; break; }
       if (gtimer() - t0 > kBarrierLimitNs) {
         atomicExch(&h->abort, 1);
@@ -175,7 +175,6 @@ __device__ __forceinline__ bool grid_barrier(EighHdr* h, unsigned target, int* s
         break;
       }
     }
-    __threadfence();
     *s_flag = ok;
   }
   __syncthreads();
@@ -241,8 +240,8 @@ struct TriArgs {
 
 __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
   extern __shared__ double sm[];
-  __shared__ double red[kTriWarps + 1];
-  __shared__ double sh[3];
+  __shared__ double red[2][kTriWarps];  // the warps' parts of the step's two sums
+  __shared__ double sh[4];              // tau, beta, scale of the reflector; alpha
   __shared__ int s_flag;
   const int N = a.N, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int G = gridDim.x;
@@ -264,27 +263,27 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
   // rows are dealt to CTAs cyclically (row i to CTA i mod G), then to the CTA's row warps, so
   // the shrinking trailing matrix stays spread over every SM; with N <= G * kRowWarps each row
   // warp owns one row at most and keeps it in registers while it is updated.  The last warp
-  // owns no row: its lane 0 forms the reflectors' scalars.
+  // owns no row: it adds the warps' sums and forms the reflectors' scalars meanwhile.
   const bool row_warp = wid < kRowWarps;
   auto row_of = [&](int t) { return blockIdx.x + G * (wid + kRowWarps * t); };
   const bool reg_rows = N <= kTriRegMaxN && N <= G * kRowWarps;
   const int myrow = row_warp ? row_of(0) : N;
   unsigned bar = 0;
 
-  // reflector of x[k0..N) (xn2 = sum over j > k0 of x_j^2): the scalars tau, beta and the
-  // scale of u's tail (0 when the column is already reduced: u = e_k0)
-  auto hh_scalars = [&](int k0, double xn2) {
-    if (tid == kScalarTid) {
+  // by the scalar warp: reflector of x[k0..N) from the warps' parts of xn2 = sum over j > k0 of
+  // x_j^2: tau, beta and the scale of u's tail (0 when the column is already reduced: u = e_k0);
+  // lane 0 divides for tau, lane 1 for the scale, in one division of the warp
+  auto hh_scalars = [&](int k0, const double* parts) {
+    const double xn2 = warps_sum_d(parts);
+    if (lane < 2) {
       const double al = x[k0];
-      double t = 0.0, b = al, sc = 0.0;
+      double q = 0.0, b = al;
       if (xn2 != 0.0) {
         b = -copysign(sqrt(fma(al, al, xn2)), al);
-        t = (b - al) / b;
-        sc = 1.0 / (al - b);
+        q = (lane == 0 ? b - al : 1.0) / (lane == 0 ? b : al - b);
       }
-      sh[0] = t;
-      sh[1] = b;
-      sh[2] = sc;
+      sh[lane == 0 ? 0 : 2] = q;
+      if (lane == 0) sh[1] = b;
     }
   };
   // after a barrier: x[k0+1..) scaled into u's tail, x[k0] = 1; CTA 0 also stores u as row
@@ -306,7 +305,10 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
     x[j] = xj;
     if (j >= 2) xn = fma(xj, xj, xn);
   }
-  hh_scalars(1, block_sum_d(xn, red));
+  xn = warp_sum_d(xn);
+  if (lane == 0) red[1][wid] = xn;
+  __syncthreads();
+  if (!row_warp) hh_scalars(1, red[1]);
   __syncthreads();
   double tau_c = sh[0], beta = sh[1];
   if (writer && tid == 0) {
@@ -329,7 +331,16 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
       if (lane == 0) a.pbuf[i] = tau_c * acc;
     }
   }
-  if (!grid_barrier(a.hdr, (++bar) * G, &s_flag)) return;
+  // the own row, column lane + 32 q in rr[q], is kept in registers from here on
+  double rr[kTriRowRegs];
+  double* Amy = A + (size_t)(myrow < N ? myrow : 0) * N;
+#pragma unroll
+  for (int q = 0; q < kTriRowRegs; ++q) {
+    const int j = lane + 32 * q;
+    rr[q] = reg_rows && myrow < N && j < N ? __ldcg(Amy + j) : 0.0;
+  }
+  grid_arrive(a.hdr);
+  if (!grid_wait(a.hdr, (++bar) * G, &s_flag)) return;
   {
     double* t = v;
     v = x;
@@ -340,7 +351,7 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
     const double* pk = a.pbuf + (size_t)(k & 1) * N;
     const double* Ak1 = A + (size_t)(k + 1) * N;
     const bool last = k + 1 == N - 2;
-    // every load of the step at once: p_k, row k+1, and (register path) the warp's own row
+    // the loads of the step at once: p_k and row k+1
     double pr[kTriVec], ar[kTriVec];
 #pragma unroll
     for (int r = 0; r < kTriVec; ++r) {
@@ -352,16 +363,7 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
         ar[r] = __ldcg(Ak1 + j);
       }
     }
-    double rr[kTriRowRegs];
     const bool has_row = reg_rows && myrow < N && myrow >= k + 2;
-    double* Amy = A + (size_t)(has_row ? myrow : 0) * N;
-    if (has_row) {
-#pragma unroll
-      for (int q = 0; q < kTriRowRegs; ++q) {
-        const int j = k + 2 + lane + 32 * q;
-        rr[q] = j < N ? __ldcg(Amy + j) : 0.0;
-      }
-    }
     double acc = 0.0;
 #pragma unroll
     for (int r = 0; r < kTriVec; ++r) {
@@ -370,9 +372,6 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
     }
     for (int j = k + 1 + tid + kTriThreads * kTriVec; j < N; j += kTriThreads)
       acc = fma(__ldcg(pk + j), v[j], acc);
-    // alpha = (tau_k / 2)(p_k . v_k); with w = p - alpha v the update A - v w^T - w v^T is
-    // A_ij - v_i p_j - (p_i - 2 alpha v_i) v_j, formed from p and v alone
-    const double al = 0.5 * tau_c * block_sum_d(acc, red);
 #pragma unroll
     for (int r = 0; r < kTriVec; ++r) {
       const int j = k + 1 + tid + kTriThreads * r;
@@ -380,7 +379,26 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
     }
     for (int j = k + 1 + tid + kTriThreads * kTriVec; j < N; j += kTriThreads)
       p[j] = __ldcg(pk + j);
+    acc = warp_sum_d(acc);
+    if (lane == 0) red[0][wid] = acc;
     __syncthreads();
+    // alpha = (tau_k / 2)(p_k . v_k); with w = p - alpha v the update A - v w^T - w v^T is
+    // A_ij - v_i p_j - (p_i - 2 alpha v_i) v_j, formed from p and v alone.  While the scalar warp
+    // forms alpha, the row warps apply the part that does not need it (not at the last step, whose
+    // 2 x 2 block is formed from the rows as they stand)
+    const double vi = has_row ? v[myrow] : 0.0;
+    if (!row_warp) {
+      const double t = warps_sum_d(red[0]);
+      if (lane == 0) sh[3] = 0.5 * tau_c * t;
+    } else if (has_row && !last) {
+#pragma unroll
+      for (int q = 0; q < kTriRowRegs; ++q) {
+        const int j = lane + 32 * q;
+        if (32 * q + 31 >= k + 2 && j >= k + 2 && j < N) rr[q] = fma(-vi, p[j], rr[q]);
+      }
+    }
+    __syncthreads();
+    const double al = sh[3];
     // row k+1 of the updated matrix (v[k+1] = 1): its column k+1 below the diagonal
     const double ck1 = fma(-2.0, al, p[k + 1]);
     xn = 0.0;
@@ -398,20 +416,9 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
       x[j] = xj;
       if (j >= k + 3) xn = fma(xj, xj, xn);
     }
-    // register path: the own row's rank-2 update, while the norm is reduced (not at the last
-    // step, whose 2 x 2 block is formed from the rows as they stand)
-    if (has_row && !last) {
-      const double vi = v[myrow], ci = fma(-2.0 * al, vi, p[myrow]);
-#pragma unroll
-      for (int q = 0; q < kTriRowRegs; ++q) {
-        const int j = k + 2 + lane + 32 * q;
-        if (j < N) {
-          rr[q] = fma(-ci, v[j], fma(-vi, p[j], rr[q]));
-          Amy[j] = rr[q];
-        }
-      }
-    }
-    const double xn2 = block_sum_d(xn, red);
+    xn = warp_sum_d(xn);
+    if (lane == 0) red[1][wid] = xn;
+    __syncthreads();
     if (last) {  // the last 2 x 2 block
       if (writer && tid == 0) {
         a.d[N - 2] = x[N - 2];
@@ -421,17 +428,29 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
       }
       break;
     }
-    // the scalar warp forms the next reflector while the row warps take the dot of their
-    // updated row with the unscaled column (u_{k+2} = 1, u_j = sc x_j beyond)
-    hh_scalars(k + 2, xn2);
+    // the scalar warp forms the next reflector while the row warps finish their row's update and
+    // take its dot with the unscaled column (u_{k+2} = 1, u_j = sc x_j beyond).  The sums run over
+    // the columns k+3+l, k+35+l, ..., whichever lane holds them, and the shuffle tree pairs the
+    // same sums in every rotation of the lanes.  Row k+2 (at the end also the last) is published
     double rawdot = 0.0, r0 = 0.0;
-    if (has_row) {
+    if (!row_warp) {
+      hh_scalars(k + 2, red[1]);
+    } else if (has_row) {
+      const double ci = fma(-2.0 * al, vi, p[myrow]);
 #pragma unroll
       for (int q = 0; q < kTriRowRegs; ++q) {
-        const int j = k + 2 + lane + 32 * q;
-        if (j < N) {
-          if (q == 0 && lane == 0) r0 = rr[0];
+        const int j = lane + 32 * q;
+        if (32 * q + 31 >= k + 2 && j >= k + 2 && j < N) {
+          rr[q] = fma(-ci, v[j], rr[q]);
+          if (j == k + 2) r0 = rr[q];
           else rawdot = fma(rr[q], x[j], rawdot);
+        }
+      }
+      if (myrow == k + 2 || k == N - 4) {
+#pragma unroll
+        for (int q = 0; q < kTriRowRegs; ++q) {
+          const int j = lane + 32 * q;
+          if (j >= k + 2 && j < N) Amy[j] = rr[q];
         }
       }
       rawdot = warp_sum_d(rawdot);
@@ -444,28 +463,30 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
       a.e[k + 1] = beta;
       a.tau[k + 1] = tau_n;
     }
-    hh_apply(k + 2, k + 1);
     // p_{k+1} = tau A u over the own rows i >= k+2
     double* pn = a.pbuf + (size_t)((k + 1) & 1) * N;
     if (reg_rows) {
-      if (has_row && lane == 0) pn[myrow] = tau_n * fma(sc, rawdot, r0);
+      if (has_row && lane == ((k + 2) & 31)) pn[myrow] = tau_n * fma(sc, rawdot, r0);
+      grid_arrive(a.hdr);
+      hh_apply(k + 2, k + 1);
     } else {
+      hh_apply(k + 2, k + 1);
       __syncthreads();  // the scaled reflector
       for (int t = 0; row_warp; ++t) {
         const int i = row_of(t);
         if (i >= N) break;
         if (i < k + 2) continue;
         double* Ar = A + (size_t)i * N;
-        const double vi = v[i], ci = fma(-2.0 * al, vi, p[i]);
+        const double vr = v[i], ci = fma(-2.0 * al, vr, p[i]);
         double acc2 = 0.0;
         int j = k + 2 + lane;
         for (; j + 96 < N; j += 128) {
           const double a0 = __ldcg(Ar + j), a1 = __ldcg(Ar + j + 32), a2 = __ldcg(Ar + j + 64),
                        a3 = __ldcg(Ar + j + 96);
-          const double b0 = fma(-ci, v[j], fma(-vi, p[j], a0));
-          const double b1 = fma(-ci, v[j + 32], fma(-vi, p[j + 32], a1));
-          const double b2 = fma(-ci, v[j + 64], fma(-vi, p[j + 64], a2));
-          const double b3 = fma(-ci, v[j + 96], fma(-vi, p[j + 96], a3));
+          const double b0 = fma(-ci, v[j], fma(-vr, p[j], a0));
+          const double b1 = fma(-ci, v[j + 32], fma(-vr, p[j + 32], a1));
+          const double b2 = fma(-ci, v[j + 64], fma(-vr, p[j + 64], a2));
+          const double b3 = fma(-ci, v[j + 96], fma(-vr, p[j + 96], a3));
           Ar[j] = b0;
           Ar[j + 32] = b1;
           Ar[j + 64] = b2;
@@ -476,15 +497,16 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
           acc2 = fma(b3, x[j + 96], acc2);
         }
         for (; j < N; j += 32) {
-          const double b0 = fma(-ci, v[j], fma(-vi, p[j], __ldcg(Ar + j)));
+          const double b0 = fma(-ci, v[j], fma(-vr, p[j], __ldcg(Ar + j)));
           Ar[j] = b0;
           acc2 = fma(b0, x[j], acc2);
         }
         acc2 = warp_sum_d(acc2);
         if (lane == 0) pn[i] = tau_n * acc2;
       }
+      grid_arrive(a.hdr);
     }
-    if (!grid_barrier(a.hdr, (++bar) * G, &s_flag)) return;
+    if (!grid_wait(a.hdr, (++bar) * G, &s_flag)) return;
     double* t = v;
     v = x;
     x = t;
@@ -610,7 +632,8 @@ __device__ __forceinline__ int sturm_count_f32(const float* __restrict__ d,
   return cnt;
 }
 
-// The same count in double: sign changes of the leading minors
+// The same count in double, bound by the FP64 pipe (16 clocks an instruction and SM) or by the one
+// chained FP64 operation of a row: a zero minor is only noted, and its rows are done again.  Sign changes of the leading minors
 // p_i = (d_i - sig) p_{i-1} - e_{i-1}^2 p_{i-2} (a zero minor counts as a tiny negative ratio),
 // the pair (p_{i-1}, p_i) rescaled by 2^-+300 after every eighth row when its larger magnitude
 // has left [2^-300, 2^300] (with ||T||_inf <= 1 and the split threshold, eight rows move it by
@@ -623,14 +646,31 @@ __device__ __forceinline__ int sturm_count_f64(const double* __restrict__ d,
   int cnt = dbl_sign(p1);
   int i = s0 + 1;
   while (i < s1) {
-    const int iend = min(i + 8, s1);
-#pragma unroll 4
-    for (; i < iend; ++i) {
-      double p2 = fma(d[i] - sig, p1, -(e2[i - 1] * p0));
-      if (dbl_is_zero(p2)) p2 = -p1 * 0x1p-60;
-      cnt += dbl_sign(p2) ^ dbl_sign(p1);
-      p0 = p1;
-      p1 = p2;
+    const int ib = i, iend = min(i + 8, s1), cb = cnt;
+    const double b0 = p0, b1 = p1;
+    bool zero = false;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (i < iend) {
+        const double p2 = fma(d[i] - sig, p1, -(e2[i - 1] * p0));
+        zero |= dbl_is_zero(p2);
+        cnt += dbl_sign(p2) ^ dbl_sign(p1);
+        p0 = p1;
+        p1 = p2;
+        ++i;
+      }
+    }
+    if (zero) {  // once more, with the zero minors replaced
+      p0 = b0;
+      p1 = b1;
+      cnt = cb;
+      for (i = ib; i < iend; ++i) {
+        double p2 = fma(d[i] - sig, p1, -(e2[i - 1] * p0));
+        if (dbl_is_zero(p2)) p2 = -p1 * 0x1p-60;
+        cnt += dbl_sign(p2) ^ dbl_sign(p1);
+        p0 = p1;
+        p1 = p2;
+      }
     }
     const int ex = max(dbl_biased_exp(p0), dbl_biased_exp(p1));
     if (ex > 1023 + 300) {
@@ -673,7 +713,7 @@ __global__ void __launch_bounds__(kBisThreads) k_bisect(int N, const double* __r
   __syncthreads();
   const int lane = threadIdx.x & 31, j = lane & 15;
   const unsigned hm = 0xffffu << (lane & 16);
-  const int s = (blockIdx.x * kBisThreads + threadIdx.x) >> 4;
+  const int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 4;
   if (s >= N) return;  // uniform over the half-warp
   if (h->abort) {
     if (j == 0) lam[s] = __longlong_as_double(0x7ff8000000000000ll);
@@ -842,6 +882,7 @@ __global__ void __launch_bounds__(32) k_twisted(int N, const double* __restrict_
     double dp = pivot_floor(ds[s0] - lm), rp = rcp_nr(dp);
     Z[s0 * ld + c] = dp;
     Wp[s0 * ld + c] = rp;
+#pragma unroll 4
     for (int i = s0 + 1; i < s1; ++i) {
       dp = pivot_floor(fma(-e2[i - 1], rp, ds[i] - lm));
       rp = rcp_nr(dp);
@@ -851,6 +892,7 @@ __global__ void __launch_bounds__(32) k_twisted(int N, const double* __restrict_
   } else {
     double dm = pivot_floor(ds[s1 - 1] - lm), rm = rcp_nr(dm);
     Wd[(s1 - 1) * ld + c] = rm;
+#pragma unroll 4
     for (int i = s1 - 2; i >= s0; --i) {
       dm = pivot_floor(fma(-e2[i], rm, ds[i] - lm));
       rm = rcp_nr(dm);
@@ -863,6 +905,7 @@ __global__ void __launch_bounds__(32) k_twisted(int N, const double* __restrict_
   const int a = side == 0 ? s0 : mid, b = side == 0 ? mid : s1;
   double best = 0.0;
   int r = -1;
+#pragma unroll 8
   for (int i = a; i < b; ++i) {
     const double g = i < s1 - 1 ? fabs(fma(-e2[i], Wd[(i + 1) * ld + c], Z[i * ld + c]))
                                 : fabs(Z[i * ld + c]);
@@ -882,30 +925,37 @@ __global__ void __launch_bounds__(32) k_twisted(int N, const double* __restrict_
     }
   }
   __syncwarp(pm);
-  // z: thread 0 upwards from r, thread 1 downwards; rescaled by 2^-500 when above 2^500
+  // z: thread 0 upwards from r, thread 1 downwards; rescaled by 2^-500 when above 2^500.  kZ rows'
+  // factors are loaded ahead of the chain of products that uses them
+  constexpr int kZ = 8;
   int nres = 0;
-  if (side == 0) {
-    Z[r * ld + c] = 1.0;
+  const int step = side == 0 ? -1 : 1, n_z = side == 0 ? r - s0 : s1 - 1 - r;
+  const double* W = side == 0 ? Wp : Wd;
+  if (side == 0) Z[r * ld + c] = 1.0;
+  {
     double z = 1.0;
-    for (int i = r - 1; i >= s0; --i) {
-      z = -es[i] * z * Wp[i * ld + c];
-      if (fabs(z) > 0x1p500) {
-        for (int u = i + 1; u <= r; ++u) Z[u * ld + c] *= 0x1p-500;
-        z *= 0x1p-500;
-        ++nres;
+    for (int q0 = 0; q0 < n_z; q0 += kZ) {
+      double ev[kZ], wv[kZ];
+#pragma unroll
+      for (int u = 0; u < kZ; ++u) {
+        const int i = r + step * (q0 + u + 1);
+        const bool in = q0 + u < n_z;
+        ev[u] = in ? es[side == 0 ? i : i - 1] : 0.0;
+        wv[u] = in ? W[i * ld + c] : 0.0;
       }
-      Z[i * ld + c] = z;
-    }
-  } else {
-    double z = 1.0;
-    for (int i = r + 1; i < s1; ++i) {
-      z = -es[i - 1] * z * Wd[i * ld + c];
-      if (fabs(z) > 0x1p500) {
-        for (int u = r + 1; u < i; ++u) Z[u * ld + c] *= 0x1p-500;
-        z *= 0x1p-500;
-        ++nres;
+#pragma unroll
+      for (int u = 0; u < kZ; ++u) {
+        if (q0 + u >= n_z) break;
+        const int i = r + step * (q0 + u + 1);
+        z = -ev[u] * z * wv[u];
+        if (fabs(z) > 0x1p500) {
+          const int v0 = side == 0 ? i + 1 : r + 1, v1 = side == 0 ? r + 1 : i;
+          for (int v = v0; v < v1; ++v) Z[v * ld + c] *= 0x1p-500;
+          z *= 0x1p-500;
+          ++nres;
+        }
+        Z[i * ld + c] = z;
       }
-      Z[i * ld + c] = z;
     }
   }
   __syncwarp(pm);
@@ -915,13 +965,21 @@ __global__ void __launch_bounds__(32) k_twisted(int N, const double* __restrict_
   for (int q = nres; q < other; ++q)
     for (int i = lo_i; i < hi_i; ++i) Z[i * ld + c] *= 0x1p-500;
   double n2 = 0.0;
+#pragma unroll 8
   for (int i = lo_i; i < hi_i; ++i) {
     const double zi = Z[i * ld + c];
     n2 = fma(zi, zi, n2);
   }
   n2 += __shfl_xor_sync(pm, n2, 1);
   const double sc = 1.0 / sqrt(n2);
-  for (int i = lo_i; i < hi_i; ++i) Z[i * ld + c] *= sc;
+  for (int i0 = lo_i; i0 < hi_i; i0 += kZ) {
+    double zv[kZ];
+#pragma unroll
+    for (int u = 0; u < kZ; ++u) zv[u] = i0 + u < hi_i ? Z[(i0 + u) * ld + c] : 0.0;
+#pragma unroll
+    for (int u = 0; u < kZ; ++u)
+      if (i0 + u < hi_i) Z[(i0 + u) * ld + c] = zv[u] * sc;
+  }
 }
 
 __device__ __forceinline__ double hash_uniform(unsigned long long key) {
@@ -1247,7 +1305,9 @@ int eigh_run(int N, const double* A, double* V, double* w, char* ws, cudaStream_
   if (!ok(cudaFuncSetAttribute(k_bisect, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)bis_smem)))
     return DONOF_ERR_CUDA;
-  k_bisect<<<(N * 16 + kBisThreads - 1) / kBisThreads, kBisThreads, bis_smem, s>>>(
+  // a warp (two eigenvalues) per CTA while that spreads them over more SMs
+  const int bis_threads = N <= 2 * sms ? 32 : kBisThreads;
+  k_bisect<<<(N * 16 + bis_threads - 1) / bis_threads, bis_threads, bis_smem, s>>>(
       N, ds, e2, df, e2f, bstart, bend, glo, ghi, hdr, lam);
   const size_t rank_smem = (size_t)N * 12;
   if (!ok(cudaFuncSetAttribute(k_rank_plan, cudaFuncAttributeMaxDynamicSharedMemorySize,
