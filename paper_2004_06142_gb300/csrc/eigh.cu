@@ -23,11 +23,13 @@
 //      the tensor cores (digits.cu).
 #include <float.h>
 
+#include <atomic>
 #include <map>
 #include <mutex>
 #include <vector>
 
 #include "common.cuh"
+#include "tcptx.cuh"
 
 namespace donof {
 namespace {
@@ -46,6 +48,9 @@ constexpr int kClDesc = 5;        // ints per cluster: first slot, members, bloc
 constexpr int kTriVec = 5;  // (kTriRegMaxN + kTriThreads - 1) / kTriThreads
 constexpr int kTriRegMaxN = 1216;
 constexpr int kTriRowRegs = (kTriRegMaxN - 2 + 31) / 32;
+// its cluster form: the most CTAs, rows per row warp, and the largest n
+constexpr int kRowGroup = 4;  // 32-column pieces of a row handled together
+constexpr int kClCtas = 16, kClRows = 1, kClCols = 128;
 constexpr double kClusterTol = 1e-5;
 constexpr unsigned long long kBarrierLimitNs = 2000000000ull;
 
@@ -225,7 +230,9 @@ __global__ void k_eigh_scale_copy(const double* __restrict__ A, long long nn, Ei
 }
 
 // ---------------------------------------------------------------------------
-// 1. Householder tridiagonalisation (cooperative launch, kTriThreads threads, one CTA per SM)
+// 1. Householder tridiagonalisation: a cooperative launch of CTAs that exchange through L2 and a
+//    grid barrier, or (CL) one cluster of up to 16 CTAs that exchange through each other's shared
+//    memory and the cluster's hardware barrier.  Both form the same sums in the same order.
 // ---------------------------------------------------------------------------
 struct TriArgs {
   int N;
@@ -238,6 +245,20 @@ struct TriArgs {
   EighHdr* hdr;
 };
 
+__device__ __forceinline__ void store_peer(double* at, uint32_t rank, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(mapa_shared(smem_u32(at), rank)), "d"(v)
+               : "memory");
+}
+
+// R rows of up to 32 Q columns per row warp in registers.  An FP64 instruction of a warp holds its
+// scheduler's FP64 unit for 64 clocks, whatever its active lanes, and takes as long.  A column is a
+// chain of two sums over the vector, a square root, a division and a barrier; at 120 that chain (7700
+// of 16700 clocks left) is all of it, at 1200 the rows' three operations per element and the vector's
+// five on every SM are half of the 15700 clocks (8 rows a CTA, two a scheduler).  So the row warps
+// work while the scalar warp runs the chain, and rows stay in registers: reading and writing them
+// through L2 with the updates between the chain's parts took 1046 us at 120 and 12.9 ms at 1200,
+// this 410 us and 8.8 ms.
+template <int R, int Q, bool CL>
 __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
   extern __shared__ double sm[];
   __shared__ double red[2][kTriWarps];  // the warps' parts of the step's two sums
@@ -245,9 +266,13 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
   __shared__ int s_flag;
   const int N = a.N, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int G = gridDim.x;
+  const int W = N < 32 * Q ? 32 * Q : N;  // width of the vectors, zero past N
   double* v = sm;           // reflector of the current step (indices k+1 .. N-1)
-  double* x = sm + N;       // next column, then its reflector
-  double* p = sm + 2 * N;   // p = tau A v of the current step
+  double* x = sm + W;       // next column, then its reflector
+  double* p = sm + 2 * W;   // p = tau A v of the current step
+  double* pb = sm + 3 * W;  // CL: p of the current and the next step, written by their owners
+  double* rb = pb + 2 * N;  // CL: row k+1 of the current and the next step
+  constexpr int kVec = CL ? 1 : kTriVec;
   double* A = a.A;
   const bool writer = blockIdx.x == 0;
   if (N <= 2) {
@@ -261,14 +286,28 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
     return;
   }
   // rows are dealt to CTAs cyclically (row i to CTA i mod G), then to the CTA's row warps, so
-  // the shrinking trailing matrix stays spread over every SM; with N <= G * kRowWarps each row
-  // warp owns one row at most and keeps it in registers while it is updated.  The last warp
-  // owns no row: it adds the warps' sums and forms the reflectors' scalars meanwhile.
+  // the shrinking trailing matrix stays spread over every CTA; with N <= G * kRowWarps * R each row
+  // warp owns R rows at most and keeps them in registers.  The last warp owns no row: it adds the
+  // warps' sums and forms the reflectors' scalars meanwhile.
   const bool row_warp = wid < kRowWarps;
   auto row_of = [&](int t) { return blockIdx.x + G * (wid + kRowWarps * t); };
-  const bool reg_rows = N <= kTriRegMaxN && N <= G * kRowWarps;
-  const int myrow = row_warp ? row_of(0) : N;
+  const bool reg_rows = CL || (N <= 32 * Q && N <= G * kRowWarps * R);
+  int myrow[R];
+#pragma unroll
+  for (int t = 0; t < R; ++t) myrow[t] = row_warp ? row_of(t) : N;
   unsigned bar = 0;
+  auto arrive = [&]() {
+    if (CL) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    else grid_arrive(a.hdr);
+  };
+  auto wait = [&]() {
+    if (!CL) return grid_wait(a.hdr, (++bar) * G, &s_flag);
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    __syncthreads();  // what the CTA wrote behind its arrival
+    return true;
+  };
+  for (int j = N + tid; j < W; j += kTriThreads) v[j] = x[j] = p[j] = 0.0;
+  if (CL) cluster_sync_all();  // every CTA's shared memory exists
 
   // by the scalar warp: reflector of x[k0..N) from the warps' parts of xn2 = sum over j > k0 of
   // x_j^2: tau, beta and the scale of u's tail (0 when the column is already reduced: u = e_k0);
@@ -328,19 +367,26 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
 #pragma unroll 4
       for (int j = 1 + lane; j < N; j += 32) acc = fma(__ldcg(Ar + j), x[j], acc);
       acc = warp_sum_d(acc);
-      if (lane == 0) a.pbuf[i] = tau_c * acc;
+      if (CL) {
+        if (lane < G) store_peer(pb + i, lane, tau_c * acc);
+      } else if (lane == 0) {
+        a.pbuf[i] = tau_c * acc;
+      }
     }
   }
-  // the own row, column lane + 32 q in rr[q], is kept in registers from here on
-  double rr[kTriRowRegs];
-  double* Amy = A + (size_t)(myrow < N ? myrow : 0) * N;
+  if (CL)
+    for (int j = tid; j < N; j += kTriThreads) rb[j] = __ldcg(A + N + j);
+  // the own rows, column lane + 32 q in rr[.][q], are kept in registers from here on
+  double rr[R][Q];
 #pragma unroll
-  for (int q = 0; q < kTriRowRegs; ++q) {
-    const int j = lane + 32 * q;
-    rr[q] = reg_rows && myrow < N && j < N ? __ldcg(Amy + j) : 0.0;
-  }
-  grid_arrive(a.hdr);
-  if (!grid_wait(a.hdr, (++bar) * G, &s_flag)) return;
+  for (int t = 0; t < R; ++t)
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const int j = lane + 32 * q;
+      rr[t][q] = reg_rows && myrow[t] < N && j < N ? __ldcg(A + (size_t)myrow[t] * N + j) : 0.0;
+    }
+  arrive();
+  if (!wait()) return;
   {
     double* t = v;
     v = x;
@@ -352,50 +398,60 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
     const double* Ak1 = A + (size_t)(k + 1) * N;
     const bool last = k + 1 == N - 2;
     // the loads of the step at once: p_k and row k+1
-    double pr[kTriVec], ar[kTriVec];
+    double pr[kVec], ar[kVec];
 #pragma unroll
-    for (int r = 0; r < kTriVec; ++r) {
+    for (int r = 0; r < kVec; ++r) {
       const int j = k + 1 + tid + kTriThreads * r;
       pr[r] = 0.0;
       ar[r] = 0.0;
       if (j < N) {
-        pr[r] = __ldcg(pk + j);
-        ar[r] = __ldcg(Ak1 + j);
+        pr[r] = CL ? pb[(k & 1) * N + j] : __ldcg(pk + j);
+        ar[r] = CL ? rb[(k & 1) * N + j] : __ldcg(Ak1 + j);
       }
     }
-    const bool has_row = reg_rows && myrow < N && myrow >= k + 2;
+    bool has_row[R];
+#pragma unroll
+    for (int t = 0; t < R; ++t) has_row[t] = reg_rows && myrow[t] < N && myrow[t] >= k + 2;
     double acc = 0.0;
 #pragma unroll
-    for (int r = 0; r < kTriVec; ++r) {
+    for (int r = 0; r < kVec; ++r) {
       const int j = k + 1 + tid + kTriThreads * r;
       if (j < N) acc = fma(pr[r], v[j], acc);
     }
-    for (int j = k + 1 + tid + kTriThreads * kTriVec; j < N; j += kTriThreads)
+    for (int j = k + 1 + tid + kTriThreads * kVec; j < N; j += kTriThreads)
       acc = fma(__ldcg(pk + j), v[j], acc);
 #pragma unroll
-    for (int r = 0; r < kTriVec; ++r) {
+    for (int r = 0; r < kVec; ++r) {
       const int j = k + 1 + tid + kTriThreads * r;
       if (j < N) p[j] = pr[r];
     }
-    for (int j = k + 1 + tid + kTriThreads * kTriVec; j < N; j += kTriThreads)
+    for (int j = k + 1 + tid + kTriThreads * kVec; j < N; j += kTriThreads)
       p[j] = __ldcg(pk + j);
-    acc = warp_sum_d(acc);
+    if (k + 1 + 32 * wid < N) acc = warp_sum_d(acc);  // (a warp past the end: zeros)
     if (lane == 0) red[0][wid] = acc;
     __syncthreads();
     // alpha = (tau_k / 2)(p_k . v_k); with w = p - alpha v the update A - v w^T - w v^T is
     // A_ij - v_i p_j - (p_i - 2 alpha v_i) v_j, formed from p and v alone.  While the scalar warp
     // forms alpha, the row warps apply the part that does not need it (not at the last step, whose
     // 2 x 2 block is formed from the rows as they stand)
-    const double vi = has_row ? v[myrow] : 0.0;
+    double vi[R];
+#pragma unroll
+    for (int t = 0; t < R; ++t) vi[t] = has_row[t] ? v[myrow[t]] : 0.0;
     if (!row_warp) {
       const double t = warps_sum_d(red[0]);
       if (lane == 0) sh[3] = 0.5 * tau_c * t;
-    } else if (has_row && !last) {
+    } else if (!last) {
 #pragma unroll
-      for (int q = 0; q < kTriRowRegs; ++q) {
-        const int j = lane + 32 * q;
-        if (32 * q + 31 >= k + 2 && j >= k + 2 && j < N) rr[q] = fma(-vi, p[j], rr[q]);
-      }
+      for (int t = 0; t < R; ++t)
+        if (has_row[t]) {
+#pragma unroll
+          for (int q0 = 0; q0 < Q; q0 += kRowGroup) {
+            if (32 * (q0 + kRowGroup) <= k + 2 || 32 * q0 >= N) continue;
+#pragma unroll
+            for (int q = q0; q < q0 + kRowGroup && q < Q; ++q)
+              rr[t][q] = fma(-vi[t], p[lane + 32 * q], rr[t][q]);
+          }
+        }
     }
     __syncthreads();
     const double al = sh[3];
@@ -403,7 +459,7 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
     const double ck1 = fma(-2.0, al, p[k + 1]);
     xn = 0.0;
 #pragma unroll
-    for (int r = 0; r < kTriVec; ++r) {
+    for (int r = 0; r < kVec; ++r) {
       const int j = k + 1 + tid + kTriThreads * r;
       if (j < N) {
         const double xj = fma(-ck1, v[j], ar[r] - pr[r]);
@@ -411,12 +467,12 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
         if (j >= k + 3) xn = fma(xj, xj, xn);
       }
     }
-    for (int j = k + 1 + tid + kTriThreads * kTriVec; j < N; j += kTriThreads) {
+    for (int j = k + 1 + tid + kTriThreads * kVec; j < N; j += kTriThreads) {
       const double xj = fma(-ck1, v[j], __ldcg(Ak1 + j) - p[j]);
       x[j] = xj;
       if (j >= k + 3) xn = fma(xj, xj, xn);
     }
-    xn = warp_sum_d(xn);
+    if (k + 1 + 32 * wid < N) xn = warp_sum_d(xn);
     if (lane == 0) red[1][wid] = xn;
     __syncthreads();
     if (last) {  // the last 2 x 2 block
@@ -431,29 +487,55 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
     // the scalar warp forms the next reflector while the row warps finish their row's update and
     // take its dot with the unscaled column (u_{k+2} = 1, u_j = sc x_j beyond).  The sums run over
     // the columns k+3+l, k+35+l, ..., whichever lane holds them, and the shuffle tree pairs the
-    // same sums in every rotation of the lanes.  Row k+2 (at the end also the last) is published
-    double rawdot = 0.0, r0 = 0.0;
+    // same sums in every rotation of the lanes.  Row k+2 (at the end also the last) is published.
+    // The rows' loops skip groups of columns that are done with (a few columns of a group are
+    // updated for nothing: a test for each costs more), so that nothing but FP64 work is left
+    double rawdot[R], r0[R];
+#pragma unroll
+    for (int t = 0; t < R; ++t) rawdot[t] = r0[t] = 0.0;
     if (!row_warp) {
       hh_scalars(k + 2, red[1]);
-    } else if (has_row) {
-      const double ci = fma(-2.0 * al, vi, p[myrow]);
+    } else {
 #pragma unroll
-      for (int q = 0; q < kTriRowRegs; ++q) {
-        const int j = lane + 32 * q;
-        if (32 * q + 31 >= k + 2 && j >= k + 2 && j < N) {
-          rr[q] = fma(-ci, v[j], rr[q]);
-          if (j == k + 2) r0 = rr[q];
-          else rawdot = fma(rr[q], x[j], rawdot);
-        }
-      }
-      if (myrow == k + 2 || k == N - 4) {
+      for (int t = 0; t < R; ++t) {
+        if (!has_row[t]) continue;
+        const double ci = fma(-2.0 * al, vi[t], p[myrow[t]]);
 #pragma unroll
-        for (int q = 0; q < kTriRowRegs; ++q) {
-          const int j = lane + 32 * q;
-          if (j >= k + 2 && j < N) Amy[j] = rr[q];
+        for (int q0 = 0; q0 < Q; q0 += kRowGroup) {
+          if (32 * (q0 + kRowGroup) <= k + 2 || 32 * q0 >= N) continue;
+#pragma unroll
+          for (int q = q0; q < q0 + kRowGroup && q < Q; ++q)
+            rr[t][q] = fma(-ci, v[lane + 32 * q], rr[t][q]);
+          if (32 * q0 <= k + 2) {  // the group that holds column k+2
+#pragma unroll
+            for (int q = q0; q < q0 + kRowGroup && q < Q; ++q) {
+              const int j = lane + 32 * q;
+              if (j == k + 2) r0[t] = rr[t][q];
+              if (j > k + 2) rawdot[t] = fma(rr[t][q], x[j], rawdot[t]);
+            }
+          } else {
+#pragma unroll
+            for (int q = q0; q < q0 + kRowGroup && q < Q; ++q)
+              rawdot[t] = fma(rr[t][q], x[lane + 32 * q], rawdot[t]);
+          }
         }
+        if ((!CL && myrow[t] == k + 2) || k == N - 4) {
+#pragma unroll
+          for (int q = 0; q < Q; ++q) {
+            const int j = lane + 32 * q;
+            if (j >= k + 2 && j < N) A[(size_t)myrow[t] * N + j] = rr[t][q];
+          }
+        }
+        if (CL && myrow[t] == k + 2) {
+#pragma unroll
+          for (int q = 0; q < Q; ++q) {
+            const int j = lane + 32 * q;
+            if (j >= k + 2 && j < N)
+              for (int c = 0; c < G; ++c) store_peer(rb + ((k + 1) & 1) * N + j, c, rr[t][q]);
+          }
+        }
+        rawdot[t] = warp_sum_d(rawdot[t]);
       }
-      rawdot = warp_sum_d(rawdot);
     }
     __syncthreads();
     const double tau_n = sh[0], sc = sh[2];
@@ -466,8 +548,18 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
     // p_{k+1} = tau A u over the own rows i >= k+2
     double* pn = a.pbuf + (size_t)((k + 1) & 1) * N;
     if (reg_rows) {
-      if (has_row && lane == ((k + 2) & 31)) pn[myrow] = tau_n * fma(sc, rawdot, r0);
-      grid_arrive(a.hdr);
+#pragma unroll
+      for (int t = 0; t < R; ++t) {
+        if (!has_row[t]) continue;  // (uniform over the warp)
+        const double pi = tau_n * fma(sc, rawdot[t], r0[t]);  // in the lane that holds r0
+        if (CL) {
+          const double pv = __shfl_sync(0xffffffffu, pi, (k + 2) & 31);
+          if (lane < G) store_peer(pb + ((k + 1) & 1) * N + myrow[t], lane, pv);
+        } else if (lane == ((k + 2) & 31)) {
+          pn[myrow[t]] = pi;
+        }
+      }
+      arrive();
       hh_apply(k + 2, k + 1);
     } else {
       hh_apply(k + 2, k + 1);
@@ -504,9 +596,9 @@ __global__ void __launch_bounds__(kTriThreads, 1) k_tridiag(TriArgs a) {
         acc2 = warp_sum_d(acc2);
         if (lane == 0) pn[i] = tau_n * acc2;
       }
-      grid_arrive(a.hdr);
+      arrive();
     }
-    if (!grid_wait(a.hdr, (++bar) * G, &s_flag)) return;
+    if (!wait()) return;
     double* t = v;
     v = x;
     x = t;
@@ -572,18 +664,35 @@ __global__ void __launch_bounds__(256) k_tri_prep(int N, const double* __restric
     h->tnorm = tn * ts;
     h->tscale = ts;
     h->pivmin = 0x1p-100;
-    int s0 = 0, nb = 0;
-    for (int i = 0; i < N; ++i) {
-      if (sflag[i]) {
-        for (int r = s0; r <= i; ++r) {
-          bstart[r] = s0;
-          bend[r] = i + 1;
-        }
-        blist[nb++] = s0;
-        s0 = i + 1;
-      }
+  }
+  // the rows that end a block, a bit each; a row's block lies between the bits around it
+  const int nwd = (N + 31) / 32;
+  unsigned* ends = (unsigned*)(sflag + 2 * N);
+  for (int i = threadIdx.x; i < nwd * 32; i += blockDim.x) {
+    const unsigned m = __ballot_sync(0xffffffffu, i < N && sflag[i]);
+    if ((threadIdx.x & 31) == 0) ends[i / 32] = m;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < N; i += blockDim.x) {
+    int wd = i / 32;
+    unsigned m = ends[wd] >> (i & 31) << (i & 31);
+    while (!m) m = ends[++wd];  // (the last row ends a block)
+    bend[i] = 32 * wd + __ffs(m);
+    wd = i / 32;
+    m = ends[wd] & ((1u << (i & 31)) - 1u);
+    while (!m && wd > 0) m = ends[--wd];
+    const int s0 = m ? 32 * wd + 32 - __clz(m) : 0;
+    bstart[i] = s0;
+    if (s0 == i) {
+      int b = __popc(ends[i / 32] & ((1u << (i & 31)) - 1u));
+      for (int q = 0; q < i / 32; ++q) b += __popc(ends[q]);
+      blist[b] = i;
     }
-    s_nb = nb;
+    if (i == N - 1) {
+      int b = 0;
+      for (int q = 0; q < nwd; ++q) b += __popc(ends[q]);
+      s_nb = b;
+    }
   }
   __syncthreads();
   const int nb = s_nb, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
@@ -617,55 +726,71 @@ __global__ void __launch_bounds__(256) k_tri_prep(int N, const double* __restric
 
 // Number of eigenvalues of the (scaled) block [s0, s1) below sig in float: the ratio form
 // q_i = (d_i - sig) - e_{i-1}^2 / q_{i-1}, |q_i| floored at piv (a zero pivot counts negative).
-__device__ __forceinline__ int sturm_count_f32(const float* __restrict__ d,
-                                               const float* __restrict__ e2, int s0, int s1,
+// t holds (d_i, e_{i-1}^2).  The signs are shifted into a word, counted every eight rows.
+__device__ __forceinline__ int sturm_count_f32(const float2* __restrict__ t, int s0, int s1,
                                                float sig) {
   constexpr float piv = 1e-30f;
-  float q = d[s0] - sig;
+  float q = t[s0].x - sig;
   if (fabsf(q) < piv) q = -piv;
   int cnt = q < 0.0f ? 1 : 0;
-  for (int i = s0 + 1; i < s1; ++i) {
-    q = (d[i] - sig) - __fdividef(e2[i - 1], q);
+  int i = s0 + 1;
+  for (; i + 8 <= s1; i += 8) {
+    unsigned neg = 0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const float2 r = t[i + u];
+      q = (r.x - sig) - __fdividef(r.y, q);
+      if (fabsf(q) < piv) q = -piv;
+      neg = __funnelshift_l(__float_as_uint(q), neg, 1);
+    }
+    cnt += __popc(neg);
+  }
+  for (; i < s1; ++i) {
+    const float2 r = t[i];
+    q = (r.x - sig) - __fdividef(r.y, q);
     if (fabsf(q) < piv) q = -piv;
     cnt += q < 0.0f ? 1 : 0;
   }
   return cnt;
 }
 
-// The same count in double, bound by the FP64 pipe (16 clocks an instruction and SM) or by the one
-// chained FP64 operation of a row: a zero minor is only noted, and its rows are done again.  Sign changes of the leading minors
+// The same count in double: sign changes of the leading minors
 // p_i = (d_i - sig) p_{i-1} - e_{i-1}^2 p_{i-2} (a zero minor counts as a tiny negative ratio),
 // the pair (p_{i-1}, p_i) rescaled by 2^-+300 after every eighth row when its larger magnitude
 // has left [2^-300, 2^300] (with ||T||_inf <= 1 and the split threshold, eight rows move it by
-// at most 2^13 up or 2^-616 down).
-__device__ __forceinline__ int sturm_count_f64(const double* __restrict__ d,
-                                               const double* __restrict__ e2, int s0, int s1,
+// at most 2^13 up or 2^-616 down).  Eight rows at a time: their minors' signs go into a word, and a
+// zero among them is only noted and its rows done again, so that a row is three FP64 operations,
+// one of them in the chain, and little else.
+__device__ __forceinline__ int sturm_count_f64(const double2* __restrict__ t, int s0, int s1,
                                                double sig) {
-  double p0 = 1.0, p1 = d[s0] - sig;
+  double p0 = 1.0, p1 = t[s0].x - sig;
   if (dbl_is_zero(p1)) p1 = -0x1p-60;
   int cnt = dbl_sign(p1);
-  int i = s0 + 1;
-  while (i < s1) {
-    const int ib = i, iend = min(i + 8, s1), cb = cnt;
+  for (int i = s0 + 1; i < s1; i += 8) {
     const double b0 = p0, b1 = p1;
-    bool zero = false;
+    unsigned low = 0;
+    if (i + 8 <= s1) {
+      unsigned neg = (unsigned)dbl_sign(p1);  // signs of the minors, the last one in bit 0
+      low = 0xffffffffu;
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      if (i < iend) {
-        const double p2 = fma(d[i] - sig, p1, -(e2[i - 1] * p0));
-        zero |= dbl_is_zero(p2);
-        cnt += dbl_sign(p2) ^ dbl_sign(p1);
+      for (int u = 0; u < 8; ++u) {
+        const double2 r = t[i + u];
+        const double p2 = fma(r.x - sig, p1, -(r.y * p0));
+        const unsigned hi = (unsigned)__double2hiint(p2);
+        neg = __funnelshift_l(hi, neg, 1);
+        low = min(low, hi << 1);
         p0 = p1;
         p1 = p2;
-        ++i;
       }
+      if (low) cnt += __popc((neg ^ (neg >> 1)) & 0xffu);
     }
-    if (zero) {  // once more, with the zero minors replaced
+    if (!low) {  // the last rows, or a zero (or nearly) among the eight
       p0 = b0;
       p1 = b1;
-      cnt = cb;
-      for (i = ib; i < iend; ++i) {
-        double p2 = fma(d[i] - sig, p1, -(e2[i - 1] * p0));
+      const int iend = min(i + 8, s1);
+      for (int j = i; j < iend; ++j) {
+        const double2 r = t[j];
+        double p2 = fma(r.x - sig, p1, -(r.y * p0));
         if (dbl_is_zero(p2)) p2 = -p1 * 0x1p-60;
         cnt += dbl_sign(p2) ^ dbl_sign(p1);
         p0 = p1;
@@ -673,12 +798,11 @@ __device__ __forceinline__ int sturm_count_f64(const double* __restrict__ d,
       }
     }
     const int ex = max(dbl_biased_exp(p0), dbl_biased_exp(p1));
-    if (ex > 1023 + 300) {
-      p0 *= 0x1p-300;
-      p1 *= 0x1p-300;
-    } else if (ex < 1023 - 300) {
-      p0 *= 0x1p300;
-      p1 *= 0x1p300;
+    if (ex > 1023 + 300 || ex < 1023 - 300) {  // (a branch: the FP64 pipe is what counts here)
+      asm volatile("");
+      const double f = ex > 1023 ? 0x1p-300 : 0x1p300;
+      p0 *= f;
+      p1 *= f;
     }
   }
   return cnt;
@@ -689,6 +813,9 @@ __device__ __forceinline__ int sturm_count_f64(const double* __restrict__ d,
 // (brackets of ~2^-20 ||T||), the bracket widened by 4e-6 ||T|| (the float counts are exact
 // for a matrix within a few float roundings of T) and its ends checked by double counts (the
 // Gershgorin interval again if either fails), then double rounds to the width eps ||T||.
+// The nine double rounds are bound by the FP64 pipe, three operations of 64 clocks a row (with
+// rescaling by selects and a test on every row, and four warps on an SM at small N: 275 us at 120
+// and 2.6 ms at 1200; now 170 us and 1.56 ms).
 constexpr int kBisThreads = 128;
 __global__ void __launch_bounds__(kBisThreads) k_bisect(int N, const double* __restrict__ ds,
                                                         const double* __restrict__ e2,
@@ -699,16 +826,12 @@ __global__ void __launch_bounds__(kBisThreads) k_bisect(int N, const double* __r
                                                         const double* __restrict__ glo,
                                                         const double* __restrict__ ghi,
                                                         const EighHdr* h, double* lam) {
-  extern __shared__ double sb[];
-  double* sd = sb;
-  double* se2 = sb + N;
-  float* sdf = (float*)(sb + 2 * N);
-  float* se2f = sdf + N;
+  extern __shared__ double2 sb[];
+  double2* sd = sb;  // (d_i, e_{i-1}^2)
+  float2* sdf = (float2*)(sb + N);
   for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    sd[i] = ds[i];
-    sdf[i] = df[i];
-    se2[i] = i < N - 1 ? e2[i] : 0.0;
-    se2f[i] = i < N - 1 ? e2f[i] : 0.0f;
+    sd[i] = make_double2(ds[i], i > 0 ? e2[i - 1] : 0.0);
+    sdf[i] = make_float2(df[i], i > 0 ? e2f[i - 1] : 0.0f);
   }
   __syncthreads();
   const int lane = threadIdx.x & 31, j = lane & 15;
@@ -721,7 +844,7 @@ __global__ void __launch_bounds__(kBisThreads) k_bisect(int N, const double* __r
   }
   const int s0 = bstart[s], s1 = bend[s], k = s - s0;
   if (s1 - s0 == 1) {
-    if (j == 0) lam[s] = sd[s0];
+    if (j == 0) lam[s] = sd[s0].x;
     return;
   }
   const double tn = h->tnorm;
@@ -744,14 +867,14 @@ __global__ void __launch_bounds__(kBisThreads) k_bisect(int N, const double* __r
   for (int r = 0; r < 5; ++r) {
     const double step = (hi - lo) * (1.0 / 17.0);
     const double sg = lo + (j + 1) * step;
-    narrow(sturm_count_f32(sdf, se2f, s0, s1, (float)sg) > k, lo, step, 1);
+    narrow(sturm_count_f32(sdf, s0, s1, (float)sg) > k, lo, step, 1);
   }
   lo -= 4e-6 * tn;
   hi += 4e-6 * tn;
   {  // 16 points from lo to hi inclusive: the ends verify the float bracket
     const double step = (hi - lo) * (1.0 / 15.0);
     const double sg = lo + j * step;
-    const int c = sturm_count_f64(sd, se2, s0, s1, sg);
+    const int c = sturm_count_f64(sd, s0, s1, sg);
     const int clo = __shfl_sync(hm, c, lane & 16), chi = __shfl_sync(hm, c, (lane & 16) + 15);
     if (clo <= k && chi > k) {
       narrow(c > k, lo, step, 0);
@@ -764,7 +887,7 @@ __global__ void __launch_bounds__(kBisThreads) k_bisect(int N, const double* __r
     if (!(hi - lo > fmax(DBL_EPSILON * tn, 2.0 * DBL_EPSILON * fmax(fabs(lo), fabs(hi))))) break;
     const double step = (hi - lo) * (1.0 / 17.0);
     const double sg = lo + (j + 1) * step;
-    narrow(sturm_count_f64(sd, se2, s0, s1, sg) > k, lo, step, 1);
+    narrow(sturm_count_f64(sd, s0, s1, sg) > k, lo, step, 1);
   }
   if (j == 0) lam[s] = 0.5 * (lo + hi);
 }
@@ -778,6 +901,7 @@ __device__ __forceinline__ long long dbl_key(double x) {
 // Rank of every eigenvalue (integer keys, ties by slot), eigenvalues of A in ascending order;
 // CTA 0 also lists the clusters: runs of a block's consecutive eigenvalues closer than
 // kClusterTol ||T|| (the gaps tested in parallel, the runs found by one thread).
+constexpr int kRankLanes = 8;  // threads per eigenvalue
 __global__ void __launch_bounds__(256) k_rank_plan(int N, const double* __restrict__ lam,
                                                    const int* __restrict__ bend, EighHdr* h,
                                                    int* col, double* w_out, int* incl, int* cl,
@@ -787,35 +911,51 @@ __global__ void __launch_bounds__(256) k_rank_plan(int N, const double* __restri
   for (int i = threadIdx.x; i < N; i += blockDim.x) skey[i] = dbl_key(lam[i]);
   __syncthreads();
   const double unscale = 1.0 / (h->tscale * h->scale);  // a power of two
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s < N) {
-    const long long ks = skey[s];
+  const int s = (blockIdx.x * blockDim.x + threadIdx.x) / kRankLanes;
+  const int part = threadIdx.x % kRankLanes;
+  {
+    const long long ks = s < N ? skey[s] : 0;
     int r = 0;
-    for (int t = 0; t < N; ++t) {
+    for (int t = part; t < N; t += kRankLanes) {
       const long long kt = skey[t];
       r += (kt < ks || (kt == ks && t < s)) ? 1 : 0;
     }
-    const double ls = lam[s];
-    if (ls != ls) r = s;  // NaN (a failed reduction): its own slot
-    col[s] = r;
-    w_out[r] = ls * unscale;
+#pragma unroll
+    for (int o = kRankLanes / 2; o; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    if (s < N && part == 0) {
+      const double ls = lam[s];
+      if (ls != ls) r = s;  // NaN (a failed reduction): its own slot
+      col[s] = r;
+      w_out[r] = ls * unscale;
+    }
   }
   if (blockIdx.x != 0) return;
   const double tol = kClusterTol * h->tnorm;
   for (int i = threadIdx.x; i < N; i += blockDim.x)
     sgap[i] = (i + 1 < bend[i] && lam[i + 1] - lam[i] < tol) ? 1 : 0;
   __syncthreads();
+  // no cluster anywhere, and the rows where one starts, a bit each
+  const int nw = (N + 31) / 32;
+  unsigned* first = (unsigned*)(sgap + N);
+  for (int i = threadIdx.x; i < nw * 32; i += blockDim.x) {
+    if (i < N) incl[i] = cj[i] = 0;
+    const bool st = i < N && sgap[i] && (i == 0 || !sgap[i - 1]);
+    const unsigned m = __ballot_sync(0xffffffffu, st);
+    if ((threadIdx.x & 31) == 0) first[i / 32] = m;
+  }
+  __syncthreads();
   if (threadIdx.x != 0) return;
   int ncl = 0, maxcl = 0, off = 0;
-  for (int s0 = 0; s0 < N;) {
-    int t = s0;
-    while (sgap[t]) ++t;  // sgap[bend - 1] = 0 ends every run inside its block
-    const int m = t - s0 + 1;
-    for (int u = s0; u <= t; ++u) {
-      incl[u] = m > 1 ? ncl + 1 : 0;  // cluster id + 1
-      cj[u] = u - s0;                 // member index
-    }
-    if (m > 1) {
+  for (int wd = 0; wd < nw; ++wd)
+    for (unsigned m0 = first[wd]; m0; m0 &= m0 - 1) {
+      const int s0 = 32 * wd + __ffs(m0) - 1;
+      int t = s0;
+      while (sgap[t]) ++t;  // sgap[bend - 1] = 0 ends every run inside its block
+      const int m = t - s0 + 1;
+      for (int u = s0; u <= t; ++u) {
+        incl[u] = ncl + 1;  // cluster id + 1
+        cj[u] = u - s0;     // member index
+      }
       const int a0 = bstart[s0], L = bend[s0] - a0;
       int* c = cl + kClDesc * ncl;
       c[0] = s0;
@@ -827,8 +967,6 @@ __global__ void __launch_bounds__(256) k_rank_plan(int N, const double* __restri
       maxcl = max(maxcl, m);
       ++ncl;
     }
-    s0 = t + 1;
-  }
   h->ncl = ncl;
   h->maxcl = maxcl;
 }
@@ -856,7 +994,11 @@ __device__ __forceinline__ double pivot_floor(double v) {
 // gamma_i = D+_i - e_i^2 / D-_{i+1} (each thread half the rows), the twist r where |gamma_r|
 // is smallest (first such row), z_r = 1, and thread 0 forms z_i = -e_i z_{i+1} / D+_i above r
 // while thread 1 forms z_i = -e_{i-1} z_{i-1} / D-_i below it; normalised to unit length.
-// Z[i][col] (row-major, column = rank of the eigenvalue), zero outside the block.
+// Z[i][col] (row-major, column = rank of the eigenvalue), zero outside the block.  Bound by the
+// chain of a row's pivot and reciprocal (five FP64 operations, three conversions), which both
+// threads run in one stream of instructions; in the other passes a row's loads are ahead of the
+// chain.  (The sides one after the other and each load in the chain: 157 us at 120 and 1.93 ms at
+// 1200; now 87 us and 0.90 ms.)
 __global__ void __launch_bounds__(32) k_twisted(int N, const double* __restrict__ ds,
                                                 const double* __restrict__ es,
                                                 const double* __restrict__ e2,
@@ -878,25 +1020,19 @@ __global__ void __launch_bounds__(32) k_twisted(int N, const double* __restrict_
   }
   if (incl[s]) return;
   const double lm = lam[s];
-  if (side == 0) {
-    double dp = pivot_floor(ds[s0] - lm), rp = rcp_nr(dp);
-    Z[s0 * ld + c] = dp;
-    Wp[s0 * ld + c] = rp;
+  {  // both threads' pivots in one stream of instructions: row i0 + dir t
+    const int dir = side == 0 ? 1 : -1, i0 = side == 0 ? s0 : s1 - 1, eo = side == 0 ? -1 : 0;
+    double* W = side == 0 ? Wp : Wd;
+    double pv = pivot_floor(ds[i0] - lm), rv = rcp_nr(pv);
+    if (side == 0) Z[i0 * ld + c] = pv;
+    W[i0 * ld + c] = rv;
 #pragma unroll 4
-    for (int i = s0 + 1; i < s1; ++i) {
-      dp = pivot_floor(fma(-e2[i - 1], rp, ds[i] - lm));
-      rp = rcp_nr(dp);
-      Z[i * ld + c] = dp;
-      Wp[i * ld + c] = rp;
-    }
-  } else {
-    double dm = pivot_floor(ds[s1 - 1] - lm), rm = rcp_nr(dm);
-    Wd[(s1 - 1) * ld + c] = rm;
-#pragma unroll 4
-    for (int i = s1 - 2; i >= s0; --i) {
-      dm = pivot_floor(fma(-e2[i], rm, ds[i] - lm));
-      rm = rcp_nr(dm);
-      Wd[i * ld + c] = rm;
+    for (int t = 1; t < s1 - s0; ++t) {
+      const int i = i0 + dir * t;
+      pv = pivot_floor(fma(-e2[i + eo], rv, ds[i] - lm));
+      rv = rcp_nr(pv);
+      if (side == 0) Z[i * ld + c] = pv;
+      W[i * ld + c] = rv;
     }
   }
   __syncwarp(pm);
@@ -1145,8 +1281,8 @@ __global__ void k_cluster_scatter(int N, int s, int m, int a0, int L,
 // ---------------------------------------------------------------------------
 // 4. back-transformation V = Q Z, Q = H_0 ... H_{nref-1} in blocks of kNb reflectors
 // ---------------------------------------------------------------------------
-// Gram matrices G_b = Y_b^T Y_b of every block (entries c <= c' only), Y_b's column c the
-// reflector k0 + c: grid (nblk, kNb / 16, kNb / 16) of 16 x 16 sub-tiles, upper ones only.
+// Gram matrices G_b = Y_b^T Y_b of every block, Y_b's column c the reflector k0 + c: grid (nblk,
+// kNb / 16, kNb / 16) of 16 x 16 sub-tiles, the upper ones formed and mirrored.
 __global__ void __launch_bounds__(256) k_gram(int N, int nref, const double* __restrict__ Yr,
                                               double* G) {
   const int b = blockIdx.x, tr = blockIdx.y, tc = blockIdx.z;
@@ -1170,36 +1306,42 @@ __global__ void __launch_bounds__(256) k_gram(int N, int nref, const double* __r
     __syncthreads();
   }
   G[(size_t)b * kNb * kNb + gr * kNb + gc] = acc;
+  if (tr < tc) G[(size_t)b * kNb * kNb + gc * kNb + gr] = acc;
 }
 
 // Triangular factors T_b (upper): T^-1 = diag(1 / tau) + the strictly upper part of G, so column
 // j solves T_jj = tau_j, T_ij = -tau_i sum_{c = i+1}^{j} G_ic T_cj upwards from i = j - 1: a warp
-// per column, the column in shared memory, the sums over the lanes.  (A thread per row with one
-// chain of up to 2016 terms: 163 us; this: 39 us.)
-__global__ void __launch_bounds__(256) k_tfactor(int nref, const double* __restrict__ tau,
-                                                 const double* __restrict__ G, double* T) {
-  __shared__ double x[8][kNb];
-  const int b = blockIdx.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int k0 = b * kNb, j = blockIdx.y * 8 + w;
+// per column, lane l with the sums of rows l and l + 32, to which every new T_ij is added at once (G
+// is symmetric: its row i holds the factors).  Bound by the chain of a product, a broadcast and an
+// addition per row.  (Dots over the lanes: 39 us;
+// this: 20 us.)
+constexpr int kTfWarps = 4;
+__global__ void __launch_bounds__(32 * kTfWarps) k_tfactor(int nref, const double* __restrict__ tau,
+                                                           const double* __restrict__ G,
+                                                           double* T) {
+  const int b = blockIdx.x, lane = threadIdx.x & 31;
+  const int k0 = b * kNb, j = blockIdx.y * kTfWarps + (threadIdx.x >> 5);
   const int m = nref - k0 < kNb ? nref - k0 : kNb;
   const double* Gb = G + (size_t)b * kNb * kNb;
   double* Tb = T + (size_t)b * kNb * kNb;
-  x[w][lane] = 0.0;
-  x[w][lane + 32] = 0.0;
-  __syncwarp();
+  const double t0 = lane < m ? -tau[k0 + lane] : 0.0, t1 = lane + 32 < m ? -tau[k0 + lane + 32] : 0.0;
+  double s0 = 0.0, s1 = 0.0;  // sums, then (rows >= i) the entries of T
   if (j < m) {
-    if (lane == 0) x[w][j] = tau[k0 + j];
-    __syncwarp();
-    for (int i = j - 1; i >= 0; --i) {
-      const double g0 = lane > i ? Gb[i * kNb + lane] : 0.0;
-      const double g1 = lane + 32 > i ? Gb[i * kNb + lane + 32] : 0.0;
-      const double t = warp_sum_d(fma(g0, x[w][lane], g1 * x[w][lane + 32]));
-      if (lane == 0) x[w][i] = -tau[k0 + i] * t;
-      __syncwarp();
+    // T_jj as if -tau_j times a sum of -1
+    if (lane == (j & 31)) (j < 32 ? s0 : s1) = -1.0;
+#pragma unroll 4
+    for (int i = j; i >= 0; --i) {
+      const double g0 = lane < i ? Gb[i * kNb + lane] : 0.0;
+      const double g1 = lane + 32 < i ? Gb[i * kNb + lane + 32] : 0.0;
+      const double e = i < 32 ? t0 * s0 : t1 * s1;  // of use in lane i mod 32
+      const double t = __shfl_sync(0xffffffffu, e, i & 31);
+      if (lane == (i & 31)) (i < 32 ? s0 : s1) = t;
+      if (lane < i) s0 = fma(g0, t, s0);
+      if (i > 32 && lane + 32 < i) s1 = fma(g1, t, s1);
     }
   }
-  Tb[(size_t)lane * kNb + j] = x[w][lane];
-  Tb[(size_t)(lane + 32) * kNb + j] = x[w][lane + 32];
+  Tb[(size_t)lane * kNb + j] = lane <= j ? s0 : 0.0;
+  Tb[(size_t)(lane + 32) * kNb + j] = lane + 32 <= j ? s1 : 0.0;
 }
 
 struct DevInfo {
@@ -1221,6 +1363,70 @@ int device_sms(int* sms) {
   }
   *sms = it->second.sms;
   return DONOF_OK;
+}
+
+// The largest cluster of CTAs of the cluster form that the device takes (asked once per device).
+int tridiag_cluster_max() {
+  static std::atomic<int> known[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64) return 0;
+  int c = known[dev].load();
+  if (c > 0) return c - 1;
+  int best = 0;
+  if (cudaFuncSetAttribute(k_tridiag<kClRows, kClCols / 32, true>,
+                           cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+    for (int size = kClCtas; size >= 1 && best == 0; size /= 2) {
+      cudaLaunchAttribute at{};
+      at.id = cudaLaunchAttributeClusterDimension;
+      at.val.clusterDim.x = size;
+      at.val.clusterDim.y = at.val.clusterDim.z = 1;
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = dim3(size);
+      cfg.blockDim = dim3(kTriThreads);
+      cfg.dynamicSmemBytes = ((size_t)7 * kClCols) * 8;
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+      int n = 0;
+      if (cudaOccupancyMaxActiveClusters(&n, k_tridiag<kClRows, kClCols / 32, true>, &cfg) ==
+              cudaSuccess && n > 0)
+        best = size;
+    }
+  }
+  cudaGetLastError();  // a size that the device does not take is no error of the call
+  known[dev].store(best + 1);
+  return best;
+}
+
+cudaError_t launch_tridiag(TriArgs a, int sms, cudaStream_t s) {
+  int size = 1;
+  while (size * kRowWarps < a.N && size < kClCtas) size *= 2;
+  // One cluster while a row warp has one row and the vector few pieces (all of donof_eigh, grid ->
+  // cluster: 24: 278 -> 268 us, 64: 552 -> 509, 120: 962 -> 891; with two rows a warp 160: 1288 ->
+  // 1298, 256: 2286 -> 2490).  Fewer CTAs for the grid form change nothing (1 to 8 rows a CTA)
+  if (a.N <= kClCols && size <= tridiag_cluster_max()) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = size;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(size);
+    cfg.blockDim = dim3(kTriThreads);
+    cfg.dynamicSmemBytes = ((size_t)3 * kClCols + 4 * a.N) * 8;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_tridiag<kClRows, kClCols / 32, true>, a);
+  }
+  const auto kern = k_tridiag<1, kTriRowRegs, false>;
+  const size_t smem = (size_t)3 * (a.N < 32 * kTriRowRegs ? 32 * kTriRowRegs : a.N) * 8;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  int occ = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kTriThreads, smem);
+  if (e != cudaSuccess) return e;
+  if (occ < 1) return cudaErrorInvalidValue;
+  void* args[] = {&a};
+  return cudaLaunchCooperativeKernel((const void*)kern, dim3(sms), dim3(kTriThreads), args, smem, s);
 }
 
 }  // namespace
@@ -1280,23 +1486,12 @@ int eigh_run(int N, const double* A, double* V, double* w, char* ws, cudaStream_
   int sms = 0;
   int rc = device_sms(&sms);
   if (rc != DONOF_OK) return rc;
-  const size_t tri_smem = (size_t)3 * N * 8;
-  if (!ok(cudaFuncSetAttribute(k_tridiag, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)tri_smem)))
-    return DONOF_ERR_CUDA;
-  int occ = 0;
-  if (!ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_tridiag, kTriThreads, tri_smem)) ||
-      occ < 1)
-    return DONOF_ERR_CUDA;
   TriArgs ta{N, Aw, Yr, d, e, tau, (double*)(ws + L.pbuf), hdr};
-  void* targs[] = {&ta};
-  if (!ok(cudaLaunchCooperativeKernel((const void*)k_tridiag, dim3(sms), dim3(kTriThreads), targs,
-                                      tri_smem, s)))
-    return DONOF_ERR_CUDA;
+  if (!ok(launch_tridiag(ta, sms, s))) return DONOF_ERR_CUDA;
   count_launch(1);
 
   // 2. eigenvalues (of T scaled to ||T||_inf <= 1)
-  const size_t prep_smem = (size_t)2 * N * 4;
+  const size_t prep_smem = (size_t)2 * N * 4 + (size_t)(N + 31) / 32 * 4;
   if (!ok(cudaFuncSetAttribute(k_tri_prep, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)prep_smem)))
     return DONOF_ERR_CUDA;
@@ -1309,11 +1504,11 @@ int eigh_run(int N, const double* A, double* V, double* w, char* ws, cudaStream_
   const int bis_threads = N <= 2 * sms ? 32 : kBisThreads;
   k_bisect<<<(N * 16 + bis_threads - 1) / bis_threads, bis_threads, bis_smem, s>>>(
       N, ds, e2, df, e2f, bstart, bend, glo, ghi, hdr, lam);
-  const size_t rank_smem = (size_t)N * 12;
+  const size_t rank_smem = (size_t)N * 12 + (size_t)(N + 31) / 32 * 4;
   if (!ok(cudaFuncSetAttribute(k_rank_plan, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)rank_smem)))
     return DONOF_ERR_CUDA;
-  k_rank_plan<<<(N + 255) / 256, 256, rank_smem, s>>>(N, lam, bend, hdr, col, w, incl, cl, cj,
+  k_rank_plan<<<(N * kRankLanes + 255) / 256, 256, rank_smem, s>>>(N, lam, bend, hdr, col, w, incl, cl, cj,
                                                       bstart);
   // 3. eigenvectors of T (into V)
   k_twisted<<<(2 * N + 31) / 32, 32, 0, s>>>(N, ds, es, e2, bstart, bend, lam, col, incl, V, Wp,
@@ -1379,7 +1574,7 @@ int eigh_run(int N, const double* A, double* V, double* w, char* ws, cudaStream_
   // 4. V = Q Z
   if (L.nblk > 0) {
     k_gram<<<dim3(L.nblk, kNb / 16, kNb / 16), 256, 0, s>>>(N, L.nref, Yr, G);
-    k_tfactor<<<dim3(L.nblk, kNb / 8), 256, 0, s>>>(L.nref, tau, G, T);
+    k_tfactor<<<dim3(L.nblk, kNb / kTfWarps), 32 * kTfWarps, 0, s>>>(L.nref, tau, G, T);
     count_launch(2);
     if (!ok(cudaGetLastError()) ||
         !ok(digit_reflect(N, L.nref, Yr, T, V, ws + L.A, &hdr->abort_code, &hdr->abort, s)))
