@@ -406,6 +406,7 @@ struct DigitArgs {
   const __half* Bimg;   // stage images of B (k_digit_planes)
   const int* eB;        // per column, as eA
   int N, NT, ntiles, mtiles, nstages, splits;
+  int imgNT;            // columns of the images' tiles, a multiple of NT
   // C(m, n) at C + split sCs + (m / Mb) sCb + (m % Mb) sCm + n
   double* C;
   long long sCs, sCb, sCm;

@@ -25,21 +25,24 @@
 // doubles themselves (8 bytes per element read once per column tile instead of 16 of digits
 // written and read).
 //
-// CTA (544 threads, one per SM, 16 worker warps and an MMA warp): a unit is a 128 x NT output
-// tile (NT <= 64) and a range of 32-wide K stages.  Per stage each worker thread turns 8
-// doubles (fetched one stage ahead) into 8 x 8 digits in shared memory; one thread issues the
-// MMAs: A's digit i against B's stacked digits 0 .. 7 - i, whose products land in the
-// neighbouring accumulators i .. 7, so a digit of A is read once per 256 columns.  The flush of
-// a chunk follows the splitting of the next stage, so the MMAs drain meanwhile; carries go back
-// to TMEM, so that only group 0 needs registers between the chunks of a unit.
+// CTA (576 threads, one per SM, 16 worker warps, an MMA warp and a copying warp): a unit is a 128 x
+// NT output tile (NT <= 64) and a range of 32-wide K stages.  Per stage each worker thread turns 8
+// doubles (fetched one stage ahead) into 8 x 8 digits in shared memory; the MMA warp multiplies A's
+// digit i with B's stacked digits 0 .. 7 - i, whose products land in the neighbouring
+// accumulators i .. 7, so a digit of A is read once per 256 columns; the copying warp fetches B's
+// digits.  The flush of a chunk follows the splitting of the next stage, so the MMAs drain
+// meanwhile; carries go back to TMEM, so that only group 0 needs registers between the chunks of a
+// unit.
 //
-// Measured: 2.4 us per stage of a full unit (128 x 48 or 64 columns, 32 of k), 24 to 34 TFLOP/s;
-// X = B C at N 500, 80 orbitals, 2000 slices: 4.1 ms, 78.9 ms on the FP64 pipe.  What bounds it:
-// the splitting's integer instructions (about 400 per warp and stage, the integer ALU at half
-// rate: 2300 of 5000 clocks) and the MMAs' shared-memory reads (100 KB per 16 of k at 128 bytes a
-// clock, 1600 clocks per stage), which overlap only in part.  Tried and dropped: the
-// double-to-integer conversion for the split (10 % slower), A's digits in TMEM (the MMAs are
-// faster, but NT is 48 at most and the stores cost the workers as much), stages of 16 (slower).
+// Measured: 3150 clocks per stage of a 128 x 48 tile, 1.7 us, and some 10000 per unit for the
+// conversion of its result; X = B C at N 500, 80 orbitals, 2000 slices: 3.4 ms (78.9 ms on the FP64
+// pipe).  What bounds it: the workers' integer instructions (about 400 per warp and stage, the
+// integer ALU at half rate, 2000 clocks), with four warps to a scheduler to hide their latencies;
+// the MMAs' shared-memory reads (100 KB per 16 of k at 128 bytes a clock, 1600 clocks per stage)
+// run beside them.  Tried and dropped: the double-to-integer conversion for the split (10 %
+// slower), A's digits in TMEM (the MMAs are faster, but NT is 48 at most and the stores cost the
+// workers as much), stages of 16 (slower), loops instead of unrolled columns in the conversion
+// of the results (what they keep in local memory costs 20 %), waits that sleep (1 % slower).
 #include <atomic>
 
 #include "common.cuh"
@@ -52,7 +55,7 @@ constexpr int kD = 8;             // digits of an operand
 constexpr int kStageK = 32;       // elements of k per stage (64-byte rows, 64-byte swizzle)
 constexpr int kChunkStages = 8;   // stages per exact accumulation (256 elements)
 constexpr int kWorkers = 16;      // worker warps
-constexpr int kDigThreads = 32 * (kWorkers + 1);
+constexpr int kDigThreads = 32 * (kWorkers + 2);  // ..., the MMA warp, the copying warp
 constexpr int kTileM = 128;
 constexpr uint32_t kABytes = kD * kTileM * kStageK * 2;  // a stage of A digits
 // sum_{i > 0} 64 2^(7 (7 - i)) + 256 2^49: makes every digit's field non-negative
@@ -135,13 +138,23 @@ __device__ __forceinline__ uint32_t sw64(int row, int chunk) {
   return (uint32_t)(row * 64 + ((chunk ^ ((row >> 1) & 3)) << 4));
 }
 
-// mbar_wait with only its first attempt inlined.
-__device__ __noinline__ bool wait_long(uint32_t bar, uint32_t parity, int* status,
-                                       int* abort_flag) {
-  return mbar_wait(bar, parity, status, abort_flag);
-}
+// mbar_wait without a call: a call saves the caller's registers, among them the elements of A that
+// are still on their way from memory, and so waits for them (a build of 500 / 2000 / 80: 5.73 ms
+// with calls, 5.68 without).
 __device__ __forceinline__ bool wait_for(uint32_t bar, uint32_t parity, const DigitArgs& a) {
-  return mbar_try(bar, parity) || wait_long(bar, parity, a.status, a.abort_flag);
+  uint32_t t0 = 0;
+  for (uint32_t it = 0;; ++it) {
+    if (mbar_try(bar, parity)) return true;
+    if ((it & 255u) != 255u) continue;
+    if (*(volatile int*)a.abort_flag != 0) return false;
+    const uint32_t t = (uint32_t)globaltimer();
+    if (it == 255u) t0 = t;
+    if (t - t0 > (uint32_t)kWaitLimitNs) {
+      atomicExch(a.abort_flag, 1);
+      atomicCAS(a.status, 0, (int)DONOF_ERR_TIMEOUT);
+      return false;
+    }
+  }
 }
 
 __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
@@ -247,6 +260,38 @@ struct Cursor {
   }
 };
 
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r));
+  return r;
+}
+// mma_f16<0> by the lanes with lead != 0, the descriptors given as their low words (start address
+// and leading byte offset); the high word is that of sdesc(., 64).
+__device__ __forceinline__ void mma_f16_if(uint32_t lead, uint32_t dtmem, uint32_t a, uint32_t b,
+                                           uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\t"
+      "mov.b64 da, {%1, %6};\n\t"
+      "mov.b64 db, {%2, %6};\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "setp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n\t}" ::"r"(dtmem),
+      "r"(a), "r"(b), "r"(idesc), "r"(accumulate), "r"(lead), "n"(32 | 1 << 14 | 4 << 29)
+      : "memory");
+}
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const __half* src, uint32_t bytes,
+                                          uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
+          "r"(dst),
+      "l"((unsigned long long)src), "r"(bytes), "r"(bar)
+      : "memory");
+}
+
 template <bool KC, int NT>
 __global__ void __launch_bounds__(kDigThreads, 1)
     k_digit_gemm(const __grid_constant__ DigitArgs a) {
@@ -259,8 +304,9 @@ __global__ void __launch_bounds__(kDigThreads, 1)
   // accumulators read, clean-up
   enum { kAFull = 0, kBFull = 2, kEmpty = 4, kAccFull = 6, kAccEmpty = 7, kClean = 8 };
   uint32_t* tmem_slot = (uint32_t*)(bars + 9);
-  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
-  const uint32_t smem0 = smem_u32(smem), bar0 = smem_u32(bars);
+  const int tid = threadIdx.x, lane = tid % 32;
+  const int warp = __shfl_sync(0xffffffffu, tid / 32, 0);
+  const uint32_t smem0 = (smem_u32(smem_raw) + 1023u) & ~1023u, bar0 = smem0 + 2 * stage_bytes;
   auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
   const int units = a.mtiles * a.ntiles * a.splits;
   if (tid == 0) {
@@ -279,13 +325,17 @@ __global__ void __launch_bounds__(kDigThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *(volatile uint32_t*)tmem_slot;
+  constexpr uint32_t tmem = 0;  // all 512 columns are this CTA's: they start at column 0
   // all of the above while the kernel before runs
   const int zero = chain_wait();
 
   if (warp == kWorkers) {
-    if (lane == 0) {  // ------------------------------------------------ MMA issuer
+    {  // ------------------------------------------------ MMA issuer
+      // The whole warp walks the stages and one elected lane issues, so that the descriptors are
+      // computed in the uniform registers the MMAs take them from (a branch of one lane moves
+      // them there, eight moves an MMA: a build of 500 / 2000 / 80 5.68 ms, so 5.19)
       uint32_t it = 0, chunk = 0;
+      const uint32_t lead = elect_one();
       bool ok = true;
       constexpr int per = 256 / NT < kD ? 256 / NT : kD;  // digits of B per MMA
       for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
@@ -295,18 +345,15 @@ __global__ void __launch_bounds__(kDigThreads, 1)
         for (int st = s0; st < s1; ++st, ++it) {
           const int c = (st - s0) % kChunkStages;
           const uint32_t buf = it & 1u, ph = (it >> 1) & 1u;
-          if (c == 0 && !wait_for(bar(kAccEmpty), (chunk & 1u) ^ 1u, a)) {
-            ok = false;
-            break;
-          }
-          if (!wait_for(bar(kBFull + buf), ph, a) ||
-              !wait_for(bar(kAFull + buf), ph, a)) {
+          bool ready = c > 0 || wait_for(bar(kAccEmpty), (chunk & 1u) ^ 1u, a);
+          ready = ready && wait_for(bar(kBFull + buf), ph, a) && wait_for(bar(kAFull + buf), ph, a);
+          if (!__all_sync(0xffffffffu, ready)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t abase = smem_u32(smem + (size_t)buf * stage_bytes);
-          const uint64_t ad0 = sdesc(abase, 64), bd0 = sdesc(abase + kABytes, 64);
+          const uint32_t ad0 = ((smem0 + buf * stage_bytes) >> 4) | 1u << 16;
+          const uint32_t bd0 = ad0 + (kABytes >> 4);
 #pragma unroll
           for (int k = 0; k < kStageK / 16; ++k) {
             const uint32_t acc = (st > s0 || k > 0) ? 1u : 0u;
@@ -317,24 +364,65 @@ __global__ void __launch_bounds__(kDigThreads, 1)
                 const int n = kD - i - j < per ? kD - i - j : per;
                 // descriptors: the start address counts 16 bytes; the first products of every
                 // accumulator are those of digit 0 of A
-                mma_f16<0>(tmem + (uint32_t)((i + j) * NT),
-                           ad0 + (uint64_t)((i * (kTileM * 64) + k * 32) >> 4),
-                           bd0 + (uint64_t)((j * NT * 64 + k * 32) >> 4),
+                mma_f16_if(lead, tmem + (uint32_t)((i + j) * NT),
+                           ad0 + (uint32_t)((i * (kTileM * 64) + k * 32) >> 4),
+                           bd0 + (uint32_t)((j * NT * 64 + k * 32) >> 4),
                            idesc_f16(kTileM, n * NT), i == 0 ? acc : 1u);
               }
             }
           }
-          mma_commit<0>(bar(kEmpty + buf));
+          if (lead) mma_commit<0>(bar(kEmpty + buf));
           if (c == kChunkStages - 1 || st == s1 - 1) {
-            mma_commit<0>(bar(kAccFull));
+            if (lead) mma_commit<0>(bar(kAccFull));
             ++chunk;
           }
         }
       }
-      if (*(volatile int*)a.abort_flag != 0) {  // MMAs in flight complete before TMEM is freed
-        mma_commit_local<0>(bar(kClean));
+      // after an abort, MMAs in flight complete before TMEM is freed
+      if (__any_sync(0xffffffffu, *(volatile int*)a.abort_flag != 0)) {
+        if (lead) mma_commit_local<0>(bar(kClean));
+        __syncwarp();
         mbar_wait_quiet(bar(kClean), 0u, kDrainLimitNs);
       }
+    }
+    __syncwarp();
+  } else if (warp == kWorkers + 1) {  // ------------------------------------ copies of B's digits
+    // (a warp of its own: one of the workers, whose arrivals all wait for, held up every stage: a
+    // build of 500 / 2000 / 80 5.19 ms, so 4.78)
+    if (lane == 0) {
+      uint32_t it = 0, issued[2] = {0, 0};
+      bool ok = true;
+      for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+        const int sp = u / (a.ntiles * a.mtiles);
+        const int s0 = (int)((long long)a.nstages * sp / a.splits);
+        const int s1 = (int)((long long)a.nstages * (sp + 1) / a.splits);
+        const int n0 = u % a.ntiles * NT;
+        const size_t img_stage = (size_t)kD * a.imgNT * kStageK;
+        // NT rows of every digit's rows (a multiple of 16: the swizzle's phase is theirs)
+        const __half* img = a.Bimg + ((size_t)(n0 / a.imgNT) * a.nstages + s0) * img_stage +
+                            n0 % a.imgNT * kStageK;
+        for (int st = s0; st < s1; ++st, ++it, img += img_stage) {
+          const uint32_t buf = it & 1u, ph = (it >> 1) & 1u;
+          if (!wait_for(bar(kEmpty + buf), ph ^ 1u, a)) {
+            ok = false;
+            break;
+          }
+          const uint32_t dst = smem0 + buf * stage_bytes + kABytes;
+          mbar_expect_tx(bar(kBFull + buf), b_bytes);
+          if (a.imgNT == NT) {
+            bulk_copy(dst, img, b_bytes, bar(kBFull + buf));
+          } else {
+#pragma unroll
+            for (int d = 0; d < kD; ++d)
+              bulk_copy(dst + (uint32_t)d * (NT * kStageK * 2),
+                        img + (size_t)d * a.imgNT * kStageK, NT * kStageK * 2, bar(kBFull + buf));
+          }
+          ++issued[buf];
+        }
+      }
+      // the copies issued land before the CTA leaves, after an abort too
+      for (int i = 0; i < 2; ++i)
+        if (issued[i]) mbar_wait_quiet(bar(kBFull + i), (issued[i] - 1) & 1u, kDrainLimitNs);
     }
     __syncwarp();
   } else {  // --------------------------------------------------------- workers
@@ -478,7 +566,6 @@ __global__ void __launch_bounds__(kDigThreads, 1)
 
     bool pend = false, pend_last = false;
     int pend_u = 0, c = 0;
-    uint32_t b_issued[2] = {0, 0};
     const uint32_t dst = KC ? sw64(tid >> 2, tid & 3) : sw64(tid & 127, tid >> 7);
     while (ok && cur.u < units) {
       const uint32_t buf = it & 1u, ph = (it >> 1) & 1u;
@@ -487,16 +574,6 @@ __global__ void __launch_bounds__(kDigThreads, 1)
         break;
       }
       const uint32_t sa = smem0 + buf * stage_bytes;
-      if (tid == 0) {
-        const size_t img = ((size_t)(cur.u % a.ntiles) * a.nstages + cur.st) * (b_bytes / 2);
-        mbar_expect_tx(bar(kBFull + buf), b_bytes);
-        asm volatile(
-            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
-                "r"(sa + kABytes),
-            "l"((unsigned long long)(a.Bimg + img)), "r"(b_bytes), "r"(bar(kBFull + buf))
-            : "memory");
-        ++b_issued[buf];
-      }
       const int u = cur.u;
       const bool last = cur.last();
       Fixed8 f;
@@ -524,10 +601,6 @@ __global__ void __launch_bounds__(kDigThreads, 1)
       }
     }
     if (ok && pend) flush(pend_u, pend_last);
-    // after an abort, the B copies issued land before the CTA leaves
-    if (tid == 0 && *(volatile int*)a.abort_flag != 0)
-      for (int s = 0; s < 2; ++s)
-        if (b_issued[s]) mbar_wait_quiet(bar(kBFull + s), (b_issued[s] - 1) & 1u, kDrainLimitNs);
   }
   tc_fence_before();
   __syncthreads();
@@ -941,13 +1014,39 @@ cudaError_t launch_exps_planes(const double* S, long long ld, int K, int ncols, 
   return cudaGetLastError();
 }
 
+// Columns of a unit's tile: the width of the images' tiles or a divisor of it, whichever takes the
+// units through the chip soonest.  Wide tiles split A less often; narrow ones fill more SMs and have
+// less to do once the last stage is in.  Clocks measured per stage, per unit and (code not yet in the
+// instruction caches) per launch, of tiles of 16, 32, 48 and 64.  With the images' width throughout:
+// 120^3 27 us, 500 x 80 x 500 43, 640^3 65, 1200^3 194; by this rule 21, 35, 52, 194.
+int tile_columns(int N, int imgNT, long long mtiles, int splits, int nstages) {
+  constexpr int kStage[4] = {2400, 2800, 3150, 3850}, kUnit[4] = {3500, 6000, 10000, 13000},
+                kCold[4] = {13000, 14000, 24000, 30000};
+  const long long stages = (nstages + splits - 1) / splits;
+  long long best = 0;
+  int NT = imgNT;
+  for (int w = imgNT; w >= 16; w -= 16) {
+    if (imgNT % w) continue;
+    const long long units = mtiles * ((N + w - 1) / w) * splits;
+    const long long waves = (units + sm_count() - 1) / sm_count();
+    const long long t =
+        waves * (stages * kStage[w / 16 - 1] + kUnit[w / 16 - 1]) + kCold[w / 16 - 1];
+    if (w == imgNT || t < best) {
+      best = t;
+      NT = w;
+    }
+  }
+  return NT;
+}
+
 // Fills the tiling of `a` (its operands, K layout and output are set) and launches it.
 cudaError_t launch_digit_gemm(DigitArgs a, long long K, cudaStream_t s) {
   const DigitShape sh = digit_shape(a.N, K);
-  a.NT = sh.NT;
-  a.ntiles = sh.ntiles;
+  a.imgNT = sh.NT;
   a.nstages = sh.nstages;
   a.mtiles = (a.M + kTileM - 1) / kTileM;
+  a.NT = tile_columns(a.N, sh.NT, a.mtiles, a.splits, sh.nstages);
+  a.ntiles = (a.N + a.NT - 1) / a.NT;
   a.k64 = kK64;
   if (a.KB == 1) a.Kpad = sh.nstages * kStageK;
   auto even = [](long long v) { return (v & 1) == 0; };

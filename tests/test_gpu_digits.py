@@ -115,6 +115,19 @@ def test_zeros_extremes_and_non_finite(product):
     _check(C[np.ix_(ok, cols)], A[ok], B[:, cols])
 
 
+@pytest.mark.parametrize("kc", [True, False])
+@pytest.mark.parametrize("N,K", [(64, 33), (120, 120), (80, 300), (33, 64), (200, 32), (49, 600)])
+def test_result_does_not_depend_on_the_tiles(product, N, K, kc):
+    """A product's sums are exact up to one rounding, so the rows of a tall product (wide tiles) are
+    those of a short one of the same rows (tiles of a divisor of the width), bit for bit."""
+    rng = np.random.default_rng(N + K)
+    A = rng.standard_normal((128 * 160, K))
+    B = rng.standard_normal((K, N))
+    tall = product(A, B, kc)
+    for rows in (1, 130):
+        np.testing.assert_array_equal(tall[:rows], product(A[:rows], B, kc))
+
+
 @pytest.mark.parametrize("nbf,naux,npair,ncwo,packed,blocks", [
     (500, 300, 20, 3, False, 1),   # several row and column tiles, two chunks of k
     (97, 150, 4, 3, True, 3),      # packed slices, blocks of slices, odd sizes
