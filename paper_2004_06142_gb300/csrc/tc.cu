@@ -1054,6 +1054,13 @@ __device__ inline double load_B_elem(const double* __restrict__ B, int layout, l
 // The passes over B below work in fp32 on elements scaled by a power of two per slice (this
 // GPU's FP64 pipe gives 1.6 operations per clock and SM, its double-to-float conversion 100): a
 // CTA per slice finds the largest (scaled) exponent, then sums elements brought to at most 2.
+// The double (hi, lo), within a normal float's range, cut to a float's 24 bits.  From the bits: the
+// conversion instruction holds the FP64 unit of its scheduler for 64 clocks, as any FP64 one does
+// (k_p_scale of 1103 packed slices of 301: 336 us with it, 281 so).
+__device__ __forceinline__ float float_of_top(uint32_t hi, uint32_t lo) {
+  const uint32_t t = __funnelshift_l(lo, hi, 3) + ((127u - 1023u) << 23);
+  return __uint_as_float((t & 0x7fffffffu) | (hi & 0x80000000u));
+}
 // two_floats: v 2^k (biased exponent e of v, e + k within a float's range) as xh + xl, xh the
 // upper 24 bits rounded half up, xl the lower 29 bits (rounded to 24), from the bits alone.
 __device__ __forceinline__ void two_floats(double v, int k, float& xh, float& xl) {
@@ -1062,17 +1069,20 @@ __device__ __forceinline__ void two_floats(double v, int k, float& xh, float& xl
   const bool tiny = (hi & 0x7ff00000u) == 0 || e < 1023 - 120;  // taken as zero
   uint32_t h2 = hi + ((uint32_t)k << 20), l2 = lo;
   asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, 0;" : "+r"(l2), "+r"(h2) : "r"(0x10000000u));
-  xh = tiny ? 0.f : (float)__hiloint2double((int)h2, (int)(l2 & 0xe0000000u));
+  xh = tiny ? 0.f : float_of_top(h2, l2);
   // the lower bits as a signed number of 2^-3: weight 2^(e - 1023 - 52 - 3)
   const float w = __int_as_float(max(e - 1078 + 127, 0) << 23);
   const float r = (float)(int)(lo << 3) * w;
   xl = tiny ? 0.f : ((int)hi < 0 ? -r : r);
 }
-// |v| 2^k rounded to a float, for sums that a few roundings do not matter to.
+// |v| 2^k rounded (half up) to a float, for sums that a few roundings do not matter to.
 __device__ __forceinline__ float one_float(double v, int k) {
-  const int hi = __double2hiint(v), e = ((hi >> 20) & 0x7ff) + k;
-  const bool tiny = (hi & 0x7ff00000) == 0 || e < 1023 - 120;
-  return tiny ? 0.f : (float)__hiloint2double((hi & 0xfffff) | (e << 20), __double2loint(v));
+  const uint32_t hi = (uint32_t)__double2hiint(v);
+  const int e = (int)((hi >> 20) & 0x7ffu) + k;
+  const bool tiny = (hi & 0x7ff00000u) == 0 || e < 1023 - 120;
+  uint32_t h2 = (hi & 0xfffffu) | ((uint32_t)e << 20), l2 = (uint32_t)__double2loint(v);
+  asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, 0;" : "+r"(l2), "+r"(h2) : "r"(0x10000000u));
+  return tiny ? 0.f : float_of_top(h2, l2);
 }
 // s + c += p, the rounding of s kept in c (Knuth's two-sum)
 __device__ __forceinline__ void add_comp(float& s, float& c, float p) {
@@ -1083,29 +1093,85 @@ __device__ __forceinline__ void add_comp(float& s, float& c, float p) {
 // What elements too small for their square to be a float can add to a row's sum, per element.
 constexpr double kStatsLost = 0x1p-118;
 
+constexpr int kBoundSlack = 64;
 // Row sums of slice P (N x N, symmetric) over its elements times 2^(-s_mu - s_nu) (s null: 0) in
 // units of 2^top: row(mu, squares, magnitudes), called by one thread per row.  EXACT: compensated
 // sums, to about 2^-40; otherwise squares only, to sum_margin.  Dense: a warp per row.  Packed: a
 // warp per stored row, whose elements also count for their columns (partial sums per warp in
-// shared memory, added in the order of the warps).  Returns top (above 4096: a NaN or an infinity).
+// shared memory, added in the order of the warps).  bound: 4096 + an upper bound of the largest
+// scaled biased exponent, less than kBoundSlack above it, the largest over the threads; negative: it
+// is found first.  Returns top, the bound or the exponent itself (above 4096: a NaN or an infinity).
 // All threads of the CTA call it; sh holds kSums N floats per warp and once more (packed), red 33
 // ints.
 template <bool PACKED, bool EXACT, class Row>
 __device__ __forceinline__ int slice_row_sums(const double* __restrict__ B, int N,
                                               const int* __restrict__ s, float* sh, int* red,
-                                              const Row& row) {
+                                              int bound, const Row& row) {
   constexpr int kSums = EXACT ? 4 : 1;  // squares, their compensation, magnitudes, theirs
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  int m = 0;  // biased; 0: the slice is zero
-  for (int mu = w; mu < N; mu += nw) {
-    const double* r = B + (PACKED ? (long long)mu * (mu + 1) / 2 : (long long)mu * N);
-    const int n = PACKED ? mu + 1 : N, smu = s ? s[mu] : 0;
-#pragma unroll 4
-    for (int nu = lane; nu < n; nu += 32) {
-      const int e = (__double2hiint(r[nu]) >> 20) & 0x7ff;
-      if (e > 0) m = max(m, e == 2047 ? 1 << 20 : e + 4096 - smu - (s ? s[nu] : 0));
+  int m = bound < 0 ? 0 : bound;  // biased; 0: the slice is zero
+  if (bound < 0 && !s) {  // the exponents alone: the slice from end to end, eight loads in flight
+    const int per = PACKED ? N * (N + 1) / 2 : N * N;
+    for (int i0 = threadIdx.x; i0 < per; i0 += 8 * blockDim.x) {
+      int h[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int i = i0 + j * blockDim.x;
+        h[j] = i < per ? __double2hiint(B[i]) : 0;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int e = (h[j] >> 20) & 0x7ff;
+        if (e > 0) m = max(m, e == 2047 ? 1 << 20 : e + 4096);
+      }
     }
   }
+  // A row at a time, kBatch loads of a lane ahead of their use, over the ends of rows too (bound by
+  // the latency of the loads otherwise: a row is a few of them per lane): at(mu, nu, v) for every
+  // element in order, end(mu) after a row
+  constexpr int kBatch = 4;
+  auto walk = [&](auto at, auto end) {
+    auto row_at = [&](int mu) {
+      return B + (PACKED ? (long long)mu * (mu + 1) / 2 : (long long)mu * N);
+    };
+    int mu = w, n0 = 0;  // the batch in v: row mu, elements n0 + lane + 32 u
+    double v[kBatch];
+    auto load = [&](int r, int c0, double (&x)[kBatch]) {
+      const int n = PACKED ? r + 1 : N;
+      const double* p = row_at(r);
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        const int nu = c0 + lane + 32 * u;
+        x[u] = r < N && nu < n ? p[nu] : 0.0;
+      }
+    };
+    if (mu < N) load(mu, 0, v);
+    while (mu < N) {
+      const int n = PACKED ? mu + 1 : N;
+      int r2 = mu, c2 = n0 + 32 * kBatch;
+      if (c2 >= n) {
+        r2 += nw;
+        c2 = 0;
+      }
+      double x[kBatch];
+      load(r2, c2, x);
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        const int nu = n0 + lane + 32 * u;
+        if (nu < n) at(mu, nu, v[u]);
+      }
+      if (r2 != mu) end(mu);
+      mu = r2;
+      n0 = c2;
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) v[u] = x[u];
+    }
+  };
+  if (bound < 0 && s)
+    walk([&](int mu, int nu, double v) {
+      const int e = (__double2hiint(v) >> 20) & 0x7ff;
+      if (e > 0) m = max(m, e == 2047 ? 1 << 20 : e + 4096 - s[mu] - s[nu]);
+    }, [](int) {});
   m = __reduce_max_sync(0xffffffffu, m);
   __syncthreads();  // red and sh are free
   if (lane == 0) red[w] = m;
@@ -1120,37 +1186,35 @@ __device__ __forceinline__ int slice_row_sums(const double* __restrict__ B, int 
   __syncthreads();
   const int top = red[32] - 4096;  // the largest scaled biased exponent
   float* cs = sh + kSums * N * w;  // this warp's partial sums of the columns
-  for (int mu = w; mu < N; mu += nw) {
-    const double* r = B + (PACKED ? (long long)mu * (mu + 1) / 2 : (long long)mu * N);
-    const int n = PACKED ? mu + 1 : N, k = 1023 - top - (s ? s[mu] : 0);
-    float ss = 0.f, sc = 0.f, l1 = 0.f, lc = 0.f;
-#pragma unroll 4
-    for (int nu = lane; nu < n; nu += 32) {
-      if (EXACT) {
-        float xh, xl;
-        two_floats(r[nu], k - (s ? s[nu] : 0), xh, xl);
-        const float q = __fmul_rn(xh, xh);
-        const float qe = fmaf(2.f * xh, xl, fmaf(xh, xh, -q)), a = fabsf(xh);
-        const float al = xh < 0.f ? -xl : xl;
-        add_comp(ss, sc, q);
-        sc += qe;
-        add_comp(l1, lc, a);
-        lc += al;
-        if (PACKED && nu < mu) {
-          float ts = cs[nu], tc = cs[N + nu], tl = cs[2 * N + nu], td = cs[3 * N + nu];
-          add_comp(ts, tc, q);
-          add_comp(tl, td, a);
-          cs[nu] = ts;
-          cs[N + nu] = tc + qe;
-          cs[2 * N + nu] = tl;
-          cs[3 * N + nu] = td + al;
-        }
-      } else {
-        const float x = one_float(r[nu], k - (s ? s[nu] : 0));
-        ss = fmaf(x, x, ss);
-        if (PACKED && nu < mu) cs[nu] = fmaf(x, x, cs[nu]);
+  float ss = 0.f, sc = 0.f, l1 = 0.f, lc = 0.f;
+  const int k0 = 1023 - top;
+  walk([&](int mu, int nu, double v) {
+    const int k = k0 - (s ? s[mu] + s[nu] : 0);
+    if (EXACT) {
+      float xh, xl;
+      two_floats(v, k, xh, xl);
+      const float q = __fmul_rn(xh, xh);
+      const float qe = fmaf(2.f * xh, xl, fmaf(xh, xh, -q)), a = fabsf(xh);
+      const float al = xh < 0.f ? -xl : xl;
+      add_comp(ss, sc, q);
+      sc += qe;
+      add_comp(l1, lc, a);
+      lc += al;
+      if (PACKED && nu < mu) {
+        float ts = cs[nu], tc = cs[N + nu], tl = cs[2 * N + nu], td = cs[3 * N + nu];
+        add_comp(ts, tc, q);
+        add_comp(tl, td, a);
+        cs[nu] = ts;
+        cs[N + nu] = tc + qe;
+        cs[2 * N + nu] = tl;
+        cs[3 * N + nu] = td + al;
       }
+    } else {
+      const float x = one_float(v, k);
+      ss = fmaf(x, x, ss);
+      if (PACKED && nu < mu) cs[nu] = fmaf(x, x, cs[nu]);
     }
+  }, [&](int mu) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       if (EXACT) {
@@ -1176,7 +1240,8 @@ __device__ __forceinline__ int slice_row_sums(const double* __restrict__ B, int 
         row(mu, (double)ss + (double)sc, (double)l1 + (double)lc);
       }
     }
-  }
+    ss = sc = l1 = lc = 0.f;
+  });
   if (PACKED) {
     __syncthreads();
     for (int mu = threadIdx.x; mu < N; mu += blockDim.x) {
@@ -1222,8 +1287,10 @@ inline size_t slice_smem(bool packed, int N) {
 // Per row (P, mu) of B: its squared L2 norm (rn2, fp32 rounded up, for the exponents of X in the
 // G contraction), the slice's largest row L1 norm (L1max, the bound on X^T rows) and the AO
 // index's largest row norm over the slices (rnmax, for the symmetric scaling); any
-// non-finite element raises DONOF_ERR_NONFINITE.  1103 packed slices of 301: 0.26 ms (in double,
-// every element gathered twice: 1.18 ms).
+// non-finite element raises DONOF_ERR_NONFINITE.  Bound by its instructions (54 float additions an
+// element, for two compensated sums over its row and over its column).  1103 packed slices of 301:
+// 0.28 ms (with a row's loads behind the reduction of the row before: 0.39; in double, every element
+// gathered twice: 1.18).
 template <bool PACKED>
 __global__ void __launch_bounds__(256) k_b_stats(const double* __restrict__ B, int Q, int N,
                                                  DevHeader* hdr, double* L1max, float* rn2,
@@ -1240,7 +1307,7 @@ __global__ void __launch_bounds__(256) k_b_stats(const double* __restrict__ B, i
     // the slice's scale is known to every thread only after the call: the rows are scaled by
     // the exponent that the call found, which it leaves in red
     const int top = slice_row_sums<PACKED, true>(
-        B + P * per, N, nullptr, sh_f, red, [&](int mu, double ss, double l1) {
+        B + P * per, N, nullptr, sh_f, red, -1, [&](int mu, double ss, double l1) {
           const int t = red[32] - 4096;
           if (t > 4096) {
             out[mu] = __int_as_float(0x7fc00000);
@@ -1265,11 +1332,12 @@ __global__ void __launch_bounds__(256) k_b_stats(const double* __restrict__ B, i
 
 // Per slice: t_P, the exponent of the largest row norm of Bt^P without t_P.  Where the fp32 sums
 // cannot tell on which side of a power of two the norm lies, the slice's sums are taken in
-// double.  1103 packed slices of 301: 0.2 ms (in double, with an ldexp per element: 1.35 ms).
+// double.  1103 packed slices of 301: 0.13 ms (with a pass for the largest element first: 0.20; with
+// the loads of a row behind the row before too: 0.28; in double, with an ldexp per element: 1.35).
 template <bool PACKED>
 __global__ void __launch_bounds__(256) k_p_scale(const double* __restrict__ B, int Q, int N,
                                                  const int* __restrict__ eS, double invT,
-                                                 int* tP) {
+                                                 const float* __restrict__ rn2, int* tP) {
   extern __shared__ float sh_f[];
   __shared__ int red[33];
   __shared__ unsigned long long redl[33];
@@ -1278,14 +1346,40 @@ __global__ void __launch_bounds__(256) k_p_scale(const double* __restrict__ B, i
   // lanes, the warps' sums, every term rounded before
   const int nw = blockDim.x >> 5;
   int* sS = (int*)(sh_f + (PACKED ? (nw + 1) * N : 0));  // the scale exponents, behind the sums
-  for (int i = threadIdx.x; i < N; i += blockDim.x) sS[i] = eS[i];
+  int lo = 1 << 20, hi = -(1 << 20);
+  for (int i = threadIdx.x; i < N; i += blockDim.x) {
+    const int e = eS[i];
+    sS[i] = e;
+    lo = min(lo, e);
+    hi = max(hi, e);
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if ((threadIdx.x & 31) == 0) {
+    red[threadIdx.x >> 5] = lo;
+    red[16 + (threadIdx.x >> 5)] = hi;
+  }
   __syncthreads();
+  for (int i = 0; i < nw; ++i) {
+    lo = min(lo, red[i]);
+    hi = max(hi, red[16 + i]);
+  }
   const double mg = (N / 32 + (PACKED ? N / nw : 0) + 32) * 0x1p-24;
   for (int P = blockIdx.x; P < Q; P += gridDim.x) {
     const double* Bp = B + P * per;
     double mx = 0.0;
+    // the scale of the sums from the rows' norms: |B_mu,nu| 2^(-s_mu - s_nu) < 2^(b - s_mu - min s),
+    // 4^b > the row's squared norm.  Not for norms near a float's range or scales that differ
+    // by more than the sums bear
+    int bound = 0, far = hi - lo > kBoundSlack - 24 ? 1 : 0;
+    for (int mu = threadIdx.x; mu < N; mu += blockDim.x) {
+      const int e = (__float_as_int(rn2[(size_t)P * N + mu]) >> 23) & 0x1ff;  // (with the sign)
+      if (e < 27 || e > 227) far = 1;
+      bound = max(bound, ((e - 125) >> 1) - sS[mu] - lo + 1022 + 4096);
+    }
+    if (__syncthreads_or(far)) bound = -1;
     const int top = slice_row_sums<PACKED, false>(
-        Bp, N, sS, sh_f, red, [&](int, double ss, double) { mx = fmax(mx, ss); });
+        Bp, N, sS, sh_f, red, bound, [&](int, double ss, double) { mx = fmax(mx, ss); });
     const double ss = block_max(mx, redl);
     const double sc = pow2d(top - 1023);
     const int e0 = intfrac_exponent_inv(sqrt(ss * (1.0 - mg)) * sc, invT);
@@ -1360,52 +1454,65 @@ __device__ __forceinline__ void intfrac_split_scaled(double v, int k, __half& h,
   f = __float2half_rn((yh - __half2float(h)) + yl);
 }
 
-// Bt^P 2^-t_P -> integer + fraction planes in the lower-triangle tile storage (SymTiles).  A warp
-// per stored row mu of a slice (rows of the last tile padded to Rlast), a lane per 8
-// consecutive stored elements; the columns reach to the end of mu's tile.
+// Bt^P 2^-t_P -> integer + fraction planes in the lower-triangle tile storage (SymTiles).  A CTA per
+// 8 stored rows of a slice (rows of the last tile padded to Rlast), their pieces of 8 consecutive
+// stored elements dealt over its threads; the columns reach to the end of the rows' tile.  Bound by
+// its integer instructions, so that pieces past the matrix are only zeroed and no lane is left
+// over at the ends of rows (1103 packed slices of 301, a warp per row and zeros converted like
+// all others: 299 us; this: 206).
 __global__ void __launch_bounds__(256) k_split_B_sym(const double* __restrict__ B, int layout,
                                                      int Q, int N, SymTiles st,
                                                      const int* __restrict__ eS,
                                                      const int* __restrict__ tP, __half* H,
                                                      __half* F) {
-  const long long npk = (long long)N * (N + 1) / 2;
+  const bool dense = layout == DONOF_B_DENSE;
+  const size_t per = dense ? (size_t)N * N : (size_t)N * (N + 1) / 2;
   const int rows = 128 * (st.T - 1) + st.Rlast;  // stored rows (= columns) per slice
-  const int lane = threadIdx.x & 31, rb = (rows + 7) / 8;
-  const long long tot = (long long)Q * rb;
-  for (long long u = blockIdx.x; u < tot; u += gridDim.x) {  // 8 rows of a slice per CTA
-    const int P = (int)(u / rb), mu = (int)(u - (long long)P * rb) * 8 + (threadIdx.x >> 5);
-    if (mu >= rows) continue;
-    const int ti = mu >> 7, r = mu & 127, Ri = sym_R(st, ti);
-    const int k0 = -tP[P] - (mu < N ? eS[mu] : 0);
-    const double* Bp = B + (layout == DONOF_B_DENSE ? (size_t)P * N * N : (size_t)P * npk);
+  const int rb = rows / 8, tot = Q * rb;
+  for (int u = blockIdx.x; u < tot; u += gridDim.x) {  // 8 rows of a slice per CTA
+    const int P = u / rb, mu0 = (u - P * rb) * 8;
+    const int ti = mu0 >> 7, Ri = sym_R(st, ti), tp = tP[P];
+    const double* Bp = B + (size_t)P * per;
     const size_t base = (size_t)P * st.perP;
-    const int ncols = 128 * ti + (ti == st.T - 1 ? st.Rlast : 128);
-    const double* row = Bp + (layout == DONOF_B_DENSE ? (size_t)mu * N
-                                                      : (size_t)((long long)mu * (mu + 1) / 2));
-    for (int c8 = lane; c8 < ncols / 8; c8 += 32) {
+    const int n8 = 16 * ti + (ti == st.T - 1 ? st.Rlast : 128) / 8;  // pieces of a row
+    const uint32_t inv = 0xffffffffu / (uint32_t)n8 + 1;  // 2^32 / n8 upwards (8 n8^2 < 2^32)
+    for (int it = threadIdx.x; it < 8 * n8; it += blockDim.x) {
+      const int r8 = (int)__umulhi((uint32_t)it, inv), c8 = it - r8 * n8, mu = mu0 + r8;
+      const int r = mu & 127, nu0 = 8 * c8;
       __align__(16) __half hv[8], fv[8];
-      const int nu0 = 8 * c8;
-      double v[8];
-      int k[8];
-      if (mu < N && (layout == DONOF_B_DENSE ? nu0 + 7 < N : nu0 + 7 <= mu)) {  // stored in a row
-        *(int4*)k = *(const int4*)(eS + nu0);
-        *(int4*)(k + 4) = *(const int4*)(eS + nu0 + 4);
+      if (mu < N && nu0 < N) {
+        const int k0 = -tp - eS[mu];
+        double v[8];
+        int k[8];
+        // element nu0 + j: in mu's row up to the diagonal, above it in row nu0 + j (packed); offsets
+        // within a slice fit an int (a slice of more would not fit the device)
+        const int row = dense ? mu * N + nu0 : mu * (mu + 1) / 2 + nu0;
+        const int diag = dense ? 8 : mu - nu0;  // the last j of the row
+        int col = nu0 * (nu0 + 1) / 2 + mu;
+        if (nu0 + 8 <= N) {
+          *(int4*)k = *(const int4*)(eS + nu0);
+          *(int4*)(k + 4) = *(const int4*)(eS + nu0 + 4);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          v[j] = __ldg(row + nu0 + j);
-          k[j] = k0 - k[j];
+          for (int j = 0; j < 8; ++j) {
+            v[j] = __ldg(Bp + (j <= diag ? row + j : col));
+            col += nu0 + j + 1;
+            k[j] = k0 - k[j];
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const bool in = nu0 + j < N;
+            v[j] = in ? __ldg(Bp + (j <= diag ? row + j : col)) : 0.0;
+            col += nu0 + j + 1;
+            k[j] = in ? k0 - eS[nu0 + j] : 0;
+          }
         }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) intfrac_split_scaled(v[j], k[j], hv[j], fv[j]);
       } else {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int nu = nu0 + j;
-          const bool in = mu < N && nu < N;
-          v[j] = in ? load_B_elem(Bp, layout, 0, mu, mu, nu, N, npk) : 0.0;
-          k[j] = in ? k0 - eS[nu] : 0;
-        }
+        for (int j = 0; j < 8; ++j) hv[j] = fv[j] = __float2half_rn(0.f);
       }
-#pragma unroll
-      for (int j = 0; j < 8; ++j) intfrac_split_scaled(v[j], k[j], hv[j], fv[j]);
       const int tj = c8 >> 4, c = (c8 >> 3) & 1, j8 = c8 & 7;
       const size_t o = base + sym_tile_off(st, ti, tj) + ((size_t)c * Ri + r) * 64 +
                        (size_t)((j8 ^ (r & 7)) * 8);
@@ -1912,7 +2019,7 @@ cudaError_t launch_prepare_split_B(const Dims& d, const double* B, char* ws, con
                                     (float*)(ws + L.rn2), (unsigned long long*)(ws + L.rnmax));
   k_sym_scale<<<1, 1024, 0, s>>>((const double*)(ws + L.rnmax), d.N, (int*)(ws + L.eS));
   const size_t smem2 = (packed ? smem / 4 : 0) + (size_t)d.N * 4;
-  scale<<<ctas, threads, smem2, s>>>(B, d.Q, d.N, eS, invT, tP);
+  scale<<<ctas, threads, smem2, s>>>(B, d.Q, d.N, eS, invT, (const float*)(ws + L.rn2), tP);
   k_sym_exps<<<num_sms() * 4, 256, 0, s>>>(tP, eS, d.Q, d.N, (int*)(ws + L.eB));
   const SymTiles st = sym_tiles(d.N);
   if (st.dense)
