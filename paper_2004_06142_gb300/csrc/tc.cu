@@ -156,7 +156,11 @@ __device__ __forceinline__ int rr_partner(int i, int r, int T) {
   int p;
   if (i == n - 1) p = r;
   else if (i == r) p = n - 1;
-  else p = ((2 * r - i) % (n - 1) + (n - 1)) % (n - 1);
+  else {
+    p = 2 * r - i;  // mod n - 1, within (-(n - 1), 2 (n - 1))
+    if (p < 0) p += n - 1;
+    if (p >= n - 1) p -= n - 1;
+  }
   return p >= T ? i : p;
 }
 
@@ -506,39 +510,52 @@ __device__ __forceinline__ void tc_body(const TcArgs* __restrict__ targs,
         nch = jj < T - 1 ? 2 : rl64;
       }
       for (int it = 0; it < iters; ++it) {
-        if (!mbar_wait(bar(kFull + stage), phase, status, abort_flag)) { ok = false; break; }
+        if (!mbar_try(bar(kFull + stage), phase) &&
+            !mbar_wait(bar(kFull + stage), phase, status, abort_flag)) {
+          ok = false;
+          break;
+        }
         tc_fence_after();
-        const uint32_t base = smem_u32(smem + (size_t)stage * stage_bytes);
+        const uint32_t base = smem_u32(smem + (size_t)stage * stage_bytes) >> 4;  // in 16 bytes
         const bool tr = amn || (sym && jj > mt);
         const uint32_t id = tr ? (idesc | (1u << 15)) : idesc;
+        // the words of the descriptors (sdesc, sdesc_mn, sdesc_plain) and their step per 16 of k
+        constexpr uint32_t kHi = ((8u * SWZ) >> 4) | 1u << 14 | (SWZ == 128 ? 2u : 4u) << 29;
+        uint32_t a_lo = base, a_hi, a_step;
+        if (il8) {  // two K-adjacent core-matrix columns (BM rows x 16 B) per step
+          a_lo |= (uint32_t)(BM * 16 >> 4) << 16;
+          a_hi = (128u >> 4) | 1u << 14;
+          a_step = 2 * BM * 16 >> 4;
+        } else if (tr) {
+          a_lo |= (mn_lbo >> 4) << 16;
+          a_hi = (mn_sbo >> 4) | 1u << 14 | 2u << 29;
+          a_step = 2048 >> 4;
+        } else {
+          a_lo |= 1u << 16;
+          a_hi = kHi;
+          a_step = 32 >> 4;
+        }
+        const uint32_t b_lo = (base + (2 * a_bytes >> 4)) | 1u << 16;
 #pragma unroll
         for (int k = 0; k < BK / 16; ++k) {
-          uint64_t ah, al;
-          if (il8) {  // two K-adjacent core-matrix columns (BM rows x 16 B) per step
-            ah = sdesc_plain(base + k * 2 * BM * 16, BM * 16, 128);
-            al = sdesc_plain(base + a_bytes + k * 2 * BM * 16, BM * 16, 128);
-          } else if (tr) {
-            ah = sdesc_mn(base + k * 2048, mn_lbo, mn_sbo);
-            al = sdesc_mn(base + a_bytes + k * 2048, mn_lbo, mn_sbo);
-          } else {
-            ah = sdesc(base + k * 32, SWZ);
-            al = sdesc(base + a_bytes + k * 32, SWZ);
-          }
-          const uint64_t bh = sdesc(base + 2 * a_bytes + k * 32, SWZ);
-          const uint64_t bl = sdesc(base + 2 * a_bytes + b_bytes + k * 32, SWZ);
+          const uint32_t ah = a_lo + (uint32_t)k * a_step, al = ah + (a_bytes >> 4);
+          const uint32_t bh = b_lo + (uint32_t)k * 2, bl = bh + (b_bytes >> 4);
           const uint32_t first = (it > 0 || k > 0) ? 1u : 0u;
+          auto mma = [&](uint32_t d, uint32_t a, uint32_t b, uint32_t acc) {
+            mma_f16_words<PAIR>(d, a, a_hi, b, kHi, id, acc);
+          };
           if (NUM == kSplit3) {
-            mma_f16<PAIR>(d0, ah, bh, id, first);
-            mma_f16<PAIR>(d0, ah, bl, id, 1u);
-            mma_f16<PAIR>(d0, al, bh, id, 1u);
+            mma(d0, ah, bh, first);
+            mma(d0, ah, bl, 1u);
+            mma(d0, al, bh, 1u);
           } else if (bcat) {  // bh: the 2 Nn rows of both planes
-            mma_f16<PAIR>(d0, ah, bh, id, first);  // [h h | h f]
-            mma_f16<PAIR>(d1, al, bh, id, first);  // [f h | f f]
+            mma(d0, ah, bh, first);  // [h h | h f]
+            mma(d1, al, bh, first);  // [f h | f f]
           } else {
-            mma_f16<PAIR>(d0, ah, bh, id, first);  // integer x integer: exact
-            mma_f16<PAIR>(d1, ah, bl, id, first);
-            mma_f16<PAIR>(d1, al, bh, id, 1u);
-            mma_f16<PAIR>(d1, al, bl, id, 1u);
+            mma(d0, ah, bh, first);  // integer x integer: exact
+            mma(d1, ah, bl, first);
+            mma(d1, al, bh, 1u);
+            mma(d1, al, bl, 1u);
           }
         }
         mma_commit<PAIR>(bar(kEmpty + stage));  // frees the stage in both CTAs of a pair

@@ -162,6 +162,13 @@ __device__ __forceinline__ void mma_f16(uint32_t dtmem, uint64_t a, uint64_t b, 
         "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
         : "memory");
 }
+// The same with the descriptors given as their low and high words.
+template <int PAIR>
+__device__ __forceinline__ void mma_f16_words(uint32_t dtmem, uint32_t alo, uint32_t ahi,
+                                              uint32_t blo, uint32_t bhi, uint32_t idesc,
+                                              uint32_t accumulate) {
+  mma_f16<PAIR>(dtmem, (uint64_t)ahi << 32 | alo, (uint64_t)bhi << 32 | blo, idesc, accumulate);
+}
 // Arrive on `bar` once the MMAs issued so far are complete: in this CTA, or (PAIR) on the
 // barrier at the same offset in both CTAs of the pair.
 template <int PAIR>
