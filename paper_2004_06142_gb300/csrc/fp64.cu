@@ -298,18 +298,24 @@ namespace {
 // one warp per orbital p: H_pp over the lanes' rows mu, and G[mu][p] = n_p (h C)[mu][p]
 __device__ __forceinline__ void k_hdiag_ginit_body(const Blk& B_, Dims d, const double* __restrict__ C, const double* __restrict__ hC,
                               const double* __restrict__ n, double* Hd, double* G, double gscale) {
-  const int p = B_.x * (blockDim.x / 32) + threadIdx.x / 32;
-  const int lane = threadIdx.x % 32;
-  if (p >= d.A) return;
+  // A CTA of 8 warps per orbital: bound by the latency of its strided loads (500 / 80, a warp per
+  // orbital: 13 us; so: 5.5)
+  const int p = B_.x, lane = threadIdx.x % 32, w = threadIdx.x / 32;
+  __shared__ double red[8];
   const double np_ = n[p];
   double s = 0.0;
-  for (int mu = lane; mu < d.N; mu += 32) {
+  for (int mu = threadIdx.x; mu < d.N; mu += blockDim.x) {
     const double v = hC[(size_t)mu * d.A + p];
     s += C[(size_t)mu * d.N + p] * v;
     G[(size_t)mu * d.A + p] = gscale * np_ * v;
   }
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) Hd[p] = s;
+  if (lane == 0) red[w] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int i = 1; i < (int)(blockDim.x / 32); ++i) s += red[i];
+    Hd[p] = s;
+  }
 }
 __global__ void k_hdiag_ginit(Dims d, const double* __restrict__ C, const double* __restrict__ hC,
                               const double* __restrict__ n, double* Hd, double* G, double gscale) {
@@ -319,7 +325,7 @@ __global__ void k_hdiag_ginit(Dims d, const double* __restrict__ C, const double
 
 cudaError_t launch_hdiag_ginit(const Dims& d, const double* C, char* ws, const Layout& L,
                                bool one_electron_G, cudaStream_t s) {
-  launch_chained(k_hdiag_ginit, (d.A + 7) / 8, 256, 0, s, d, C, (const double*)(ws + L.hC),
+  launch_chained(k_hdiag_ginit, d.A, 256, 0, s, d, C, (const double*)(ws + L.hC),
                  (const double*)(ws + L.n), (double*)(ws + L.Hd), (double*)(ws + L.G),
                  one_electron_G ? 1.0 : 0.0);
   count_launch(1);

@@ -176,26 +176,39 @@ __device__ __forceinline__ void k_jk_eY_body(const Blk& B_, const double* __rest
           j += jv[u];
         }
       }
-      for (; sp < splits; ++sp) {
-        k += Ksp[(size_t)sp * AA + src];
-        j += Jsp[(size_t)sp * AA + src];
+      if (sp < splits) {  // the rest, its loads in flight together too
+        double kv[7], jv[7];
+#pragma unroll
+        for (int u = 0; u < 7; ++u) {
+          const bool in = sp + u < splits;
+          kv[u] = in ? Ksp[(size_t)(sp + u) * AA + src] : 0.0;
+          jv[u] = in ? Jsp[(size_t)(sp + u) * AA + src] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 7; ++u) {
+          if (sp + u >= splits) break;
+          k += kv[u];
+          j += jv[u];
+        }
       }
       K[i] += k;
       J[i] += j;
     }
     return;
   }
-  // one warp per (split, row p), rows p >= A get exponent 0
-  const int lane = threadIdx.x % 32;
+  // one warp per (split, row p), rows p >= A get exponent 0; the exponents of a CTA's rows by one
+  // warp, a lane each: an FP64 instruction takes its scheduler 64 clocks for one lane as for 32, and
+  // these were most of the kernel (500 / 2000 / 80: 33 us with every warp's own, 27 so)
+  __shared__ double bounds[32];
+  const int lane = threadIdx.x % 32, w = threadIdx.x / 32, nw = blockDim.x / 32;
   const int nrow = splits * Ap;
-  for (int t = ((B_.x - n0) * blockDim.x + threadIdx.x) / 32; t < nrow;
-       t += (B_.gx - n0) * blockDim.x / 32) {
-    const int sp = t / Ap, p = t % Ap;
+  for (int t0 = (B_.x - n0) * nw; t0 < nrow; t0 += (B_.gx - n0) * nw) {
+    const int t = t0 + w, sp = t / Ap, p = t % Ap;
     // the squared norm in fp32 (this GPU's FP64 pipe is narrow): ss, and sa the sum of the
     // terms' magnitudes; fewer than 64 roundings of 2^-24 each (conversions included) keep
     // ss within 2^-17 sa of the exact sum, so ss + 2^-16 sa bounds it from above
     float ss = 0.f, sa = 0.f;
-    if (p < A) {
+    if (t < nrow && p < A) {
       const double* Ks = Ksp + (size_t)sp * AA;
       for (int q = lane; q < A; q += 32) {
         const float bc = BcF[(size_t)q * Ap + p];
@@ -217,10 +230,15 @@ __device__ __forceinline__ void k_jk_eY_body(const Blk& B_, const double* __rest
       ss += __shfl_xor_sync(0xffffffffu, ss, o);
       sa += __shfl_xor_sync(0xffffffffu, sa, o);
     }
-    const double bound = (double)ss + 0x1p-16 * (double)sa;
-    // row length of the G contraction over this split: (slices in it) x Ap
-    const double Kc = (double)(np * (sp + 1LL) / splits - np * (long long)sp / splits) * Ap;
-    if (lane == 0) eY[t] = intfrac_exponent(sqrt(fmax(bound, 0.0)) * (1.0 + 1e-6), Kc);
+    if (lane == 0) bounds[w] = (double)ss + 0x1p-16 * (double)sa;
+    __syncthreads();
+    if (w == 0 && lane < nw && t0 + lane < nrow) {
+      // row length of the G contraction over this split: (slices in it) x Ap
+      const int s = (t0 + lane) / Ap;
+      const double Kc = (double)(np * (s + 1LL) / splits - np * (long long)s / splits) * Ap;
+      eY[t0 + lane] = intfrac_exponent(sqrt(fmax(bounds[lane], 0.0)) * (1.0 + 1e-6), Kc);
+    }
+    __syncthreads();
   }
 }
 __global__ void __launch_bounds__(256) k_jk_eY(const double* __restrict__ Ksp,
