@@ -1,12 +1,12 @@
 // Symmetric FP64 eigensolver of the orbital update (Sec. III.B: the new orbitals are the
 // eigenvectors of the symmetric matrix F of Eq. Fockian, and its eigenvalues the next
 // diagonal).  Laid out for this GPU's narrow FP64 pipe and large L2:
-//   1. A = Q T Q^T by Householder reflections in one cooperative launch (one CTA per SM, one
-//      grid barrier per column).  Each step forms the next column of the rank-2-updated
-//      matrix in every CTA (from one row, by symmetry) and its reflector; every row warp
-//      updates its own row of the trailing matrix and takes its part of the next
-//      matrix-vector product while a scalar warp forms the reflector's scalars; the matrix
-//      stays in L2.  A is first scaled by a power of two (exact) to a largest element in
+//   1. A = Q T Q^T by Householder reflections, one barrier per column: small matrices in one
+//      cluster of CTAs, larger ones in a cooperative launch of one CTA per SM.  Each step forms
+//      the next column of the rank-2-updated matrix in every CTA (from one row, by symmetry) and
+//      its reflector; every row warp updates its own row of the trailing matrix, which it keeps
+//      in registers (in L2 above n 1216), and takes its part of the next matrix-vector product
+//      while a scalar warp forms the reflector's scalars.  A is first scaled by a power of two (exact) to a largest element in
 //      [1/2, 1).
 //   2. T is split where an off-diagonal element is at most 16 N eps ||T||_inf (a perturbation
 //      of that size moves no eigenvalue by more) and scaled by a power of two to
@@ -236,7 +236,7 @@ __global__ void k_eigh_scale_copy(const double* __restrict__ A, long long nn, Ei
 // ---------------------------------------------------------------------------
 struct TriArgs {
   int N;
-  double* A;     // N x N, row-major, symmetric; trailing rows updated in place
+  double* A;     // N x N, row-major, symmetric; the updated rows that others need (rows in memory: all)
   double* Yr;    // reflector k in row k, columns k+1 .. N-1 (zero elsewhere)
   double* d;     // diagonal of T
   double* e;     // off-diagonal of T (N - 1)

@@ -1,6 +1,6 @@
-// FP64 kernels of the PNOF build: the strided batched DGEMM that carries every
-// contraction of the plain-double path (and the small double contractions of the
-// mixed path), and the per-orbital / per-pair kernels of both paths:
+// FP64 kernels of the PNOF build: the per-orbital / per-pair kernels of both paths, and the strided
+// batched DGEMM, J / K and Y on the FP64 pipe, which carry the plain-double path where its
+// workspace has no room for digit products (digits.cu):
 //   occupations n(gamma) and Jacobians ........ Eqs. soo, woo
 //   coefficient matrices of E in J and K ........ Eqs. Eg, Efg, Efg_s
 //   J / K accumulation over P, the Y^P operands . Eqs. JKpq (density-fitted)
