@@ -183,8 +183,8 @@ dim3 kind_grid(int kind, const Dims& d, const donof_instance& x, bool backward) 
     case GK_XEXP: return dim3(std::max(1, ceil_div((long long)sp3 * N, 256)), 2, 1);
     case GK_DIAGW: return dim3(ceil_div(np, kDiagWTileSlices), ceil_div(A, kDiagWTileCols), 1);
     case GK_KPART: return dim3(ceil_div(kpart_quads(A), 256), sp3, 1);
-    case GK_JKEY:  // the sums a thread per entry; the exponents a warp per (split, row)
-      return dim3(ceil_div((long long)A * A, 256) + ceil_div((long long)sp3 * Ap, 8), 1, 1);
+    case GK_JKEY:  // the sums kJkEntries a block; the exponents a warp per (split, row)
+      return dim3(ceil_div((long long)A * A, kJkEntries) + ceil_div((long long)sp3 * Ap, 8), 1, 1);
     case GK_YQUANT: return dim3(ceil_div(np, 8), 1, 1);  // eight slices a block
     case GK_REDUCEG: return dim3(ceil_div((long long)N * (Ap / 4), 256), 1, 1);
     case GK_EROWS: return dim3(ceil_div(A, 8), 1, 1);

@@ -246,6 +246,8 @@ __host__ __device__ inline int kpart_quads(int A) {
   return 2 * kb * (kb + 1) + (A % 4) * (kb + 1);
 }
 
+// Entries of K and J per CTA of k_jk_eY's sums (mid.cu).
+constexpr int kJkEntries = 64;
 // Tiles of k_diag_w (mid.cu): a CTA per 32 slices and 64 columns.
 constexpr int kDiagWTileSlices = 32, kDiagWTileCols = 64;
 

@@ -153,47 +153,39 @@ __device__ __forceinline__ void k_jk_eY_body(const Blk& B_, const double* __rest
                                                int Ap, int splits, double* K, double* J,
                                                int* eY) {
   const int AA = A * A;
-  // blocks x < n0: the K, J sums (a thread per entry); the others: the exponents
-  const int n0 = (AA + blockDim.x - 1) / blockDim.x;
+  // blocks x < n0: the K, J sums, kJkEntries entries each, K by the first threads and J by the next (a
+  // warp per scheduler, whose FP64 unit a chain of additions fills; a thread for both sums of an
+  // entry and 256 entries a CTA kept 25 SMs busy for most of the kernel's 27 us at 500 / 2000 /
+  // 80, 14 so); the others: the exponents
+  const int n0 = (AA + kJkEntries - 1) / kJkEntries;
   if (B_.x < n0) {
-    {
-      const int i = B_.x * blockDim.x + threadIdx.x;
-      if (i >= AA) return;
-      const int qi = i / A, pi = i % A;
-      const int src = pi <= qi ? i : pi * A + qi;  // the partials hold p <= q
-      double k = 0.0, j = 0.0;
-      int sp = 0;
-      for (; sp + 8 <= splits; sp += 8) {  // eight splits in flight, summed in order
-        double kv[8], jv[8];
+    const int which = threadIdx.x / kJkEntries;
+    const int i = B_.x * kJkEntries + threadIdx.x % kJkEntries;
+    if (which > 1 || i >= AA) return;
+    const int qi = i / A, pi = i % A;
+    const int src = pi <= qi ? i : pi * A + qi;  // the partials hold p <= q
+    const double* part = which == 0 ? Ksp : Jsp;
+    double t = 0.0;
+    int sp = 0;
+    for (; sp + 8 <= splits; sp += 8) {  // eight splits in flight, summed in order
+      double v[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          kv[u] = Ksp[(size_t)(sp + u) * AA + src];
-          jv[u] = Jsp[(size_t)(sp + u) * AA + src];
-        }
+      for (int u = 0; u < 8; ++u) v[u] = part[(size_t)(sp + u) * AA + src];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          k += kv[u];
-          j += jv[u];
-        }
-      }
-      if (sp < splits) {  // the rest, its loads in flight together too
-        double kv[7], jv[7];
-#pragma unroll
-        for (int u = 0; u < 7; ++u) {
-          const bool in = sp + u < splits;
-          kv[u] = in ? Ksp[(size_t)(sp + u) * AA + src] : 0.0;
-          jv[u] = in ? Jsp[(size_t)(sp + u) * AA + src] : 0.0;
-        }
-#pragma unroll
-        for (int u = 0; u < 7; ++u) {
-          if (sp + u >= splits) break;
-          k += kv[u];
-          j += jv[u];
-        }
-      }
-      K[i] += k;
-      J[i] += j;
+      for (int u = 0; u < 8; ++u) t += v[u];
     }
+    if (sp < splits) {  // the rest, its loads in flight together too
+      double v[7];
+#pragma unroll
+      for (int u = 0; u < 7; ++u) v[u] = sp + u < splits ? part[(size_t)(sp + u) * AA + src] : 0.0;
+#pragma unroll
+      for (int u = 0; u < 7; ++u) {
+        if (sp + u >= splits) break;
+        t += v[u];
+      }
+    }
+    double* out = which == 0 ? K : J;
+    out[i] += t;
     return;
   }
   // one warp per (split, row p), rows p >= A get exponent 0; the exponents of a CTA's rows by one
@@ -383,7 +375,7 @@ cudaError_t launch_mid_mixed(const Dims& d, int np, int splits, char* ws, const 
   launch_chained(k_kpart, dim3((kpart_quads(A) + 255) / 256, splits), 256, 0, s, b, D, np, A, Ap,
                  splits, (double*)(ws + L.Ksp), (double*)(ws + L.Jsp));
   const int ncta_e = (splits * Ap + 7) / 8;  // a warp per (split, row) of the exponents
-  launch_chained(k_jk_eY, (A * A + 255) / 256 + ncta_e, 256, 0, s, (const double*)(ws + L.Ksp),
+  launch_chained(k_jk_eY, (A * A + kJkEntries - 1) / kJkEntries + ncta_e, 256, 0, s, (const double*)(ws + L.Ksp),
                  (const double*)(ws + L.Jsp), D, W, BcF, np, A, Ap, splits, (double*)(ws + L.K),
                  (double*)(ws + L.J), (int*)(ws + L.eY));
   launch_chained(k_y_quant, np < sm_count() * 8 ? np : sm_count() * 8, dim3(Ap / 4, 8), 0, s,

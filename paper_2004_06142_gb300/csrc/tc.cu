@@ -1603,8 +1603,8 @@ struct SplitJobs {
 };
 
 // Column norms of job.S -> exponents of the integer + fraction split of S^T: e[c] for
-// c < nrows_out.  A CTA of at least 32 x G threads per 32 columns, G = norm_groups(N) (row
-// groups enough for the columns' length): thread (c, g < G) sums rows g, g + G, ...
+// c < nrows_out.  A CTA of (at least) columns x G threads per kNormCols columns (32 where the split
+// follows), G = norm_groups(N) (row groups enough for the columns' length): thread (c, g < G) sums rows g, g + G, ...
 // (coalesced across c, four loads in flight, in order of mu), the G partial sums of a column
 // are then added in order.
 __host__ __device__ inline int norm_groups(int N) { return N > 256 ? 32 : 8; }
@@ -1645,19 +1645,23 @@ __device__ __forceinline__ int colnorm_finish(const SplitJob& jb, int c, const d
   if (jb.norm) jb.norm[c] = nr;
   return e;
 }
+// kNormCols columns a CTA: the FP64 work of a CTA is what bounds it (64 clocks a warp instruction
+// and scheduler), so that many narrow CTAs beat few of whole lines (500 columns of 500: 14.5 us by
+// 32 columns, 11.2 by 8).
+constexpr int kNormCols = 8;
 __device__ __forceinline__ void k_colnorms_body(const Blk& B_, SplitJobs jobs, double invT, DevHeader* hdr) {
   const SplitJob& jb = jobs.j[B_.y];
-  if ((int)B_.x * 32 >= jb.nrows_out) return;  // uniform over the CTA
+  if ((int)B_.x * kNormCols >= jb.nrows_out) return;  // uniform over the CTA
   __shared__ double red[32][33];
-  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
+  const int tx = threadIdx.x % kNormCols, ty = threadIdx.x / kNormCols;
   const int G = norm_groups(jb.N);
-  const int c = B_.x * 32 + tx;
+  const int c = B_.x * kNormCols + tx;
   if (ty < G) red[ty][tx] = colnorm_partial(jb, c, ty, G);
   __syncthreads();
   if (ty == 0 && c < jb.nrows_out) colnorm_finish(jb, c, red, tx, G, invT, hdr);
 }
 // The row of CTAs behind the jobs', if any, clears `zero`.
-__global__ void __launch_bounds__(1024) k_colnorms(SplitJobs jobs, double invT, DevHeader* hdr,
+__global__ void __launch_bounds__(32 * kNormCols) k_colnorms(SplitJobs jobs, double invT, DevHeader* hdr,
                                                    const ZeroJob zero) {
   const Blk b = native_blk();
   if (b.y == jobs.count) {
@@ -1834,8 +1838,8 @@ cudaError_t launch_split_jobs(const SplitJobs& jobs, int Np, double invT, DevHea
     if (jobs.j[k].nrows_out > rmax) rmax = jobs.j[k].nrows_out;
   const bool clear = zero.flag || zero.n[0] > 0;
   launch_chained_to(first ? 0 : kChainCtas, k_colnorms,
-                    dim3((rmax + 31) / 32, jobs.count + (clear ? 1 : 0)),
-                    32 * norm_groups(jobs.j[0].N), 0, s, jobs, invT, hdr, zero);
+                    dim3((rmax + kNormCols - 1) / kNormCols, jobs.count + (clear ? 1 : 0)),
+                    kNormCols * norm_groups(jobs.j[0].N), 0, s, jobs, invT, hdr, zero);
   launch_chained(k_split_T, dim3((Np + 31) / 32, (rmax + 31) / 32, jobs.count), 256, 0, s, jobs, Np);
   count_launch(2);
   return cudaGetLastError();
