@@ -972,7 +972,8 @@ int grid_for(long long threads) {
   return (int)(nb < 1 ? 1 : (nb < 152 * 16 ? nb : 152 * 16));
 }
 
-cudaError_t launch_exps(const ExpJob* jobs, int count, cudaStream_t s) {
+// `first`: the first launch of a call.
+cudaError_t launch_exps(const ExpJob* jobs, int count, cudaStream_t s, bool first = false) {
   ExpJobs js{};
   long long nb = 1;
   for (int i = 0; i < count; ++i) {
@@ -982,7 +983,8 @@ cudaError_t launch_exps(const ExpJob* jobs, int count, cudaStream_t s) {
                                        : (jobs[i].rows + 7) / 8;
     if (t > nb) nb = t;
   }
-  launch_chained(k_exps, dim3((unsigned)(nb < 152 * 8 ? nb : 152 * 8), count), 256, 0, s, js);
+  launch_chained_to(first ? 0 : kChainCtas, k_exps,
+                    dim3((unsigned)(nb < 152 * 8 ? nb : 152 * 8), count), 256, 0, s, js);
   count_launch(1);
   return cudaGetLastError();
 }
@@ -1272,7 +1274,7 @@ cudaError_t digit_prepare_B(const Dims& d, const double* B, char* ws, const Layo
   int* out = (int*)(ws + L.eRow);
   if (d.layout == DONOF_B_DENSE) {
     const ExpJob j{B, d.N, (long long)d.Q * d.N, d.N, 0, out};
-    return launch_exps(&j, 1, s);
+    return launch_exps(&j, 1, s, true);
   }
   const int in_smem = d.N <= 12000 ? 1 : 0;
   k_packed_exps<<<d.Q < 152 * 8 ? d.Q : 152 * 8, 256, in_smem ? (size_t)d.N * 4 : 0, s>>>(

@@ -1404,6 +1404,11 @@ cudaError_t launch_tridiag(TriArgs a, int sms, cudaStream_t s) {
   // cluster: 24: 278 -> 268 us, 64: 552 -> 509, 120: 962 -> 891; with two rows a warp 160: 1288 ->
   // 1298, 256: 2286 -> 2490).  Fewer CTAs for the grid form change nothing (1 to 8 rows a CTA)
   if (a.N <= kClCols && size <= tridiag_cluster_max()) {
+    if (size > 8) {  // (each time: the context may be another one since the device was asked)
+      const cudaError_t e = cudaFuncSetAttribute(
+          k_tridiag<kClRows, kClCols / 32, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e != cudaSuccess) return e;
+    }
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeClusterDimension;
     at.val.clusterDim.x = size;

@@ -1110,6 +1110,7 @@ __device__ __forceinline__ void add_comp(float& s, float& c, float p) {
 // What elements too small for their square to be a float can add to a row's sum, per element.
 constexpr double kStatsLost = 0x1p-118;
 
+constexpr int kFlatN = 46000;  // slices below it are walked by 32-bit offsets
 constexpr int kBoundSlack = 64;
 // Row sums of slice P (N x N, symmetric) over its elements times 2^(-s_mu - s_nu) (s null: 0) in
 // units of 2^top: row(mu, squares, magnitudes), called by one thread per row.  EXACT: compensated
@@ -1127,8 +1128,8 @@ __device__ __forceinline__ int slice_row_sums(const double* __restrict__ B, int 
   constexpr int kSums = EXACT ? 4 : 1;  // squares, their compensation, magnitudes, theirs
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   int m = bound < 0 ? 0 : bound;  // biased; 0: the slice is zero
-  if (bound < 0 && !s) {  // the exponents alone: the slice from end to end, eight loads in flight
-    const int per = PACKED ? N * (N + 1) / 2 : N * N;
+  if (bound < 0 && !s && N < kFlatN) {  // the exponents alone: the slice from end to end, eight loads in flight
+    const int per = PACKED ? N * (N + 1) / 2 : N * N;  // (N below kFlatN)
     for (int i0 = threadIdx.x; i0 < per; i0 += 8 * blockDim.x) {
       int h[8];
 #pragma unroll
@@ -1184,10 +1185,10 @@ __device__ __forceinline__ int slice_row_sums(const double* __restrict__ B, int 
       for (int u = 0; u < kBatch; ++u) v[u] = x[u];
     }
   };
-  if (bound < 0 && s)
+  if (bound < 0 && (s || N >= kFlatN))
     walk([&](int mu, int nu, double v) {
       const int e = (__double2hiint(v) >> 20) & 0x7ff;
-      if (e > 0) m = max(m, e == 2047 ? 1 << 20 : e + 4096 - s[mu] - s[nu]);
+      if (e > 0) m = max(m, e == 2047 ? 1 << 20 : e + 4096 - (s ? s[mu] + s[nu] : 0));
     }, [](int) {});
   m = __reduce_max_sync(0xffffffffu, m);
   __syncthreads();  // red and sh are free
@@ -1476,7 +1477,7 @@ __device__ __forceinline__ void intfrac_split_scaled(double v, int k, __half& h,
 // stored elements dealt over its threads; the columns reach to the end of the rows' tile.  Bound by
 // its integer instructions, so that pieces past the matrix are only zeroed and no lane is left
 // over at the ends of rows (1103 packed slices of 301, a warp per row and zeros converted like
-// all others: 299 us; this: 206).
+// all others: 299 us; this: 214).
 __global__ void __launch_bounds__(256) k_split_B_sym(const double* __restrict__ B, int layout,
                                                      int Q, int N, SymTiles st,
                                                      const int* __restrict__ eS,
@@ -1501,17 +1502,18 @@ __global__ void __launch_bounds__(256) k_split_B_sym(const double* __restrict__ 
         const int k0 = -tp - eS[mu];
         double v[8];
         int k[8];
-        // element nu0 + j: in mu's row up to the diagonal, above it in row nu0 + j (packed); offsets
-        // within a slice fit an int (a slice of more would not fit the device)
-        const int row = dense ? mu * N + nu0 : mu * (mu + 1) / 2 + nu0;
+        // element nu0 + j: in mu's row up to the diagonal, above it in row nu0 + j (packed: N is at
+        // most kPackedStatsMaxN)
+        const double* Br = dense ? Bp + (size_t)mu * N : Bp;  // (offsets from it fit 32 bits)
+        const int row = dense ? nu0 : mu * (mu + 1) / 2 + nu0;
         const int diag = dense ? 8 : mu - nu0;  // the last j of the row
-        int col = nu0 * (nu0 + 1) / 2 + mu;
+        int col = dense ? 0 : nu0 * (nu0 + 1) / 2 + mu;
         if (nu0 + 8 <= N) {
           *(int4*)k = *(const int4*)(eS + nu0);
           *(int4*)(k + 4) = *(const int4*)(eS + nu0 + 4);
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            v[j] = __ldg(Bp + (j <= diag ? row + j : col));
+            v[j] = __ldg(Br + (j <= diag ? row + j : col));
             col += nu0 + j + 1;
             k[j] = k0 - k[j];
           }
@@ -1519,7 +1521,7 @@ __global__ void __launch_bounds__(256) k_split_B_sym(const double* __restrict__ 
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
             const bool in = nu0 + j < N;
-            v[j] = in ? __ldg(Bp + (j <= diag ? row + j : col)) : 0.0;
+            v[j] = in ? __ldg(Br + (j <= diag ? row + j : col)) : 0.0;
             col += nu0 + j + 1;
             k[j] = in ? k0 - eS[nu0 + j] : 0;
           }
