@@ -1127,10 +1127,11 @@ cudaError_t digit_product(int M, int N, int K, const double* A, long long sAm, l
 // ------------------------------------------------------------------ reflectors
 namespace {
 constexpr int kRefBlk = 64;   // reflectors per block
-constexpr int kRefCols = 8;   // columns of Z per CTA of k_reflect_w
+constexpr int kRefCols = 4;   // columns of Z per CTA of k_reflect_w
 // W = T (sum over the splits of part[s][n][c]) for the columns n of Z, c < 64 reflectors, and its
 // stage images (k = c, two stages): the sums and W in shared memory, a thread per reflector and
-// two columns; then a thread per column and 8 reflectors.
+// column; then a thread per column and 8 reflectors.  Bound by the FP64 units of a CTA's SM: 8
+// columns a CTA and two a thread took 18.5 us at 120 columns, 21.4 at 1200; this 13.6 and 19.4.
 __global__ void __launch_bounds__(256) k_reflect_w(const double* __restrict__ part, int splits,
                                                    int N, const double* __restrict__ T,
                                                    uint32_t k64, int* eW, __half* img, int NT,
@@ -1149,24 +1150,18 @@ __global__ void __launch_bounds__(256) k_reflect_w(const double* __restrict__ pa
   }
   __syncthreads();
   {
-    const int r = tid % kRefBlk, g = tid / kRefBlk * 2;  // T is upper triangular
-    double a0 = 0.0, a1 = 0.0, b0 = 0.0, b1 = 0.0;       // two chains each
+    const int r = tid % kRefBlk, g = tid / kRefBlk;  // T is upper triangular
+    double a0 = 0.0, a1 = 0.0;                       // two chains
     int c = r;
     for (; c + 1 < kRefBlk; c += 2) {
       a0 = fma(Ts[r][c], Ws[g][c], a0);
-      b0 = fma(Ts[r][c], Ws[g + 1][c], b0);
       a1 = fma(Ts[r][c + 1], Ws[g][c + 1], a1);
-      b1 = fma(Ts[r][c + 1], Ws[g + 1][c + 1], b1);
     }
-    if (c < kRefBlk) {
-      a0 = fma(Ts[r][c], Ws[g][c], a0);
-      b0 = fma(Ts[r][c], Ws[g + 1][c], b0);
-    }
+    if (c < kRefBlk) a0 = fma(Ts[r][c], Ws[g][c], a0);
     Wt[g][r] = a0 + a1;
-    Wt[g + 1][r] = b0 + b1;
   }
   __syncthreads();
-  if (tid < kRefCols * 8) {  // (two whole warps; 8 neighbouring lanes per column)
+  if (tid < kRefCols * 8) {  // (a whole warp; 8 neighbouring lanes per column)
     const int j = tid / 8, kc = tid % 8, n = n0 + j;
     double x[8];
     int m = 0;
