@@ -270,7 +270,7 @@ __device__ __forceinline__ uint32_t elect_one() {
   return r;
 }
 // mma_f16<0> by the lanes with lead != 0, the descriptors given as their low words (start address
-// and leading byte offset); the high word is that of sdesc(., 64).
+// and leading byte offset); the high word is that of 64-byte rows.
 __device__ __forceinline__ void mma_f16_if(uint32_t lead, uint32_t dtmem, uint32_t a, uint32_t b,
                                            uint32_t idesc, uint32_t accumulate) {
   asm volatile(
@@ -280,7 +280,7 @@ __device__ __forceinline__ void mma_f16_if(uint32_t lead, uint32_t dtmem, uint32
       "setp.ne.b32 p, %4, 0;\n\t"
       "setp.ne.b32 q, %5, 0;\n\t"
       "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n\t}" ::"r"(dtmem),
-      "r"(a), "r"(b), "r"(idesc), "r"(accumulate), "r"(lead), "n"(32 | 1 << 14 | 4 << 29)
+      "r"(a), "r"(b), "r"(idesc), "r"(accumulate), "r"(lead), "n"(sdesc_hi(8 * 64, 4))
       : "memory");
 }
 __device__ __forceinline__ void bulk_copy(uint32_t dst, const __half* src, uint32_t bytes,

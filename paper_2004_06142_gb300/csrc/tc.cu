@@ -519,16 +519,16 @@ __device__ __forceinline__ void tc_body(const TcArgs* __restrict__ targs,
         const uint32_t base = smem_u32(smem + (size_t)stage * stage_bytes) >> 4;  // in 16 bytes
         const bool tr = amn || (sym && jj > mt);
         const uint32_t id = tr ? (idesc | (1u << 15)) : idesc;
-        // the words of the descriptors (sdesc, sdesc_mn, sdesc_plain) and their step per 16 of k
-        constexpr uint32_t kHi = ((8u * SWZ) >> 4) | 1u << 14 | (SWZ == 128 ? 2u : 4u) << 29;
+        // the words of the descriptors and their step per 16 of k
+        constexpr uint32_t kHi = sdesc_hi(8 * SWZ, SWZ == 128 ? 2 : 4);
         uint32_t a_lo = base, a_hi, a_step;
         if (il8) {  // two K-adjacent core-matrix columns (BM rows x 16 B) per step
           a_lo |= (uint32_t)(BM * 16 >> 4) << 16;
-          a_hi = (128u >> 4) | 1u << 14;
+          a_hi = sdesc_hi(128, 0);
           a_step = 2 * BM * 16 >> 4;
         } else if (tr) {
           a_lo |= (mn_lbo >> 4) << 16;
-          a_hi = (mn_sbo >> 4) | 1u << 14 | 2u << 29;
+          a_hi = sdesc_hi(mn_sbo, 2);
           a_step = 2048 >> 4;
         } else {
           a_lo |= 1u << 16;

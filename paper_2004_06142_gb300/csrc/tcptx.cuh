@@ -103,39 +103,17 @@ __device__ __forceinline__ void tc_fence_before() {
 __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
-// Shared-memory matrix descriptor of a K-major tile with rows of `swz` bytes
-// (swizzle 128B: layout 2, 64B: layout 4), 8-row core groups `8*swz` bytes apart.
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr, int swz) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)1 << 16;                          // leading byte offset (unused, K-major swz)
-  d |= (uint64_t)((8u * (uint32_t)swz) >> 4) << 32;  // stride byte offset
-  d |= (uint64_t)1 << 46;                          // descriptor version
-  d |= (uint64_t)(swz == 128 ? 2 : 4) << 61;       // swizzle mode
-  return d;
-}
-// Shared-memory descriptor of an MN-major operand with the 128-byte swizzle: K rows of 64
-// MN elements (128 B each), the 64-wide MN chunks `chunk` bytes apart, groups of 8 K rows
-// 1024 bytes apart.
-__device__ __forceinline__ uint64_t sdesc_mn(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
-  return d;
-}
-// Shared-memory descriptor of a K-major operand without swizzle, stored as core matrices of
-// 8 rows x 16 bytes: rows 16 bytes apart, 8-row groups `sbo` bytes apart, K-adjacent core
-// matrices `lbo` bytes apart.
-__device__ __forceinline__ uint64_t sdesc_plain(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;
-  return d;  // layout type 0: no swizzle
+// Shared-memory matrix descriptors as two words.  Low: the start address and the leading byte
+// offset, (address >> 4) | (lbo >> 4) << 16.  High: the stride byte offset, the descriptor version
+// and the swizzle mode (sdesc_hi).
+//  * K-major tile with rows of 128 or 64 bytes, swizzled over them (layouts 2 and 4): sbo the 8
+//    rows of a core group; lbo unused, 1.
+//  * MN-major operand with the 128-byte swizzle (layout 2), K rows of 64 MN elements: lbo from one
+//    64-wide MN chunk to the next, sbo 1024, a group of 8 K rows.
+//  * K-major core matrices of 8 rows x 16 bytes without swizzle (layout 0): sbo from one 8-row
+//    group to the next, lbo between K-adjacent core matrices.
+__host__ __device__ constexpr uint32_t sdesc_hi(uint32_t sbo, uint32_t layout) {
+  return (sbo >> 4) | 1u << 14 | layout << 29;
 }
 // Instruction descriptor, kind::f16: fp16 A and B, fp32 D, both K-major, M x N.
 __host__ __device__ constexpr uint32_t idesc_f16(int M, int N) {
