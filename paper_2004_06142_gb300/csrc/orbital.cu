@@ -146,7 +146,8 @@ int opt_layout(int N, int A, int depth, OptLayout* o) {
   o->Fbar = take(nn);
   o->hist = take(2 * (size_t)m * nn);  // per slot: F_AO, then e_AO
   o->eps = take((size_t)N * 8);
-  o->scal = take(8 * 8);                // [0] E, [1] asym bits, [2] E of the occupation step
+  o->scal = take(8 * 8);                // [0] E, [1] asym bits, [2] E of the occupation step,
+                                        // [3] the products' status and abort words
   o->B = take((size_t)kMaxDepth * kMaxDepth * 8);
   o->c = take((size_t)(kMaxDepth + 2) * 8);  // c[0..n]; the restart flag kept at [kMaxDepth + 1]
   o->work = take(eigh_workspace_bytes(N));  // the eigensolver's workspace
@@ -349,6 +350,14 @@ struct Loop {
 
 bool ok(cudaError_t e) { return e == cudaSuccess; }
 
+// The products' operands go to the eigensolver's workspace, their status and abort words to words
+// of the loop's own, cleared when the loop starts (the eigensolver's are undefined before its
+// first call).
+EighScratch loop_scratch(const Loop& lp) {
+  int* words = (int*)(lp.ows + lp.L.scal + 24);
+  return EighScratch{eigh_scratch(lp.N, lp.ows + lp.L.work).mem, words, words + 1};
+}
+
 // one build at (C, gamma): E and lambda into the loop workspace, asym computed; returns
 // DONOF_OK and the host copies of E and asym
 int loop_build(Loop& lp, double* E, double* asym) {
@@ -385,7 +394,7 @@ int loop_reorthonormalise(Loop& lp) {
   const int N = lp.N;
   double* T1 = (double*)(lp.ows + lp.L.T1);
   double* T2 = (double*)(lp.ows + lp.L.T2);
-  const EighScratch sc = eigh_scratch(N, lp.ows + lp.L.work);
+  const EighScratch sc = loop_scratch(lp);
   if (product(N, N, N, lp.C, 1, N, lp.C, N, 1, T1, sc, lp.s) != DONOF_OK) return DONOF_ERR_CUDA;
   k_newton_schulz<<<152 * 4, 256, 0, lp.s>>>(T1, N, T1);
   count_launch(1);
@@ -423,7 +432,7 @@ int loop_orbital_step(Loop& lp, double zeta, int depth, std::vector<int>& active
   double* W = (double*)(o + lp.L.T2);  // R_a C^T, nact x N
   k_halve_block<<<152, 256, 0, lp.s>>>(Emo, N, A);
   count_launch(1);
-  const EighScratch sc = eigh_scratch(N, o + lp.L.work);
+  const EighScratch sc = loop_scratch(lp);
   if (product(A, N, N, Emo, N, 1, lp.C, 1, N, W, sc, lp.s) != DONOF_OK ||
       product(N, N, A, lp.C, N, 1, W, N, 1, T1, sc, lp.s) != DONOF_OK)
     return DONOF_ERR_CUDA;
@@ -488,7 +497,7 @@ int loop_initial_diagonal(Loop& lp) {
   const int rc = eigh_run(N, S, S, (double*)(o + lp.L.eps), o + lp.L.work, lp.s);
   if (rc != DONOF_OK) return rc;
   // T1 = C V, V[i][j] = S[i * N + j] (ascending eigenvalues)
-  if (product(N, N, N, lp.C, N, 1, S, N, 1, T1, eigh_scratch(N, o + lp.L.work), lp.s) != DONOF_OK ||
+  if (product(N, N, N, lp.C, N, 1, S, N, 1, T1, loop_scratch(lp), lp.s) != DONOF_OK ||
       !ok(cudaMemcpyAsync(lp.C, T1, (size_t)N * N * 8, cudaMemcpyDeviceToDevice, lp.s)))
     return DONOF_ERR_CUDA;
   k_negate<<<8, 256, 0, lp.s>>>((const double*)(o + lp.L.eps), N, lp.Fdiag);
@@ -536,6 +545,7 @@ extern "C" int donof_optimize(const donof_problem* prob, const donof_opt_params*
   lp.N = prob->nbf;
   lp.s = (cudaStream_t)stream;
   opt_layout(lp.N, prob->npair * (1 + prob->ncwo) + prob->nsingle, prm->diis_depth, &lp.L);
+  if (!ok(cudaMemsetAsync(lp.ows + lp.L.scal, 0, 8 * 8, lp.s))) return DONOF_ERR_CUDA;
 
   int nE = 0;
   auto record = [&](double E) {
