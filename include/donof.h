@@ -215,7 +215,8 @@ int donof_optimize_occupations(const donof_problem* prob, const int32_t* pair_ma
  * C_new <- C_new (3 I - C_new^T C_new) / 2.  lam, Fdiag[nbf], C (device, as in
  * donof_energy_lagrangian) in; C_new[nbf*nbf] (column j = new orbital j) and eps[nbf]
  * (device) out; nbf <= 4096.  Workspace: donof_orbital_update_workspace_size bytes (device,
- * 256-byte aligned).  Note: with lambda as defined here (lambda = C^T G, G = dE/dC / 4) the first-order
+ * 256-byte aligned).  A device-side wait that runs out leaves NaN in C_new and eps.  Note: with
+ * lambda as defined here (lambda = C^T G, G = dE/dC / 4) the first-order
  * energy change of this update is 4 sum_{q<p} F_qp^2 / (F_pp - F_qq), so a diagonal that
  * decreases with the orbital index lowers E (the paper's Eq. ene1 prints the opposite sign). */
 int donof_orbital_update_workspace_size(int32_t nbf, size_t* bytes);
@@ -335,7 +336,8 @@ int donof_nofmp2_static(const donof_problem* prob, const int32_t* pair_map,
  * h, B, pair_map as for donof_energy_lagrangian (B already prepared in build_ws); C[nbf*nbf],
  * gamma[npair*ncwo] and Fdiag[nbf] are device arrays updated in place.  opt_ws: device,
  * 256-byte aligned, donof_optimize_workspace_size bytes.  The call is synchronous: the host
- * reads E and the asymmetry after every build.  *result (host) receives the final E and
+ * reads E and the asymmetry after every build, and returns DONOF_ERR_TIMEOUT when a device-side
+ * wait of an orbital step ran out.  *result (host) receives the final E and
  * asymmetry, the iteration counts and whether it converged; energies (host, optional)
  * receives the energy of every orbital-iteration build, at most energies_cap of them. */
 typedef struct {

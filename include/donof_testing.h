@@ -59,6 +59,10 @@ int donof_testing_digit_product(const double* A, int64_t sAm, int64_t sAk, const
                                 int64_t ldb, double* C, int64_t ldc, int32_t M, int32_t N,
                                 int32_t K, void* workspace, size_t workspace_bytes, void* stream);
 
+/* The next `products` matrix products of the orbital step (donof_orbital_update, donof_optimize) of
+ * the calling host thread leave the abort word that a wait which ran out leaves. */
+int donof_testing_orbital_timeouts(int32_t products);
+
 /* The bounded device wait of the tensor-core kernel, run out on purpose: one CTA whose two
  * roles wait on mbarriers that nothing completes, the first with a limit of limit_a_ns
  * (at most 2 s), the second with limit_b_ns (at most 20 s).  The first wait's time-out

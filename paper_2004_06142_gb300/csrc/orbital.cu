@@ -2,6 +2,8 @@
 // Lagrangian lambda and a given diagonal, its FP64 eigendecomposition, the rotated orbitals
 // C V and their FP64 reorthonormalisation (one Newton-Schulz step C (3I - C^T C) / 2).
 // The eigendecomposition is this library's own FP64 solver (eigh.cu).
+#include <string.h>
+
 #include <vector>
 
 #include "common.cuh"
@@ -37,13 +39,30 @@ __global__ void k_newton_schulz(const double* __restrict__ S, int N, double* M) 
 // C = A B to double precision (M x N, row-major; A(m, k) at m sAm + k sAk, B(k, n) at k sBk +
 // n sBn, one stride of each 1), by exact digit products on the tensor cores: 0.17 ms at 1200^3
 // (1.7 ms and more on the FP64 pipe).  The operands' digits go to the eigensolver's workspace,
-// which is free between its calls.
+// which is free between its calls.  A wait that runs out raises the abort word and leaves C partly
+// unwritten: whoever calls this reads the word after its last product.  (t_timeouts: products of this
+// host thread still to be treated so, for tests.)
+thread_local int t_timeouts = 0;
 int product(int M, int N, int K, const double* A, long long sAm, long long sAk, const double* B,
             long long sBk, long long sBn, double* C, const EighScratch& w, cudaStream_t s) {
-  return digit_product(M, N, K, A, sAm, sAk, B, sBk, sBn, C, N, w.mem, w.status, w.abort_flag, s) ==
-                 cudaSuccess
-             ? DONOF_OK
-             : DONOF_ERR_CUDA;
+  cudaError_t e =
+      digit_product(M, N, K, A, sAm, sAk, B, sBk, sBn, C, N, w.mem, w.status, w.abort_flag, s);
+  if (e == cudaSuccess && t_timeouts > 0) {
+    --t_timeouts;
+    e = cudaMemsetAsync(w.abort_flag, 1, sizeof(int), s);
+  }
+  return e == cudaSuccess ? DONOF_OK : DONOF_ERR_CUDA;
+}
+
+// The orbitals and eigenvalues of an update one of whose waits ran out: NaN.
+__global__ void __launch_bounds__(256) k_void_timed_out(const int* abort_flag, double* C, long long nn,
+                                                        double* eps, int n) {
+  const int z = chain_begin();
+  if (*(const volatile int*)(abort_flag + z) == 0) return;
+  const double nan = __longlong_as_double(0x7ff8000000000000ll);
+  const long long t0 = blockIdx.x * 256ll + threadIdx.x;
+  for (long long i = t0; i < nn; i += 256ll * gridDim.x) C[i] = nan;
+  for (long long i = t0; i < n; i += 256ll * gridDim.x) eps[i] = nan;
 }
 
 }  // namespace
@@ -93,6 +112,13 @@ extern "C" int donof_orbital_update(int32_t nbf, const double* lam, const double
   count_launch(1);
   if (cudaGetLastError() != cudaSuccess) return DONOF_ERR_CUDA;
   if (product(N, N, N, T, N, 1, S, N, 1, C_new, sc, s) != DONOF_OK) return DONOF_ERR_CUDA;
+  // (this call has no status of its own: the workspace is the caller's, and the call may return
+  // before the device is done)
+  const long long n2 = (long long)N * N;
+  launch_chained(k_void_timed_out, (int)(n2 < 152 * 256 ? (n2 + 255) / 256 : 152), 256, 0, s,
+                 sc.abort_flag, C_new, n2, eps, N);
+  count_launch(1);
+  if (cudaGetLastError() != cudaSuccess) return DONOF_ERR_CUDA;
   prof_end(DONOF_PHASE_ORBITAL_UPDATE, s);
   return DONOF_OK;
 }
@@ -309,9 +335,14 @@ __global__ void k_diis_combine(const double* __restrict__ hist, const double* __
 }
 
 // Eigenvectors (columns of the row-major eigenvector matrix W) in decreasing eigenvalue order
-// as the columns of C; the eigenvalues in that order as the next diagonal.
+// as the columns of C; the eigenvalues in that order as the next diagonal.  The eigensolver's abort
+// word, which its next call clears, is passed on to the loop's words.
+__device__ __forceinline__ void pass_on_timeout(const int* from, int* words) {
+  if (blockIdx.x == 0 && threadIdx.x == 0 && *(const volatile int*)from != 0) words[1] = 1;
+}
 __global__ void k_take_descending(const double* __restrict__ W, const double* __restrict__ eps,
-                                  int N, double* C, double* Fdiag) {
+                                  int N, double* C, double* Fdiag, const int* eig_abort, int* words) {
+  pass_on_timeout(eig_abort, words);
   const long long tot = (long long)N * N;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < tot;
        i += (long long)gridDim.x * blockDim.x) {
@@ -330,7 +361,9 @@ __global__ void k_symmetrise(const double* __restrict__ lam, int N, double* S) {
     S[i] = 0.5 * (lam[i] + lam[(size_t)p * N + q]);
   }
 }
-__global__ void k_negate(const double* __restrict__ x, int n, double* y) {
+__global__ void k_negate(const double* __restrict__ x, int n, double* y, const int* eig_abort,
+                         int* words) {
+  pass_on_timeout(eig_abort, words);
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
     y[i] = -x[i];
 }
@@ -353,13 +386,15 @@ bool ok(cudaError_t e) { return e == cudaSuccess; }
 // The products' operands go to the eigensolver's workspace, their status and abort words to words
 // of the loop's own, cleared when the loop starts (the eigensolver's are undefined before its
 // first call).
+int* loop_words(const Loop& lp) { return (int*)(lp.ows + lp.L.scal + 24); }
 EighScratch loop_scratch(const Loop& lp) {
-  int* words = (int*)(lp.ows + lp.L.scal + 24);
+  int* words = loop_words(lp);
   return EighScratch{eigh_scratch(lp.N, lp.ows + lp.L.work).mem, words, words + 1};
 }
 
 // one build at (C, gamma): E and lambda into the loop workspace, asym computed; returns
-// DONOF_OK and the host copies of E and asym
+// DONOF_OK and the host copies of E and asym.  Every orbital step is followed by a build, so that
+// the steps' timed-out waits are found here.
 int loop_build(Loop& lp, double* E, double* asym) {
   char* o = lp.ows;
   int rc = donof_energy_lagrangian(lp.prob, lp.h, lp.B, lp.C, lp.gamma, lp.pm, lp.bws, lp.bbytes,
@@ -371,13 +406,16 @@ int loop_build(Loop& lp, double* E, double* asym) {
                                      (unsigned long long*)(o + lp.L.scal + 8));
   count_launch(1);
   if (!ok(cudaGetLastError())) return DONOF_ERR_CUDA;
-  double hv[2];
-  if (!ok(cudaMemcpyAsync(hv, o + lp.L.scal, 16, cudaMemcpyDeviceToHost, lp.s)) ||
+  double hv[4];
+  if (!ok(cudaMemcpyAsync(hv, o + lp.L.scal, 32, cudaMemcpyDeviceToHost, lp.s)) ||
       !ok(cudaStreamSynchronize(lp.s)))
     return DONOF_ERR_CUDA;
   int32_t st = 0;
   rc = donof_read_status(lp.bws, &st, lp.s);
   if (rc != DONOF_OK) return rc;
+  int32_t words[2];
+  memcpy(words, hv + 3, 8);
+  if (words[1] != 0) return DONOF_ERR_TIMEOUT;
   if (st != DONOF_OK) return st;
   *E = hv[0];
   *asym = hv[1];
@@ -470,7 +508,8 @@ int loop_orbital_step(Loop& lp, double zeta, int depth, std::vector<int>& active
   int rc = eigh_run(N, Fbar, Fbar, (double*)(o + lp.L.eps), o + lp.L.work, lp.s);
   if (rc != DONOF_OK) return rc;
   k_take_descending<<<152 * 4, 256, 0, lp.s>>>(Fbar, (const double*)(o + lp.L.eps), N, lp.C,
-                                               lp.Fdiag);
+                                               lp.Fdiag, eigh_scratch(N, o + lp.L.work).abort_flag,
+                                               loop_words(lp));
   count_launch(1);
   if (!ok(cudaGetLastError())) return DONOF_ERR_CUDA;
   rc = loop_reorthonormalise(lp);
@@ -500,7 +539,8 @@ int loop_initial_diagonal(Loop& lp) {
   if (product(N, N, N, lp.C, N, 1, S, N, 1, T1, loop_scratch(lp), lp.s) != DONOF_OK ||
       !ok(cudaMemcpyAsync(lp.C, T1, (size_t)N * N * 8, cudaMemcpyDeviceToDevice, lp.s)))
     return DONOF_ERR_CUDA;
-  k_negate<<<8, 256, 0, lp.s>>>((const double*)(o + lp.L.eps), N, lp.Fdiag);
+  k_negate<<<8, 256, 0, lp.s>>>((const double*)(o + lp.L.eps), N, lp.Fdiag,
+                                eigh_scratch(N, o + lp.L.work).abort_flag, loop_words(lp));
   count_launch(1);
   return ok(cudaGetLastError()) ? DONOF_OK : DONOF_ERR_CUDA;
 }
@@ -608,5 +648,13 @@ extern "C" int donof_optimize(const donof_problem* prob, const donof_opt_params*
   result->E = E;
   result->max_asym = asym;
   result->energies_recorded = nE;
+  return DONOF_OK;
+}
+
+#include "../../include/donof_testing.h"
+
+extern "C" int donof_testing_orbital_timeouts(int32_t products) {
+  if (products < 0) return DONOF_ERR_INVALID_ARG;
+  t_timeouts = products;
   return DONOF_OK;
 }
