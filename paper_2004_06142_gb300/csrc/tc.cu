@@ -1298,6 +1298,7 @@ inline int slice_warps(bool packed, int N) {
   while (packed && nw > 1 && (size_t)(nw + 1) * 16 * N > 200 * 1024) --nw;
   return nw;
 }
+constexpr int kSliceSmemMax = 224 * 1024;
 inline size_t slice_smem(bool packed, int N) {
   return packed ? (size_t)(slice_warps(true, N) + 1) * 16 * N : 0;  // (k_b_stats)
 }
@@ -2040,21 +2041,23 @@ cudaError_t launch_prepare_split_B(const Dims& d, const double* B, char* ws, con
   const bool packed = d.layout == DONOF_B_PACKED;
   if (packed && d.N > kPackedStatsMaxN) return cudaErrorInvalidValue;  // (no B of that size fits)
   const size_t smem = slice_smem(packed, d.N);
+  const size_t smem2 = (packed ? smem / 4 : 0) + (size_t)d.N * 4;
   const int threads = 32 * slice_warps(packed, d.N), ctas = d.Q < num_sms() * 8 ? d.Q : num_sms() * 8;
   auto stats = packed ? k_b_stats<true> : k_b_stats<false>;
   auto scale = packed ? k_p_scale<true> : k_p_scale<false>;
-  if (smem > 48 * 1024 || (size_t)d.N * 4 > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(stats, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(scale, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)((packed ? smem / 4 : 0) + (size_t)d.N * 4));
-    if (e != cudaSuccess) return e;
-  }
+  // the 48 KB that need no attribute are for the kernels' static shared memory too; one limit for
+  // every size, so that calls from several threads don't lower each other's
+  auto raise = [](const void* fn, size_t bytes) {
+    return bytes <= 47 * 1024 ? cudaSuccess
+                              : cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                     kSliceSmemMax);
+  };
+  cudaError_t e = raise((const void*)stats, smem);
+  if (e == cudaSuccess) e = raise((const void*)scale, smem2);
+  if (e != cudaSuccess) return e;
   stats<<<ctas, threads, smem, s>>>(B, d.Q, d.N, hdr, (double*)(ws + L.L1max),
                                     (float*)(ws + L.rn2), (unsigned long long*)(ws + L.rnmax));
   k_sym_scale<<<1, 1024, 0, s>>>((const double*)(ws + L.rnmax), d.N, (int*)(ws + L.eS));
-  const size_t smem2 = (packed ? smem / 4 : 0) + (size_t)d.N * 4;
   scale<<<ctas, threads, smem2, s>>>(B, d.Q, d.N, eS, invT, (const float*)(ws + L.rn2), tP);
   k_sym_exps<<<num_sms() * 4, 256, 0, s>>>(tP, eS, d.Q, d.N, (int*)(ws + L.eB));
   const SymTiles st = sym_tiles(d.N);
