@@ -1112,24 +1112,29 @@ constexpr double kStatsLost = 0x1p-118;
 
 constexpr int kFlatN = 46000;  // slices below it are walked by 32-bit offsets
 constexpr int kBoundSlack = 64;
+// How a slice is walked: dense rows; a packed lower triangle's stored rows; or its whole rows, the
+// part above the diagonal gathered from the columns (packed slices whose sums of columns have no
+// room in shared memory).
+enum SliceForm { kSliceDense = 0, kSlicePacked = 1, kSliceGathered = 2 };
 // Row sums of slice P (N x N, symmetric) over its elements times 2^(-s_mu - s_nu) (s null: 0) in
 // units of 2^top: row(mu, squares, magnitudes), called by one thread per row.  EXACT: compensated
-// sums, to about 2^-40; otherwise squares only, to sum_margin.  Dense: a warp per row.  Packed: a
+// sums, to about 2^-40; otherwise squares only, to sum_margin.  Whole rows: a warp per row.  Packed: a
 // warp per stored row, whose elements also count for their columns (partial sums per warp in
 // shared memory, added in the order of the warps).  bound: 4096 + an upper bound of the largest
 // scaled biased exponent, less than kBoundSlack above it, the largest over the threads; negative: it
 // is found first.  Returns top, the bound or the exponent itself (above 4096: a NaN or an infinity).
 // All threads of the CTA call it; sh holds kSums N floats per warp and once more (packed), red 33
 // ints.
-template <bool PACKED, bool EXACT, class Row>
+template <SliceForm FORM, bool EXACT, class Row>
 __device__ __forceinline__ int slice_row_sums(const double* __restrict__ B, int N,
                                               const int* __restrict__ s, float* sh, int* red,
                                               int bound, const Row& row) {
+  constexpr bool PACKED = FORM == kSlicePacked;
   constexpr int kSums = EXACT ? 4 : 1;  // squares, their compensation, magnitudes, theirs
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   int m = bound < 0 ? 0 : bound;  // biased; 0: the slice is zero
   if (bound < 0 && !s && N < kFlatN) {  // the exponents alone: the slice from end to end, eight loads in flight
-    const int per = PACKED ? N * (N + 1) / 2 : N * N;  // (N below kFlatN)
+    const int per = FORM != kSliceDense ? N * (N + 1) / 2 : N * N;  // (N below kFlatN)
     for (int i0 = threadIdx.x; i0 < per; i0 += 8 * blockDim.x) {
       int h[8];
 #pragma unroll
@@ -1150,7 +1155,7 @@ __device__ __forceinline__ int slice_row_sums(const double* __restrict__ B, int 
   constexpr int kBatch = 4;
   auto walk = [&](auto at, auto end) {
     auto row_at = [&](int mu) {
-      return B + (PACKED ? (long long)mu * (mu + 1) / 2 : (long long)mu * N);
+      return B + (FORM != kSliceDense ? (long long)mu * (mu + 1) / 2 : (long long)mu * N);
     };
     int mu = w, n0 = 0;  // the batch in v: row mu, elements n0 + lane + 32 u
     double v[kBatch];
@@ -1160,7 +1165,10 @@ __device__ __forceinline__ int slice_row_sums(const double* __restrict__ B, int 
 #pragma unroll
       for (int u = 0; u < kBatch; ++u) {
         const int nu = c0 + lane + 32 * u;
-        x[u] = r < N && nu < n ? p[nu] : 0.0;
+        if (FORM == kSliceGathered && nu > r)
+          x[u] = r < N && nu < n ? B[(long long)nu * (nu + 1) / 2 + r] : 0.0;
+        else
+          x[u] = r < N && nu < n ? p[nu] : 0.0;
       }
     };
     if (mu < N) load(mu, 0, v);
@@ -1290,17 +1298,20 @@ __device__ __forceinline__ double block_max(double v, unsigned long long* red) {
   for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t = max(t, red[i]);
   return __longlong_as_double((long long)t);
 }
-// Warps of a slice's CTA and its shared memory (the largest N of packed slices whose sums fit one
-// warp's share is 6400; no B of that size fits the device).
+// Warps of a slice's CTA and its shared memory.  Packed slices of more than 6400 functions, whose
+// sums of columns do not fit even one warp's share, are gathered by rows.
 constexpr int kPackedStatsMaxN = 6400;
-inline int slice_warps(bool packed, int N) {
+inline SliceForm slice_form(bool packed, int N) {
+  return !packed ? kSliceDense : N <= kPackedStatsMaxN ? kSlicePacked : kSliceGathered;
+}
+inline int slice_warps(SliceForm form, int N) {
   int nw = 8;
-  while (packed && nw > 1 && (size_t)(nw + 1) * 16 * N > 200 * 1024) --nw;
+  while (form == kSlicePacked && nw > 1 && (size_t)(nw + 1) * 16 * N > 200 * 1024) --nw;
   return nw;
 }
 constexpr int kSliceSmemMax = 224 * 1024;
-inline size_t slice_smem(bool packed, int N) {
-  return packed ? (size_t)(slice_warps(true, N) + 1) * 16 * N : 0;  // (k_b_stats)
+inline size_t slice_smem(SliceForm form, int N) {
+  return form == kSlicePacked ? (size_t)(slice_warps(form, N) + 1) * 16 * N : 0;  // (k_b_stats)
 }
 
 // Per row (P, mu) of B: its squared L2 norm (rn2, fp32 rounded up, for the exponents of X in the
@@ -1310,14 +1321,14 @@ inline size_t slice_smem(bool packed, int N) {
 // element, for two compensated sums over its row and over its column).  1103 packed slices of 301:
 // 0.28 ms (with a row's loads behind the reduction of the row before: 0.39; in double, every element
 // gathered twice: 1.18).
-template <bool PACKED>
+template <SliceForm FORM>
 __global__ void __launch_bounds__(256) k_b_stats(const double* __restrict__ B, int Q, int N,
                                                  DevHeader* hdr, double* L1max, float* rn2,
                                                  unsigned long long* rnmax_bits) {
   extern __shared__ float sh_f[];
   __shared__ int red[33];
   __shared__ unsigned long long redl[33];
-  const long long per = PACKED ? (long long)N * (N + 1) / 2 : (long long)N * N;
+  const long long per = FORM != kSliceDense ? (long long)N * (N + 1) / 2 : (long long)N * N;
   constexpr double kUp = 1.0 + 0x1p-36;  // above the compensated sums' error
   const double lost = N * kStatsLost;
   for (int P = blockIdx.x; P < Q; P += gridDim.x) {
@@ -1325,7 +1336,7 @@ __global__ void __launch_bounds__(256) k_b_stats(const double* __restrict__ B, i
     float* out = rn2 + (size_t)P * N;
     // the slice's scale is known to every thread only after the call: the rows are scaled by
     // the exponent that the call found, which it leaves in red
-    const int top = slice_row_sums<PACKED, true>(
+    const int top = slice_row_sums<FORM, true>(
         B + P * per, N, nullptr, sh_f, red, -1, [&](int mu, double ss, double l1) {
           const int t = red[32] - 4096;
           if (t > 4096) {
@@ -1353,22 +1364,26 @@ __global__ void __launch_bounds__(256) k_b_stats(const double* __restrict__ B, i
 // cannot tell on which side of a power of two the norm lies, the slice's sums are taken in
 // double.  1103 packed slices of 301: 0.13 ms (with a pass for the largest element first: 0.20; with
 // the loads of a row behind the row before too: 0.28; in double, with an ldexp per element: 1.35).
-template <bool PACKED>
+template <SliceForm FORM>
 __global__ void __launch_bounds__(256) k_p_scale(const double* __restrict__ B, int Q, int N,
-                                                 const int* __restrict__ eS, double invT,
-                                                 const float* __restrict__ rn2, int* tP) {
+                                                 const int* __restrict__ eS, int s_in_smem,
+                                                 double invT, const float* __restrict__ rn2,
+                                                 int* tP) {
+  constexpr bool PACKED = FORM == kSlicePacked;
   extern __shared__ float sh_f[];
   __shared__ int red[33];
   __shared__ unsigned long long redl[33];
-  const long long npk = (long long)N * (N + 1) / 2, per = PACKED ? npk : (long long)N * N;
+  const long long npk = (long long)N * (N + 1) / 2;
+  const long long per = FORM != kSliceDense ? npk : (long long)N * N;
   // rounding of the sums: N / 32 terms a lane, N / nw in a warp's sum of a column, the tree over
   // lanes, the warps' sums, every term rounded before
   const int nw = blockDim.x >> 5;
-  int* sS = (int*)(sh_f + (PACKED ? (nw + 1) * N : 0));  // the scale exponents, behind the sums
+  int* sh_s = (int*)(sh_f + (PACKED ? (nw + 1) * N : 0));  // the scale exponents, behind the sums
+  const int* sS = s_in_smem ? sh_s : eS;
   int lo = 1 << 20, hi = -(1 << 20);
   for (int i = threadIdx.x; i < N; i += blockDim.x) {
     const int e = eS[i];
-    sS[i] = e;
+    if (s_in_smem) sh_s[i] = e;
     lo = min(lo, e);
     hi = max(hi, e);
   }
@@ -1397,7 +1412,7 @@ __global__ void __launch_bounds__(256) k_p_scale(const double* __restrict__ B, i
       bound = max(bound, ((e - 125) >> 1) - sS[mu] - lo + 1022 + 4096);
     }
     if (__syncthreads_or(far)) bound = -1;
-    const int top = slice_row_sums<PACKED, false>(
+    const int top = slice_row_sums<FORM, false>(
         Bp, N, sS, sh_f, red, bound, [&](int, double ss, double) { mx = fmax(mx, ss); });
     const double ss = block_max(mx, redl);
     const double sc = pow2d(top - 1023);
@@ -1411,8 +1426,8 @@ __global__ void __launch_bounds__(256) k_p_scale(const double* __restrict__ B, i
     for (int mu = threadIdx.x >> 5; mu < N; mu += nw) {
       double t = 0.0;
       for (int nu = threadIdx.x & 31; nu < N; nu += 32) {
-        const double v = ldexp(load_B_elem(Bp, PACKED ? DONOF_B_PACKED : DONOF_B_DENSE, 0, mu, mu,
-                                           nu, N, npk),
+        const double v = ldexp(load_B_elem(Bp, FORM != kSliceDense ? DONOF_B_PACKED : DONOF_B_DENSE,
+                                           0, mu, mu, nu, N, npk),
                                -eS[mu] - eS[nu]);
         t = fma(v, v, t);
       }
@@ -1478,7 +1493,8 @@ __device__ __forceinline__ void intfrac_split_scaled(double v, int k, __half& h,
 // stored elements dealt over its threads; the columns reach to the end of the rows' tile.  Bound by
 // its integer instructions, so that pieces past the matrix are only zeroed and no lane is left
 // over at the ends of rows (1103 packed slices of 301, a warp per row and zeros converted like
-// all others: 299 us; this: 214).
+// all others: 299 us; this: 214).  Off: the offsets within a slice, 64 bits from kFlatN on.
+template <class Off>
 __global__ void __launch_bounds__(256) k_split_B_sym(const double* __restrict__ B, int layout,
                                                      int Q, int N, SymTiles st,
                                                      const int* __restrict__ eS,
@@ -1503,12 +1519,11 @@ __global__ void __launch_bounds__(256) k_split_B_sym(const double* __restrict__ 
         const int k0 = -tp - eS[mu];
         double v[8];
         int k[8];
-        // element nu0 + j: in mu's row up to the diagonal, above it in row nu0 + j (packed: N is at
-        // most kPackedStatsMaxN)
-        const double* Br = dense ? Bp + (size_t)mu * N : Bp;  // (offsets from it fit 32 bits)
-        const int row = dense ? nu0 : mu * (mu + 1) / 2 + nu0;
+        // element nu0 + j: in mu's row up to the diagonal, above it in row nu0 + j
+        const double* Br = dense ? Bp + (size_t)mu * N : Bp;
+        const Off row = dense ? (Off)nu0 : (Off)mu * (mu + 1) / 2 + nu0;
         const int diag = dense ? 8 : mu - nu0;  // the last j of the row
-        int col = dense ? 0 : nu0 * (nu0 + 1) / 2 + mu;
+        Off col = dense ? 0 : (Off)nu0 * (nu0 + 1) / 2 + mu;
         if (nu0 + 8 <= N) {
           *(int4*)k = *(const int4*)(eS + nu0);
           *(int4*)(k + 4) = *(const int4*)(eS + nu0 + 4);
@@ -2038,13 +2053,17 @@ cudaError_t launch_prepare_split_B(const Dims& d, const double* B, char* ws, con
   int* tP = (int*)(ws + L.tmax);
   const int* eS = (const int*)(ws + L.eS);
   const double invT = intfrac_inv_target(d.N);
-  const bool packed = d.layout == DONOF_B_PACKED;
-  if (packed && d.N > kPackedStatsMaxN) return cudaErrorInvalidValue;  // (no B of that size fits)
-  const size_t smem = slice_smem(packed, d.N);
-  const size_t smem2 = (packed ? smem / 4 : 0) + (size_t)d.N * 4;
-  const int threads = 32 * slice_warps(packed, d.N), ctas = d.Q < num_sms() * 8 ? d.Q : num_sms() * 8;
-  auto stats = packed ? k_b_stats<true> : k_b_stats<false>;
-  auto scale = packed ? k_p_scale<true> : k_p_scale<false>;
+  const SliceForm form = slice_form(d.layout == DONOF_B_PACKED, d.N);
+  const size_t smem = slice_smem(form, d.N);
+  const int s_in_smem = smem / 4 + (size_t)d.N * 4 <= kSliceSmemMax ? 1 : 0;
+  const size_t smem2 = smem / 4 + (s_in_smem ? (size_t)d.N * 4 : 0);
+  const int threads = 32 * slice_warps(form, d.N), ctas = d.Q < num_sms() * 8 ? d.Q : num_sms() * 8;
+  auto stats = form == kSliceDense    ? k_b_stats<kSliceDense>
+               : form == kSlicePacked ? k_b_stats<kSlicePacked>
+                                      : k_b_stats<kSliceGathered>;
+  auto scale = form == kSliceDense    ? k_p_scale<kSliceDense>
+               : form == kSlicePacked ? k_p_scale<kSlicePacked>
+                                      : k_p_scale<kSliceGathered>;
   // the 48 KB that need no attribute are for the kernels' static shared memory too; one limit for
   // every size, so that calls from several threads don't lower each other's
   auto raise = [](const void* fn, size_t bytes) {
@@ -2058,15 +2077,15 @@ cudaError_t launch_prepare_split_B(const Dims& d, const double* B, char* ws, con
   stats<<<ctas, threads, smem, s>>>(B, d.Q, d.N, hdr, (double*)(ws + L.L1max),
                                     (float*)(ws + L.rn2), (unsigned long long*)(ws + L.rnmax));
   k_sym_scale<<<1, 1024, 0, s>>>((const double*)(ws + L.rnmax), d.N, (int*)(ws + L.eS));
-  scale<<<ctas, threads, smem2, s>>>(B, d.Q, d.N, eS, invT, (const float*)(ws + L.rn2), tP);
+  scale<<<ctas, threads, smem2, s>>>(B, d.Q, d.N, eS, s_in_smem, invT, (const float*)(ws + L.rn2), tP);
   k_sym_exps<<<num_sms() * 4, 256, 0, s>>>(tP, eS, d.Q, d.N, (int*)(ws + L.eB));
   const SymTiles st = sym_tiles(d.N);
   if (st.dense)
     k_split_B_dense<<<num_sms() * 8, 256, 0, s>>>(B, d.layout, d.Q, d.N, st.ld, eS, tP,
                                                   (__half*)(ws + L.Bhi), (__half*)(ws + L.Blo));
   else
-    k_split_B_sym<<<num_sms() * 8, 256, 0, s>>>(B, d.layout, d.Q, d.N, st, eS, tP,
-                                                (__half*)(ws + L.Bhi), (__half*)(ws + L.Blo));
+    (d.N < kFlatN ? k_split_B_sym<int> : k_split_B_sym<long long>)<<<num_sms() * 8, 256, 0, s>>>(
+        B, d.layout, d.Q, d.N, st, eS, tP, (__half*)(ws + L.Bhi), (__half*)(ws + L.Blo));
   count_launch(5);
   return cudaGetLastError();
 }

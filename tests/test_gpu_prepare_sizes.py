@@ -59,3 +59,20 @@ def test_dense_at_the_default_limit(nbf):
     b.prepare(_slices(nbf, 1))
     torch.cuda.synchronize()
     assert b.status() == 0
+
+
+# the largest packed slices whose column sums fit shared memory, and whole rows gathered beyond
+@pytest.mark.parametrize("nbf,naux", [(6400, 1), (6401, 2), (6559, 1)])
+def test_packed_beyond_shared_memory(nbf, naux):
+    _agree(nbf, naux)
+
+
+def test_packed_beyond_shared_memory_reports_non_finite():
+    import torch
+    import paper_2004_06142_gb300 as dn
+    b = dn.Builder(6500, 1, 2, 1, dn.PNOF7, dn.B_PACKED, dn.MIXED)
+    B = torch.ones(1, 6500 * 6501 // 2, dtype=torch.float64, device="cuda")
+    B[0, 6499 * 6500 // 2 + 17] = float("inf")  # in the last row: part of column 17 too
+    b.prepare(B)
+    torch.cuda.synchronize()
+    assert b.status() == -3
