@@ -1298,9 +1298,9 @@ __device__ __forceinline__ double block_max(double v, unsigned long long* red) {
   for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t = max(t, red[i]);
   return __longlong_as_double((long long)t);
 }
-// Warps of a slice's CTA and its shared memory.  Packed slices of more than 6400 functions, whose
-// sums of columns do not fit even one warp's share, are gathered by rows.
-constexpr int kPackedStatsMaxN = 6400;
+// Warps of a slice's CTA and its shared memory.  Packed slices whose sums of columns leave a CTA
+// fewer than two warps are gathered by rows (5000 functions, 152 slices: 154 ms with one warp).
+constexpr int kPackedStatsMaxN = 4266;
 inline SliceForm slice_form(bool packed, int N) {
   return !packed ? kSliceDense : N <= kPackedStatsMaxN ? kSlicePacked : kSliceGathered;
 }
@@ -1437,6 +1437,72 @@ __global__ void __launch_bounds__(256) k_p_scale(const double* __restrict__ B, i
     const double exact = block_max(sqrt(t2), redl);
     if (threadIdx.x == 0) tP[P] = intfrac_exponent_inv(exact, invT);
   }
+}
+
+// The same two passes for a B of few slices, whose CTAs would leave most of the chip idle: a warp per
+// row (P, mu) of the whole B, in double, the part above a packed row's diagonal gathered.  L1max and
+// tmax start at zero; k_t_exps then gives t_P.
+__global__ void __launch_bounds__(256) k_b_stats_rows(const double* __restrict__ B, int layout,
+                                                      long long Q, int N, DevHeader* hdr,
+                                                      unsigned long long* L1max_bits, float* rn2,
+                                                      unsigned long long* rnmax_bits) {
+  const long long rows = Q * N, npk = (long long)N * (N + 1) / 2;
+  const int lane = threadIdx.x % 32;
+  bool bad = false;
+  for (long long row = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / 32; row < rows;
+       row += (long long)gridDim.x * blockDim.x / 32) {
+    const long long P = row / N;
+    const int mu = (int)(row % N);
+    double ss = 0.0, l1 = 0.0;
+    for (int nu = lane; nu < N; nu += 32) {
+      const double v = load_B_elem(B, layout, P, row, mu, nu, N, npk);
+      ss = fma(v, v, ss);
+      l1 += fabs(v);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      ss += __shfl_xor_sync(0xffffffffu, ss, o);
+      l1 += __shfl_xor_sync(0xffffffffu, l1, o);
+    }
+    const double nr = sqrt(ss);
+    if (lane == 0) {
+      rn2[row] = __double2float_ru(ss);
+      atomic_max_nonneg(L1max_bits + P, l1);
+      atomic_max_nonneg(rnmax_bits + mu, nr);
+    }
+    bad = bad || !isfinite(nr);
+  }
+  if (lane == 0 && bad) set_status(hdr, DONOF_ERR_NONFINITE);
+}
+__global__ void __launch_bounds__(256) k_p_scale_rows(const double* __restrict__ B, int layout,
+                                                      long long Q, int N,
+                                                      const int* __restrict__ eS,
+                                                      unsigned long long* tmax_bits) {
+  const long long rows = Q * N, npk = (long long)N * (N + 1) / 2;
+  const int lane = threadIdx.x % 32;
+  for (long long row = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / 32; row < rows;
+       row += (long long)gridDim.x * blockDim.x / 32) {
+    const long long P = row / N;
+    const int mu = (int)(row % N);
+    double ss = 0.0;
+    for (int nu = lane; nu < N; nu += 32) {
+      const double v = ldexp(load_B_elem(B, layout, P, row, mu, nu, N, npk), -eS[mu] - eS[nu]);
+      ss = fma(v, v, ss);
+    }
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    if (lane == 0) atomic_max_nonneg(tmax_bits + P, sqrt(ss));
+  }
+}
+__global__ void k_t_exps(const double* __restrict__ tmax, int Q, double invT, int* tP) {
+  for (int P = blockIdx.x * blockDim.x + threadIdx.x; P < Q; P += gridDim.x * blockDim.x)
+    tP[P] = intfrac_exponent_inv(tmax[P], invT);
+}
+// Whether the passes go by rows: a slice's CTA takes about 1.1 ns an element, the chip by rows 15 ps.
+// Both measured (donof_prepare_B, ms, slices / rows): 1200 dense, 16 slices 2.52 / 0.47, 64 slices
+// 2.61 / 1.63; 1200 packed, 16 1.27 / 0.47, 64 1.48 / 1.64; 3000 packed, 64 19.1 / 8.8, 152 20 / 21;
+// 200 dense, 16 0.140 / 0.085, 64 0.149 / 0.143; 5000 gathered, 64 50 / 24, 152 50 / 56.
+inline bool slices_by_rows(SliceForm form, int Q, int N) {
+  const int few = form == kSliceDense ? 80 : form == kSliceGathered ? 130 : 384 / slice_warps(form, N);
+  return N > 1 && Q < few;
 }
 
 // Symmetric scaling of B: B^P_{mu nu} = 2^(t_P + s_mu + s_nu) Bt^P_{mu nu} keeps Bt^P
@@ -2055,6 +2121,7 @@ cudaError_t launch_prepare_split_B(const Dims& d, const double* B, char* ws, con
   const double invT = intfrac_inv_target(d.N);
   const SliceForm form = slice_form(d.layout == DONOF_B_PACKED, d.N);
   const size_t smem = slice_smem(form, d.N);
+  const bool by_rows = slices_by_rows(form, d.Q, d.N);
   const int s_in_smem = smem / 4 + (size_t)d.N * 4 <= kSliceSmemMax ? 1 : 0;
   const size_t smem2 = smem / 4 + (s_in_smem ? (size_t)d.N * 4 : 0);
   const int threads = 32 * slice_warps(form, d.N), ctas = d.Q < num_sms() * 8 ? d.Q : num_sms() * 8;
@@ -2071,13 +2138,31 @@ cudaError_t launch_prepare_split_B(const Dims& d, const double* B, char* ws, con
                               : cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                      kSliceSmemMax);
   };
-  cudaError_t e = raise((const void*)stats, smem);
-  if (e == cudaSuccess) e = raise((const void*)scale, smem2);
-  if (e != cudaSuccess) return e;
-  stats<<<ctas, threads, smem, s>>>(B, d.Q, d.N, hdr, (double*)(ws + L.L1max),
-                                    (float*)(ws + L.rn2), (unsigned long long*)(ws + L.rnmax));
+  double* L1max = (double*)(ws + L.L1max);
+  float* rn2 = (float*)(ws + L.rn2);
+  auto* rnmax = (unsigned long long*)(ws + L.rnmax);
+  double* tmax = (double*)(ws + L.eB);  // by rows: in the space of the exponents made from it
+  if (by_rows) {
+    cudaError_t e = cudaMemsetAsync(L1max, 0, (size_t)d.Q * 8, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(tmax, 0, (size_t)d.Q * 8, s);
+    if (e != cudaSuccess) return e;
+    k_b_stats_rows<<<num_sms() * 8, 256, 0, s>>>(B, d.layout, d.Q, d.N, hdr,
+                                                 (unsigned long long*)L1max, rn2, rnmax);
+  } else {
+    cudaError_t e = raise((const void*)stats, smem);
+    if (e == cudaSuccess) e = raise((const void*)scale, smem2);
+    if (e != cudaSuccess) return e;
+    stats<<<ctas, threads, smem, s>>>(B, d.Q, d.N, hdr, L1max, rn2, rnmax);
+  }
   k_sym_scale<<<1, 1024, 0, s>>>((const double*)(ws + L.rnmax), d.N, (int*)(ws + L.eS));
-  scale<<<ctas, threads, smem2, s>>>(B, d.Q, d.N, eS, s_in_smem, invT, (const float*)(ws + L.rn2), tP);
+  if (by_rows) {
+    k_p_scale_rows<<<num_sms() * 8, 256, 0, s>>>(B, d.layout, d.Q, d.N, eS,
+                                                 (unsigned long long*)tmax);
+    k_t_exps<<<1, 256, 0, s>>>(tmax, d.Q, invT, tP);
+    count_launch(1);
+  } else {
+    scale<<<ctas, threads, smem2, s>>>(B, d.Q, d.N, eS, s_in_smem, invT, rn2, tP);
+  }
   k_sym_exps<<<num_sms() * 4, 256, 0, s>>>(tP, eS, d.Q, d.N, (int*)(ws + L.eB));
   const SymTiles st = sym_tiles(d.N);
   if (st.dense)

@@ -48,31 +48,41 @@ def _agree(nbf, naux):
 # dynamic shared memory just below 48 KB: packed slices' sums, dense slices' scale exponents
 @pytest.mark.parametrize("nbf", [338, 339, 340, 341, 342])
 def test_packed_at_the_default_limit(nbf):
-    _agree(nbf, 3)
+    _agree(nbf, 60)
 
 
 @pytest.mark.parametrize("nbf", [12032, 12200, 12288])
 def test_dense_at_the_default_limit(nbf):
     import torch
     import paper_2004_06142_gb300 as dn
-    b = dn.Builder(nbf, 1, 2, 1, dn.PNOF7, dn.B_DENSE, dn.MIXED)
-    b.prepare(_slices(nbf, 1))
+    b = dn.Builder(nbf, 80, 2, 1, dn.PNOF7, dn.B_DENSE, dn.MIXED)
+    b.prepare(torch.ones(80, nbf, nbf, dtype=torch.float64, device="cuda"))
     torch.cuda.synchronize()
     assert b.status() == 0
 
 
-# the largest packed slices whose column sums fit shared memory, and whole rows gathered beyond
-@pytest.mark.parametrize("nbf,naux", [(6400, 1), (6401, 2), (6559, 1)])
+# the largest packed slices whose column sums get two warps' shares of shared memory, and whole rows
+# gathered beyond, each with slices enough for a CTA each and with few
+@pytest.mark.parametrize("nbf,naux", [(4266, 192), (4267, 130), (4267, 3), (6400, 1), (6401, 2)])
 def test_packed_beyond_shared_memory(nbf, naux):
     _agree(nbf, naux)
 
 
-def test_packed_beyond_shared_memory_reports_non_finite():
+# the fewest slices that get a CTA each (80 dense, 384 / 8 packed) and the most that do not
+@pytest.mark.parametrize("nbf", [4, 9, 130, 257, 301])
+@pytest.mark.parametrize("naux", [1, 47, 48, 79, 80])
+def test_few_slices(nbf, naux):
+    _agree(nbf, naux)
+
+
+@pytest.mark.parametrize("naux", [1, 130])
+def test_packed_beyond_shared_memory_reports_non_finite(naux):
     import torch
     import paper_2004_06142_gb300 as dn
-    b = dn.Builder(6500, 1, 2, 1, dn.PNOF7, dn.B_PACKED, dn.MIXED)
-    B = torch.ones(1, 6500 * 6501 // 2, dtype=torch.float64, device="cuda")
-    B[0, 6499 * 6500 // 2 + 17] = float("inf")  # in the last row: part of column 17 too
-    b.prepare(B)
-    torch.cuda.synchronize()
-    assert b.status() == -3
+    for bad in (float("inf"), float("nan")):
+        b = dn.Builder(4300, naux, 2, 1, dn.PNOF7, dn.B_PACKED, dn.MIXED)
+        B = torch.ones(naux, 4300 * 4301 // 2, dtype=torch.float64, device="cuda")
+        B[naux - 1, 4299 * 4300 // 2 + 17] = bad  # in the last row: part of column 17 too
+        b.prepare(B)
+        torch.cuda.synchronize()
+        assert b.status() == -3
