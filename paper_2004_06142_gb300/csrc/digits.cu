@@ -1351,6 +1351,10 @@ int digit_block(const Dims& d, const double* Bblk, int p0, int np, char* ws, con
     int *bmax = (int*)(ws + L.bmax), *wmax = (int*)(ws + L.wmax), *eY = (int*)(ws + L.eY64);
     const double *Ac = (const double*)(ws + L.Acoef), *Bc = (const double*)(ws + L.Bcoef);
     const int js = jk_splits64(A, np), wc = np < 152 * 4 ? np : 152 * 4;
+    // (a slice's diagonal in shared memory: above 48 KB with the attribute, the largest there is, so
+    // that calls of several sizes don't lower each other's)
+    if ((size_t)A * 8 > 47 * 1024)
+      CKI(cudaFuncSetAttribute(k_w_jk64, cudaFuncAttributeMaxDynamicSharedMemorySize, 16384 * 8));
     launch_chained(k_w_jk64, wc + jb * js, 256, (size_t)A * 8, s, b, np, A, Ac, W, wmax, wc, js,
                    part, bmax);
     launch_chained(k_jk_final64, jb + (A + 7) / 8, 256, 0, s, part, js, A, Bc, bmax, wmax,
