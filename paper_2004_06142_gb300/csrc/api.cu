@@ -51,17 +51,23 @@ void choose_digit(Dims& d, uint64_t x_budget) {
   const int nblk0 = d.nblk, pb0 = d.pb;
   const size_t per = per_slice_fp64(d, 1);
   d.digit = 1;
-  for (int nblk = nblk0; nblk <= 4 * nblk0; ++nblk) {
+  // From the fewest blocks on, each number of slices a block once (every call comes through here):
+  // first those that the budget and the row and unit indices' 32 bits allow.
+  long long most = (1ll << 30) / d.N;
+  if (x_budget > 0 && x_budget / per < (uint64_t)most) most = (long long)(x_budget / per);
+  if (most < 1) most = 1;
+  long long nblk = nblk0;
+  if ((d.Q + nblk - 1) / nblk > most) nblk = (d.Q + most - 1) / most;
+  while (nblk <= 4ll * nblk0) {
     const long long pb = (d.Q + nblk - 1) / nblk;
-    if (x_budget > 0 && pb > 1 && (size_t)pb * per > x_budget) continue;
     set_blocks(d, pb);
-    if ((long long)d.pb * d.N > (1ll << 30)) continue;  // row and unit indices in 32 bits
     const size_t total = make_layout(d).total;
     if (total <= limit) {
       d.ws_total = total > plain ? total : plain;
       return;
     }
     if (pb == 1) break;
+    nblk = (d.Q + pb - 2) / (pb - 1);  // the fewest blocks of fewer slices
   }
   d.digit = 0;
   set_blocks(d, pb0);
