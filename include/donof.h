@@ -60,10 +60,12 @@ enum { DONOF_PNOF5 = 5, DONOF_PNOF7 = 7, DONOF_PNOF7S = 8 };
 enum { DONOF_B_DENSE = 0, DONOF_B_PACKED = 1 };
 /* DONOF_FP64: every contraction to double precision.  Where their buffers fit (almost always),
  * as exact digit products on the tensor cores: operands in fixed point of 57 bits and a sign
- * relative to the largest element of their row, eight digits each, the digit products summed in
- * integers and rounded once; errors are those of a double GEMM or below, relative to the largest
- * elements (elements below 2^-57 of their row's largest are lost).  Otherwise in IEEE double on
- * the CUDA cores.
+ * relative to the largest element of their row (elements below 2^-57 of it are lost), eight digits
+ * each, the digit products summed in integers, the sum cut to 62 bits and rounded once; sums over
+ * splits and blocks of the auxiliary index are added in double.  The contractions over AO indices
+ * take powers of two off B and h and put them on C, so that errors do not depend on the norms of the
+ * AO functions; they are those of a double GEMM or below, relative to the largest elements.
+ * Otherwise in IEEE double on the CUDA cores.
  * DONOF_MIXED: the large contractions (X = B C, b = C^T X, G += X Y, lambda = C^T G) on the
  * tensor cores.  Every operand row is stored as 2^e (h + f): h an fp16 integer with the
  * row's L2 norm bounding ||h||_2 below 2^12, f the fp16 remainder.  The integer products
@@ -111,8 +113,8 @@ int donof_workspace_size(const donof_problem* prob, size_t* bytes);
 
 /* Register B (device) with the workspace.  DONOF_MIXED: converts B once into the
  * integer + fraction fp16 copy that every later build streams (B is fixed across orbital
- * iterations, Sec. III.D).  DONOF_FP64: records B and the largest exponents of its
- * rows, which later builds scale by.  Must be called again when B
+ * iterations, Sec. III.D).  DONOF_FP64: records B, the scales of its AO indices and the largest
+ * exponents of its rows, which later builds scale by.  Must be called again when B
  * changes; the build calls must then pass the same B pointer. */
 int donof_prepare_B(const donof_problem* prob, const double* B, void* workspace,
                     size_t workspace_bytes, void* stream);

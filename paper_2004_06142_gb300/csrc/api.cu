@@ -178,11 +178,14 @@ Layout make_layout(const Dims& d) {
     if (!d.digit) L.skp = take(ks > 1 ? ks * N * A * 8 : 0);
   }
   if (d.precision == DONOF_FP64) {
-    L.X64 = take(pb * N * A * 8);
+    const size_t x = pb * N * A * 8, kb = d.digit ? kscale_bytes(d.N) : 0;
+    L.X64 = take(x > kb ? x : kb);
+    L.sH = L.X64;  // (a build's end alone, which has no X)
     L.b64 = take(pb * A * A * 8);
     L.Bun = d.layout == DONOF_B_PACKED ? take(pb * N * N * 8) : 0;
     if (d.digit) {
       L.eRow = take((size_t)d.Q * N * 4);
+      L.sB = take(kscale_bytes(d.N));
       L.eH64 = take(N * 4);
       L.eC64 = take(N * 4);      // eC64 .. exend: zeroed per build
       L.eG64 = take(A * 4);
@@ -484,7 +487,7 @@ int run_build(const donof_problem* prob, const double* h, const double* B, const
     rc = run_hc_tc(d, ws, L, s);
     if (rc != DONOF_OK) return rc;
   } else if (d.digit) {
-    CK(digit_hc(d, h, C, ws, L, zero, s));
+    CK(digit_hc(d, h, C, mode != kFinish, ws, L, zero, s));
   } else {
     CK(cudaMemsetAsync(zero.flag, 0, sizeof(int32_t), s));
     for (int i = 0; i < 4; ++i)
@@ -585,7 +588,7 @@ int run_build(const donof_problem* prob, const double* h, const double* B, const
       rc = run_lambda_tc(d, C, ws, L, lam, s);
       if (rc != DONOF_OK) return rc;
     } else if (d.digit) {
-      CK(digit_lambda(d, C, ws, L, lam, s));
+      CK(digit_lambda(d, C, mode != kFinish, ws, L, lam, s));
     } else {
       CK(cudaMemsetAsync(lam, 0, (size_t)N * N * 8, s));
       CK(launch_dgemm(split_k_args(N, A, N, C, 1, N, (const double*)(ws + L.G), A, 1, lam, N, 1,

@@ -47,8 +47,9 @@ struct Layout {
   size_t X64, b64, Y64, Bun;
   // FP64 path on digit products: largest biased exponents of B's rows (eRow, from
   // prepare), of C's columns, h's rows and G's columns, of X per (P, q) and per mu, of b and
-  // w, and Y's columns; the stage images of C_act (then of G) and of Y; w^P
-  size_t eRow, eC64, eH64, eG64, exq, exm, bmax, wmax, exend, eY64, Cimg, Yimg, W64;
+  // w, and Y's columns; the stage images of C_act (then of G) and of Y; w^P; the AO indices' scales
+  // (KScale) of B and, for a build's end without a B, of h
+  size_t eRow, eC64, eH64, eG64, exq, exm, bmax, wmax, exend, eY64, Cimg, Yimg, W64, sB, sH;
   // mixed path
   // integer + fraction planes (h, f) of the tensor-core operands and their per-row
   // exponents: B (Bhi/Blo, eB), C_act^T (Chi/Clo, eC), X^T for b (Xthi/Xtlo, eXt), X for G
@@ -397,6 +398,19 @@ struct DgemmArgs {
 };
 cudaError_t launch_dgemm(const DgemmArgs& a, cudaStream_t s);
 
+// Powers of two taken off one operand of a contraction, along its k, and put on the other: info =
+// {whether any s is not zero, the largest s}, s >= 0, kp = s 2^20, kn = -s 2^20, padded with zeros
+// to kscale_pad (digits.cu).
+struct KScale {
+  const int* info;
+  const uint32_t *kp, *kn;
+};
+__host__ __device__ inline int kscale_pad(int K) { return (K + 31) / 32 * 32; }
+inline size_t kscale_bytes(int K) { return 256 + (size_t)2 * kscale_pad(K) * 4; }
+inline KScale kscale_at(char* p, int K) {
+  const uint32_t* w = (const uint32_t*)(p + 256);
+  return KScale{(const int*)p, w, w + kscale_pad(K)};
+}
 // Products of doubles as exact digit products on the tensor cores (digits.cu).
 struct DigitArgs {
   // A(m, k): row m = b Mb + r at A + b sAb + r sAm; k = kb Kpad + q at kb sAkb + q sAk
@@ -405,6 +419,9 @@ struct DigitArgs {
   long long sAb, sAm, sAk, sAkb;
   int M, Mb, Kin, Kpad, KB;
   const int* eA;        // per row: the largest biased exponent in it, or a larger one; null: 1023
+  // when set (KB 1): A(m, k) is taken times 2^-s_k, ks the words of KScale; where *ks_on is 0, s = 0
+  const uint32_t* ks;
+  const int* ks_on;
   const __half* Bimg;   // stage images of B (k_digit_planes)
   const int* eB;        // per column, as eA
   int N, NT, ntiles, mtiles, nstages, splits;
@@ -413,9 +430,11 @@ struct DigitArgs {
   double* C;
   long long sCs, sCb, sCm;
   // when set: the largest biased exponents of the result, per (m / Mb, n) in exq[.. exq_ld + n]
-  // and per m % Mb in exm (atomic maxima; zeroed by the caller)
+  // and per m % Mb in exm (atomic maxima; zeroed by the caller); exq's of the result times
+  // 2^-row_s[m % Mb]
   int *exq, *exm;
   int exq_ld;
+  const uint32_t* row_s;  // as kp
   int sub;              // C -= A B
   int vecA, vecC;       // 16-byte loads of A / stores of C are aligned
   int *status, *abort_flag;
@@ -473,12 +492,13 @@ cudaError_t digit_reflect(int N, int nref, const double* Yr, const double* T, do
 // slices (X, b, J, K, G; Bblk: its slices, dense), lambda.
 cudaError_t digit_prepare_B(const Dims& d, const double* B, char* ws, const Layout& L,
                             cudaStream_t s);
-cudaError_t digit_hc(const Dims& d, const double* h, const double* C, char* ws, const Layout& L,
-                     ZeroJob zero, cudaStream_t s);
+// (prepared: the workspace holds a B, whose scales of the AO indices are taken; else h's)
+cudaError_t digit_hc(const Dims& d, const double* h, const double* C, bool prepared, char* ws,
+                     const Layout& L, ZeroJob zero, cudaStream_t s);
 int digit_block(const Dims& d, const double* Bblk, int p0, int np, char* ws, const Layout& L,
                 cudaStream_t s);
-cudaError_t digit_lambda(const Dims& d, const double* C, char* ws, const Layout& L, double* lam,
-                         cudaStream_t s);
+cudaError_t digit_lambda(const Dims& d, const double* C, bool prepared, char* ws, const Layout& L,
+                         double* lam, cudaStream_t s);
 // The split count split_k_args uses for an M x N output with contraction length K.
 int splitk_count(int M, int N, int K);
 // Symmetric FP64 eigensolver (eigh.cu): A (N x N, row-major, symmetric; not modified) =

@@ -10,23 +10,28 @@
 // relative to 2^(EA + EB)).  Over kChunk = 256 elements of k no partial sum of a group exceeds
 //   256 * 256^2 = 2^24 (g = 0),  256 (2 * 256 * 64 + (g - 1) 64^2) <= 14.7e6 (g > 0),
 // so every accumulation is exact whatever the tensor core's rounding; after each chunk the
-// groups are added up in integers (92 bits, so a contraction may have 2^17 chunks) and the sum
-// is rounded once, to the double that is stored.
+// groups are added up in integers (group 0 in 32 bits: at most 127 chunks; contractions are cut at
+// 64, K <= 16384), and the sum, cut to its leading 62 bits, is rounded once, to the double that is
+// stored.  (Splitting operands so that products of low precision are exact: Ozaki, Ogita, Oishi and
+// Rump, "Error-free transformations of matrix multiplication".)
 //
 // Error: elements within 2^4 of their row's (column's) largest are represented exactly, smaller
 // ones to 2^-57 of it; the digit products left out add about 2^-57 sqrt(K) of the product of the
-// two maxima.  A chain of K double FMAs rounds its running sum K times, which over the
-// contractions of a build is as much or more (measured over 64-bit references: see
-// tests/test_gpu_digits.py).  Rows or columns that hold a NaN or an infinity give NaN; elements
-// below 2^-958 count as zero.
+// two maxima.  A chain of K double FMAs rounds its running sum K times, relative to the terms:
+// as much or more where the terms are of one size (tests/test_gpu_digits.py), but less where small
+// elements of one operand meet large ones of the other.  In a build that is so when the AO
+// functions' norms differ, and there the scales of k_scales take it off (tests/
+// test_gpu_ao_scaling.py).  Rows or columns that hold a NaN or an infinity give NaN; elements below
+// 2^-958 (scaled) count as zero.
 //
 // The B operand's digits are written once per product, as the images of the shared-memory
 // stages (k_digit_planes); the digits of A are formed on the way into shared memory from the
 // doubles themselves (8 bytes per element read once per column tile instead of 16 of digits
 // written and read).
 //
-// CTA (576 threads, one per SM, 16 worker warps, an MMA warp and a copying warp): a unit is a 128 x
-// NT output tile (NT <= 64) and a range of 32-wide K stages.  Per stage each worker thread turns 8
+// CTA (one per SM: 16 worker warps, an MMA warp, a copying warp and, for wide tiles, two idle ones
+// that leave their registers to the workers): a unit is a 128 x NT output tile (NT <= 64) and a range
+// of 32-wide K stages.  Per stage each worker thread turns 8
 // doubles (fetched one stage ahead) into 8 x 8 digits in shared memory; the MMA warp multiplies A's
 // digit i with B's stacked digits 0 .. 7 - i, whose products land in the neighbouring
 // accumulators i .. 7, so a digit of A is read once per 256 columns; the copying warp fetches B's
@@ -34,8 +39,8 @@
 // meanwhile; carries go back to TMEM, so that only group 0 needs registers between the chunks of a
 // unit.
 //
-// Measured: 3150 clocks per stage of a 128 x 48 tile, 1.7 us, and some 10000 per unit for the
-// conversion of its result; X = B C at N 500, 80 orbitals, 2000 slices: 3.4 ms (78.9 ms on the FP64
+// Measured: about 2850 clocks per stage of a 128 x 48 tile, 1.5 us, and some 10000 per unit for the
+// conversion of its result; X = B C at N 500, 80 orbitals, 2000 slices: 3.14 ms (78.9 ms on the FP64
 // pipe).  What bounds it: the workers' integer instructions (about 400 per warp and stage, the
 // integer ALU at half rate, 2000 clocks), with four warps to a scheduler to hide their latencies;
 // the MMAs' shared-memory reads (100 KB per 16 of k at 128 bytes a clock, 1600 clocks per stage)
@@ -44,6 +49,7 @@
 // workers as much), stages of 16 (slower), loops instead of unrolled columns in the conversion
 // of the results (what they keep in local memory costs 20 %), waits that sleep (1 % slower).
 #include <atomic>
+#include <type_traits>
 
 #include "common.cuh"
 #include "tcptx.cuh"
@@ -55,16 +61,30 @@ constexpr int kD = 8;             // digits of an operand
 constexpr int kStageK = 32;       // elements of k per stage (64-byte rows, 64-byte swizzle)
 constexpr int kChunkStages = 8;   // stages per exact accumulation (256 elements)
 constexpr int kWorkers = 16;      // worker warps
-constexpr int kDigThreads = 32 * (kWorkers + 2);  // ..., the MMA warp, the copying warp
+// Registers a thread of the wide tiles once the roles part: the launch's 96 (five warps on a
+// scheduler) leave the workers' elements and columns spilled, which the scales' words make worse (a
+// build of 500 / 2000 / 80 4.75 ms without the scales, 5.12 with them, 4.45 so; narrow tiles do not
+// spill, and a short product pays about 0.5 us for the exchange).
+constexpr int kWorkerRegs = 112, kOtherRegs = 32;
+constexpr bool split_regs(int NT) { return NT >= 48; }
+constexpr int dig_threads(int NT) { return 32 * (kWorkers + (split_regs(NT) ? 4 : 2)); }
 constexpr int kTileM = 128;
 constexpr uint32_t kABytes = kD * kTileM * kStageK * 2;  // a stage of A digits
 // sum_{i > 0} 64 2^(7 (7 - i)) + 256 2^49: makes every digit's field non-negative
 constexpr long long kBias = 64ll * (((1ll << 49) - 1) / 127) + (256ll << 49);
 
+// The biased exponent of x; of a NaN or an infinity kNanMark, above every finite (and scaled) one.
+constexpr int kNanMark = 1 << 14;
+__device__ __forceinline__ int exp_of(double x) {
+  const int e = (__double2hiint(x) >> 20) & 0x7ff;
+  return e == 2047 ? kNanMark : e;
+}
 // The exponent word of a row (or column) whose largest biased exponent is em, for its products'
 // scale (a row with a NaN or an infinity: far above every finite scale, which marks its results).
 constexpr int kNanExp = 1 << 20;
-__device__ __forceinline__ int scale_exp(int em) { return em >= 2047 ? kNanExp : (em < 64 ? 64 : em); }
+__device__ __forceinline__ int scale_exp(int em) {
+  return em >= kNanMark / 2 ? kNanExp : (em < 64 ? 64 : em);
+}
 // ... and as split_exp, (em + 7) << 20, for the shift of its elements' mantissas.
 __device__ __forceinline__ uint32_t split_exp(int em) { return (uint32_t)((em < 64 ? 64 : em) + 7) << 20; }
 
@@ -113,7 +133,7 @@ __device__ __forceinline__ uint32_t digit_pair(const Fixed& a, const Fixed& b, u
                                      __float2half2_rn(-1024.0f / (1 << s) - 64.0f));
   return *reinterpret_cast<const uint32_t*>(&d);
 }
-// The digits of 8 consecutive elements of k, one 16-byte word per digit, `step` bytes apart.
+// The digits of 8 consecutive elements of k, one 16-byte word per digit.
 struct Fixed8 {
   Fixed f[8];
   uint32_t k64;
@@ -122,6 +142,15 @@ __device__ __forceinline__ void to_fixed8(const double (&x)[8], uint32_t e20, ui
                                           Fixed8& r) {
 #pragma unroll
   for (int j = 0; j < 8; ++j) r.f[j] = to_fixed(x[j], e20);
+  r.k64 = k64;
+}
+// The same with the elements scaled by the powers of two of their k (ks: KScale's words of the 8).
+__device__ __forceinline__ void to_fixed8(const double (&x)[8], uint32_t e20,
+                                          const uint32_t* __restrict__ ks, uint32_t k64, Fixed8& r) {
+  const uint4 a = __ldg((const uint4*)ks), b = __ldg((const uint4*)ks + 1);
+  const uint32_t k[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+  for (int j = 0; j < 8; ++j) r.f[j] = to_fixed(x[j], e20 + k[j]);
   r.k64 = k64;
 }
 template <int D = 0, class Put>
@@ -292,8 +321,15 @@ __device__ __forceinline__ void bulk_copy(uint32_t dst, const __half* src, uint3
       : "memory");
 }
 
+// Whether a contraction's k are scaled: the word is loaded before the chain's wait (it is written
+// before the first kernel of a call, which is launched plainly) and looked at behind it, by adding the
+// wait's zero.
+__device__ __forceinline__ int scales_word(const int* info) {
+  return info ? *(const volatile int*)info : 0;
+}
+
 template <bool KC, int NT>
-__global__ void __launch_bounds__(kDigThreads, 1)
+__global__ void __launch_bounds__(dig_threads(NT), 1)
     k_digit_gemm(const __grid_constant__ DigitArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -326,11 +362,14 @@ __global__ void __launch_bounds__(kDigThreads, 1)
   __syncthreads();
   tc_fence_after();
   constexpr uint32_t tmem = 0;  // all 512 columns are this CTA's: they start at column 0
+  const int scales = scales_word(a.ks_on);
   // all of the above while the kernel before runs
   const int zero = chain_wait();
+  const bool scaled = scales + zero != 0;
 
-  if (warp == kWorkers) {
-    {  // ------------------------------------------------ MMA issuer
+  if (warp >= kWorkers) {
+    if constexpr (split_regs(NT)) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kOtherRegs));
+    if (warp == kWorkers) {  // ---------------------------------------- MMA issuer
       // The whole warp walks the stages and one elected lane issues, so that the descriptors are
       // computed in the uniform registers the MMAs take them from (a branch of one lane moves
       // them there, eight moves an MMA: a build of 500 / 2000 / 80 5.68 ms, so 5.19)
@@ -384,48 +423,49 @@ __global__ void __launch_bounds__(kDigThreads, 1)
         __syncwarp();
         mbar_wait_quiet(bar(kClean), 0u, kDrainLimitNs);
       }
-    }
-    __syncwarp();
-  } else if (warp == kWorkers + 1) {  // ------------------------------------ copies of B's digits
-    // (a warp of its own: one of the workers, whose arrivals all wait for, held up every stage: a
-    // build of 500 / 2000 / 80 5.19 ms, so 4.78)
-    if (lane == 0) {
-      uint32_t it = 0, issued[2] = {0, 0};
-      bool ok = true;
-      for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
-        const int sp = u / (a.ntiles * a.mtiles);
-        const int s0 = (int)((long long)a.nstages * sp / a.splits);
-        const int s1 = (int)((long long)a.nstages * (sp + 1) / a.splits);
-        const int n0 = u % a.ntiles * NT;
-        const size_t img_stage = (size_t)kD * a.imgNT * kStageK;
-        // NT rows of every digit's rows (a multiple of 16: the swizzle's phase is theirs)
-        const __half* img = a.Bimg + ((size_t)(n0 / a.imgNT) * a.nstages + s0) * img_stage +
-                            n0 % a.imgNT * kStageK;
-        for (int st = s0; st < s1; ++st, ++it, img += img_stage) {
-          const uint32_t buf = it & 1u, ph = (it >> 1) & 1u;
-          if (!wait_for(bar(kEmpty + buf), ph ^ 1u, a)) {
-            ok = false;
-            break;
-          }
-          const uint32_t dst = smem0 + buf * stage_bytes + kABytes;
-          mbar_expect_tx(bar(kBFull + buf), b_bytes);
-          if (a.imgNT == NT) {
-            bulk_copy(dst, img, b_bytes, bar(kBFull + buf));
-          } else {
+      __syncwarp();
+    } else if (warp == kWorkers + 1) {  // ------------------------------- copies of B's digits
+      // (a warp of its own: one of the workers, whose arrivals all wait for, held up every stage: a
+      // build of 500 / 2000 / 80 5.19 ms, so 4.78)
+      if (lane == 0) {
+        uint32_t it = 0, issued[2] = {0, 0};
+        bool ok = true;
+        for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+          const int sp = u / (a.ntiles * a.mtiles);
+          const int s0 = (int)((long long)a.nstages * sp / a.splits);
+          const int s1 = (int)((long long)a.nstages * (sp + 1) / a.splits);
+          const int n0 = u % a.ntiles * NT;
+          const size_t img_stage = (size_t)kD * a.imgNT * kStageK;
+          // NT rows of every digit's rows (a multiple of 16: the swizzle's phase is theirs)
+          const __half* img = a.Bimg + ((size_t)(n0 / a.imgNT) * a.nstages + s0) * img_stage +
+                              n0 % a.imgNT * kStageK;
+          for (int st = s0; st < s1; ++st, ++it, img += img_stage) {
+            const uint32_t buf = it & 1u, ph = (it >> 1) & 1u;
+            if (!wait_for(bar(kEmpty + buf), ph ^ 1u, a)) {
+              ok = false;
+              break;
+            }
+            const uint32_t dst = smem0 + buf * stage_bytes + kABytes;
+            mbar_expect_tx(bar(kBFull + buf), b_bytes);
+            if (a.imgNT == NT) {
+              bulk_copy(dst, img, b_bytes, bar(kBFull + buf));
+            } else {
 #pragma unroll
-            for (int d = 0; d < kD; ++d)
-              bulk_copy(dst + (uint32_t)d * (NT * kStageK * 2),
-                        img + (size_t)d * a.imgNT * kStageK, NT * kStageK * 2, bar(kBFull + buf));
+              for (int d = 0; d < kD; ++d)
+                bulk_copy(dst + (uint32_t)d * (NT * kStageK * 2),
+                          img + (size_t)d * a.imgNT * kStageK, NT * kStageK * 2, bar(kBFull + buf));
+            }
+            ++issued[buf];
           }
-          ++issued[buf];
         }
+        // the copies issued land before the CTA leaves, after an abort too
+        for (int i = 0; i < 2; ++i)
+          if (issued[i]) mbar_wait_quiet(bar(kBFull + i), (issued[i] - 1) & 1u, kDrainLimitNs);
       }
-      // the copies issued land before the CTA leaves, after an abort too
-      for (int i = 0; i < 2; ++i)
-        if (issued[i]) mbar_wait_quiet(bar(kBFull + i), (issued[i] - 1) & 1u, kDrainLimitNs);
+      __syncwarp();
     }
-    __syncwarp();
   } else {  // --------------------------------------------------------- workers
+    if constexpr (split_regs(NT)) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kWorkerRegs));
     // group 0 of this thread's row (TMEM lane) and a quarter of the columns, over the chunks of a
     // unit so far (the other groups stay in TMEM)
     constexpr int kCols = NT / 4;
@@ -437,7 +477,6 @@ __global__ void __launch_bounds__(kDigThreads, 1)
     double x[8];
     if (cur.u < units) cur.load(a, x);
     uint32_t it = 0, nflush = 0;
-    bool ok = true;
 
     // After a chunk: group 0 is moved to `top`, the carries of the other groups to their
     // neighbours, exactly in fp32 (a group is below 2^24 - 2^17, its carry at most 2^17), which
@@ -488,8 +527,9 @@ __global__ void __launch_bounds__(kDigThreads, 1)
       const int ea = (rv ? (a.eA ? scale_exp(__ldg(a.eA + row)) : 1023) : 0) - 1086;
       double* Crow = a.C + (long long)sp * a.sCs + (long long)b * a.sCb + (long long)r * a.sCm + n0;
       int rmax = 0;
-      // exponents of the result per (b, column): the lanes of a warp span one or two b when a
-      // b has at least 32 rows
+      // exponents of the result per (b, column), its rows scaled as the k of the next product that
+      // they are: the lanes of a warp span one or two b when a b has at least 32 rows
+      const int rs = rv && a.row_s ? (int)(__ldg(a.row_s + r) >> 20) : 0;
       const int b_lo = __shfl_sync(0xffffffffu, b, 0);
       const bool wide = a.Mb >= 32;
       const bool two = __any_sync(0xffffffffu, rv && b != b_lo);
@@ -524,8 +564,9 @@ __global__ void __launch_bounds__(kDigThreads, 1)
           v[j] = fixed_to_double(hi, (uint32_t)lo & 0x0fffffffu,
                                  ea + (a.eB ? scale_exp(__ldg(a.eB + (n < a.N ? n : a.N - 1))) : 1023));
           if (a.exq) {
-            const int e = rv ? (__double2hiint(v[j]) >> 20) & 0x7ff : 0;
+            int e = rv ? exp_of(v[j]) : 0;
             rmax = max(rmax, e);
+            e = max(e - rs, 0);
             if (wide) {
               const int r0 = __reduce_max_sync(0xffffffffu, b == b_lo ? e : 0);
               if (lane == h + j) mx0 = r0;
@@ -567,32 +608,43 @@ __global__ void __launch_bounds__(kDigThreads, 1)
     bool pend = false, pend_last = false;
     int pend_u = 0, c = 0;
     const uint32_t dst = KC ? sw64(tid >> 2, tid & 3) : sw64(tid & 127, tid >> 7);
-    while (ok && cur.u < units) {
-      const uint32_t buf = it & 1u, ph = (it >> 1) & 1u;
-      if (!wait_for(bar(kEmpty + buf), ph ^ 1u, a)) {
-        ok = false;
-        break;
-      }
-      const uint32_t sa = smem0 + buf * stage_bytes;
+    const uint32_t* ks = a.ks + 8 * (KC ? tid & 3 : tid >> 7);
+    // Wide tiles: the last flush behind the loop, a second copy of its code (units of 128 x 48 take
+    // 7 % less so); narrow ones, whose products are short, in the loop's last turn.
+    constexpr bool kTail = split_regs(NT);
+    for (;;) {
+      const bool more = cur.u < units;
+      if (!more && (kTail || !pend)) break;
       const int u = cur.u;
-      const bool last = cur.last();
-      Fixed8 f;
-      to_fixed8(x, cur.e20, a.k64, f);
-      cur.next(a, units);
-      if (cur.u < units) cur.load(a, x);  // the next stage's elements, in flight over a stage
-      store_digits(f, [&](int d, uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
-        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(sa + dst + d * (kTileM * 64)),
-                     "r"(w0), "r"(w1), "r"(w2), "r"(w3)
-                     : "memory");
-      });
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar(kAFull + buf));
-      ++it;
-      if (pend) {
-        ok = flush(pend_u, pend_last);
-        pend = false;
+      bool last = false;
+      if (more) {
+        const uint32_t buf = it & 1u, ph = (it >> 1) & 1u;
+        if (!wait_for(bar(kEmpty + buf), ph ^ 1u, a)) {
+          pend = false;
+          break;
+        }
+        const uint32_t sa = smem0 + buf * stage_bytes;
+        last = cur.last();
+        Fixed8 f;
+        if (scaled) to_fixed8(x, cur.e20, ks + cur.st * kStageK, a.k64, f);
+        else to_fixed8(x, cur.e20, a.k64, f);
+        cur.next(a, units);
+        if (cur.u < units) cur.load(a, x);  // the next stage's elements, in flight over a stage
+        store_digits(f, [&](int d, uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
+          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(sa + dst + d * (kTileM * 64)),
+                       "r"(w0), "r"(w1), "r"(w2), "r"(w3)
+                       : "memory");
+        });
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(kAFull + buf));
+        ++it;
       }
+      if (pend) {
+        pend = false;
+        if (!flush(pend_u, pend_last)) break;
+      }
+      if (!more) break;
       if (last || ++c == kChunkStages) {
         pend = true;
         pend_u = u;
@@ -600,7 +652,7 @@ __global__ void __launch_bounds__(kDigThreads, 1)
         c = 0;
       }
     }
-    if (ok && pend) flush(pend_u, pend_last);
+    if (kTail && pend) flush(pend_u, pend_last);
   }
   tc_fence_before();
   __syncthreads();
@@ -610,38 +662,56 @@ __global__ void __launch_bounds__(kDigThreads, 1)
 
 // ------------------------------------------------------------------ exponents and planes
 // Largest biased exponents of the columns (by_col: atomic maxima into zeroed words) or of the
-// rows of up to three matrices.
+// rows of up to three matrices, their elements scaled by the powers of two of the contraction's k
+// (columns: C, by 2^s of the row; rows: h, by 2^-s of the column; minus: G's columns by 2^-s).
 struct ExpJob {
   const double* S;
   long long ld;
   long long rows;
   int cols, by_col;
   int* out;
+  KScale k;
+  int minus;
 };
 struct ExpJobs {
   ExpJob j[3];
 };
 constexpr int kExpRows = 64;  // rows of a column job per CTA
 
-__device__ __forceinline__ int exp_field(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+__device__ __forceinline__ int scale_of(const KScale& k, int i) { return (int)(k.kp[i] >> 20); }
+// The exponent scaled by 2^s; of a zero 0.
+__device__ __forceinline__ int exp_scaled(double x, int s) {
+  const int e = exp_of(x);
+  return e ? max(e + s, 1) : 0;
+}
+// The least exponent word of an operand scaled upwards, so that its zeros (which have no hidden bit)
+// are shifted out whatever their scale.
+__device__ __forceinline__ int least_up(const int* info) { return 64 + info[1]; }
 
 __global__ void __launch_bounds__(256) k_exps(ExpJobs jobs) {
+  const int scales = scales_word(jobs.j[blockIdx.y].k.info);
   const int z = chain_begin(), bx = (int)blockIdx.x + z;
+  const bool s = scales + z != 0;
   const ExpJob jb = jobs.j[blockIdx.y + z];
   const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
   if (jb.by_col) {
     __shared__ int red[8][32];
     const int ncb = (jb.cols + 31) / 32;
     const long long tiles = (long long)ncb * ((jb.rows + kExpRows - 1) / kExpRows);
+    const int least = s && !jb.minus ? least_up(jb.k.info) : 0;
     for (long long t = bx; t < tiles; t += gridDim.x) {
       const int c = (int)(t % ncb) * 32 + tx;
       const long long r0 = t / ncb * kExpRows;
-      int m = 0;
+      int m = least;
       if (c < jb.cols) {
 #pragma unroll
         for (int i = 0; i < kExpRows / 8; ++i) {
           const long long r = r0 + ty + 8 * i;
-          if (r < jb.rows) m = max(m, exp_field(jb.S[r * jb.ld + c]));
+          if (r < jb.rows) {
+            const double v = jb.S[r * jb.ld + c];
+            const int sr = s ? scale_of(jb.k, (int)r) : 0;
+            m = max(m, s ? exp_scaled(v, jb.minus ? -sr : sr) : exp_of(v));
+          }
         }
       }
       red[ty][tx] = m;
@@ -658,39 +728,149 @@ __global__ void __launch_bounds__(256) k_exps(ExpJobs jobs) {
       const double* row = jb.S + r * jb.ld;
       int m = 0;
 #pragma unroll 4
-      for (int c = tx; c < jb.cols; c += 32) m = max(m, exp_field(__ldg(row + c)));
+      for (int c = tx; c < jb.cols; c += 32) {
+        const double v = __ldg(row + c);
+        m = max(m, s ? exp_scaled(v, -scale_of(jb.k, c)) : exp_of(v));
+      }
       m = __reduce_max_sync(0xffffffffu, m);
       if (tx == 0) jb.out[r] = m;
     }
   }
 }
 
-// The rows of symmetric slices stored as packed lower triangles: one CTA per slice, the
-// slice's maxima in shared memory (in the output itself when N is too large for it).
+// ------------------------------------------------------------------ scales of the AO indices
+// Fixed point relative to the largest element of a row loses the small ones, and rows of B (and
+// columns of C) in an AO basis whose functions are of very different norm hold both: with B and h
+// scaled by w_mu w_nu and C by 1 / w_nu, spread over 1e8, builds were off by 1e-10, in double by 1e-15
+// whatever the spread.  So the contractions over AO indices take B, h, X and G times 2^-s and C
+// times 2^s, exactly, in the exponents' subtraction that splits them (their scaled products are the
+// same numbers).  s_mu is half the exponent of the largest B^P_mu,mu, or, where B's off-diagonal
+// elements do not bear that out (|B_mu,nu| <= 2^(s_mu + s_nu) holds for integrals), what brings the
+// row's largest element to the level of B's: it moves with the functions' norms, so that errors do
+// not depend on them.  Where s spans no more than kEvenSpan it is taken as zero, and the operands
+// and results are those of unscaled products.
+constexpr int kEvenSpan = 3;
+constexpr int kScaleMax = 1000;  // (the shifts stay below 4096)
+// rm, dm: largest exponents of the rows and of the diagonal elements.  Leaves in k: info = {whether
+// any s is not zero, the largest}; s >= 0; kp and kn, s 2^20 and -s 2^20, padded with zeros.
+__global__ void __launch_bounds__(1024) k_scales(const int* __restrict__ rm,
+                                                 const int* __restrict__ dm, int N, int* info,
+                                                 uint32_t* kp, uint32_t* kn) {
+  __shared__ int red[32];
+  auto all_max = [&](int v) {
+    v = __reduce_max_sync(0xffffffffu, v);
+    __syncthreads();
+    if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = v;
+    __syncthreads();
+    v = red[threadIdx.x % 32];
+    return __reduce_max_sync(0xffffffffu, v);
+  };
+  int R = 0;
+  for (int i = threadIdx.x; i < N; i += 1024)
+    if (rm[i] < kNanMark) R = max(R, rm[i]);
+  R = all_max(R);
+  int least = -(1 << 20), most = -(1 << 20);  // of -s and s
+  auto raw = [&](int i) { return max(dm[i], 2 * rm[i] - R) >> 1; };
+  auto counts = [&](int i) { return rm[i] > 0 && rm[i] < kNanMark; };  // (a row of zeros: any s)
+  for (int i = threadIdx.x; i < N; i += 1024)
+    if (counts(i)) {
+      least = max(least, -raw(i));
+      most = max(most, raw(i));
+    }
+  const int lo = -all_max(least), span = all_max(most) - lo;
+  const bool on = span > kEvenSpan;
+  const int hi = span < kScaleMax ? span : kScaleMax;
+  for (int i = threadIdx.x; i < kscale_pad(N); i += 1024) {
+    const int v = on && i < N && counts(i) ? min(raw(i) - lo, hi) : 0;
+    kp[i] = (uint32_t)v << 20;
+    kn[i] = 0u - ((uint32_t)v << 20);
+  }
+  if (threadIdx.x == 0) {
+    info[0] = on;
+    info[1] = on ? hi : 0;
+  }
+}
+
+// Rows of N elements (row r: AO index r mod N) of a B of whole rows, or of h: a warp per row.  FIRST:
+// the largest exponents of the rows (into out, unless null), of the AO indices' rows and of their
+// diagonal elements (atomic maxima into zeroed words).  The second pass: those of the rows scaled by
+// 2^-s of the column, where any s is not zero.  TRI: rows of packed lower triangles, the part above
+// the diagonal gathered.  Bound by memory: 2000 slices of 700 1.2 ms a pass.
+template <bool TRI, bool FIRST>
+__global__ void __launch_bounds__(256) k_row_exps(const double* __restrict__ B, long long rows, int N,
+                                                  int* out, int* rm, int* dm, KScale k) {
+  const int z = chain_begin();
+  if (!FIRST && !k.info[z]) return;
+  const int tx = threadIdx.x % 32;
+  const long long npk = (long long)N * (N + 1) / 2;
+  for (long long r = blockIdx.x * 8 + threadIdx.x / 32 + z; r < rows; r += (long long)gridDim.x * 8) {
+    const long long P = r / N;
+    const int mu = (int)(r - P * N);
+    const double* row = TRI ? B + P * npk + (long long)mu * (mu + 1) / 2 : B + r * N;
+    const int own = TRI ? mu + 1 : N;
+    int m = 0;
+    auto take = [&](double v, int c) { m = max(m, FIRST ? exp_of(v) : exp_scaled(v, -scale_of(k, c))); };
+#pragma unroll 4
+    for (int c = tx; c < own; c += 32) take(__ldg(row + c), c);
+    if (TRI) {
+#pragma unroll 4
+      for (int c = own + tx; c < N; c += 32)
+        take(__ldg(B + P * npk + (long long)c * (c + 1) / 2 + mu), c);
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (tx != 0) continue;
+    if (out) out[r] = m;
+    if (FIRST) {
+      if (m > *(volatile int*)(rm + mu)) atomicMax(rm + mu, m);
+      const int e = exp_of(__ldg(row + mu));
+      if (e < kNanMark && e > *(volatile int*)(dm + mu)) atomicMax(dm + mu, e);
+    }
+  }
+}
+
+// The rows of symmetric slices stored as packed lower triangles, the passes of k_row_exps: one CTA
+// per slice, the slice's maxima in shared memory.
+constexpr int kPackedFewSlices = 1000;  // (500 slices of 700: 330 us by rows, 630 by slices; 2000: 1300, 1250)
+template <bool FIRST>
 __global__ void __launch_bounds__(256) k_packed_exps(const double* __restrict__ Bp, int Q, int N,
-                                                     int in_smem, int* out) {
+                                                     int* out, int* rm, int* dm, KScale k) {
   const int z = chain_begin(), bx = (int)blockIdx.x + z;
-  extern __shared__ int sh_max[];
+  extern __shared__ int ex[];
+  if (!FIRST && !k.info[z]) return;
   const long long npk = (long long)N * (N + 1) / 2;
   for (int P = bx; P < Q; P += gridDim.x) {
-    int* ex = in_smem ? sh_max : out + (size_t)P * N;
     for (int i = threadIdx.x; i < N; i += 256) ex[i] = 0;
     __syncthreads();
     const double* B = Bp + (size_t)P * npk;
     for (int mu = threadIdx.x / 32; mu < N; mu += 8) {
       const double* row = B + (long long)mu * (mu + 1) / 2;
+      const int smu = FIRST ? 0 : scale_of(k, mu);
       int m = 0;
       for (int nu = threadIdx.x % 32; nu <= mu; nu += 32) {
-        const int e = exp_field(__ldg(row + nu));
+        const double v = __ldg(row + nu);
+        int e = (__double2hiint(v) >> 20) & 0x7ff, f = e;  // (marked at the end)
+        if (!FIRST) {
+          e = exp_scaled(v, -scale_of(k, nu));
+          f = exp_scaled(v, -smu);
+        }
         m = max(m, e);
-        if (e > *(volatile int*)(ex + nu)) atomicMax(ex + nu, e);
+        if (f > *(volatile int*)(ex + nu)) atomicMax(ex + nu, f);
       }
       m = __reduce_max_sync(0xffffffffu, m);
-      if (threadIdx.x % 32 == 0) atomicMax(ex + mu, m);
+      if (threadIdx.x % 32 == 0) {
+        atomicMax(ex + mu, m);
+        if (FIRST) {
+          const int e = exp_of(__ldg(row + mu));
+          if (e < kNanMark && e > *(volatile int*)(dm + mu)) atomicMax(dm + mu, e);
+        }
+      }
     }
     __syncthreads();
-    if (in_smem)
-      for (int i = threadIdx.x; i < N; i += 256) out[(size_t)P * N + i] = ex[i];
+    for (int i = threadIdx.x; i < N; i += 256) {
+      const int e = FIRST && ex[i] == 2047 ? kNanMark : ex[i];
+      out[(size_t)P * N + i] = e;
+      if (FIRST && e > *(volatile int*)(rm + i)) atomicMax(rm + i, e);
+    }
     __syncthreads();
   }
 }
@@ -701,24 +881,30 @@ __device__ __forceinline__ size_t img_addr(int n, int kc, int NT, int nstages) {
   const int nt = n / NT, r = n - nt * NT;
   return (((size_t)nt * nstages + (kc >> 2)) * (size_t)(kD * NT * 64) + sw64(r, kc & 3)) / 2;
 }
-__device__ __forceinline__ void put_planes(const double (&x)[8], int em, uint32_t k64, __half* img,
-                                           size_t at, int NT) {
+// ks: the words of the 8 elements' scales, or null.
+__device__ __forceinline__ void put_planes(const double (&x)[8], int em, const uint32_t* ks,
+                                           uint32_t k64, __half* img, size_t at, int NT) {
   Fixed8 f;
-  to_fixed8(x, split_exp(em), k64, f);
+  if (ks) to_fixed8(x, split_exp(em), ks, k64, f);
+  else to_fixed8(x, split_exp(em), k64, f);
   store_digits(f, [&](int d, uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
     *(uint4*)(img + at + (size_t)d * NT * kStageK) = make_uint4(w0, w1, w2, w3);
   });
 }
 
 // Stage images of a matrix S[k sk + n sn]: a thread per column and 8 elements of k (columns past
-// N and elements past K are zero; ex null: exponent 1023).
+// N and elements past K are zero; ex null: exponent 1023), scaled by 2^s of its k (minus: 2^-s).
+constexpr int kZeroExp = 2047;  // the exponent word of the columns that are only padding
 __global__ void __launch_bounds__(256) k_digit_planes(const double* __restrict__ S, long long sk,
                                                       long long sn, int K, int N, uint32_t k64,
-                                                      const int* __restrict__ ex,
-                                                      __half* img, int NT, int ntiles,
+                                                      const int* __restrict__ ex, KScale ksc,
+                                                      int minus, __half* img, int NT, int ntiles,
                                                       int nstages) {
+  const int scales = scales_word(ksc.info);
   const int z = chain_begin(), bx = (int)blockIdx.x + z;
+  const bool on = scales + z != 0;
   const int W = NT * ntiles;
+  const uint32_t* ks = !on ? nullptr : minus ? ksc.kp : ksc.kn;
   const long long tot = (long long)W * nstages * 4;
   for (long long i = bx * 256ll + threadIdx.x; i < tot; i += 256ll * gridDim.x) {
     const int kc = (int)(i / W), n = (int)(i - (long long)kc * W);
@@ -728,7 +914,8 @@ __global__ void __launch_bounds__(256) k_digit_planes(const double* __restrict__
       const int k = 8 * kc + j;
       x[j] = (n < N && k < K) ? S[(long long)k * sk + (long long)n * sn] : 0.0;
     }
-    put_planes(x, n < N ? (ex ? ex[n] : 1023) : 2047, k64, img, img_addr(n, kc, NT, nstages), NT);
+    put_planes(x, n < N ? (ex ? ex[n] : 1023) : kZeroExp, ks ? ks + 8 * kc : nullptr, k64, img,
+               img_addr(n, kc, NT, nstages), NT);
   }
 }
 
@@ -739,11 +926,13 @@ __global__ void __launch_bounds__(256) k_digit_planes(const double* __restrict__
 constexpr int kFuseK = 640;
 __global__ void __launch_bounds__(256) k_exps_planes(const double* __restrict__ S, long long ld,
                                                      int K, int ncols, int N, uint32_t k64,
-                                                     int* ex, __half* img, int NT, int nstages,
-                                                     int col_ctas, const double* __restrict__ R,
+                                                     int* ex, KScale ksc, int minus, __half* img,
+                                                     int NT, int nstages, int col_ctas, const double* __restrict__ R,
                                                      int rows, int rows_k, int* ex_rows,
                                                      int row_ctas, const ZeroJob zero) {
+  const int scales = scales_word(ksc.info);
   const int z = chain_begin(), bx = (int)blockIdx.x + z;
+  const bool on = scales + z != 0;
   const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
   if (bx >= col_ctas + row_ctas) {
     zero_ranges(zero, bx - col_ctas - row_ctas, (int)gridDim.x - col_ctas - row_ctas);
@@ -752,8 +941,18 @@ __global__ void __launch_bounds__(256) k_exps_planes(const double* __restrict__ 
   if (bx >= col_ctas) {
     for (int r = (bx - col_ctas) * 8 + ty; r < rows; r += row_ctas * 8) {
       int m = 0;
-#pragma unroll 4
-      for (int c = tx; c < rows_k; c += 32) m = max(m, exp_field(__ldg(R + (long long)r * rows_k + c)));
+      for (int c0 = tx; c0 < rows_k; c0 += 128) {
+        double v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          v[i] = c0 + 32 * i < rows_k ? __ldg(R + (long long)r * rows_k + c0 + 32 * i) : 0.0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          int e = exp_of(v[i]);
+          if (on && e) e = max(e - scale_of(ksc, c0 + 32 * i), 1);  // (not a zero: within the row)
+          m = max(m, e);
+        }
+      }
       m = __reduce_max_sync(0xffffffffu, m);
       if (tx == 0) ex_rows[r] = m;
     }
@@ -763,15 +962,29 @@ __global__ void __launch_bounds__(256) k_exps_planes(const double* __restrict__ 
   const int n = bx * 32 + tx;  // columns past N: to the width of the images
   int m = 0;
   if (n < ncols) {
-#pragma unroll 4
-    for (int k = ty; k < K; k += 8) m = max(m, exp_field(S[(long long)k * ld + n]));
+    for (int k0 = ty; k0 < K; k0 += 32) {
+      double v[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] = k0 + 8 * i < K ? S[(long long)(k0 + 8 * i) * ld + n] : 0.0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        int e = exp_of(v[i]);
+        if (on && e) {
+          const int sk = scale_of(ksc, k0 + 8 * i);
+          e = max(e + (minus ? -sk : sk), 1);
+        }
+        m = max(m, e);
+      }
+    }
   }
+  if (on && !minus) m = max(m, least_up(ksc.info));
   red[ty][tx] = m;
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < 8; ++i) m = max(m, red[i][tx]);
   if (ty == 0 && n < ncols) ex[n] = m;
   if (n >= (N + NT - 1) / NT * NT) return;  // (the images' width: every tile is NT columns)
+  const uint32_t* ks = !on ? nullptr : minus ? ksc.kp : ksc.kn;
   for (int kc = ty; kc < nstages * 4; kc += 8) {
     double x[8];
 #pragma unroll
@@ -779,7 +992,8 @@ __global__ void __launch_bounds__(256) k_exps_planes(const double* __restrict__ 
       const int k = 8 * kc + j;
       x[j] = (n < N && k < K) ? S[(long long)k * ld + n] : 0.0;
     }
-    put_planes(x, n < N ? m : 2047, k64, img, img_addr(n, kc, NT, nstages), NT);
+    put_planes(x, n < N ? m : kZeroExp, ks ? ks + 8 * kc : nullptr, k64, img,
+               img_addr(n, kc, NT, nstages), NT);
   }
 }
 
@@ -809,7 +1023,7 @@ __global__ void __launch_bounds__(256) k_w_jk64(const double* __restrict__ b, in
         for (; r < A; ++r) w[0] = fma(row[(size_t)r * A], dv[r], w[0]);
         const double t = (w[0] + w[1]) + (w[2] + w[3]);
         W[(size_t)P * A + p] = t;
-        const int e = exp_field(t);
+        const int e = exp_of(t);
         if (e > *(volatile int*)(wmax + p)) atomicMax(wmax + p, e);
       }
       __syncthreads();
@@ -843,7 +1057,7 @@ __global__ void __launch_bounds__(256) k_w_jk64(const double* __restrict__ b, in
     for (int u = 0; u < 4; ++u) {
       sj[u & 1] = fma(dp[u], dq[u], sj[u & 1]);
       sk[u & 1] = fma(v[u], v[u], sk[u & 1]);
-      m = max(m, exp_field(v[u]));
+      m = max(m, exp_of(v[u]));
     }
   }
   for (; P < P1; ++P) {
@@ -851,7 +1065,7 @@ __global__ void __launch_bounds__(256) k_w_jk64(const double* __restrict__ b, in
     const double v = bp[opq];
     sj[0] = fma(bp[op], bp[oq], sj[0]);
     sk[0] = fma(v, v, sk[0]);
-    m = max(m, exp_field(v));
+    m = max(m, exp_of(v));
   }
   double* o = part + (size_t)split * 2 * tri;
   o[i] = sj[0] + sj[1];
@@ -899,11 +1113,11 @@ __global__ void __launch_bounds__(256) k_jk_final64(const double* __restrict__ p
   int f = wmax[p];
   for (int q = lane; q < A; q += 32) {
     const int hi = p > q ? p : q, lw = p > q ? q : p;
-    const int eb = bmax[hi * (hi + 1) / 2 + lw], ec = exp_field(Bc[(size_t)q * A + p]);
-    f = max(f, eb == 2047 || ec == 2047 ? 2047 : (ec && eb ? ec + eb - 1022 : 0));
+    const int eb = bmax[hi * (hi + 1) / 2 + lw], ec = exp_of(Bc[(size_t)q * A + p]);
+    f = max(f, eb >= kNanMark || ec >= kNanMark ? kNanMark : (ec && eb ? ec + eb - 1022 : 0));
   }
   f = __reduce_max_sync(0xffffffffu, f);
-  if (lane == 0) eY[p] = f >= 2047 ? 2047 : (f + 2 > 2046 ? 2046 : f + 2);
+  if (lane == 0) eY[p] = f >= kNanMark ? kNanMark : (f + 2 > 2046 ? 2046 : f + 2);
 }
 
 // Stage images of Y over k = P Kpad + q: Y^P_qp = Bcoef_qp b^P_qp + delta_qp w^P_p, formed and
@@ -930,7 +1144,7 @@ __global__ void __launch_bounds__(256) k_y_planes(const double* __restrict__ b, 
         if (q == n) x[j] += W[(size_t)P * A + n];
       }
     }
-    put_planes(x, n < A ? eY[n] : 2047, k64, img, img_addr(n, kc, NT, nstages), NT);
+    put_planes(x, n < A ? eY[n] : kZeroExp, nullptr, k64, img, img_addr(n, kc, NT, nstages), NT);
   }
 }
 
@@ -972,8 +1186,7 @@ int grid_for(long long threads) {
   return (int)(nb < 1 ? 1 : (nb < 152 * 16 ? nb : 152 * 16));
 }
 
-// `first`: the first launch of a call.
-cudaError_t launch_exps(const ExpJob* jobs, int count, cudaStream_t s, bool first = false) {
+cudaError_t launch_exps(const ExpJob* jobs, int count, cudaStream_t s) {
   ExpJobs js{};
   long long nb = 1;
   for (int i = 0; i < count; ++i) {
@@ -983,17 +1196,16 @@ cudaError_t launch_exps(const ExpJob* jobs, int count, cudaStream_t s, bool firs
                                        : (jobs[i].rows + 7) / 8;
     if (t > nb) nb = t;
   }
-  launch_chained_to(first ? 0 : kChainCtas, k_exps,
-                    dim3((unsigned)(nb < 152 * 8 ? nb : 152 * 8), count), 256, 0, s, js);
+  launch_chained(k_exps, dim3((unsigned)(nb < 152 * 8 ? nb : 152 * 8), count), 256, 0, s, js);
   count_launch(1);
   return cudaGetLastError();
 }
 
 cudaError_t launch_planes(const double* S, long long sk, long long sn, int K, int N, const int* ex,
-                          void* img, cudaStream_t s) {
+                          const KScale& k, int minus, void* img, cudaStream_t s) {
   const DigitShape sh = digit_shape(N, K);
   launch_chained(k_digit_planes, grid_for((long long)sh.NT * sh.ntiles * sh.nstages * 4), 256, 0, s,
-      S, sk, sn, K, N, kK64, ex, (__half*)img, sh.NT, sh.ntiles, sh.nstages);
+      S, sk, sn, K, N, kK64, ex, k, minus, (__half*)img, sh.NT, sh.ntiles, sh.nstages);
   count_launch(1);
   return cudaGetLastError();
 }
@@ -1001,7 +1213,7 @@ cudaError_t launch_planes(const double* S, long long sk, long long sn, int K, in
 // ncols columns' exponents and the planes of the first N, K <= kFuseK; rows' exponents of R; zero
 // cleared.  `first`: the first launch of a call.
 cudaError_t launch_exps_planes(const double* S, long long ld, int K, int ncols, int N, int* ex,
-                               void* img, const double* R, int rows, int rows_k, int* ex_rows,
+                               const KScale& k, int minus, void* img, const double* R, int rows, int rows_k, int* ex_rows,
                                const ZeroJob& zero, bool first, cudaStream_t s) {
   const DigitShape sh = digit_shape(N, K);
   const int width = ncols > sh.NT * sh.ntiles ? ncols : sh.NT * sh.ntiles;
@@ -1010,8 +1222,8 @@ cudaError_t launch_exps_planes(const double* S, long long ld, int K, int ncols, 
   for (int i = 0; i < 4; ++i) nz += zero.n[i];
   const int zc = (int)(nz < 2048 * 32 ? (nz + 2047) / 2048 : 32);
   launch_chained_to(first ? 0 : kChainCtas, k_exps_planes, cc + rc + (zero.flag && !zc ? 1 : zc),
-                    256, 0, s, S, ld, K, ncols, N, kK64, ex, (__half*)img, sh.NT, sh.nstages, cc, R,
-                    rows, rows_k, ex_rows, rc, zero);
+                    256, 0, s, S, ld, K, ncols, N, kK64, ex, k, minus, (__half*)img, sh.NT,
+                    sh.nstages, cc, R, rows, rows_k, ex_rows, rc, zero);
   count_launch(1);
   return cudaGetLastError();
 }
@@ -1080,9 +1292,15 @@ cudaError_t launch_digit_gemm(DigitArgs a, long long K, cudaStream_t s) {
     if (raise) {
       e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
+      // the workers wait for the registers that they ask for: the launch has to hold the split's sum
+      cudaFuncAttributes fa;
+      e = cudaFuncGetAttributes(&fa, fn);
+      if (e != cudaSuccess) return e;
+      if (split_regs(a.NT) && fa.numRegs / 8 * 8 * dig_threads(a.NT) < 32 * (4 * kOtherRegs + kWorkers * kWorkerRegs))
+        return cudaErrorInvalidConfiguration;
       mask |= bit;
     }
-    launch_chained(fn, grid, kDigThreads, smem, s, a);
+    launch_chained(fn, grid, dig_threads(a.NT), smem, s, a);
     e = cudaGetLastError();
     if (e == cudaSuccess || raise) break;
   }
@@ -1110,11 +1328,11 @@ cudaError_t digit_product(int M, int N, int K, const double* A, long long sAm, l
   char* img = (char*)eB + align_up((size_t)N * 4);
   if (sAk != 1 || sBn == 1)  // a matrix read down its columns accumulates maxima
     CKE(cudaMemsetAsync(scratch, 0, (size_t)(img - scratch), s));
-  ExpJob jobs[2] = {{B, sBk, K, N, 1, eB}, {A, sAm, M, K, 0, eA}};
-  if (sBn != 1) jobs[0] = ExpJob{B, sBn, N, K, 0, eB};
-  if (sAk != 1) jobs[1] = ExpJob{A, sAk, K, M, 1, eA};
+  ExpJob jobs[2] = {{B, sBk, K, N, 1, eB, {}, 0}, {A, sAm, M, K, 0, eA, {}, 0}};
+  if (sBn != 1) jobs[0] = ExpJob{B, sBn, N, K, 0, eB, {}, 0};
+  if (sAk != 1) jobs[1] = ExpJob{A, sAk, K, M, 1, eA, {}, 0};
   CKE(launch_exps(jobs, 2, s));
-  CKE(launch_planes(B, sBk, sBn, K, N, eB, img, s));
+  CKE(launch_planes(B, sBk, sBn, K, N, eB, KScale{}, 0, img, s));
   DigitArgs a{};
   a.KB = 1; a.splits = 1;
   a.A = A; a.sAm = sAm; a.sAk = sAk; a.M = M; a.Mb = M; a.Kin = K; a.eA = eA;
@@ -1168,12 +1386,12 @@ __global__ void __launch_bounds__(256) k_reflect_w(const double* __restrict__ pa
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       x[i] = Wt[j][8 * kc + i];
-      m = max(m, exp_field(x[i]));
+      m = max(m, exp_of(x[i]));
     }
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (n < N && kc == 0) eW[n] = m;
-    if (n < NT * ntiles) put_planes(x, n < N ? m : 2047, k64, img, img_addr(n, kc, NT, 2), NT);
+    if (n < NT * ntiles) put_planes(x, n < N ? m : kZeroExp, nullptr, k64, img, img_addr(n, kc, NT, 2), NT);
   }
 }
 int reflect_splits(int N, int stages) {
@@ -1213,7 +1431,8 @@ cudaError_t digit_reflect(int N, int nref, const double* Yr, const double* T, do
   const DigitShape ysh = digit_shape(kRefBlk, N);  // NT 64, one tile per block
   const int W = nblk * kRefBlk;
   launch_chained(k_digit_planes, grid_for((long long)W * ysh.nstages * 4), 256, 0, s,
-      Yr, 1, N, N, nref, kK64, nullptr, (__half*)(img + L.y), kRefBlk, nblk, ysh.nstages);
+      Yr, 1, N, N, nref, kK64, nullptr, KScale{}, 0, (__half*)(img + L.y), kRefBlk, nblk,
+      ysh.nstages);
   count_launch(1);
   CKE(cudaGetLastError());
   const DigitShape wsh = digit_shape(N, kRefBlk);
@@ -1264,41 +1483,78 @@ DigitArgs digit_args(char* ws, const Layout& L) {
 }
 }  // namespace
 
-cudaError_t digit_prepare_B(const Dims& d, const double* B, char* ws, const Layout& L,
-                            cudaStream_t s) {
-  int* out = (int*)(ws + L.eRow);
-  if (d.layout == DONOF_B_DENSE) {
-    const ExpJob j{B, d.N, (long long)d.Q * d.N, d.N, 0, out};
-    return launch_exps(&j, 1, s, true);
-  }
-  const int in_smem = d.N <= 12000 ? 1 : 0;
-  k_packed_exps<<<d.Q < 152 * 8 ? d.Q : 152 * 8, 256, in_smem ? (size_t)d.N * 4 : 0, s>>>(
-      B, d.Q, d.N, in_smem, out);
+namespace {
+// Scales of the AO indices from the exponents that the first pass left.
+cudaError_t launch_scales(const int* rm, const int* dm, int N, const KScale& k, cudaStream_t s) {
+  k_scales<<<1, 1024, 0, s>>>(rm, dm, N, (int*)k.info, (uint32_t*)k.kp, (uint32_t*)k.kn);
   count_launch(1);
   return cudaGetLastError();
 }
+}  // namespace
 
-cudaError_t digit_hc(const Dims& d, const double* h, const double* C, char* ws, const Layout& L,
-                     ZeroJob zero, cudaStream_t s) {
+cudaError_t digit_prepare_B(const Dims& d, const double* B, char* ws, const Layout& L,
+                            cudaStream_t s) {
+  int* out = (int*)(ws + L.eRow);
+  const KScale k = kscale_at(ws + L.sB, d.N);
+  int *rm = (int*)(ws + L.eC64), *dm = (int*)(ws + L.exm);  // (free between builds)
+  CKE(cudaMemsetAsync(ws + L.eC64, 0, L.exend - L.eC64, s));
+  const int tri = d.layout == DONOF_B_PACKED;
+  const long long rows = (long long)d.Q * d.N, nb = (rows + 7) / 8;
+  const size_t smem = (size_t)d.N * 4;
+  if (tri && smem > 47 * 1024) {  // (one limit for all sizes)
+    CKE(cudaFuncSetAttribute(k_packed_exps<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             16384 * 4));
+    CKE(cudaFuncSetAttribute(k_packed_exps<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             16384 * 4));
+  }
+  const dim3 slices(d.Q < 152 * 8 ? d.Q : 152 * 8), by_rows((unsigned)(nb < 152 * 8 ? nb : 152 * 8));
+  for (int pass = 0; pass < 2; ++pass) {
+    if (tri && d.Q >= kPackedFewSlices)
+      (pass ? k_packed_exps<false> : k_packed_exps<true>)<<<slices, 256, smem, s>>>(B, d.Q, d.N, out,
+                                                                                   rm, dm, k);
+    else
+      (tri ? (pass ? k_row_exps<true, false> : k_row_exps<true, true>)
+           : (pass ? k_row_exps<false, false> : k_row_exps<false, true>))<<<by_rows, 256, 0, s>>>(
+          B, rows, d.N, out, rm, dm, k);
+    count_launch(1);
+    CKE(cudaGetLastError());
+    if (pass == 0) CKE(launch_scales(rm, dm, d.N, k, s));
+  }
+  return cudaSuccess;
+}
+
+cudaError_t digit_hc(const Dims& d, const double* h, const double* C, bool prepared, char* ws,
+                     const Layout& L, ZeroJob zero, cudaStream_t s) {
   const int N = d.N;
+  const KScale k = kscale_at(ws + (prepared ? L.sB : L.sH), N);
+  if (!prepared) {  // no B in this workspace: the scales that h shows
+    int *rm = (int*)(ws + L.eC64), *dm = (int*)(ws + L.exm);
+    CKE(cudaMemsetAsync(ws + L.eC64, 0, L.exend - L.eC64, s));
+    k_row_exps<false, true><<<(N + 7) / 8 < 152 * 8 ? (N + 7) / 8 : 152 * 8, 256, 0, s>>>(
+        h, N, N, nullptr, rm, dm, k);
+    count_launch(1);
+    CKE(cudaGetLastError());
+    CKE(launch_scales(rm, dm, N, k, s));
+  }
   // exponents of C's columns (the operand planes, and lambda's rows) and of h's rows
   if (N <= kFuseK) {
     zero.add(ws + L.exq, L.exend - L.exq);
-    CKE(launch_exps_planes(C, N, N, N, d.A, (int*)(ws + L.eC64), ws + L.Cimg, h, N, N,
+    CKE(launch_exps_planes(C, N, N, N, d.A, (int*)(ws + L.eC64), k, 0, ws + L.Cimg, h, N, N,
                            (int*)(ws + L.eH64), zero, true, s));
   } else {
     CKE(cudaMemsetAsync(ws + L.eC64, 0, L.exend - L.eC64, s));
     if (zero.flag) CKE(cudaMemsetAsync(zero.flag, 0, sizeof(int), s));
     for (int i = 0; i < 4; ++i)
       if (zero.n[i] > 0) CKE(cudaMemsetAsync(zero.p[i], 0, (size_t)zero.n[i] * 8, s));
-    const ExpJob jobs[2] = {{C, N, N, N, 1, (int*)(ws + L.eC64)},
-                            {h, N, N, N, 0, (int*)(ws + L.eH64)}};
+    const ExpJob jobs[2] = {{C, N, N, N, 1, (int*)(ws + L.eC64), k, 0},
+                            {h, N, N, N, 0, (int*)(ws + L.eH64), k, 0}};
     CKE(launch_exps(jobs, 2, s));
-    CKE(launch_planes(C, N, 1, N, d.A, (const int*)(ws + L.eC64), ws + L.Cimg, s));
+    CKE(launch_planes(C, N, 1, N, d.A, (const int*)(ws + L.eC64), k, 0, ws + L.Cimg, s));
   }
   DigitArgs a = digit_args(ws, L);
   a.A = h; a.sAm = N; a.sAk = 1; a.M = N; a.Mb = N; a.Kin = N;
   a.eA = (const int*)(ws + L.eH64);
+  a.ks = k.kp; a.ks_on = k.info;
   a.Bimg = (const __half*)(ws + L.Cimg); a.eB = (const int*)(ws + L.eC64);
   a.N = d.A;
   a.C = (double*)(ws + L.hC); a.sCm = d.A;
@@ -1313,6 +1569,7 @@ int digit_block(const Dims& d, const double* Bblk, int p0, int np, char* ws, con
     if ((x) != cudaSuccess) return DONOF_ERR_CUDA; \
   } while (0)
   const int N = d.N, A = d.A;
+  const KScale k = kscale_at(ws + L.sB, N);
   double* X = (double*)(ws + L.X64);
   double* b = (double*)(ws + L.b64);
   int* exq = (int*)(ws + L.exq);
@@ -1323,10 +1580,11 @@ int digit_block(const Dims& d, const double* Bblk, int p0, int np, char* ws, con
     a.A = Bblk; a.sAb = (long long)N * N; a.sAm = N; a.sAk = 1;
     a.M = np * N; a.Mb = N; a.Kin = N;
     a.eA = (const int*)(ws + L.eRow) + (size_t)p0 * N;
+    a.ks = k.kp; a.ks_on = k.info;
     a.Bimg = (const __half*)(ws + L.Cimg); a.eB = (const int*)(ws + L.eC64);
     a.N = A;
     a.C = X; a.sCb = (long long)N * A; a.sCm = A;
-    a.exq = exq; a.exq_ld = A; a.exm = exm;
+    a.exq = exq; a.exq_ld = A; a.exm = exm; a.row_s = k.kp;
     CKI(launch_digit_gemm(a, N, s));
   }
   prof_end(DONOF_PHASE_HALF_TRANSFORM, s);
@@ -1336,6 +1594,7 @@ int digit_block(const Dims& d, const double* Bblk, int p0, int np, char* ws, con
     a.A = X; a.sAb = (long long)N * A; a.sAm = 1; a.sAk = A;
     a.M = np * A; a.Mb = A; a.Kin = N;
     a.eA = exq;
+    a.ks = k.kp; a.ks_on = k.info;
     a.Bimg = (const __half*)(ws + L.Cimg); a.eB = (const int*)(ws + L.eC64);
     a.N = A;
     a.C = b; a.sCb = (long long)A * A; a.sCm = A;
@@ -1384,25 +1643,28 @@ int digit_block(const Dims& d, const double* Bblk, int p0, int np, char* ws, con
   return DONOF_OK;
 }
 
-cudaError_t digit_lambda(const Dims& d, const double* C, char* ws, const Layout& L, double* lam,
-                         cudaStream_t s) {
+cudaError_t digit_lambda(const Dims& d, const double* C, bool prepared, char* ws, const Layout& L,
+                         double* lam, cudaStream_t s) {
   const int N = d.N, A = d.A;
+  const KScale k = kscale_at(ws + (prepared ? L.sB : L.sH), N);
   const double* G = (const double*)(ws + L.G);
   int* eG = (int*)(ws + L.eG64);
   // C's planes are done with
   if (N <= kFuseK) {
     ZeroJob zero{};
     zero.add(lam, (size_t)N * N * 8);
-    CKE(launch_exps_planes(G, A, N, A, A, eG, ws + L.Cimg, nullptr, 0, 0, nullptr, zero, false, s));
+    CKE(launch_exps_planes(G, A, N, A, A, eG, k, 1, ws + L.Cimg, nullptr, 0, 0, nullptr, zero, false,
+                           s));
   } else {
     CKE(cudaMemsetAsync(lam, 0, (size_t)N * N * 8, s));
-    const ExpJob jobs[1] = {{G, A, N, A, 1, eG}};
+    const ExpJob jobs[1] = {{G, A, N, A, 1, eG, k, 1}};
     CKE(launch_exps(jobs, 1, s));
-    CKE(launch_planes(G, A, 1, N, A, eG, ws + L.Cimg, s));
+    CKE(launch_planes(G, A, 1, N, A, eG, k, 1, ws + L.Cimg, s));
   }
   DigitArgs a = digit_args(ws, L);
   a.A = C; a.sAm = 1; a.sAk = N; a.M = N; a.Mb = N; a.Kin = N;
   a.eA = (const int*)(ws + L.eC64);
+  a.ks = k.kn; a.ks_on = k.info;  // C's side of the scales
   a.Bimg = (const __half*)(ws + L.Cimg); a.eB = eG;
   a.N = A;
   a.C = lam; a.sCm = N;
