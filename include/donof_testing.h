@@ -12,6 +12,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include "donof.h"
+
 #ifdef __cplusplus
 extern "C" {
 #endif
@@ -49,6 +51,10 @@ int donof_testing_tc_gemm_il8(const uint16_t* A_hi, const uint16_t* A_lo, const 
 int donof_testing_tc_gemm_ex(const uint16_t* A_hi, const uint16_t* A_lo, const uint16_t* B_hi,
                              const uint16_t* B_lo, float* D, int32_t M, int32_t N, int32_t K,
                              int32_t layout, int32_t pair, void* stream);
+
+/* *digits (host): 1 where the contractions of a DONOF_FP64 build of `prob` are digit products, 0
+ * where they run on the FP64 pipe. */
+int donof_testing_fp64_digits(const donof_problem* prob, int32_t* digits);
 
 /* C = A B in double by exact digit products on the tensor cores (the FP64 path's contraction):
  * A(m, k) at A[m sAm + k sAk] with sAm = 1 or sAk = 1, B(k, n) at B[k ldb + n], C(m, n) at

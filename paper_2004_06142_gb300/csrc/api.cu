@@ -803,3 +803,13 @@ extern "C" const char* donof_status_string(int status) {
     default: return "unknown status";
   }
 }
+
+#include "../../include/donof_testing.h"
+
+extern "C" int donof_testing_fp64_digits(const donof_problem* prob, int32_t* digits) {
+  const int rc = check_problem(prob);
+  if (rc != DONOF_OK) return rc;
+  if (!digits || prob->precision != DONOF_FP64) return DONOF_ERR_INVALID_ARG;
+  *digits = make_dims(prob).digit;
+  return DONOF_OK;
+}
