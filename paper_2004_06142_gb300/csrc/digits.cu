@@ -920,10 +920,13 @@ __global__ void __launch_bounds__(256) k_digit_planes(const double* __restrict__
 }
 
 // The same with the exponents found on the way, for K <= kFuseK: a CTA per 32 columns passes over
-// them twice (the second time from L1 or L2), so that a short product needs one launch less;
+// them twice (the second time from L1 or L2), so that a short product needs one launch less, and the
+// call no memsets; but few CTAs, each with all of K, take longer the larger K is (a whole build with
+// separate launches / so: nbf 24 99 / 90 us, 100 134 / 123, 300 166 / 165, 500 253 / 263, 640 233 /
+// 248, 1200 472 / 507);
 // the CTAs from col_ctas on find the rows' exponents of a second matrix (R, rows of `rows_k`
 // elements), a warp per row, and those behind them clear `zero`.
-constexpr int kFuseK = 640;
+constexpr int kFuseK = 320;
 __global__ void __launch_bounds__(256) k_exps_planes(const double* __restrict__ S, long long ld,
                                                      int K, int ncols, int N, uint32_t k64,
                                                      int* ex, KScale ksc, int minus, __half* img,
