@@ -235,21 +235,24 @@ int donof_orbital_update(int32_t nbf, const double* lam, const double* Fdiag, co
  *   w[n]:   device, eigenvalues in ascending order.
  * 1 <= n <= 4096.  Workspace: donof_eigh_workspace_size(n) bytes of device memory, 256-byte
  * aligned, owned by the caller (one call at a time per workspace).  Method: Householder
- * reduction to tridiagonal T in one cooperative launch (one CTA per SM); T split where an
+ * reduction to tridiagonal T, for n <= 128 in one cluster of up to 16 CTAs (where the device takes
+ * it), else in one cooperative launch (one CTA per SM); T split where an
  * off-diagonal element is at most 16 n eps ||T||_inf; eigenvalues by bisection on Sturm
  * counts; eigenvectors of T from twisted factorisations, and by inverse iteration with
  * block orthonormalisation for eigenvalues of one block closer than 1e-5 ||T||_inf (every
  * member's own inverse iteration; clusters of more than 32 members in panels on the GEMM
- * kernel); V = Q Z in blocks of 64 reflectors.  The call waits once for `stream` (after the
- * eigenvalues, to read the clusters' layout on the host), so it cannot be captured into a
+ * kernel); V = Q Z in blocks of 64 reflectors, as exact digit products on the tensor cores.  The
+ * call waits once for `stream` (after the eigenvalues, to read the clusters' layout on the host), so it cannot be captured into a
  * CUDA graph; donof_orbital_update and donof_optimize inherit that wait.  Each eigenvalue is
  * within a small multiple of n eps ||A|| of the exact one and each eigenvector within that
  * over its gap; columns of V are orthonormal to about n eps ||A|| / (smallest gap outside the
  * clusters).
  * Returns DONOF_ERR_INVALID_ARG (n out of range, NULL pointer), DONOF_ERR_WORKSPACE, or
  * DONOF_ERR_CUDA (a failed launch, also when the cooperative launch cannot make its grid
- * co-resident).  Device-side outcomes (A not finite; a grid-barrier wait that ran out after
- * 2 s, which leaves NaN eigenvalues) are read with donof_eigh_read_status, which waits for
+ * co-resident).  Device-side outcomes (A not finite; a wait that ran out after 2 s: of the
+ * cooperative launch's grid barrier, which leaves NaN eigenvalues, or of a digit product, which leaves
+ * V unfinished; the cluster form's hardware barrier has no limit of its own) are read with
+ * donof_eigh_read_status, which waits for
  * `stream` and writes DONOF_OK, DONOF_ERR_NONFINITE or DONOF_ERR_TIMEOUT to *status. */
 int donof_eigh_workspace_size(int32_t n, size_t* bytes);
 int donof_eigh(int32_t n, const double* A, double* V, double* w, void* workspace,

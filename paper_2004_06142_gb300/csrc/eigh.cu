@@ -618,8 +618,8 @@ __device__ __forceinline__ int dbl_biased_exp(double x) { return (__double2hiint
 __device__ __forceinline__ int dbl_sign(double x) { return (int)((unsigned)__double2hiint(x) >> 31); }
 
 // One CTA.  ||T||_inf and the scale ts; the split off-diagonal (es, es^2) and the diagonal
-// scaled by ts (double and float copies); the blocks (bstart/bend of every row, found by one
-// thread from integer flags); each block's Gershgorin interval (at its first row, one warp
+// scaled by ts (double and float copies); the blocks (bstart/bend of every row, from a bit mask of
+// the rows that end one); each block's Gershgorin interval (at its first row, one warp
 // per block); the twisted factorisations' pivot floor.
 __global__ void __launch_bounds__(256) k_tri_prep(int N, const double* __restrict__ d,
                                                   const double* __restrict__ e, EighHdr* h,
