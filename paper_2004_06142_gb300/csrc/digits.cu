@@ -1236,8 +1236,8 @@ cudaError_t launch_exps_planes(const double* S, long long ld, int K, int ncols, 
 // less to do once the last stage is in.  Clocks measured per stage, per unit and (code not yet in the
 // instruction caches) per launch, of tiles of 16, 32, 48 and 64.  With the images' width throughout:
 // 120^3 27 us, 500 x 80 x 500 43, 640^3 65, 1200^3 194; by this rule 21, 35, 52, 194.
-// (Measured before the wide tiles' registers: their stages, now about 2850 and 3500 clocks, would
-// change the choice in 9 of 1710 products tried, between near ties.)
+// (Measured before the wide tiles' registers, which make their stages a tenth shorter; that changes
+// the choice in 9 of 1710 products tried, near ties.)
 int tile_columns(int N, int imgNT, long long mtiles, int splits, int nstages) {
   constexpr int kStage[4] = {2400, 2800, 3150, 3850}, kUnit[4] = {3500, 6000, 10000, 13000},
                 kCold[4] = {13000, 14000, 24000, 30000};
