@@ -751,10 +751,10 @@ __global__ void __launch_bounds__(256) k_exps(ExpJobs jobs) {
 // and results are those of unscaled products.
 constexpr int kEvenSpan = 3;
 constexpr int kScaleMax = 1000;  // (the shifts stay below 4096)
-// rm, dm: largest exponents of the rows and of the diagonal elements.  Leaves in k: info = {whether
+// rm, dm: largest exponents of the rows and of the diagonal elements, `copies` of each, the first of
+// which takes the others' maxima.  Leaves in k: info = {whether
 // any s is not zero, the largest}; s >= 0; kp and kn, s 2^20 and -s 2^20, padded with zeros.
-__global__ void __launch_bounds__(1024) k_scales(const int* __restrict__ rm,
-                                                 const int* __restrict__ dm, int N, int* info,
+__global__ void __launch_bounds__(1024) k_scales(int* rm, int* dm, int copies, int N, int* info,
                                                  uint32_t* kp, uint32_t* kn) {
   __shared__ int red[32];
   auto all_max = [&](int v) {
@@ -766,8 +766,17 @@ __global__ void __launch_bounds__(1024) k_scales(const int* __restrict__ rm,
     return __reduce_max_sync(0xffffffffu, v);
   };
   int R = 0;
-  for (int i = threadIdx.x; i < N; i += 1024)
-    if (rm[i] < kNanMark) R = max(R, rm[i]);
+  for (int i = threadIdx.x; i < N; i += 1024) {  // (a thread's own i throughout)
+    int m = 0, e = 0;
+#pragma unroll 4
+    for (int c = 0; c < copies; ++c) {
+      m = max(m, rm[(size_t)c * N + i]);
+      e = max(e, dm[(size_t)c * N + i]);
+    }
+    rm[i] = m;
+    dm[i] = e;
+    if (m < kNanMark) R = max(R, m);
+  }
   R = all_max(R);
   int least = -(1 << 20), most = -(1 << 20);  // of -s and s
   auto raw = [&](int i) { return max(dm[i], 2 * rm[i] - R) >> 1; };
@@ -793,14 +802,20 @@ __global__ void __launch_bounds__(1024) k_scales(const int* __restrict__ rm,
 
 // Rows of N elements (row r: AO index r mod N) of a B of whole rows, or of h: a warp per row.  FIRST:
 // the largest exponents of the rows (into out, unless null), of the AO indices' rows and of their
-// diagonal elements (atomic maxima into zeroed words).  The second pass: those of the rows scaled by
+// diagonal elements (atomic maxima into zeroed words, `copies` of them, which k_scales puts together:
+// with one copy the first rows of all CTAs queued for the same few lines, 140 us instead of 95 for
+// 4000 slices of 97).  The second pass: those of the rows scaled by
 // 2^-s of the column, where any s is not zero.  TRI: rows of packed lower triangles, the part above
 // the diagonal gathered.  Bound by memory: 2000 slices of 700 1.2 ms a pass.
 template <bool TRI, bool FIRST>
 __global__ void __launch_bounds__(256) k_row_exps(const double* __restrict__ B, long long rows, int N,
-                                                  int* out, int* rm, int* dm, KScale k) {
+                                                  int* out, int* rm, int* dm, int copies, KScale k) {
   const int z = chain_begin();
   if (!FIRST && !k.info[z]) return;
+  if (FIRST) {
+    rm += (size_t)(blockIdx.x % copies) * N;
+    dm += (size_t)(blockIdx.x % copies) * N;
+  }
   const int tx = threadIdx.x % 32;
   const long long npk = (long long)N * (N + 1) / 2;
   for (long long r = blockIdx.x * 8 + threadIdx.x / 32 + z; r < rows; r += (long long)gridDim.x * 8) {
@@ -829,14 +844,21 @@ __global__ void __launch_bounds__(256) k_row_exps(const double* __restrict__ B, 
 }
 
 // The rows of symmetric slices stored as packed lower triangles, the passes of k_row_exps: one CTA
-// per slice, the slice's maxima in shared memory.
-constexpr int kPackedFewSlices = 1000;  // (500 slices of 700: 330 us by rows, 630 by slices; 2000: 1300, 1250)
+// per slice, the slice's maxima in shared memory, and its diagonal's (FIRST).
+// (A wave of slices takes its CTAs' time however few they are: 1500 functions 2.1 ms for 500 slices as
+// for 1000, by rows 1.6 and 3.2; 700 functions 0.51 and 0.53, by rows 0.30 and 0.6.)
+constexpr int kPackedFewSlices = 700;
 template <bool FIRST>
 __global__ void __launch_bounds__(256) k_packed_exps(const double* __restrict__ Bp, int Q, int N,
-                                                     int* out, int* rm, int* dm, KScale k) {
+                                                     int* out, int* rm, int* dm, int copies,
+                                                     KScale k) {
   const int z = chain_begin(), bx = (int)blockIdx.x + z;
   extern __shared__ int ex[];
   if (!FIRST && !k.info[z]) return;
+  if (FIRST) {
+    rm += (size_t)(bx % copies) * N;
+    dm += (size_t)(bx % copies) * N;
+  }
   const long long npk = (long long)N * (N + 1) / 2;
   for (int P = bx; P < Q; P += gridDim.x) {
     for (int i = threadIdx.x; i < N; i += 256) ex[i] = 0;
@@ -859,17 +881,18 @@ __global__ void __launch_bounds__(256) k_packed_exps(const double* __restrict__ 
       m = __reduce_max_sync(0xffffffffu, m);
       if (threadIdx.x % 32 == 0) {
         atomicMax(ex + mu, m);
-        if (FIRST) {
-          const int e = exp_of(__ldg(row + mu));
-          if (e < kNanMark && e > *(volatile int*)(dm + mu)) atomicMax(dm + mu, e);
-        }
+        if (FIRST) ex[N + mu] = exp_of(__ldg(row + mu));
       }
     }
     __syncthreads();
     for (int i = threadIdx.x; i < N; i += 256) {
       const int e = FIRST && ex[i] == 2047 ? kNanMark : ex[i];
       out[(size_t)P * N + i] = e;
-      if (FIRST && e > *(volatile int*)(rm + i)) atomicMax(rm + i, e);
+      if (FIRST) {
+        const int ed = ex[N + i];
+        if (e > *(volatile int*)(rm + i)) atomicMax(rm + i, e);
+        if (ed < kNanMark && ed > *(volatile int*)(dm + i)) atomicMax(dm + i, ed);
+      }
     }
     __syncthreads();
   }
@@ -1490,8 +1513,8 @@ DigitArgs digit_args(char* ws, const Layout& L) {
 
 namespace {
 // Scales of the AO indices from the exponents that the first pass left.
-cudaError_t launch_scales(const int* rm, const int* dm, int N, const KScale& k, cudaStream_t s) {
-  k_scales<<<1, 1024, 0, s>>>(rm, dm, N, (int*)k.info, (uint32_t*)k.kp, (uint32_t*)k.kn);
+cudaError_t launch_scales(int* rm, int* dm, int copies, int N, const KScale& k, cudaStream_t s) {
+  k_scales<<<1, 1024, 0, s>>>(rm, dm, copies, N, (int*)k.info, (uint32_t*)k.kp, (uint32_t*)k.kn);
   count_launch(1);
   return cudaGetLastError();
 }
@@ -1501,29 +1524,31 @@ cudaError_t digit_prepare_B(const Dims& d, const double* B, char* ws, const Layo
                             cudaStream_t s) {
   int* out = (int*)(ws + L.eRow);
   const KScale k = kscale_at(ws + L.sB, d.N);
-  int *rm = (int*)(ws + L.eC64), *dm = (int*)(ws + L.exm);  // (free between builds)
-  CKE(cudaMemsetAsync(ws + L.eC64, 0, L.exend - L.eC64, s));
+  // (X's space, free between builds, holds at least 8 N pb A bytes)
+  const int copies = (long long)d.pb * d.A < 16 ? d.pb * d.A : 16;
+  int *rm = (int*)(ws + L.X64), *dm = rm + (size_t)copies * d.N;
+  CKE(cudaMemsetAsync(rm, 0, (size_t)2 * copies * d.N * 4, s));
   const int tri = d.layout == DONOF_B_PACKED;
   const long long rows = (long long)d.Q * d.N, nb = (rows + 7) / 8;
-  const size_t smem = (size_t)d.N * 4;
+  const size_t smem = (size_t)d.N * 8;
   if (tri && smem > 47 * 1024) {  // (one limit for all sizes)
     CKE(cudaFuncSetAttribute(k_packed_exps<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             16384 * 4));
+                             16384 * 8));
     CKE(cudaFuncSetAttribute(k_packed_exps<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             16384 * 4));
+                             16384 * 8));
   }
   const dim3 slices(d.Q < 152 * 8 ? d.Q : 152 * 8), by_rows((unsigned)(nb < 152 * 8 ? nb : 152 * 8));
   for (int pass = 0; pass < 2; ++pass) {
     if (tri && d.Q >= kPackedFewSlices)
-      (pass ? k_packed_exps<false> : k_packed_exps<true>)<<<slices, 256, smem, s>>>(B, d.Q, d.N, out,
-                                                                                   rm, dm, k);
+      (pass ? k_packed_exps<false> : k_packed_exps<true>)<<<slices, 256, smem, s>>>(
+          B, d.Q, d.N, out, rm, dm, copies, k);
     else
       (tri ? (pass ? k_row_exps<true, false> : k_row_exps<true, true>)
            : (pass ? k_row_exps<false, false> : k_row_exps<false, true>))<<<by_rows, 256, 0, s>>>(
-          B, rows, d.N, out, rm, dm, k);
+          B, rows, d.N, out, rm, dm, copies, k);
     count_launch(1);
     CKE(cudaGetLastError());
-    if (pass == 0) CKE(launch_scales(rm, dm, d.N, k, s));
+    if (pass == 0) CKE(launch_scales(rm, dm, copies, d.N, k, s));
   }
   return cudaSuccess;
 }
@@ -1536,10 +1561,10 @@ cudaError_t digit_hc(const Dims& d, const double* h, const double* C, bool prepa
     int *rm = (int*)(ws + L.eC64), *dm = (int*)(ws + L.exm);
     CKE(cudaMemsetAsync(ws + L.eC64, 0, L.exend - L.eC64, s));
     k_row_exps<false, true><<<(N + 7) / 8 < 152 * 8 ? (N + 7) / 8 : 152 * 8, 256, 0, s>>>(
-        h, N, N, nullptr, rm, dm, k);
+        h, N, N, nullptr, rm, dm, 1, k);
     count_launch(1);
     CKE(cudaGetLastError());
-    CKE(launch_scales(rm, dm, N, k, s));
+    CKE(launch_scales(rm, dm, 1, N, k, s));
   }
   // exponents of C's columns (the operand planes, and lambda's rows) and of h's rows
   if (N <= kFuseK) {

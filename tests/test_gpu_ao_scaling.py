@@ -54,8 +54,8 @@ def _check(out, ref, w, keys=("J", "K", "lam", "dE_dgamma", "dE_dC")):
 # by rows and a CTA each; one block of slices and several
 @pytest.mark.parametrize("nbf,naux,npair,ncwo,packed,blocks", [
     (24, 96, 5, 1, False, 1), (24, 96, 5, 1, True, 3), (97, 60, 4, 3, True, 1),
-    (120, 300, 8, 4, False, 4), (161, 110, 3, 2, True, 1), (320, 12, 6, 3, False, 1),
-    (321, 12, 6, 3, True, 1), (700, 12, 6, 3, False, 1)])
+    (120, 300, 8, 4, False, 4), (161, 110, 3, 2, True, 1), (41, 703, 4, 2, True, 1),
+    (320, 12, 6, 3, False, 1), (321, 12, 6, 3, True, 1), (700, 12, 6, 3, False, 1)])
 @pytest.mark.parametrize("spread", [2, 8, 20])
 @pytest.mark.parametrize("order", ["random", "sorted"])
 def test_errors_do_not_depend_on_the_norms(nbf, naux, npair, ncwo, packed, blocks, spread, order):
